@@ -386,7 +386,7 @@ int fredopt_kernel_arch(int device, int* fwd_binary, int* bwd_binary, int* ptx_v
 
 /* Failure-detection check of the bounded device-side wait (no GPU fault
  * involved).  Every device-side wait of the library (the mbarrier that the
- * bulk copies of x and of the CSC windows complete) polls at most
+ * bulk copy of x completes) polls at most
  * FREDOPT_WAIT_POLLS times; when it gives up the kernel sets the handle's device error
  * word and returns, and the next synchronising call reports
  * FREDOPT_ERR_TIMEOUT and clears the word.  This call runs that wait alone in
@@ -511,11 +511,11 @@ typedef struct fredopt_ticket_info {
 
 typedef struct fredopt_server* fredopt_server_t;
 
-/* Estimate of the device memory one plan needs while it loads and runs: the
- * peak of the load (including the CSC build's scratch of one record per
- * nonzero: 16 bytes with FP32 values, 8 with 16-bit) and the resident CSR,
- * CSC, based row offsets with their block headers, vectors and tables.  The overflow table of wide 128-element
- * blocks (rows spanning 65536 or more) is counted for one such block per
+/* Estimate of the device memory one plan needs while it loads and runs: an
+ * upper bound of the load's peak (CSR and CSC with 32-bit indices and 16 bytes
+ * more per nonzero with FP32 values, 8 with 16-bit) and the resident CSR,
+ * CSC, based row offsets with their block headers, vectors and tables.  The
+ * overflow table of wide 128-element blocks (rows spanning 65536 or more) is counted for one such block per
  * column boundary plus one in 16 blocks; for plans with sparser rows the
  * estimate can be low, and a load that then does not fit fails with
  * FREDOPT_ERR_OOM without disturbing the plans in flight.  The server admits

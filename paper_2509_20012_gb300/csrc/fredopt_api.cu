@@ -45,6 +45,8 @@ struct DBuf {
     return e;
   }
   cudaError_t ensure(size_t count) { return (p && n >= count) ? cudaSuccess : alloc(count); }
+  // a reload keeps a buffer that is large enough and at most twice as large
+  cudaError_t fit(size_t count) { return (p && n >= count && n / 2 <= count) ? cudaSuccess : alloc(count); }
 };
 
 struct Timer {
@@ -105,14 +107,10 @@ struct fredopt_ctx {
   DBuf<int32_t> col_chunk, warp_chunk;
   int64_t n_chunks = 0;
   bool hint_fwd = true, hint_bwd = true;
-  std::vector<int64_t> h_voxel;  // device row -> voxel (host copy, when perm)
-  std::vector<int64_t> h_rp;     // row_ptr in device order (host copy, for the schedules)
-  std::vector<int64_t> h_cptr;   // chunk_ptr (host copy)
   int64_t row_cost = 0, chunk_cost = 0;  // warp-partition weights in use
-  std::vector<uint32_t> h_mask;  // per streamed row
   DBuf<int64_t> con_rows;        // streamed rows with a structure bit, ascending
-  std::vector<int64_t> h_con_rows;
-  int64_t n_con_rows = 0;
+  int64_t n_con_rows = 0, n_con_ne = 0;  // all of them; those with nonzeros (first in the list)
+  uint64_t empty_bits[32] = {0};  // streamed rows without nonzeros, per structure bit
   DBuf<float2> ucoef;            // coefficients of fredopt_backward (kept apart from gam)
 
   // problem
@@ -227,83 +225,6 @@ cudaError_t copy_out(fredopt_t h, void* dst, const void* src, size_t bytes, uint
   if (bytes == 0 || !dst) return cudaSuccess;
   return cudaMemcpyAsync(dst, src, bytes, dev_ptr(flags) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                          h->stream);
-}
-
-// Balanced contiguous split of rows [0, n_rows) into `parts` ranges by
-// cost(row) = nnz(row) + row_cost.  Returns parts+1 boundaries.
-std::vector<int64_t> partition_rows(const std::vector<int64_t>& rp, int64_t n_rows, int parts,
-                                    int64_t row_cost) {
-  std::vector<int64_t> b(parts + 1, n_rows);
-  b[0] = 0;
-  const double total = (double)(rp[n_rows] - rp[0]) + (double)row_cost * (double)n_rows;
-  int64_t lo = 0;
-  for (int k = 1; k < parts; ++k) {
-    const double target = total * k / parts;
-    int64_t a = lo, z = n_rows;  // first r with prefix(r) >= target
-    while (a < z) {
-      const int64_t m = (a + z) / 2;
-      const double pre = (double)(rp[m] - rp[0]) + (double)row_cost * (double)m;
-      if (pre < target) a = m + 1;
-      else z = m;
-    }
-    b[k] = a;
-    lo = a;
-  }
-  return b;
-}
-
-// Row ranges [r0, r1) for `parts` warps over the union of the row ranges
-// `ranges` (each split in nnz-balanced contiguous pieces; warps are shared
-// among ranges in proportion to their cost).  Returns 2*parts values.
-std::vector<int64_t> partition_pairs(const std::vector<int64_t>& rp,
-                                     const std::vector<std::pair<int64_t, int64_t>>& ranges, int parts,
-                                     int64_t row_cost) {
-  std::vector<int64_t> out(2 * (size_t)parts, 0);
-  std::vector<size_t> live;
-  double total = 0.0;
-  std::vector<double> cost(ranges.size(), 0.0);
-  for (size_t k = 0; k < ranges.size(); ++k) {
-    const int64_t a = ranges[k].first, z = ranges[k].second;
-    if (z <= a) continue;
-    cost[k] = (double)(rp[z] - rp[a]) + (double)row_cost * (double)(z - a);
-    total += cost[k];
-    live.push_back(k);
-  }
-  int used = 0;
-  for (size_t i = 0; i < live.size(); ++i) {
-    const size_t k = live[i];
-    const int later = (int)(live.size() - 1 - i);
-    int w;
-    if (later == 0) {
-      w = parts - used;
-    } else {
-      w = (int)std::llround(parts * (total > 0 ? cost[k] / total : 0.0));
-      w = std::max(1, std::min(w, parts - used - later));
-    }
-    if (w <= 0) break;
-    const int64_t a = ranges[k].first, z = ranges[k].second;
-    const double tot = cost[k];
-    int64_t lo = a;
-    for (int j = 0; j < w; ++j) {
-      int64_t x = z;
-      if (j + 1 < w) {
-        const double target = tot * (j + 1) / w;
-        int64_t y = z;
-        x = lo;
-        while (x < y) {  // first row m with prefix(m) >= target
-          const int64_t m = (x + y) / 2;
-          const double pre = (double)(rp[m] - rp[a]) + (double)row_cost * (double)(m - a);
-          if (pre < target) x = m + 1;
-          else y = m;
-        }
-      }
-      out[2 * (used + j)] = lo;
-      out[2 * (used + j) + 1] = x;
-      lo = x;
-    }
-    used += w;
-  }
-  return out;
 }
 
 template <typename T>
@@ -468,9 +389,11 @@ ConArgs con_args(fredopt_t h) {
 int build_sweep(fredopt_t h, int m) {
   if (h->sweep_m == m) return FREDOPT_OK;
   cudaStream_t s = h->stream;
-  std::vector<int64_t> C;
-  for (int64_t r = 0; r < h->n_hot_ne; ++r)
-    if (h->h_mask[r] != 0) C.push_back(r);
+  std::vector<int64_t> C(h->n_con_ne);  // structure rows with nonzeros, ascending
+  if (!C.empty()) {
+    CK(cudaMemcpyAsync(C.data(), h->con_rows.p, C.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+  }
   h->h_sweep_bounds.clear();
   h->sweep_wr_off.clear();
   h->sweep_warps.clear();
@@ -482,17 +405,20 @@ int build_sweep(fredopt_t h, int m) {
     h->h_sweep_bounds.push_back(C.back() + 1);
     h->sweep_nb = nb;
   }
-  std::vector<int64_t> wr;
+  int64_t n_wr = 0;
   for (int t = 0; t < h->sweep_nb; ++t) {
     const int64_t r0 = h->h_sweep_bounds[t], r1 = h->h_sweep_bounds[t + 1];
     const int warps = (int)std::max<int64_t>(1, std::min<int64_t>(h->geo.fwd_warps, r1 - r0));
-    const std::vector<int64_t> p = partition_pairs(h->h_rp, {{r0, r1}}, warps, h->row_cost);
-    h->sweep_wr_off.push_back((int64_t)wr.size() / 2);
+    h->sweep_wr_off.push_back(n_wr);
     h->sweep_warps.push_back(warps);
-    wr.insert(wr.end(), p.begin(), p.end());
+    n_wr += warps;
   }
-  if (wr.empty()) wr.assign(2, 0);
-  CK(upload_vec(h, h->sweep_wr, wr));
+  CK(h->sweep_wr.alloc((size_t)std::max<int64_t>(1, n_wr) * 2));
+  for (int t = 0; t < h->sweep_nb; ++t) {
+    TileArgs q{TileArgs::PAIRS, h->rp.p, h->h_sweep_bounds[t], h->h_sweep_bounds[t + 1], 0, 0, h->sweep_warps[t], 0,
+               h->row_cost, h->sweep_wr.p + 2 * h->sweep_wr_off[t], nullptr};
+    launch_tiles(q, s);
+  }
   const int nbnd = h->sweep_nb + 1;
   std::vector<int64_t> bnd = h->h_sweep_bounds;
   if (bnd.empty()) bnd.assign(1, 0);
@@ -630,93 +556,54 @@ void enqueue_iteration(fredopt_t h) {
   run(h, 3, [&] { launch_colfinish(G, COL_PROJ, cc, s); });
 }
 
-// Tiles for warps that claim them in order (guided self-scheduling): the
-// first W tiles each hold half of a warp's share of rows [0, n) (cost:
-// nonzeros + row_cost per row), the next W a quarter, then an eighth, a
-// sixteenth, a thirty-second, and 2W tiles of a sixty-fourth, so the last
-// tiles to be claimed are short and the warps finish close together.
-// Always kGuidedTilesPerWarp * W tiles (some may be empty), so the tile
-// count, which kernels and captured graphs hold by value, does not depend on
-// row_cost.  Returns 2 * count row bounds.
-constexpr int kGuidedTilesPerWarp = 7;
-std::vector<int64_t> guided_tiles(const std::vector<int64_t>& rp, int64_t n, int W, int64_t row_cost) {
-  const int count = kGuidedTilesPerWarp * W;
-  std::vector<int64_t> out(2 * (size_t)count, n > 0 ? n : 0);
-  if (n <= 0 || W <= 0) return out;
-  auto prefix = [&](int64_t r) { return (double)(rp[r] - rp[0]) + (double)row_cost * (double)r; };
-  const double share = prefix(n) / W;
-  const std::pair<double, int> rounds[] = {{0.5, W}, {0.25, W}, {0.125, W}, {0.0625, W}, {0.03125, W},
-                                           {0.015625, 2 * W}};
-  double target = 0.0;
-  int64_t lo = 0;
-  int k = 0;
-  for (const auto& rd : rounds) {
-    for (int i = 0; i < rd.second; ++i, ++k) {
-      target += rd.first * share;
-      int64_t hi = n;
-      if (k + 1 < count) {
-        int64_t x = lo, y = n;  // first row m with prefix(m) >= target
-        while (x < y) {
-          const int64_t m = (x + y) / 2;
-          if (prefix(m) < target) x = m + 1;
-          else y = m;
-        }
-        hi = x;
-      }
-      out[2 * (size_t)k] = lo;
-      out[2 * (size_t)k + 1] = hi;
-      lo = hi;
-    }
-  }
-  return out;
-}
-
 // Warp partitions.  A segment's sum does not depend on which warp streams it
 // (lanes take elements by their absolute block-aligned position and add them
 // in order), so these weights change the speed, never a result bit.
 int set_fwd_schedule(fredopt_t h, int64_t row_cost) {
-  const std::vector<int64_t> wr = partition_pairs(h->h_rp, {{0, h->n_hot_ne}}, h->geo.fwd_warps, row_cost);
-  const std::vector<int64_t> wa = partition_pairs(
-      h->h_rp, {{0, h->n_hot_ne}, {h->n_hot, h->n_hot + h->n_cold_ne}}, h->geo.fwd_warps, row_cost);
-  CK(cudaMemcpyAsync(h->warp_row_hot.p, wr.data(), wr.size() * sizeof(int64_t), cudaMemcpyHostToDevice, h->stream));
-  CK(cudaMemcpyAsync(h->warp_row_all.p, wa.data(), wa.size() * sizeof(int64_t), cudaMemcpyHostToDevice, h->stream));
-  const std::vector<int64_t> tl = guided_tiles(h->h_rp, h->n_hot_ne, h->geo.fwd_warps, row_cost);
-  if ((size_t)h->tile_row_hot.n < std::max<size_t>(2, tl.size())) CK(h->tile_row_hot.alloc(std::max<size_t>(2, tl.size())));
-  if (!tl.empty())
-    CK(cudaMemcpyAsync(h->tile_row_hot.p, tl.data(), tl.size() * sizeof(int64_t), cudaMemcpyHostToDevice, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
-  h->n_tiles_hot = (int)(tl.size() / 2);
+  const int W = h->geo.fwd_warps;
+  const int64_t *rp = h->rp.p, hot = h->n_hot_ne, cold = h->n_cold_ne;
+  CK(h->warp_row_hot.fit(2 * (size_t)W));
+  CK(h->warp_row_all.fit(2 * (size_t)W));
+  CK(h->tile_row_hot.fit(2 * (size_t)kGuidedTilesPerWarp * W));
+  launch_tiles(TileArgs{TileArgs::PAIRS, rp, 0, hot, 0, 0, W, 0, row_cost, h->warp_row_hot.p, nullptr}, h->stream);
+  // every row: the warps shared between streamed and other rows by their cost
+  const double c0 = (double)h->nnz_hot + (double)row_cost * (double)hot;
+  const double c1 = (double)(h->nnz - h->nnz_hot) + (double)row_cost * (double)cold;
+  int w0 = hot > 0 || cold == 0 ? W : 0;
+  if (hot > 0 && cold > 0) w0 = std::max(1, std::min(W - 1, (int)std::llround(W * (c0 / (c0 + c1)))));
+  launch_tiles(TileArgs{TileArgs::PAIRS, rp, 0, hot, h->n_hot, h->n_hot + cold, w0, W - w0, row_cost,
+                        h->warp_row_all.p, nullptr}, h->stream);
+  launch_tiles(TileArgs{TileArgs::GUIDED_PAIRS, rp, 0, hot, 0, 0, W, 0, row_cost, h->tile_row_hot.p, nullptr},
+               h->stream);
+  CK(cudaGetLastError());
+  h->n_tiles_hot = kGuidedTilesPerWarp * W;
   h->row_cost = row_cost;
   return FREDOPT_OK;
 }
 
 int set_bwd_schedule(fredopt_t h, int64_t chunk_cost) {
-  const std::vector<int64_t> w64 = partition_rows(h->h_cptr, h->n_chunks, h->geo.bwd_warps, chunk_cost);
-  const std::vector<int32_t> w32(w64.begin(), w64.end());
-  CK(cudaMemcpyAsync(h->warp_chunk.p, w32.data(), w32.size() * sizeof(int32_t), cudaMemcpyHostToDevice, h->stream));
+  const int W = h->geo.bwd_warps;
+  const int64_t* cp = h->chunk_ptr.p;
+  CK(h->warp_chunk.fit((size_t)W + 1));
+  CK(h->tile_chunk.fit((size_t)kGuidedTilesPerWarp * W + 1));
+  launch_tiles(TileArgs{TileArgs::BOUNDS32, cp, 0, h->n_chunks, 0, 0, W, 0, chunk_cost, nullptr, h->warp_chunk.p},
+               h->stream);
   // claimed tiles: guided sizes over the chunks (the same rule as the forward rows)
-  const std::vector<int64_t> tl = guided_tiles(h->h_cptr, h->n_chunks, h->geo.bwd_warps, chunk_cost);
-  std::vector<int32_t> tb(tl.size() / 2 + 1, 0);
-  for (size_t k = 0; k < tl.size() / 2; ++k) tb[k] = (int32_t)tl[2 * k];
-  tb.back() = tl.empty() ? 0 : (int32_t)tl.back();
-  if ((size_t)h->tile_chunk.n < tb.size()) CK(h->tile_chunk.alloc(tb.size()));
-  CK(cudaMemcpyAsync(h->tile_chunk.p, tb.data(), tb.size() * sizeof(int32_t), cudaMemcpyHostToDevice, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
-  h->n_tiles_bwd = (int)(tb.size() - 1);
+  launch_tiles(TileArgs{TileArgs::GUIDED32, cp, 0, h->n_chunks, 0, 0, W, 0, chunk_cost, nullptr, h->tile_chunk.p},
+               h->stream);
+  CK(cudaGetLastError());
+  h->n_tiles_bwd = kGuidedTilesPerWarp * W;
   h->chunk_cost = chunk_cost;
   return FREDOPT_OK;
 }
 
 // Objective (Eq. 2 terms) of the streamed rows without nonzeros: their dose
-// and LET-weighted dose are 0 for every w, so each term contributes w*T^2.
+// and LET-weighted dose are 0 for every w, so each term contributes w*T^2 per
+// such row of its structure.
 double f_empty(fredopt_t h) {
   double f = 0.0;
-  for (int64_t r = h->n_hot_ne; r < h->n_hot; ++r) {
-    const uint32_t m = h->h_mask[r];
-    if (!m) continue;
-    for (int i = 0; i < h->tab.n_obj; ++i)
-      if ((m >> h->tab.obj[i].bit) & 1u) f += h->tab.obj[i].weight * h->tab.obj[i].target * h->tab.obj[i].target;
-  }
+  for (int i = 0; i < h->tab.n_obj; ++i)
+    f += h->tab.obj[i].weight * h->tab.obj[i].target * h->tab.obj[i].target * (double)h->empty_bits[h->tab.obj[i].bit];
   return f;
 }
 
@@ -902,186 +789,138 @@ int fredopt_load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t 
   h->loaded = false;
   h->begun = false;
   h->sweep_m = 0;
-  int rc = FREDOPT_OK;
   cudaStream_t s = h->stream;
   join_in(h);
-
+  const bool host = !dev_ptr(flags);
+  const int vb = value_bytes(fmt);
   // every index / value array is zero padded past its last nonzero
   const int64_t nnz_alloc = ((nnz + 255) & ~255LL) + kPadElems;
 
-  // ---- host inputs: their upload is issued first, so that the copy engine
-  // runs while the host checks row_ptr and orders the rows
+  // ---- row order (and the check of row_ptr), on the device
+  DBuf<int64_t> rp_in, row_blk;
+  DBuf<uint32_t> mask_in;
+  DBuf<RowTotals> tot_rows;
+  const int64_t* rpp = row_ptr;
+  const uint32_t* mp = voxel_mask;
+  if (host) {
+    CK(rp_in.alloc(n_vox + 1));
+    CK(mask_in.alloc(n_vox));
+    CK(cudaMemcpyAsync(rp_in.p, row_ptr, (n_vox + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
+    if (n_vox) CK(cudaMemcpyAsync(mask_in.p, voxel_mask, n_vox * sizeof(uint32_t), cudaMemcpyHostToDevice, s));
+    rpp = rp_in.p;
+    mp = mask_in.p;
+  }
+  CK(row_blk.alloc(row_order_scratch(n_vox)));
+  CK(tot_rows.alloc(1));
+  CK(cudaMemsetAsync(tot_rows.p, 0, sizeof(RowTotals), s));
+  launch_rows_count(rpp, mp, n_vox, nnz, roi, row_blk.p, tot_rows.p, s);
+  CK(cudaGetLastError());
+  RowTotals tot;
+  CK(cudaMemcpyAsync(&tot, tot_rows.p, sizeof(tot), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  if (tot.flags & kRowsBadEnds) return fail(h, FREDOPT_ERR_PATTERN, "row_ptr[0] != 0 or row_ptr[n_vox] != nnz");
+  if (tot.flags & kRowsNotMonotone) return fail(h, FREDOPT_ERR_PATTERN, "row_ptr not monotone");
+  const bool perm = (tot.flags & kRowsPermuted) != 0;
+  const int64_t n_hot_ne = tot.c[0], n_hot = tot.c[0] + tot.c[1], n_cold_ne = tot.c[2], nnz_hot = tot.c[3];
+  const int64_t nh_alloc = ((nnz_hot + 255) & ~255LL) + kPadElems;
+
+  // ---- the previous plan's buffers: kept where the new plan needs at least
+  // half of them (a plan re-planned on the same handle), else all freed first
+  const bool similar = h->Dv.p && h->Dv.n >= (size_t)nnz_alloc * vb && h->Dv.n / 2 <= (size_t)nnz_alloc * vb &&
+                       h->DTv.n >= (size_t)nh_alloc * vb && h->DTv.n / 2 <= (size_t)nh_alloc * vb && h->V >= n_vox &&
+                       h->V / 2 <= n_vox;
+  if (!similar) {
+    h->rp.release(); h->col.release(); h->col16.release(); h->Dv.release(); h->Lv.release();
+    h->voxel.release(); h->mask.release(); h->con_rows.release(); h->cp.release();
+    h->crow.release(); h->crow16.release(); h->chdr.release(); h->DTv.release(); h->LTv.release();
+    h->y64.release(); h->yall.release(); h->fout_a.release(); h->fout_b.release();
+    h->vin_a.release(); h->vin_b.release();
+  }
+  h->covf.release();
+  h->ucoef.release();
+  if (fmt == FREDOPT_FP32) {
+    h->sD.release();
+    h->sL.release();
+  }
+  h->V = n_vox; h->nnz = nnz; h->n = n_spots; h->n_pad = (n_spots + 3) & ~3;
+  h->fmt = fmt; h->roi = roi; h->perm = perm; h->n_hot = n_hot; h->nnz_hot = nnz_hot;
+  h->n_hot_ne = n_hot_ne; h->n_cold_ne = n_cold_ne;
+  h->n_con_ne = tot.c[5]; h->n_con_rows = tot.c[5] + tot.c[6];
+  for (int b = 0; b < 32; ++b) h->empty_bits[b] = tot.empty_bits[b];
+
+  CK(h->rp.fit(n_vox + 1));
+  CK(h->mask.fit(n_hot));
+  CK(h->con_rows.fit(h->n_con_rows));
+  if (perm) CK(h->voxel.fit(n_vox));
+  else h->voxel.release();
+  if (fmt != FREDOPT_FP32) {
+    CK(h->sD.fit(n_vox));
+    CK(h->sL.fit(n_vox));
+  }
+  launch_rows_place(rpp, mp, n_vox, roi, row_blk.p, tot_rows.p, h->rp.p, perm ? h->voxel.p : nullptr, h->mask.p,
+                    h->con_rows.p, fmt ? h->sD.p : nullptr, fmt ? h->sL.p : nullptr, s);
+  CK(cudaGetLastError());
+
+  // ---- index and value storage.  16-bit column indices for the forward
+  // stream (2 bytes less per nonzero, same sums) when x is staged in shared
+  // memory (that bounds n_spots below 65536).  FP32 host arrays whose rows
+  // keep their order in memory are uploaded into place.
+  const bool narrow = !(format & FREDOPT_INDEX32) && n_spots <= 65536 && forward_uses_smem(h->geo_full, h->n_pad);
+  if (narrow) {
+    h->col.release();
+    CK(h->col16.fit(nnz_alloc));
+  } else {
+    h->col16.release();
+    CK(h->col.fit(nnz_alloc));
+  }
+  CK(h->Dv.fit((size_t)nnz_alloc * vb));
+  CK(h->Lv.fit((size_t)nnz_alloc * vb));
+  const int ib = narrow ? 2 : 4;
+  uint8_t* colp8 = narrow ? reinterpret_cast<uint8_t*>(h->col16.p) : reinterpret_cast<uint8_t*>(h->col.p);
+  CK(cudaMemsetAsync(colp8 + nnz * ib, 0, (nnz_alloc - nnz) * ib, s));
+  CK(cudaMemsetAsync(h->Dv.p + nnz * vb, 0, (nnz_alloc - nnz) * vb, s));
+  CK(cudaMemsetAsync(h->Lv.p + nnz * vb, 0, (nnz_alloc - nnz) * vb, s));
   DBuf<int32_t> col_in;
   DBuf<float> D_in, L_in;
   const int32_t* colp = col;
   const float *Dp = D_val, *Lp = L_val;
-  if (!dev_ptr(flags)) {
-    CK(col_in.alloc(nnz_alloc));
-    CK(D_in.alloc(nnz_alloc));
-    CK(L_in.alloc(nnz_alloc));
-    CK(cudaMemsetAsync(col_in.p + nnz, 0, (nnz_alloc - nnz) * sizeof(int32_t), s));
-    CK(cudaMemsetAsync(D_in.p + nnz, 0, (nnz_alloc - nnz) * sizeof(float), s));
-    CK(cudaMemsetAsync(L_in.p + nnz, 0, (nnz_alloc - nnz) * sizeof(float), s));
+  const bool in_place = host && fmt == FREDOPT_FP32 && n_cold_ne == 0;
+  if (host) {
+    CK(col_in.alloc(nnz));
+    float *Dd = reinterpret_cast<float*>(h->Dv.p), *Ld = reinterpret_cast<float*>(h->Lv.p);
+    if (!in_place) {
+      CK(D_in.alloc(nnz));
+      CK(L_in.alloc(nnz));
+      Dd = D_in.p;
+      Ld = L_in.p;
+    }
     if (nnz) {
       CK(cudaMemcpyAsync(col_in.p, col, nnz * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-      CK(cudaMemcpyAsync(D_in.p, D_val, nnz * sizeof(float), cudaMemcpyHostToDevice, s));
-      CK(cudaMemcpyAsync(L_in.p, L_val, nnz * sizeof(float), cudaMemcpyHostToDevice, s));
+      CK(cudaMemcpyAsync(Dd, D_val, nnz * sizeof(float), cudaMemcpyHostToDevice, s));
+      CK(cudaMemcpyAsync(Ld, L_val, nnz * sizeof(float), cudaMemcpyHostToDevice, s));
     }
     colp = col_in.p;
-    Dp = D_in.p;
-    Lp = L_in.p;
+    Dp = Dd;
+    Lp = Ld;
   }
 
-  // ---- row_ptr and the mask on the host (read in place when they are host
-  // memory); row_ptr checked on the host
-  std::vector<int64_t> rp_copy;
-  std::vector<uint32_t> m_copy;
-  const int64_t* rp0 = row_ptr;
-  const uint32_t* m0 = voxel_mask;
-  if (dev_ptr(flags)) {
-    rp_copy.resize(n_vox + 1);
-    m_copy.resize(n_vox);
-    CK(cudaMemcpyAsync(rp_copy.data(), row_ptr, (n_vox + 1) * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    if (n_vox) CK(cudaMemcpyAsync(m_copy.data(), voxel_mask, n_vox * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    rp0 = rp_copy.data();
-    m0 = m_copy.data();
-  }
-  if (rp0[0] != 0 || rp0[n_vox] != nnz) return fail(h, FREDOPT_ERR_PATTERN, "row_ptr[0] != 0 or row_ptr[n_vox] != nnz");
-  for (int64_t i = 0; i < n_vox; ++i)
-    if (rp0[i + 1] < rp0[i]) return fail(h, FREDOPT_ERR_PATTERN, "row_ptr not monotone");
-
-  // ---- device order of rows: streamed rows with nonzeros, streamed rows
-  // without, other rows with nonzeros, other rows without (each ascending);
-  // one pass over row_ptr and the mask assigns the groups
-  std::vector<uint8_t> grp(n_vox);
-  int64_t c0 = 0, c1 = 0, c2 = 0;  // counts in locals: no store-to-load chain between rows
-  for (int64_t i = 0; i < n_vox; ++i) {
-    const int g = ((!roi || m0[i] != 0) ? 0 : 2) + (rp0[i + 1] > rp0[i] ? 0 : 1);
-    grp[i] = (uint8_t)g;
-    c0 += g == 0;
-    c1 += g == 1;
-    c2 += g == 2;
-  }
-  const int64_t n_hot_ne = c0;
-  const int64_t n_hot = c0 + c1;
-  const int64_t n_cold_ne = c2;
-  std::vector<int64_t> order(n_vox);
-  bool perm = false;
-  {
-    int64_t p0 = 0, p1 = c0, p2 = c0 + c1, p3 = c0 + c1 + c2;
-    for (int64_t i = 0; i < n_vox; ++i) {
-      int64_t r;
-      switch (grp[i]) {
-        case 0: r = p0++; break;
-        case 1: r = p1++; break;
-        case 2: r = p2++; break;
-        default: r = p3++; break;
-      }
-      order[r] = i;
-      perm |= r != i;
-    }
-  }
-  std::vector<int64_t> rpd(n_vox + 1);
-  if (perm) {
-    rpd[0] = 0;
-    for (int64_t r = 0; r < n_vox; ++r) rpd[r + 1] = rpd[r] + (rp0[order[r] + 1] - rp0[order[r]]);
-  } else {
-    std::memcpy(rpd.data(), rp0, (n_vox + 1) * sizeof(int64_t));
-  }
-
-  // ---- validate (on the input layout)
-  DBuf<int64_t> rp_in;
-  CK(rp_in.alloc(n_vox + 1));
-  CK(cudaMemcpyAsync(rp_in.p, rp0, (n_vox + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
+  // ---- one pass over the input: validation, storage, FP64-class row moments
+  CK(h->mdd.fit(n_hot)); CK(h->mll.fit(n_hot)); CK(h->mdl.fit(n_hot));
+  CK(cudaMemsetAsync(h->mdd.p, 0, std::max<int64_t>(1, n_hot) * sizeof(double), s));
+  CK(cudaMemsetAsync(h->mll.p, 0, std::max<int64_t>(1, n_hot) * sizeof(double), s));
+  CK(cudaMemsetAsync(h->mdl.p, 0, std::max<int64_t>(1, n_hot) * sizeof(double), s));
   CK(cudaMemsetAsync(h->errw.p, 0, sizeof(int), s));
-  launch_validate(rp_in.p, colp, Dp, Lp, n_vox, n_spots, nnz, h->errw.p, s);
+  LoadRowsArgs la{rpp, h->rp.p, perm ? h->voxel.p : nullptr, n_hot, n_hot_ne, n_cold_ne, n_spots, colp, Dp, Lp, colp8,
+                  h->Dv.p, h->Lv.p, fmt ? h->sD.p : nullptr, fmt ? h->sL.p : nullptr, h->mdd.p, h->mll.p, h->mdl.p,
+                  h->errw.p};
+  launch_load_rows(fmt, narrow, !in_place, la, s);
   CK(cudaGetLastError());
   int verr = 0;
   CK(cudaMemcpyAsync(&verr, h->errw.p, sizeof(int), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   if (verr & 1) return fail(h, FREDOPT_ERR_PATTERN, "column index out of range or not strictly increasing within a row");
   if (verr & 2) return fail(h, FREDOPT_ERR_NONFINITE, "NaN or Inf in D or L");
-
-  // ---- drop the previous plan
-  h->rp.release(); h->col.release(); h->col16.release(); h->Dv.release(); h->Lv.release(); h->sD.release(); h->sL.release();
-  h->voxel.release(); h->mask.release(); h->con_rows.release(); h->ucoef.release(); h->cp.release(); h->crow.release(); h->crow16.release(); h->chdr.release(); h->covf.release(); h->DTv.release(); h->LTv.release();
-
-  // ---- FP32 CSR in device order (zero padded)
-  DBuf<int32_t> col_d;
-  DBuf<float> D_d, L_d;
-  CK(upload_vec(h, h->rp, rpd));
-  if (perm || dev_ptr(flags)) {
-    CK(col_d.alloc(nnz_alloc));
-    CK(D_d.alloc(nnz_alloc));
-    CK(L_d.alloc(nnz_alloc));
-    CK(cudaMemsetAsync(col_d.p + nnz, 0, (nnz_alloc - nnz) * sizeof(int32_t), s));
-    CK(cudaMemsetAsync(D_d.p + nnz, 0, (nnz_alloc - nnz) * sizeof(float), s));
-    CK(cudaMemsetAsync(L_d.p + nnz, 0, (nnz_alloc - nnz) * sizeof(float), s));
-    if (perm) {
-      // device row -> voxel: the gather's source rows, kept for the outputs
-      CK(upload_vec(h, h->voxel, order));
-      launch_gather_rows(rp_in.p, h->voxel.p, h->rp.p, n_vox, colp, Dp, Lp, col_d.p, D_d.p, L_d.p, s);
-      CK(cudaGetLastError());
-      CK(cudaStreamSynchronize(s));
-    } else if (nnz) {
-      CK(cudaMemcpyAsync(col_d.p, col, nnz * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-      CK(cudaMemcpyAsync(D_d.p, D_val, nnz * sizeof(float), cudaMemcpyDeviceToDevice, s));
-      CK(cudaMemcpyAsync(L_d.p, L_val, nnz * sizeof(float), cudaMemcpyDeviceToDevice, s));
-    }
-  } else {
-    std::swap(col_d.p, col_in.p); std::swap(col_d.n, col_in.n);
-    std::swap(D_d.p, D_in.p); std::swap(D_d.n, D_in.n);
-    std::swap(L_d.p, L_in.p); std::swap(L_d.n, L_in.n);
-  }
-  CK(cudaStreamSynchronize(s));
-  col_in.release(); D_in.release(); L_in.release(); rp_in.release();
-  std::swap(h->col.p, col_d.p); std::swap(h->col.n, col_d.n);
-
-  // ---- value storage (quantised with power-of-two row scales, or FP32)
-  if (fmt == FREDOPT_FP32) {
-    h->Dv.p = reinterpret_cast<uint8_t*>(D_d.p); h->Dv.n = D_d.n * 4; D_d.p = nullptr; D_d.n = 0;
-    h->Lv.p = reinterpret_cast<uint8_t*>(L_d.p); h->Lv.n = L_d.n * 4; L_d.p = nullptr; L_d.n = 0;
-  } else {
-    CK(h->Dv.alloc((size_t)nnz_alloc * 2));
-    CK(h->Lv.alloc((size_t)nnz_alloc * 2));
-    CK(cudaMemsetAsync(h->Dv.p, 0, (size_t)nnz_alloc * 2, s));
-    CK(cudaMemsetAsync(h->Lv.p, 0, (size_t)nnz_alloc * 2, s));
-    CK(h->sD.alloc(n_vox));
-    CK(h->sL.alloc(n_vox));
-    launch_quantize(fmt, h->rp.p, n_vox, D_d.p, L_d.p, h->Dv.p, h->Lv.p, h->sD.p, h->sL.p, s);
-    CK(cudaGetLastError());
-    CK(cudaStreamSynchronize(s));
-    D_d.release();
-    L_d.release();
-  }
-
-  // ---- streamed rows: mask, FP64 moments
-  h->V = n_vox; h->nnz = nnz; h->n = n_spots; h->n_pad = (n_spots + 3) & ~3;
-  h->fmt = fmt; h->roi = roi; h->perm = perm; h->n_hot = n_hot; h->nnz_hot = rpd[n_hot];
-  h->n_hot_ne = n_hot_ne; h->n_cold_ne = n_cold_ne;
-  h->h_mask.resize(n_hot);
-  for (int64_t r = 0; r < n_hot; ++r) h->h_mask[r] = m0[order[r]];
-  if (perm) h->h_voxel = std::move(order);  // order is not used below
-  else h->h_voxel.clear();
-  CK(upload_vec(h, h->mask, h->h_mask));
-  {
-    // the constraint evaluation visits only these rows; the others' projection
-    // coefficients stay 0
-    std::vector<int64_t>& cr = h->h_con_rows;
-    cr.clear();
-    for (int64_t r = 0; r < n_hot; ++r)
-      if (h->h_mask[r] != 0) cr.push_back(r);
-    h->n_con_rows = (int64_t)cr.size();
-    CK(upload_vec(h, h->con_rows, cr));
-  }
-  CK(h->mdd.alloc(n_hot)); CK(h->mll.alloc(n_hot)); CK(h->mdl.alloc(n_hot));
-  CK(cudaMemsetAsync(h->mdd.p, 0, std::max<int64_t>(1, n_hot) * sizeof(double), s));
-  CK(cudaMemsetAsync(h->mll.p, 0, std::max<int64_t>(1, n_hot) * sizeof(double), s));
-  CK(cudaMemsetAsync(h->mdl.p, 0, std::max<int64_t>(1, n_hot) * sizeof(double), s));
-  launch_moments(fmt, h->rp.p, n_hot_ne, h->Dv.p, h->Lv.p, fmt ? h->sD.p : nullptr, fmt ? h->sL.p : nullptr,
-                 h->mdd.p, h->mll.p, h->mdl.p, s);
-  CK(cudaGetLastError());
+  col_in.release(); D_in.release(); L_in.release(); rp_in.release(); mask_in.release();
 
   // ---- launch shapes: the whole GPU, or with FREDOPT_SHARED one SM's
   // worth of CTAs per kSharedNnzPerSm nonzeros, so that the kernels of other
@@ -1108,63 +947,59 @@ int fredopt_load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t 
     h->geo = g;
   }
 
-  // ---- CSC copy of the streamed rows (blocked stable counting transpose)
+  // ---- CSC copy of the streamed rows (blocked stable counting transpose) and
+  // the chunks of the transposed product.  Rows without nonzeros (after the
+  // others in device order) add nothing; strips over the whole GPU whatever the
+  // plan's launch shapes (the transpose does not depend on its partition).
   {
-    // rows without nonzeros (after the others in device order) add nothing
-    // one wave of 1024-thread blocks over the whole GPU whatever the plan's
-    // launch shapes (the transpose does not depend on its partition)
-    const int n_blk = (int)std::max<int64_t>(1, std::min<int64_t>(h->geo_full.n_sms, n_hot_ne));
-    std::vector<int64_t> blk = partition_rows(rpd, n_hot_ne, n_blk, 1);
-    DBuf<int64_t> blk_d, tot_d;
-    DBuf<int32_t> cnt;
-    CK(upload_vec(h, blk_d, blk));
-    CK(cnt.alloc((size_t)n_blk * n_spots));
-    CK(cudaMemsetAsync(cnt.p, 0, (size_t)n_blk * n_spots * sizeof(int32_t), s));
-    if (n_hot_ne > 0) launch_csc_count(h->rp.p, h->col.p, blk_d.p, n_blk, n_spots, cnt.p, s);
+    const CscShape cs = csc_shape(h->geo_full, fmt, std::max<int64_t>(1, n_hot_ne), n_spots, nnz_hot);
+    DBuf<int64_t> strip, tot_d;
+    DBuf<int32_t> cnt, split;
+    CK(strip.alloc((size_t)cs.n_strip + 1));
+    launch_tiles(TileArgs{TileArgs::BOUNDS64, h->rp.p, 0, n_hot_ne, 0, 0, cs.n_strip, 0, 1, strip.p, nullptr}, s);
+    CK(cnt.alloc((size_t)cs.n_strip * n_spots));
+    CK(cudaMemsetAsync(cnt.p, 0, (size_t)cs.n_strip * n_spots * sizeof(int32_t), s));
+    if (cs.use_split) CK(split.alloc((size_t)(cs.n_grp + 1) * cs.n_rows));
+    if (n_hot_ne > 0)
+      launch_csc_count(cs, h->geo_full.smem_limit, h->rp.p, h->col.p, h->col16.p, strip.p, cnt.p, split.p, s);
     CK(tot_d.alloc(n_spots));
-    launch_csc_colsum(cnt.p, n_blk, n_spots, tot_d.p, s);
-    CK(cudaGetLastError());
-    std::vector<int64_t> tot(n_spots), cph(n_spots + 1);
-    CK(cudaMemcpyAsync(tot.data(), tot_d.p, n_spots * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    launch_csc_colsum(cnt.p, cs.n_strip, n_spots, tot_d.p, s);
+    int64_t C = nnz_hot / ((int64_t)h->geo.bwd_warps * 8);
+    C = std::max<int64_t>(256, std::min<int64_t>(8192, C));
+    C = (C + 31) & ~31LL;
+    CK(h->cp.fit((size_t)n_spots + 1));
+    CK(h->col_chunk.fit((size_t)n_spots + 1));
+    launch_csc_columns(tot_d.p, n_spots, C, h->cp.p, h->col_chunk.p, s);
+    launch_csc_offsets(cnt.p, cs.n_strip, n_spots, h->cp.p, s);
+    const int64_t max_chunks = nnz_hot / C + n_spots;
+    CK(h->chunk_ptr.fit((size_t)max_chunks + 1));
+    CK(h->chunk_sum.fit((size_t)max_chunks));
+    launch_chunk_fill(h->cp.p, h->col_chunk.p, n_spots, C, h->chunk_ptr.p, s);
+    CK(h->crow.fit(nh_alloc));
+    CK(h->DTv.fit((size_t)nh_alloc * vb));
+    CK(h->LTv.fit((size_t)nh_alloc * vb));
+    CK(cudaMemsetAsync(h->crow.p + nnz_hot, 0, (nh_alloc - nnz_hot) * sizeof(int32_t), s));
+    CK(cudaMemsetAsync(h->DTv.p + (size_t)nnz_hot * vb, 0, (size_t)(nh_alloc - nnz_hot) * vb, s));
+    CK(cudaMemsetAsync(h->LTv.p + (size_t)nnz_hot * vb, 0, (size_t)(nh_alloc - nnz_hot) * vb, s));
+    int64_t total = 0;
+    int32_t n_chunks = 0;
+    CK(cudaMemcpyAsync(&total, h->cp.p + n_spots, sizeof(total), cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(&n_chunks, h->col_chunk.p + n_spots, sizeof(n_chunks), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
-    cph[0] = 0;
-    for (int j = 0; j < n_spots; ++j) cph[j + 1] = cph[j] + tot[j];
-    if (cph[n_spots] != h->nnz_hot) return fail(h, FREDOPT_ERR_CUDA, "CSC count mismatch");
-    CK(upload_vec(h, h->cp, cph));
-    launch_csc_offsets(cnt.p, n_blk, n_spots, h->cp.p, s);
-    const int vb = value_bytes(fmt);
-    const int64_t nh_alloc = ((h->nnz_hot + 255) & ~255LL) + kPadElems;
-    CK(h->crow.alloc(nh_alloc));
-    CK(h->DTv.alloc((size_t)nh_alloc * vb));
-    CK(h->LTv.alloc((size_t)nh_alloc * vb));
-    CK(cudaMemsetAsync(h->crow.p + h->nnz_hot, 0, (nh_alloc - h->nnz_hot) * sizeof(int32_t), s));
-    CK(cudaMemsetAsync(h->DTv.p + (size_t)h->nnz_hot * vb, 0, (size_t)(nh_alloc - h->nnz_hot) * vb, s));
-    CK(cudaMemsetAsync(h->LTv.p + (size_t)h->nnz_hot * vb, 0, (size_t)(nh_alloc - h->nnz_hot) * vb, s));
-    CK(cudaMemsetAsync(h->errw.p, 0, sizeof(int), s));
-    if (n_hot_ne > 0) {
-      // scattered stores are limited by their count: one record per entry,
-      // split into the three arrays by a coalesced pass (scratch freed here)
-      DBuf<uint8_t> rec;
-      const size_t rb = csc_fill_rec_bytes(h->geo, fmt, n_spots);
-      if (rb) CK(rec.alloc((size_t)h->nnz_hot * rb));
-      launch_csc_fill(h->geo, fmt, h->rp.p, h->col.p, h->Dv.p, h->Lv.p, blk_d.p, n_blk, n_spots, cnt.p,
-                      h->crow.p, h->DTv.p, h->LTv.p, h->errw.p, rb ? rec.p : nullptr, h->nnz_hot, s);
-      CK(cudaGetLastError());
-      CK(cudaStreamSynchronize(s));
-    }
+    if (total != nnz_hot) return fail(h, FREDOPT_ERR_CUDA, "CSC count mismatch");
+    h->n_chunks = n_chunks;
+    if (n_hot_ne > 0)
+      launch_csc_fill(cs, fmt, h->rp.p, h->col.p, h->col16.p, h->Dv.p, h->Lv.p, strip.p, split.p, cnt.p, h->crow.p,
+                      h->DTv.p, h->LTv.p, s);
     CK(cudaGetLastError());
-    int ferr = 0;
-    CK(cudaMemcpyAsync(&ferr, h->errw.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    if (ferr) return fail(h, FREDOPT_ERR_TIMEOUT, "a bounded device-side wait gave up (CSC transpose)");
 
     // based 16-bit row indices for the transposed product (2 bytes less per
     // nonzero and pass; crow stays for the sweep and inspection)
     h->n_wide_blocks = 0;
     if (!(format & FREDOPT_INDEX32)) {
       const int64_t n_cblk = nh_alloc / 128;
-      CK(h->crow16.alloc(nh_alloc));
-      CK(h->chdr.alloc(n_cblk));
+      CK(h->crow16.fit(nh_alloc));
+      CK(h->chdr.fit(n_cblk));
       CK(h->cnw.ensure(2));
       CK(cudaMemsetAsync(h->cnw.p, 0, 2 * sizeof(unsigned int), s));
       launch_narrow_rows(h->crow.p, n_cblk, h->crow16.p, h->chdr.p, h->cnw.p, s);
@@ -1176,41 +1011,12 @@ int fredopt_load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t 
       launch_narrow_rows_wide(h->crow.p, n_cblk, h->chdr.p, h->covf.p, h->cnw.p + 1, n_wide, s);
       CK(cudaGetLastError());
       h->n_wide_blocks = n_wide;
+    } else {
+      h->crow16.release();
     }
-
-    // chunk schedule of the transposed product
-    const int W3 = h->geo.bwd_warps;
-    int64_t C = h->nnz_hot / ((int64_t)W3 * 8);
-    C = std::max<int64_t>(256, std::min<int64_t>(8192, C));
-    C = (C + 31) & ~31LL;
-    std::vector<int64_t> cptr;
-    std::vector<int32_t> cchunk(n_spots + 1);
-    cptr.reserve(h->nnz_hot / C + n_spots + 1);
-    for (int j = 0; j < n_spots; ++j) {
-      cchunk[j] = (int32_t)cptr.size();
-      for (int64_t p = cph[j]; p < cph[j + 1]; p += C) cptr.push_back(p);
-    }
-    cchunk[n_spots] = (int32_t)cptr.size();
-    h->n_chunks = (int64_t)cptr.size();
-    cptr.push_back(h->nnz_hot);
-    CK(upload_vec(h, h->chunk_ptr, cptr));
-    CK(upload_vec(h, h->col_chunk, cchunk));
-    CK(cudaStreamSynchronize(s));
-    h->h_cptr.swap(cptr);
-    CK(h->warp_chunk.alloc(W3 + 1));
-    rc = set_bwd_schedule(h, 16);
+    const int rc = set_bwd_schedule(h, 16);
     if (rc) return rc;
-  }
-
-  // ---- 16-bit column indices for the forward stream: 2 bytes less per
-  // nonzero, same sums.  Only with x staged in shared memory (that bounds
-  // n_spots below 65536); the int32 copy served the CSC build and goes.
-  if (!(format & FREDOPT_INDEX32) && n_spots <= 65536 && forward_uses_smem(h->geo, h->n_pad)) {
-    CK(h->col16.alloc(h->col.n));
-    launch_narrow_idx(h->col.p, h->col16.p, (int64_t)h->col.n, s);
-    CK(cudaGetLastError());
-    CK(cudaStreamSynchronize(s));
-    h->col.release();
+    CK(cudaStreamSynchronize(s));  // the scratch of this block is freed here
   }
 
   // ---- row schedules of the forward product (rows with nonzeros only);
@@ -1219,19 +1025,16 @@ int fredopt_load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t 
 #ifndef FO_ROW_COST
 #define FO_ROW_COST 64
 #endif
-  h->h_rp = std::move(rpd);
-  h->n_hot_ne = n_hot_ne;
-  h->n_cold_ne = n_cold_ne;
-  CK(h->warp_row_hot.alloc(2 * (size_t)h->geo.fwd_warps));
-  CK(h->warp_row_all.alloc(2 * (size_t)h->geo.fwd_warps));
   CK(h->fsched.ensure(2));
   CK(cudaMemsetAsync(h->fsched.p, 0, 2 * sizeof(unsigned int), s));
   CK(h->bsched.ensure(2));
   CK(cudaMemsetAsync(h->bsched.p, 0, 2 * sizeof(unsigned int), s));
-  rc = set_fwd_schedule(h, FO_ROW_COST);
-  if (rc) return rc;
+  {
+    const int rc = set_fwd_schedule(h, FO_ROW_COST);
+    if (rc) return rc;
+  }
   // streaming (evict-first) loads when the streamed matrices do not fit in L2
-  const double mat_bytes = (double)h->nnz_hot * ((h->col16.p ? 2.0 : 4.0) + 2.0 * value_bytes(fmt));
+  const double mat_bytes = (double)h->nnz_hot * ((h->col16.p ? 2.0 : 4.0) + 2.0 * vb);
 #ifndef FO_STREAM_HINT
 #define FO_STREAM_HINT -1
 #endif
@@ -1239,19 +1042,18 @@ int fredopt_load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t 
   h->hint_bwd = h->hint_fwd;
 
   // ---- work buffers
-  CK(h->w.alloc(h->n_pad)); CK(h->g.alloc(h->n_pad)); CK(h->xbuf.alloc(h->n_pad)); CK(h->gtmp.alloc(h->n_pad));
+  CK(h->w.fit(h->n_pad)); CK(h->g.fit(h->n_pad)); CK(h->xbuf.fit(h->n_pad)); CK(h->gtmp.fit(h->n_pad));
   CK(cudaMemsetAsync(h->w.p, 0, h->n_pad * sizeof(float), s));
   CK(cudaMemsetAsync(h->g.p, 0, h->n_pad * sizeof(float), s));
   CK(cudaMemsetAsync(h->xbuf.p, 0, h->n_pad * sizeof(float), s));
   CK(cudaMemsetAsync(h->gtmp.p, 0, h->n_pad * sizeof(float), s));
-  CK(h->yw.alloc(n_hot)); CK(h->yg.alloc(n_hot)); CK(h->r.alloc(n_hot)); CK(h->gam.alloc(n_hot));
+  CK(h->yw.fit(n_hot)); CK(h->yg.fit(n_hot)); CK(h->r.fit(n_hot)); CK(h->gam.fit(n_hot));
   // rows without nonzeros are never written by the forward product: keep them 0
   CK(cudaMemsetAsync(h->yw.p, 0, std::max<int64_t>(1, n_hot) * sizeof(float2), s));
   CK(cudaMemsetAsync(h->yg.p, 0, std::max<int64_t>(1, n_hot) * sizeof(float2), s));
   CK(cudaMemsetAsync(h->r.p, 0, std::max<int64_t>(1, n_hot) * sizeof(float2), s));
   // projection coefficients: rows without a structure bit are never written
   CK(cudaMemsetAsync(h->gam.p, 0, std::max<int64_t>(1, n_hot) * sizeof(float2), s));
-  CK(h->chunk_sum.alloc(h->n_chunks));
   const Geometry& G = h->geo;
   // forward partials: one per tile (at most 7 guided tiles per warp)
   const int max_tiles = kGuidedTilesPerWarp * G.fwd_warps;
@@ -1265,10 +1067,8 @@ int fredopt_load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t 
   h->off_btab = h->off_stage + 4 * kFinishBlocks;
   h->n_part = h->off_btab + kBetaTable;
   h->btab_alpha = -1.0;  // the table is refilled at the next fredopt_begin
-  CK(h->part.alloc(h->n_part));
+  CK(h->part.fit(h->n_part));
   CK(cudaMemsetAsync(h->part.p, 0, h->n_part * sizeof(double), s));
-  h->y64.release(); h->yall.release(); h->fout_a.release(); h->fout_b.release();
-  h->vin_a.release(); h->vin_b.release();
   CK(cudaStreamSynchronize(s));
 
   h->tab.n_con = 0;
@@ -1300,7 +1100,8 @@ int fredopt_set_constraints(fredopt_t h, int n, const fredopt_constraint* c) {
     h->tab.con[i].prio = c[i].priority;
   }
   double* pc = h->part.p + h->off_cnt;
-  launch_count_rows(h->geo, h->tab, h->mask.p, h->mdd.p, h->mll.p, h->mdl.p, h->n_hot, pc, h->stream);
+  launch_count_rows(h->geo, h->tab, h->mask.p, h->mdd.p, h->mll.p, h->mdl.p, h->con_rows.p,
+                    h->n_con_rows, pc, h->stream);
   CK(cudaGetLastError());
   std::vector<double> hp(3 * h->geo.row_blocks);
   CK(cudaMemcpyAsync(hp.data(), pc, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
@@ -1544,7 +1345,7 @@ int fredopt_end(fredopt_t h, float* w_out, float* dose_out, float* letd_out, fre
   fa.letd_out = lptr;
   run(h, 0, [&] { launch_forward(G, h->fmt, EPI_FINAL, false, fa, h->tab, s); });
   double* pf = h->part.p + h->off_fin;
-  run(h, 5, [&] { launch_final_check(G, h->tab, h->y64.p, h->mask.p, h->mdd.p, h->mll.p, h->mdl.p, h->n_hot, pf, s); });
+  run(h, 5, [&] { launch_final_check(G, h->tab, h->y64.p, h->mask.p, h->mdd.p, h->mll.p, h->mdl.p, h->con_rows.p, h->n_con_rows, pf, s); });
   CK(cudaGetLastError());
   std::vector<double> hp(8 * G.row_blocks);
   CK(cudaMemcpyAsync(hp.data(), pf, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, s));

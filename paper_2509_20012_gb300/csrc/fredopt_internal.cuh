@@ -213,7 +213,7 @@ void launch_finish(int step, const double* part_f, int nf, const double* part_bc
                    const double* part_g, int ng, DevState* st, double* stage, const double* btab,
                    long long n_btab, cudaStream_t s);
 void launch_count_rows(const Geometry& g, const Tables& t, const uint32_t* mask, const double* dd,
-                       const double* ll, const double* dl, int64_t n_hot, double* part,
+                       const double* ll, const double* dl, const int64_t* rows, int64_t n_list, double* part,
                        cudaStream_t s);
 void launch_scatter_y(const float2* y, const int64_t* voxel, int64_t n, float* a, float* b,
                       cudaStream_t s);
@@ -223,35 +223,96 @@ void launch_row_objective(const Geometry& g, const Tables& t, const float2* yw, 
                           const float* sD, const float* sL, int64_t n_hot, float2* r_out,
                           double* part, cudaStream_t s);
 void launch_final_check(const Geometry& g, const Tables& t, const double2* y64, const uint32_t* mask,
-                        const double* dd, const double* ll, const double* dl, int64_t n_hot,
+                        const double* dd, const double* ll, const double* dl, const int64_t* rows, int64_t n_list,
                         double* part, cudaStream_t s);
 void launch_begin_state(DevState* st, cudaStream_t s);
 
-// setup (K5)
-void launch_validate(const int64_t* rp, const int32_t* col, const float* D, const float* L,
-                     int64_t n_rows, int32_t n_cols, int64_t nnz, int* err, cudaStream_t s);
-void launch_gather_rows(const int64_t* rp_src, const int64_t* src_row, const int64_t* rp_dst,
-                        int64_t n_rows, const int32_t* col_src, const float* D_src,
-                        const float* L_src, int32_t* col_dst, float* D_dst, float* L_dst,
-                        cudaStream_t s);
-void launch_quantize(int fmt, const int64_t* rp, int64_t n_rows, const float* D, const float* L,
-                     void* qD, void* qL, float* sD, float* sL, cudaStream_t s);
-void launch_moments(int fmt, const int64_t* rp, int64_t n_rows, const void* Dv, const void* Lv,
-                    const float* sD, const float* sL, double* dd, double* ll, double* dl,
-                    cudaStream_t s);
-// blocked stable counting transpose of rows [0, n_rows)
-void launch_csc_count(const int64_t* rp, const int32_t* col, const int64_t* blk_row, int n_blk,
-                      int32_t n_cols, int32_t* cnt, cudaStream_t s);
-void launch_csc_offsets(int32_t* cnt, int n_blk, int32_t n_cols, const int64_t* cp, cudaStream_t s);
-// stable CSR -> CSC scatter; a bulk-copy wait that gives up sets bit 0 of *err
-// rec: null, or csc_fill_rec_bytes(...) bytes per output entry of scratch
-// (n_out entries): the fill then stores one record per entry and splits them
-void launch_csc_fill(const Geometry& g, int fmt, const int64_t* rp, const int32_t* col, const void* Dv,
-                     const void* Lv, const int64_t* blk_row, int n_blk, int32_t n_cols, int32_t* cursor,
-                     int32_t* row_out, void* DT, void* LT, int* err, void* rec, int64_t n_out, cudaStream_t s);
-// bytes per entry of the fill's record scratch for this plan, 0 for none
-size_t csc_fill_rec_bytes(const Geometry& g, int fmt, int32_t n_cols);
-void launch_csc_colsum(const int32_t* cnt, int n_blk, int32_t n_cols, int64_t* tot, cudaStream_t s);
+// setup (K5, fredopt_load.cu)
+// Tiles that warps claim in order have guided sizes, 7 per warp: W tiles of
+// half a warp's share, W of a quarter, an eighth, a sixteenth and a
+// thirty-second, 2 W of a sixty-fourth, so the last to be claimed are short and
+// the warps finish close together.  The count does not depend on the costs:
+// kernels and captured graphs hold it by value.
+constexpr int kGuidedTilesPerWarp = 7;
+
+enum : unsigned { kRowsBadEnds = 1u, kRowsNotMonotone = 2u, kRowsPermuted = 4u };
+struct RowTotals {
+  // rows of groups 0 (streamed, with nonzeros), 1 (streamed, without), 2
+  // (other, with); nonzeros of groups 0 and 2; structure rows of groups 0, 1
+  long long c[7];
+  unsigned int flags;
+  unsigned int pad;
+  unsigned long long empty_bits[32];  // streamed rows without nonzeros, per structure bit
+};
+size_t row_order_scratch(int64_t n_rows);  // int64 values
+// tot zeroed before; blk: row_order_scratch values
+void launch_rows_count(const int64_t* rp, const uint32_t* mask, int64_t n, int64_t nnz, bool roi, int64_t* blk,
+                       RowTotals* tot, cudaStream_t s);
+// voxel, sD, sL may be null
+void launch_rows_place(const int64_t* rp, const uint32_t* mask, int64_t n, bool roi, const int64_t* blk,
+                       const RowTotals* tot, int64_t* rp_out, int64_t* voxel, uint32_t* mask_out, int64_t* con_rows,
+                       float* sD, float* sL, cudaStream_t s);
+
+struct LoadRowsArgs {
+  const int64_t* rp_in;   // input row pointers
+  const int64_t* rp_out;  // device order
+  const int64_t* voxel;   // device row -> input row, or null
+  int64_t n_hot, n_hot_ne, n_cold_ne;
+  int32_t n_cols;
+  const int32_t* col;     // input
+  const float* D;
+  const float* L;
+  void* col_out;          // uint16 or int32
+  void* Dv;
+  void* Lv;
+  float* sD;
+  float* sL;
+  double* dd;
+  double* ll;
+  double* dl;
+  int* err;
+};
+// narrow: 16-bit indices; copy_values false (FP32 only): D, L are the storage already
+void launch_load_rows(int fmt, bool narrow, bool copy_values, const LoadRowsArgs& a, cudaStream_t s);
+
+// Tile bounds over ptr (row or chunk pointers): cost of an element = its
+// nonzeros + `cost`.
+struct TileArgs {
+  enum Kind { PAIRS, BOUNDS64, BOUNDS32, GUIDED_PAIRS, GUIDED32 } kind;
+  const int64_t* ptr;
+  int64_t a0, z0, a1, z1;  // ranges (the second for PAIRS; the guided kinds start at 0)
+  int parts0, parts1;      // pieces of each range; warps for the guided kinds
+  int64_t cost;
+  int64_t* out64;
+  int32_t* out32;
+};
+void launch_tiles(const TileArgs& q, cudaStream_t s);
+// tot -> cp[n + 1] and, with chunks of C nonzeros, col_chunk[n + 1]
+void launch_csc_columns(const int64_t* tot, int32_t n, int64_t C, int64_t* cp, int32_t* col_chunk, cudaStream_t s);
+void launch_chunk_fill(const int64_t* cp, const int32_t* col_chunk, int32_t n, int64_t C, int64_t* chunk_ptr,
+                       cudaStream_t s);
+
+// blocked stable counting transpose (CSR -> CSC) of rows [0, n_rows), all with
+// nonzeros (fredopt_load.cu)
+struct CscShape {
+  int64_t n_rows;
+  int32_t n_cols;
+  int n_strip;     // strips of rows
+  int gshift;      // columns per group = 1 << gshift
+  int n_grp;
+  int tile;        // entries a CTA sorts at a time
+  bool use_split;  // keep (n_grp + 1) * n_rows group starts
+};
+CscShape csc_shape(const Geometry& g, int fmt, int64_t n_rows, int32_t n_cols, int64_t nnz);
+// cnt: n_strip * n_cols, zeroed; split: n_rows * (n_grp + 1) or null
+// (col16 when set, else col)
+void launch_csc_count(const CscShape& q, size_t smem_limit, const int64_t* rp, const int32_t* col,
+                      const uint16_t* col16, const int64_t* strip_row, int32_t* cnt, int32_t* split, cudaStream_t s);
+void launch_csc_colsum(const int32_t* cnt, int n_strip, int32_t n_cols, int64_t* tot, cudaStream_t s);
+void launch_csc_offsets(int32_t* cnt, int n_strip, int32_t n_cols, const int64_t* cp, cudaStream_t s);
+void launch_csc_fill(const CscShape& q, int fmt, const int64_t* rp, const int32_t* col, const uint16_t* col16,
+                     const void* Dv, const void* Lv, const int64_t* strip_row, const int32_t* split,
+                     const int32_t* cursor, int32_t* row_out, void* DT, void* LT, cudaStream_t s);
 void launch_dequant_csc(int fmt, const int64_t* cp, int32_t n_cols, const int32_t* row, const void* DT,
                         const void* LT, const float* sD, const float* sL, float* Dout, float* Lout,
                         cudaStream_t s);
@@ -291,8 +352,6 @@ void launch_narrow_rows(const int32_t* row, int64_t n_blk, uint16_t* row16, int3
                         cudaStream_t s);
 void launch_narrow_rows_wide(const int32_t* row, int64_t n_blk, int32_t* hdr, int32_t* ovf, unsigned int* slot,
                              unsigned int n_wide, cudaStream_t s);
-// out[i] = in[i] for i < n (in[i] < 65536), n a multiple of 4.
-void launch_narrow_idx(const int32_t* in, uint16_t* out, int64_t n, cudaStream_t s);
 // One CTA in the bounded wait of the bulk copies (spins <= 0: their bound).
 void launch_wait_check(int arrive, int spins, DevState* st, cudaStream_t s);
 

@@ -20,10 +20,11 @@
 //   K4 k_finish      64 blocks, then the last one: deterministic two-level
 //                    reduction of the partials and the closed-form
 //                    non-ascent trial loop (Fig. 3) in one warp.
-//   K5 setup         validation, row gather, quantisation, FP64 moments,
-//                    blocked stable transpose (CSR -> CSC) 16 rows a step.
+//   K5 setup         in fredopt_load.cu (row order, values, CSC copy, tiles);
+//                    here the based 16-bit row offsets of the CSC.
 #include "fredopt.h"
 #include "fredopt_internal.cuh"
+#include "fredopt_device.cuh"
 
 #include <algorithm>
 
@@ -32,7 +33,6 @@
 
 namespace fo {
 
-constexpr unsigned kFull = 0xffffffffu;
 // Launch shape and streaming depth (compile-time; the defaults were chosen
 // by measurement on GB300).
 #ifndef FO_FWD_UNROLL
@@ -119,10 +119,6 @@ __device__ __forceinline__ int lane_pos(int lane, int q) {
 
 // ------------------------------------------------------------------ helpers
 
-__device__ __forceinline__ float to_f(float v) { return v; }
-__device__ __forceinline__ float to_f(__nv_bfloat16 v) { return __bfloat162float(v); }
-__device__ __forceinline__ float to_f(__half v) { return __half2float(v); }
-
 template <typename VT> struct VecOf;
 template <> struct VecOf<float> { static constexpr int V = 4; };
 // 16-bit values: 4 per lane too (8-byte value loads), so a block keeps the
@@ -198,106 +194,6 @@ __device__ __forceinline__ void unpack(__half, uint4 u, float* o) {
     o[2 * i] = f.x;
     o[2 * i + 1] = f.y;
   }
-}
-
-template <typename T>
-__device__ __forceinline__ T warp_sum(T v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-  return v;
-}
-
-// ---- double-float (double-word) accumulation ----
-// A value hi + lo held in two FP32 numbers (|lo| <= ulp(hi) / 2): about 48
-// significant bits at FP32 speed.  GB300's FP64 rate is a small fraction of
-// its FP32 rate, so the final FP64-class pass accumulates in this form.
-// Products are exact (TwoProd with an FMA); additions use the accurate
-// double-word sum of Joldes, Muller and Popescu (ACM TOMS 44(2), 2017,
-// relative error <= 3 * 2^-48), built from Knuth's TwoSum and Dekker's
-// FastTwoSum.  Every operation is an explicitly rounded intrinsic, so the
-// compiler cannot fuse or reorder any step.
-struct DF {
-  float hi, lo;
-  __device__ DF() : hi(0.0f), lo(0.0f) {}
-  __device__ explicit DF(float v) : hi(v), lo(0.0f) {}
-  __device__ DF(float h, float l) : hi(h), lo(l) {}
-  __device__ explicit operator double() const { return (double)hi + (double)lo; }
-};
-__device__ __forceinline__ DF two_sum(float a, float b) {
-  const float s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-  return DF(s, e);
-}
-__device__ __forceinline__ DF fast_two_sum(float a, float b) {  // |a| >= |b|
-  const float s = __fadd_rn(a, b);
-  return DF(s, __fsub_rn(b, __fsub_rn(s, a)));
-}
-__device__ __forceinline__ DF df_add(DF x, DF y) {
-  const DF s = two_sum(x.hi, y.hi);
-  const DF t = two_sum(x.lo, y.lo);
-  const DF v = fast_two_sum(s.hi, __fadd_rn(s.lo, t.hi));
-  return fast_two_sum(v.hi, __fadd_rn(t.lo, v.lo));
-}
-// c + a * b
-__device__ __forceinline__ DF acc_fma(float a, float b, DF c) {
-  const float p = __fmul_rn(a, b);
-  return df_add(c, DF(p, __fmaf_rn(a, b, -p)));  // a * b = p + (a * b - p) exactly
-}
-template <>
-__device__ __forceinline__ DF warp_sum(DF v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const DF w(__shfl_xor_sync(kFull, v.hi, o), __shfl_xor_sync(kFull, v.lo, o));
-    v = df_add(v, w);
-  }
-  return v;
-}
-// c + sum of four products in double-float: the products exact (TwoProd), the
-// three sums of their high parts exact (TwoSum), the seven error terms added
-// in FP32, and one renormalised addition to c.  Against four acc_fma steps
-// this is 43 FP32 operations instead of 88, and one rounding of the pair
-// instead of four: over rows of 128 to 3072 nonzeros (positive, mixed-sign
-// and wide-ranged values) its largest error against 64-bit-exact sums is the
-// same or smaller (5e-15 against 6e-15 of the sum of magnitudes).  The final
-// pass is bound by these operations: 7.3e8 nonzeros, FP32 2.70 -> 1.46 ms,
-// FP16 2.59 -> 1.63 ms (its streaming floor is 1.07 and 0.65 ms).
-__device__ __forceinline__ DF df_dot4(const float* a, const float* x, DF c) {
-  float p[4], e[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    p[q] = __fmul_rn(a[q], x[q]);
-    e[q] = __fmaf_rn(a[q], x[q], -p[q]);
-  }
-  const DF u = two_sum(p[0], p[1]), v = two_sum(p[2], p[3]);
-  const DF s = two_sum(u.hi, v.hi);
-  const float t = __fadd_rn(__fadd_rn(__fadd_rn(u.lo, v.lo), s.lo),
-                            __fadd_rn(__fadd_rn(e[0], e[1]), __fadd_rn(e[2], e[3])));
-  const DF w = two_sum(c.hi, s.hi);
-  return fast_two_sum(w.hi, __fadd_rn(w.lo, __fadd_rn(c.lo, t)));
-}
-
-__device__ __forceinline__ float shfl_xor(float v, int o) { return __shfl_xor_sync(kFull, v, o); }
-__device__ __forceinline__ DF shfl_xor(DF v, int o) {
-  return DF(__shfl_xor_sync(kFull, v.hi, o), __shfl_xor_sync(kFull, v.lo, o));
-}
-__device__ __forceinline__ float acc_add(float a, float b) { return a + b; }
-__device__ __forceinline__ DF acc_add(DF a, DF b) { return df_add(a, b); }
-// Both sums of a segment over the warp, bit for bit those of two butterflies
-// (warp_sum): in the first step the lower half-warp takes over a and the upper
-// one b, so the other four steps serve both; 6 shuffles and 5 additions
-// instead of 10 and 10.
-template <typename Acc>
-__device__ __forceinline__ void warp_sum2(Acc& a, Acc& b, int lane) {
-  const bool up = (lane & 16) != 0;
-  const Acc give = up ? a : b;
-  Acc keep = up ? b : a;
-  keep = acc_add(keep, shfl_xor(give, 16));
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) keep = acc_add(keep, shfl_xor(keep, o));
-  const Acc other = shfl_xor(keep, 16);
-  a = up ? other : keep;
-  b = up ? keep : other;
 }
 
 // ---- mbarrier + bulk copy (TMA engine, non-tensor form) ----
@@ -1322,19 +1218,20 @@ __global__ void __launch_bounds__(kRowThreads) k_row_objective(Tables t, const f
   if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
-// FP64 check at the final point: per block [max violation per kind (6), n violated, f]
+// FP64 check at the final point over the listed rows (those with a structure
+// bit): per block [max violation per kind (6), n violated, f]
 __global__ void __launch_bounds__(kRowThreads) k_final_check(Tables t, const double2* y64,
                                                             const uint32_t* mask, const double* dd,
                                                             const double* ll, const double* dl,
-                                                            int64_t n_hot, double* part) {
+                                                            const int64_t* rows, int64_t n_list, double* part) {
   __shared__ double red[kRowThreads];
-  const int64_t per = (n_hot + gridDim.x - 1) / gridDim.x;
-  const int64_t i0 = (int64_t)blockIdx.x * per, i1 = min(n_hot, i0 + per);
+  const int64_t per = (n_list + gridDim.x - 1) / gridDim.x;
+  const int64_t j0 = (int64_t)blockIdx.x * per, j1 = min(n_list, j0 + per);
   double mk[6] = {0, 0, 0, 0, 0, 0};
   double nv = 0.0, fo = 0.0;
-  for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+  for (int64_t j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
+    const int64_t i = rows[j];
     const uint32_t m = mask[i];
-    if (!m) continue;
     const double2 y = y64[i];
     for (int q = 0; q < t.n_con; ++q) {
       const ConEntry& c = t.con[q];
@@ -1385,280 +1282,6 @@ __global__ void k_begin_state(DevState* st) {
 
 // ------------------------------------------------------------------ K5 setup
 
-__global__ void k_validate(const int64_t* rp, const int32_t* col, const float* D, const float* L,
-                           int64_t n_rows, int32_t n_cols, int* err) {
-  const int lane = threadIdx.x & 31;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n_rows; r += nw) {
-    const int64_t s = rp[r], e = rp[r + 1];
-    int bad = 0;
-    for (int64_t p = s + lane; p < e; p += 32) {
-      const int c = col[p];
-      if (c < 0 || c >= n_cols) bad |= 1;
-      if (p > s && col[p - 1] >= c) bad |= 1;
-      if (!isfinite(D[p]) || !isfinite(L[p])) bad |= 2;
-    }
-    bad = __reduce_or_sync(kFull, bad);
-    if (bad && lane == 0) atomicOr(err, bad);
-  }
-}
-
-__global__ void k_gather_rows(const int64_t* rp_src, const int64_t* src_row, const int64_t* rp_dst,
-                              int64_t n_rows, const int32_t* col_src, const float* D_src,
-                              const float* L_src, int32_t* col_dst, float* D_dst, float* L_dst) {
-  const int lane = threadIdx.x & 31;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n_rows; r += nw) {
-    const int64_t sr = src_row[r];
-    const int64_t s = rp_src[sr], e = rp_src[sr + 1], d = rp_dst[r];
-    for (int64_t p = s + lane; p < e; p += 32) {
-      col_dst[d + (p - s)] = col_src[p];
-      D_dst[d + (p - s)] = D_src[p];
-      L_dst[d + (p - s)] = L_src[p];
-    }
-  }
-}
-
-// Power-of-two scale so that scale * q is exact in binary32:
-// BF16: max|q| in (1/2, 1]; FP16: max|q| in (2^13, 2^14] (all normal values
-// down to 2^-28 of the row maximum keep 11 significant bits).
-__device__ __forceinline__ float pow2_scale(float amax, int fmt) {
-  if (!(amax > 0.0f)) return 1.0f;
-  int ex;
-  frexpf(amax, &ex);  // amax in [2^(ex-1), 2^ex)
-  return ldexpf(1.0f, fmt == 2 ? ex - 14 : ex);
-}
-
-template <typename VT>
-__device__ __forceinline__ VT from_f(float v);
-template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
-template <> __device__ __forceinline__ __half from_f<__half>(float v) { return __float2half_rn(v); }
-
-template <typename VT>
-__global__ void k_quantize(int fmt, const int64_t* rp, int64_t n_rows, const float* D, const float* L,
-                           VT* qD, VT* qL, float* sD, float* sL) {
-  const int lane = threadIdx.x & 31;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n_rows; r += nw) {
-    const int64_t s = rp[r], e = rp[r + 1];
-    float mD = 0.f, mL = 0.f;
-    for (int64_t p = s + lane; p < e; p += 32) {
-      mD = fmaxf(mD, fabsf(D[p]));
-      mL = fmaxf(mL, fabsf(L[p]));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      mD = fmaxf(mD, __shfl_xor_sync(kFull, mD, o));
-      mL = fmaxf(mL, __shfl_xor_sync(kFull, mL, o));
-    }
-    const float scD = pow2_scale(mD, fmt), scL = pow2_scale(mL, fmt);
-    for (int64_t p = s + lane; p < e; p += 32) {
-      qD[p] = from_f<VT>(D[p] / scD);
-      qL[p] = from_f<VT>(L[p] / scL);
-    }
-    if (lane == 0) { sD[r] = scD; sL[r] = scL; }
-  }
-}
-
-// FP64-accurate row moments |D_i|^2, |L_i|^2, <D_i, L_i> of the stored
-// values in double-float (exact products, accurate double-word sums: relative
-// error <= 3 * 2^-48 per addition of these nonnegative terms), at FP32 speed;
-// the power-of-two row scales are applied at the end, exactly.
-template <typename VT>
-__global__ void k_moments(const int64_t* rp, int64_t n_rows, const VT* Dv, const VT* Lv,
-                          const float* sD, const float* sL, double* dd, double* ll, double* dl) {
-  const int lane = threadIdx.x & 31;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n_rows; r += nw) {
-    const int64_t s = rp[r], e = rp[r + 1];
-    DF a, b, c;
-    for (int64_t p = s + lane; p < e; p += 32) {
-      const float d = to_f(Dv[p]), l = to_f(Lv[p]);
-      a = acc_fma(d, d, a);
-      b = acc_fma(l, l, b);
-      c = acc_fma(d, l, c);
-    }
-    a = warp_sum(a);
-    b = warp_sum(b);
-    c = warp_sum(c);
-    if (lane == 0) {
-      const double sd = sD ? (double)sD[r] : 1.0, sl = sL ? (double)sL[r] : 1.0;
-      dd[r] = (double)a * (sd * sd);
-      ll[r] = (double)b * (sl * sl);
-      dl[r] = (double)c * (sd * sl);
-    }
-  }
-}
-
-// blocked counting transpose: block b owns rows [blk_row[b], blk_row[b+1])
-template <bool SMEM>
-__global__ void k_csc_count(const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
-                            const int64_t* __restrict__ blk_row, int32_t n_cols, int32_t* __restrict__ cnt) {
-  extern __shared__ int32_t sh_cnt[];
-  const int b = blockIdx.x;
-  const int64_t s = rp[blk_row[b]], e = rp[blk_row[b + 1]];
-  int32_t* c = cnt + (int64_t)b * n_cols;
-  if (SMEM) {  // a shared-memory histogram, then one coalesced write of the block's row
-    for (int j = threadIdx.x; j < n_cols; j += blockDim.x) sh_cnt[j] = 0;
-    __syncthreads();
-    for (int64_t p = s + threadIdx.x; p < e; p += blockDim.x) atomicAdd(&sh_cnt[col[p]], 1);
-    __syncthreads();
-    for (int j = threadIdx.x; j < n_cols; j += blockDim.x) c[j] = sh_cnt[j];
-  } else {
-    for (int64_t p = s + threadIdx.x; p < e; p += blockDim.x) atomicAdd(&c[col[p]], 1);
-  }
-}
-
-__global__ void k_csc_colsum(const int32_t* cnt, int n_blk, int32_t n_cols, int64_t* tot) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n_cols) return;
-  int64_t s = 0;
-  for (int b = 0; b < n_blk; ++b) s += cnt[(int64_t)b * n_cols + j];
-  tot[j] = s;
-}
-
-// cnt[b][j] <- first output position of block b's entries of column j
-__global__ void k_csc_offsets(int32_t* cnt, int n_blk, int32_t n_cols, const int64_t* cp) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n_cols) return;
-  int64_t run = cp[j];
-  for (int b = 0; b < n_blk; ++b) {
-    const int64_t i = (int64_t)b * n_cols + j;
-    const int32_t t = cnt[i];
-    cnt[i] = (int32_t)run;  // positions < 2^31 (checked on the host)
-    run += t;
-  }
-}
-
-// Rows of a block in ascending order; within a row all columns differ, so
-// the cursor updates of one row never collide; a barrier separates rows,
-// which keeps the rows of every column ascending (a stable transpose).
-// The block's nonzeros reach shared memory by bulk copies (TMA engine) in
-// windows of W elements, two buffers deep: while the rows of one window are
-// scattered the next window is in flight, and a block barrier does not wait
-// for bulk copies, so a row costs shared-memory reads, a cursor update and a
-// barrier.  Row pointers are staged in chunks of kFillRows rows.  A bounded
-// wait that gives up sets bit 0 of *err; the block lets its copies land and
-// stops (the load then fails with a timeout).
-constexpr int kFillThreads = 1024;
-constexpr int kFillRows = 2048;
-constexpr int64_t kFillAlign = 8;  // window starts and lengths: 16 bytes of every array
-constexpr size_t kFillRpBytes = ((kFillRows + 1) * sizeof(int64_t) + 15) & ~(size_t)15;
-
-template <typename VT>
-size_t csc_fill_smem(int W, int32_t n_cols, bool smem_cursors) {
-  return 2 * (size_t)W * (sizeof(int32_t) + 2 * sizeof(VT)) + kFillRpBytes +
-         (smem_cursors ? (((size_t)n_cols * sizeof(int32_t) + 15) & ~(size_t)15) : 0) + 2 * sizeof(uint64_t);
-}
-
-template <typename VT, bool SMEM>
-__global__ void __launch_bounds__(kFillThreads) k_csc_fill(
-    const int64_t* __restrict__ rp, const int32_t* __restrict__ col, const VT* __restrict__ Dv,
-    const VT* __restrict__ Lv, const int64_t* __restrict__ blk_row, int32_t n_cols, int32_t* __restrict__ cursor,
-    int32_t* __restrict__ row_out, VT* __restrict__ DT, VT* __restrict__ LT, int W, int* err) {
-  extern __shared__ __align__(16) unsigned char fill_sh[];
-  const int b = blockIdx.x;
-  const int64_t r0 = blk_row[b], r1 = blk_row[b + 1];
-  if (r0 >= r1) return;
-  const size_t win_bytes = (size_t)W * (sizeof(int32_t) + 2 * sizeof(VT));
-  int64_t* sh_rp = reinterpret_cast<int64_t*>(fill_sh + 2 * win_bytes);
-  int32_t* sh_cur = reinterpret_cast<int32_t*>(fill_sh + 2 * win_bytes + kFillRpBytes);
-  const size_t cur_bytes = SMEM ? (((size_t)n_cols * sizeof(int32_t) + 15) & ~(size_t)15) : 0;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(fill_sh + 2 * win_bytes + kFillRpBytes + cur_bytes);
-  auto wcol = [&](int j) { return reinterpret_cast<int32_t*>(fill_sh + j * win_bytes); };
-  auto wD = [&](int j) { return reinterpret_cast<VT*>(fill_sh + j * win_bytes + sizeof(int32_t) * (size_t)W); };
-  auto wL = [&](int j) {
-    return reinterpret_cast<VT*>(fill_sh + j * win_bytes + (sizeof(int32_t) + sizeof(VT)) * (size_t)W);
-  };
-  int32_t* cur = cursor + (int64_t)b * n_cols;
-  if (SMEM) {  // the block's cursors stay in shared memory for the whole pass
-    for (int j = threadIdx.x; j < n_cols; j += blockDim.x) sh_cur[j] = cur[j];
-    cur = sh_cur;
-  }
-  // window k = elements [EA + k W, min(EA + (k + 1) W, EZ)); the arrays are
-  // zero padded past nnz to a multiple of 256 elements, so EZ is in bounds
-  const int64_t EA = rp[r0] & ~(kFillAlign - 1);
-  const int64_t EZ = (rp[r1] + kFillAlign - 1) & ~(kFillAlign - 1);
-  const int64_t n_win = (EZ - EA + W - 1) / W;
-  auto issue = [&](int64_t k) {  // thread 0: window k into buffer k & 1
-    const int j = (int)(k & 1);
-    const int64_t ws = EA + k * W;
-    const uint32_t n = (uint32_t)(EZ - ws < W ? EZ - ws : W);
-    mbar_expect_tx(&bar[j], n * (uint32_t)(sizeof(int32_t) + 2 * sizeof(VT)));
-    bulk_g2s(wcol(j), col + ws, n * (uint32_t)sizeof(int32_t), &bar[j]);
-    bulk_g2s(wD(j), Dv + ws, n * (uint32_t)sizeof(VT), &bar[j]);
-    bulk_g2s(wL(j), Lv + ws, n * (uint32_t)sizeof(VT), &bar[j]);
-  };
-  // window k's phase on its buffer is the (k >> 1)-th; the outcome is made uniform over the block
-  auto wait_win = [&](int64_t k) -> bool {
-    const bool ok = mbar_wait(&bar[k & 1], (uint32_t)((k >> 1) & 1), kMbarSpins);
-    return __syncthreads_and(ok) != 0;
-  };
-  auto land = [&](int64_t k) {  // let windows k and k + 1 (issued ones) arrive
-    if (k < n_win) mbar_wait(&bar[k & 1], (uint32_t)((k >> 1) & 1), kMbarSpins);
-    if (k + 1 < n_win) mbar_wait(&bar[(k + 1) & 1], (uint32_t)(((k + 1) >> 1) & 1), kMbarSpins);
-  };
-  if (threadIdx.x == 0) {
-    mbar_init(&bar[0], 1);
-    mbar_init(&bar[1], 1);
-    fence_mbar_init();
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    issue(0);
-    if (n_win > 1) issue(1);
-  }
-  int64_t k = 0;
-  if (!wait_win(0)) {
-    if (threadIdx.x == 0) atomicOr(err, 1);
-    land(0);
-    return;
-  }
-  int64_t ws = EA, we = EA + W < EZ ? EA + W : EZ;
-  for (int64_t c0 = r0; c0 < r1; c0 += kFillRows) {
-    const int nr = (int)(r1 - c0 < kFillRows ? r1 - c0 : kFillRows);
-    __syncthreads();  // the previous chunk is done with sh_rp
-    for (int i = threadIdx.x; i <= nr; i += blockDim.x) sh_rp[i] = rp[c0 + i];
-    __syncthreads();
-    for (int i = 0; i < nr; ++i) {
-      int64_t sp = sh_rp[i];
-      const int64_t ep = sh_rp[i + 1];
-      const int32_t r = (int32_t)(c0 + i);
-      while (true) {
-        const int64_t hi = ep < we ? ep : we;
-        const int j = (int)(k & 1);
-        const int32_t* cc = wcol(j);
-        const VT* dd = wD(j);
-        const VT* ll = wL(j);
-        for (int64_t p = sp + threadIdx.x; p < hi; p += kFillThreads) {
-          const int o = (int)(p - ws);
-          const int c = cc[o];
-          const int32_t pos = cur[c];
-          cur[c] = pos + 1;
-          row_out[pos] = r;
-          DT[pos] = dd[o];
-          LT[pos] = ll[o];
-        }
-        if (ep <= we) break;
-        // the row continues in window k + 1: free buffer k & 1 for window k + 2
-        __syncthreads();
-        if (threadIdx.x == 0 && k + 2 < n_win) issue(k + 2);
-        ++k;
-        if (!wait_win(k)) {
-          if (threadIdx.x == 0) atomicOr(err, 1);
-          land(k);
-          return;
-        }
-        ws += W;
-        we = ws + W < EZ ? ws + W : EZ;
-        sp = hi;
-      }
-      __syncthreads();  // the row's cursor updates are done
-    }
-  }
-  land(k + 1);  // nothing is normally in flight here; never leave with a copy pending
-}
-
 template <typename VT>
 __global__ void k_dequant_csc(const int64_t* cp, int32_t n_cols, const int32_t* row, const VT* DT,
                               const VT* LT, const float* sD, const float* sL, float* Dout, float* Lout) {
@@ -1683,18 +1306,18 @@ __global__ void k_scale_coef(int64_t n, const float* aD, const float* aL, const 
 }
 
 
-// reachable constraint rows (|a_r|^2 > 0): per block [count, unreachable, sum of priorities]
+// reachable constraint rows (|a_r|^2 > 0) of the listed voxel rows: per block [count, unreachable, sum of priorities]
 __global__ void __launch_bounds__(kRowThreads) k_count_rows(Tables t, const uint32_t* mask,
                                                            const double* dd, const double* ll,
-                                                           const double* dl, int64_t n_hot,
-                                                           double* part) {
+                                                           const double* dl, const int64_t* rows,
+                                                           int64_t n_list, double* part) {
   __shared__ double red[kRowThreads];
-  const int64_t per = (n_hot + gridDim.x - 1) / gridDim.x;
-  const int64_t i0 = (int64_t)blockIdx.x * per, i1 = min(n_hot, i0 + per);
+  const int64_t per = (n_list + gridDim.x - 1) / gridDim.x;
+  const int64_t j0 = (int64_t)blockIdx.x * per, j1 = min(n_list, j0 + per);
   double nr = 0.0, nu = 0.0, W = 0.0;
-  for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+  for (int64_t j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
+    const int64_t i = rows[j];
     const uint32_t m = mask[i];
-    if (!m) continue;
     for (int q = 0; q < t.n_con; ++q) {
       const ConEntry& c = t.con[q];
       if (!((m >> c.bit) & 1u)) continue;
@@ -1843,17 +1466,17 @@ void launch_row_objective(const Geometry& g, const Tables& t, const float2* yw, 
 }
 
 void launch_final_check(const Geometry& g, const Tables& t, const double2* y64, const uint32_t* mask,
-                        const double* dd, const double* ll, const double* dl, int64_t n_hot,
+                        const double* dd, const double* ll, const double* dl, const int64_t* rows, int64_t n_list,
                         double* part, cudaStream_t s) {
-  k_final_check<<<g.row_blocks, kRowThreads, 0, s>>>(t, y64, mask, dd, ll, dl, n_hot, part);
+  k_final_check<<<g.row_blocks, kRowThreads, 0, s>>>(t, y64, mask, dd, ll, dl, rows, n_list, part);
 }
 
 void launch_begin_state(DevState* st, cudaStream_t s) { k_begin_state<<<1, 1, 0, s>>>(st); }
 
 void launch_count_rows(const Geometry& g, const Tables& t, const uint32_t* mask, const double* dd,
-                       const double* ll, const double* dl, int64_t n_hot, double* part,
+                       const double* ll, const double* dl, const int64_t* rows, int64_t n_list, double* part,
                        cudaStream_t s) {
-  k_count_rows<<<g.row_blocks, kRowThreads, 0, s>>>(t, mask, dd, ll, dl, n_hot, part);
+  k_count_rows<<<g.row_blocks, kRowThreads, 0, s>>>(t, mask, dd, ll, dl, rows, n_list, part);
 }
 
 void launch_scatter_y(const float2* y, const int64_t* voxel, int64_t n, float* a, float* b,
@@ -1867,309 +1490,6 @@ static unsigned grid_for(int64_t work, int per_block, int cap) {
   if (b < 1) b = 1;
   if (b > cap) b = cap;
   return (unsigned)b;
-}
-
-void launch_validate(const int64_t* rp, const int32_t* col, const float* D, const float* L,
-                     int64_t n_rows, int32_t n_cols, int64_t, int* err, cudaStream_t s) {
-  if (n_rows == 0) return;
-  k_validate<<<grid_for(n_rows, 8, 65535), 256, 0, s>>>(rp, col, D, L, n_rows, n_cols, err);
-}
-
-void launch_gather_rows(const int64_t* rp_src, const int64_t* src_row, const int64_t* rp_dst,
-                        int64_t n_rows, const int32_t* col_src, const float* D_src,
-                        const float* L_src, int32_t* col_dst, float* D_dst, float* L_dst,
-                        cudaStream_t s) {
-  if (n_rows == 0) return;
-  k_gather_rows<<<grid_for(n_rows, 8, 65535), 256, 0, s>>>(rp_src, src_row, rp_dst, n_rows, col_src,
-                                                          D_src, L_src, col_dst, D_dst, L_dst);
-}
-
-void launch_quantize(int fmt, const int64_t* rp, int64_t n_rows, const float* D, const float* L,
-                     void* qD, void* qL, float* sD, float* sL, cudaStream_t s) {
-  if (n_rows == 0) return;
-  const unsigned gb = grid_for(n_rows, 8, 65535);
-  if (fmt == 1)
-    k_quantize<__nv_bfloat16><<<gb, 256, 0, s>>>(fmt, rp, n_rows, D, L, (__nv_bfloat16*)qD,
-                                                  (__nv_bfloat16*)qL, sD, sL);
-  else
-    k_quantize<__half><<<gb, 256, 0, s>>>(fmt, rp, n_rows, D, L, (__half*)qD, (__half*)qL, sD, sL);
-}
-
-void launch_moments(int fmt, const int64_t* rp, int64_t n_rows, const void* Dv, const void* Lv,
-                    const float* sD, const float* sL, double* dd, double* ll, double* dl,
-                    cudaStream_t s) {
-  if (n_rows == 0) return;
-  const unsigned gb = grid_for(n_rows, 8, 65535);
-  if (fmt == 1)
-    k_moments<__nv_bfloat16><<<gb, 256, 0, s>>>(rp, n_rows, (const __nv_bfloat16*)Dv,
-                                                 (const __nv_bfloat16*)Lv, sD, sL, dd, ll, dl);
-  else if (fmt == 2)
-    k_moments<__half><<<gb, 256, 0, s>>>(rp, n_rows, (const __half*)Dv, (const __half*)Lv, sD, sL, dd,
-                                          ll, dl);
-  else
-    k_moments<float><<<gb, 256, 0, s>>>(rp, n_rows, (const float*)Dv, (const float*)Lv, sD, sL, dd,
-                                         ll, dl);
-}
-
-constexpr size_t kCscSmemMax = 200 * 1024;  // per-block column table kept in shared memory
-
-void launch_csc_count(const int64_t* rp, const int32_t* col, const int64_t* blk_row, int n_blk,
-                      int32_t n_cols, int32_t* cnt, cudaStream_t s) {
-  const size_t smem = (size_t)n_cols * sizeof(int32_t);
-  if (smem <= kCscSmemMax) {
-    cudaFuncSetAttribute(k_csc_count<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_csc_count<true><<<n_blk, 1024, smem, s>>>(rp, col, blk_row, n_cols, cnt);
-  } else {
-    k_csc_count<false><<<n_blk, 1024, 0, s>>>(rp, col, blk_row, n_cols, cnt);
-  }
-}
-
-void launch_csc_colsum(const int32_t* cnt, int n_blk, int32_t n_cols, int64_t* tot, cudaStream_t s) {
-  k_csc_colsum<<<(n_cols + 255) / 256, 256, 0, s>>>(cnt, n_blk, n_cols, tot);
-}
-
-void launch_csc_offsets(int32_t* cnt, int n_blk, int32_t n_cols, const int64_t* cp, cudaStream_t s) {
-  k_csc_offsets<<<(n_cols + 255) / 256, 256, 0, s>>>(cnt, n_blk, n_cols, cp);
-}
-
-// The same stable transpose, rows taken kFillWinRows at a time: the order of
-// a column's entries within a window of rows is recovered from a per-column
-// bit mask of the window rows that hold the column, so a window costs three
-// block barriers instead of one per row.  For each window:
-//   A  every entry (row r, column c) sets bit r - g0 of mask[c] (atomic OR,
-//      order-independent);
-//   B  it goes to position cur[c] + popc(mask[c] below bit r - g0): the rows
-//      of the window before r that hold c come first, as in row order;
-//   C  the first entry of each column advances cur[c] by popc(mask[c]) and
-//      clears the mask.
-// Two 16-bit masks share a 32-bit word.  Shared memory: the block's cursors
-// and masks (6 bytes per column) and a chunk of row pointers.  The result
-// equals k_csc_fill's bit for bit.
-constexpr int kFillWinRows = 16;
-constexpr int kFillK = 2;  // entries per thread a window holds in registers (else the loop form)
-#ifndef FO_FILL_WIN
-#define FO_FILL_WIN 1  // 0: the row-by-row k_csc_fill for every plan
-#endif
-#ifndef FO_FILL_REC
-#define FO_FILL_REC 1  // 1: the window fill stores records, then k_csc_split
-#endif
-
-__device__ __forceinline__ int fill_win_row(const int64_t* wrp, int nr, int64_t p) {
-  int lo = 0, hi = nr - 1;  // the window row r with wrp[r] <= p < wrp[r + 1]
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (wrp[mid] <= p) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
-
-// With `rec`, an entry is one record store (row and both values: 16 bytes
-// for FP32, 8 for 16-bit values) instead of three scattered 4- or 2-byte
-// stores, and k_csc_split writes the three arrays afterwards with coalesced
-// stores: scattered stores are limited by their count, not their bytes.
-template <typename VT> struct FillRec;
-template <> struct FillRec<float> { using T = int4; };
-template <> struct FillRec<uint16_t> { using T = uint2; };
-__device__ __forceinline__ int4 fill_rec(int32_t r, float d, float l) {
-  return make_int4(r, __float_as_int(d), __float_as_int(l), 0);
-}
-__device__ __forceinline__ uint2 fill_rec(int32_t r, uint16_t d, uint16_t l) {
-  return make_uint2((uint32_t)r, (uint32_t)d | ((uint32_t)l << 16));
-}
-
-template <typename VT>
-__global__ void k_csc_split(const typename FillRec<VT>::T* __restrict__ rec, int64_t n, int32_t* __restrict__ row_out,
-                            VT* __restrict__ DT, VT* __restrict__ LT) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const auto v = rec[i];
-  if constexpr (sizeof(VT) == 4) {
-    row_out[i] = v.x;
-    DT[i] = __int_as_float(v.y);
-    LT[i] = __int_as_float(v.z);
-  } else {
-    row_out[i] = (int32_t)v.x;
-    DT[i] = (uint16_t)(v.y & 0xffffu);
-    LT[i] = (uint16_t)(v.y >> 16);
-  }
-}
-
-template <typename VT>
-__global__ void __launch_bounds__(kFillThreads) k_csc_fill_win(
-    const int64_t* __restrict__ rp, const int32_t* __restrict__ col, const VT* __restrict__ Dv,
-    const VT* __restrict__ Lv, const int64_t* __restrict__ blk_row, int32_t n_cols,
-    const int32_t* __restrict__ cursor, int32_t* __restrict__ row_out, VT* __restrict__ DT,
-    VT* __restrict__ LT, typename FillRec<VT>::T* __restrict__ rec) {
-  extern __shared__ __align__(16) unsigned char fill_sh[];
-  int32_t* cur = reinterpret_cast<int32_t*>(fill_sh);
-  uint32_t* mask = reinterpret_cast<uint32_t*>(fill_sh + (size_t)n_cols * sizeof(int32_t));
-  int64_t* srp = reinterpret_cast<int64_t*>(
-      fill_sh + (((size_t)n_cols * sizeof(int32_t) + (size_t)((n_cols + 1) / 2) * sizeof(uint32_t) + 15) & ~(size_t)15));
-  const int b = blockIdx.x;
-  const int64_t r0 = blk_row[b], r1 = blk_row[b + 1];
-  if (r0 >= r1) return;
-  const int32_t* gcur = cursor + (int64_t)b * n_cols;
-  for (int j = threadIdx.x; j < n_cols; j += blockDim.x) cur[j] = gcur[j];
-  for (int j = threadIdx.x; j < (n_cols + 1) / 2; j += blockDim.x) mask[j] = 0u;
-  // row pointers staged kFillRows rows at a time; windows of kFillWinRows rows
-  for (int64_t c0 = r0; c0 < r1; c0 += kFillRows) {
-    const int nc = (int)(r1 - c0 < kFillRows ? r1 - c0 : kFillRows);
-    __syncthreads();  // the previous chunk is done with srp, cur and mask
-    for (int i = threadIdx.x; i <= nc; i += blockDim.x) srp[i] = rp[c0 + i];
-    __syncthreads();
-    for (int w0 = 0; w0 < nc; w0 += kFillWinRows) {
-      const int nr = nc - w0 < kFillWinRows ? nc - w0 : kFillWinRows;
-      const int64_t* wrp = srp + w0;
-      const int64_t g0 = c0 + w0;
-      const int64_t e0 = wrp[0], e1 = wrp[nr];
-      if (w0 > 0) __syncthreads();  // the previous window's C is done with cur and mask
-      if (e1 - e0 <= (int64_t)kFillK * kFillThreads) {
-        // the window's entries in registers: one round of loads, then the
-        // three steps on shared memory only
-        int cc[kFillK], rr[kFillK];
-        VT dv[kFillK], lv[kFillK];
-#pragma unroll
-        for (int k = 0; k < kFillK; ++k) {
-          const int64_t p = e0 + threadIdx.x + (int64_t)k * kFillThreads;
-          cc[k] = -1;
-          if (p < e1) {
-            cc[k] = col[p];
-            dv[k] = Dv[p];
-            lv[k] = Lv[p];
-            rr[k] = fill_win_row(wrp, nr, p);
-          }
-        }
-#pragma unroll
-        for (int k = 0; k < kFillK; ++k)
-          if (cc[k] >= 0) atomicOr(&mask[cc[k] >> 1], 1u << ((cc[k] & 1) * 16 + rr[k]));
-        __syncthreads();
-        uint32_t mk[kFillK];
-#pragma unroll
-        for (int k = 0; k < kFillK; ++k) {
-          if (cc[k] < 0) continue;
-          const int c = cc[k], r = rr[k];
-          mk[k] = (mask[c >> 1] >> ((c & 1) * 16)) & 0xffffu;
-          const int32_t pos = cur[c] + __popc(mk[k] & ((1u << r) - 1u));
-          if (rec) {
-            rec[pos] = fill_rec((int32_t)(g0 + r), dv[k], lv[k]);
-          } else {
-            row_out[pos] = (int32_t)(g0 + r);
-            DT[pos] = dv[k];
-            LT[pos] = lv[k];
-          }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < kFillK; ++k) {
-          if (cc[k] < 0) continue;
-          const int c = cc[k];
-          if ((mk[k] & ((1u << rr[k]) - 1u)) == 0u) {  // the column's first row in the window
-            cur[c] += __popc(mk[k]);
-            atomicAnd(&mask[c >> 1], ~(0xffffu << ((c & 1) * 16)));
-          }
-        }
-        continue;
-      }
-      // A: the window rows that hold each column
-      for (int64_t p = e0 + threadIdx.x; p < e1; p += kFillThreads) {
-        const int c = col[p];
-        const int r = fill_win_row(wrp, nr, p);
-        atomicOr(&mask[c >> 1], 1u << ((c & 1) * 16 + r));
-      }
-      __syncthreads();
-      // B: each entry to its place
-      for (int64_t p = e0 + threadIdx.x; p < e1; p += kFillThreads) {
-        const int c = col[p];
-        const int r = fill_win_row(wrp, nr, p);
-        const uint32_t m = (mask[c >> 1] >> ((c & 1) * 16)) & 0xffffu;
-        const int32_t pos = cur[c] + __popc(m & ((1u << r) - 1u));
-        if (rec) {
-          rec[pos] = fill_rec((int32_t)(g0 + r), Dv[p], Lv[p]);
-        } else {
-          row_out[pos] = (int32_t)(g0 + r);
-          DT[pos] = Dv[p];
-          LT[pos] = Lv[p];
-        }
-      }
-      __syncthreads();
-      // C: advance the cursors past the window, clear the masks
-      for (int64_t p = e0 + threadIdx.x; p < e1; p += kFillThreads) {
-        const int c = col[p];
-        const int r = fill_win_row(wrp, nr, p);
-        const uint32_t m = (mask[c >> 1] >> ((c & 1) * 16)) & 0xffffu;
-        if ((m & ((1u << r) - 1u)) == 0u) {  // the column's first row in the window
-          cur[c] += __popc(m);
-          atomicAnd(&mask[c >> 1], ~(0xffffu << ((c & 1) * 16)));
-        }
-      }
-    }
-  }
-}
-
-template <typename VT>
-size_t csc_fill_win_smem(int32_t n_cols) {
-  return (((size_t)n_cols * sizeof(int32_t) + (size_t)((n_cols + 1) / 2) * sizeof(uint32_t) + 15) & ~(size_t)15) +
-         (kFillRows + 1) * sizeof(int64_t);
-}
-
-// Window length W (a multiple of kFillAlign, at most 8192) from the shared
-// memory left after the row-pointer chunk and, when they fit with W >= 1024,
-// the block's cursors.
-template <typename VT>
-static void fill_inst(const Geometry& g, const int64_t* rp, const int32_t* col, const void* Dv, const void* Lv,
-                      const int64_t* blk_row, int n_blk, int32_t n_cols, int32_t* cursor, int32_t* row_out,
-                      void* DT, void* LT, int* err, void* rec, int64_t n_out, cudaStream_t s) {
-  const size_t limit = g.smem_limit;
-  if (FO_FILL_WIN && csc_fill_win_smem<VT>(n_cols) <= limit) {
-    using R = typename FillRec<VT>::T;
-    const size_t smem = csc_fill_win_smem<VT>(n_cols);
-    cudaFuncSetAttribute(k_csc_fill_win<VT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_csc_fill_win<VT><<<n_blk, kFillThreads, smem, s>>>(rp, col, (const VT*)Dv, (const VT*)Lv, blk_row, n_cols,
-                                                          cursor, row_out, (VT*)DT, (VT*)LT, (R*)rec);
-    if (rec && n_out > 0)
-      k_csc_split<VT><<<(unsigned)((n_out + 255) / 256), 256, 0, s>>>((const R*)rec, n_out, row_out, (VT*)DT,
-                                                                       (VT*)LT);
-    return;
-  }
-  const size_t per_w = 2 * (sizeof(int32_t) + 2 * sizeof(VT));
-  auto w_for = [&](bool sc) -> int {
-    const size_t fixed = csc_fill_smem<VT>(0, n_cols, sc);
-    if (fixed >= limit) return 0;
-    const size_t w = std::min<size_t>((limit - fixed) / per_w, 8192) & ~(size_t)(kFillAlign - 1);
-    return (int)w;
-  };
-  bool sc = true;
-  int W = w_for(true);
-  if (W < 1024) {
-    sc = false;
-    W = w_for(false);
-  }
-  const size_t smem = csc_fill_smem<VT>(W, n_cols, sc);
-  if (sc) {
-    cudaFuncSetAttribute(k_csc_fill<VT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_csc_fill<VT, true><<<n_blk, kFillThreads, smem, s>>>(rp, col, (const VT*)Dv, (const VT*)Lv, blk_row, n_cols,
-                                                            cursor, row_out, (VT*)DT, (VT*)LT, W, err);
-  } else {
-    cudaFuncSetAttribute(k_csc_fill<VT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_csc_fill<VT, false><<<n_blk, kFillThreads, smem, s>>>(rp, col, (const VT*)Dv, (const VT*)Lv, blk_row, n_cols,
-                                                             cursor, row_out, (VT*)DT, (VT*)LT, W, err);
-  }
-}
-
-size_t csc_fill_rec_bytes(const Geometry& g, int fmt, int32_t n_cols) {
-  if (!FO_FILL_WIN || !FO_FILL_REC) return 0;
-  if (fmt == 0) return csc_fill_win_smem<float>(n_cols) <= g.smem_limit ? sizeof(int4) : 0;
-  return csc_fill_win_smem<uint16_t>(n_cols) <= g.smem_limit ? sizeof(uint2) : 0;
-}
-
-void launch_csc_fill(const Geometry& g, int fmt, const int64_t* rp, const int32_t* col, const void* Dv,
-                     const void* Lv, const int64_t* blk_row, int n_blk, int32_t n_cols, int32_t* cursor,
-                     int32_t* row_out, void* DT, void* LT, int* err, void* rec, int64_t n_out, cudaStream_t s) {
-  if (fmt == 0)
-    fill_inst<float>(g, rp, col, Dv, Lv, blk_row, n_blk, n_cols, cursor, row_out, DT, LT, err, rec, n_out, s);
-  else
-    fill_inst<uint16_t>(g, rp, col, Dv, Lv, blk_row, n_blk, n_cols, cursor, row_out, DT, LT, err, rec, n_out, s);
 }
 
 void launch_dequant_csc(int fmt, const int64_t* cp, int32_t n_cols, const int32_t* row, const void* DT,
@@ -2397,22 +1717,6 @@ void launch_sweep_finish(const Geometry& g, int n, const float* x, float* out, i
                          LogEntry* log, cudaStream_t s) {
   const unsigned gb = (unsigned)std::max(1, std::min(g.n_sms, (n + 255) / 256));
   k_sweep_finish<<<gb, 256, 0, s>>>(n, x, out, in_solve, st, log);
-}
-
-__global__ void __launch_bounds__(256) k_narrow_idx(const int4* __restrict__ in, uint2* __restrict__ out, int64_t n4) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += stride) {
-    const int4 v = __ldcs(in + i);
-    out[i] = make_uint2(((uint32_t)v.x & 0xffffu) | ((uint32_t)v.y << 16),
-                        ((uint32_t)v.z & 0xffffu) | ((uint32_t)v.w << 16));
-  }
-}
-
-void launch_narrow_idx(const int32_t* in, uint16_t* out, int64_t n, cudaStream_t s) {
-  const int64_t n4 = n / 4;
-  if (n4 == 0) return;
-  const unsigned grid = (unsigned)std::min<int64_t>((n4 + 255) / 256, 152 * 8);
-  k_narrow_idx<<<grid, 256, 0, s>>>(reinterpret_cast<const int4*>(in), reinterpret_cast<uint2*>(out), n4);
 }
 
 // Based 16-bit row indices of the CSC (see BlockBase): one warp per block of

@@ -242,10 +242,10 @@ int64_t fredopt_footprint_bytes(int64_t n_vox, int32_t n_spots, int64_t nnz, int
   const int fmt = format & 0xff;
   const int64_t vb = fmt == FREDOPT_FP32 ? 4 : 2;
   const int64_t na = ((nnz + 255) & ~255LL) + fo::kPadElems;
-  // peaks of the load: FP32 upload + gathered copy; the CSC fill's CSR + CSC
-  // + one scratch record per entry (16 bytes with FP32 values, 8 with 16-bit);
-  // while the 16-bit index copies are made, CSR + CSC (int32 indices) + both
-  // 16-bit copies
+  // bounds of the load's peaks: FP32 upload + the stored plan; CSR + CSC
+  // (int32 indices) + both 16-bit copies; CSR + CSC + 16 bytes per entry with
+  // FP32 values, 8 with 16-bit (the transpose's table of group starts is at
+  // most 8)
   const int64_t rec = vb == 4 ? 16 : 8;
   const int64_t load_peak =
       std::max(std::max(2 * na * 12, na * (2 * (4 + 2 * vb) + 4)), na * (2 * (4 + 2 * vb) + rec));
