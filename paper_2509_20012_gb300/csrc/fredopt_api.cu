@@ -124,6 +124,9 @@ struct fredopt_ctx {
   DBuf<float> w, g, xbuf, gtmp;
   DBuf<float2> yw, yg, r, gam, yall;
   DBuf<double2> y64;
+  // y64 / yall were zeroed since the load: the products write rows with
+  // nonzeros only, so the other rows stay 0
+  bool y64_zeroed = false, yall_zeroed = false;
   DBuf<float> chunk_sum, fout_a, fout_b, vin_a, vin_b;
   DBuf<uint8_t> vol_buf;  // volume statistics scratch
 
@@ -317,7 +320,7 @@ FwdArgs fwd_args(fredopt_t h, bool hot) {
   a.n_x_pad = h->n_pad;
   a.mask = h->mask.p;
   a.n_hot = h->n_hot;
-  a.n_warps = a.sched ? h->n_tiles_hot : h->geo.fwd_warps;
+  a.n_warps = a.sched ? h->n_tiles_hot : hot ? h->geo.fwd_warps : h->geo_full.fwd_warps;
   a.st = h->st.p;
   a.voxel = h->perm ? h->voxel.p : nullptr;
   return a;
@@ -563,15 +566,18 @@ int set_fwd_schedule(fredopt_t h, int64_t row_cost) {
   const int W = h->geo.fwd_warps;
   const int64_t *rp = h->rp.p, hot = h->n_hot_ne, cold = h->n_cold_ne;
   CK(h->warp_row_hot.fit(2 * (size_t)W));
-  CK(h->warp_row_all.fit(2 * (size_t)W));
+  // every row: single products and final passes use the whole GPU whatever
+  // the plan's launch shapes (a row's sums do not depend on them)
+  const int A = h->geo_full.fwd_warps;
+  CK(h->warp_row_all.fit(2 * (size_t)A));
   CK(h->tile_row_hot.fit(2 * (size_t)kGuidedTilesPerWarp * W));
   launch_tiles(TileArgs{TileArgs::PAIRS, rp, 0, hot, 0, 0, W, 0, row_cost, h->warp_row_hot.p, nullptr}, h->stream);
-  // every row: the warps shared between streamed and other rows by their cost
+  // the warps shared between streamed and other rows by their cost
   const double c0 = (double)h->nnz_hot + (double)row_cost * (double)hot;
   const double c1 = (double)(h->nnz - h->nnz_hot) + (double)row_cost * (double)cold;
-  int w0 = hot > 0 || cold == 0 ? W : 0;
-  if (hot > 0 && cold > 0) w0 = std::max(1, std::min(W - 1, (int)std::llround(W * (c0 / (c0 + c1)))));
-  launch_tiles(TileArgs{TileArgs::PAIRS, rp, 0, hot, h->n_hot, h->n_hot + cold, w0, W - w0, row_cost,
+  int w0 = hot > 0 || cold == 0 ? A : 0;
+  if (hot > 0 && cold > 0) w0 = std::max(1, std::min(A - 1, (int)std::llround(A * (c0 / (c0 + c1)))));
+  launch_tiles(TileArgs{TileArgs::PAIRS, rp, 0, hot, h->n_hot, h->n_hot + cold, w0, A - w0, row_cost,
                         h->warp_row_all.p, nullptr}, h->stream);
   launch_tiles(TileArgs{TileArgs::GUIDED_PAIRS, rp, 0, hot, 0, 0, W, 0, row_cost, h->tile_row_hot.p, nullptr},
                h->stream);
@@ -636,9 +642,24 @@ int check_sticky(fredopt_t h) {
   return FREDOPT_OK;
 }
 
-// FP64 pass of every row for w (host or device per flags; null = the current
-// iterate of a begun solve) into y64, as in fredopt_end.
-int final_pass_y64(fredopt_t h, const float* w, uint32_t flags) {
+// CTAs of the passes over the listed structure rows
+int list_blocks(fredopt_t h) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>(h->geo_full.row_blocks, (h->n_con_rows + 255) / 256));
+}
+
+int ready_y64(fredopt_t h) {
+  const size_t n = (size_t)std::max<int64_t>(1, h->V);
+  if (!h->y64.p || h->y64.n < n) h->y64_zeroed = false;
+  CK(h->y64.ensure(n));
+  if (!h->y64_zeroed) CK(cudaMemsetAsync(h->y64.p, 0, n * sizeof(double2), h->stream));
+  h->y64_zeroed = true;
+  return FREDOPT_OK;
+}
+
+// Double-float pass for w (host or device per flags; null = the current
+// iterate of a begun solve) into y64, as in fredopt_end: over every row, or
+// over the structure rows alone (one row per tile, claimed in order).
+int final_pass_y64(fredopt_t h, const float* w, uint32_t flags, bool structures) {
   cudaStream_t s = h->stream;
   const float* x = nullptr;
   if (w) {
@@ -649,27 +670,22 @@ int final_pass_y64(fredopt_t h, const float* w, uint32_t flags) {
     if (!h->begun) return fail(h, FREDOPT_ERR_NOT_LOADED, "w is null and no solve is begun");
     x = h->w.p;
   }
-  CK(h->y64.ensure(std::max<int64_t>(1, h->V)));
-  CK(cudaMemsetAsync(h->y64.p, 0, std::max<int64_t>(1, h->V) * sizeof(double2), s));
+  const int rc = ready_y64(h);
+  if (rc) return rc;
   FwdArgs fa = fwd_args(h, false);
   fa.x = x;
   fa.y64 = h->y64.p;
   fa.dose_out = nullptr;
   fa.letd_out = nullptr;
-  run(h, 0, [&] { launch_forward(h->geo, h->fmt, EPI_FINAL, false, fa, h->tab, s); });
+  if (structures) {
+    if (h->n_con_ne == 0) return FREDOPT_OK;  // every structure value is 0
+    fa.rows = h->con_rows.p;
+    fa.sched = h->fsched.p;
+    fa.n_warps = (int32_t)h->n_con_ne;
+  }
+  run(h, 0, [&] { launch_forward(h->geo_full, h->fmt, EPI_FINAL, false, fa, h->tab, s); });
   CK(cudaGetLastError());
   return FREDOPT_OK;
-}
-
-// Rank k (1 = largest) of the value received by the fraction `frac` of n
-// voxels: ceil(frac * n), a product within 1e-9 * max(1, product) of an
-// integer counting as that integer, kept in [1, n].
-int64_t at_volume_rank(double frac, int64_t n) {
-  volatile double t = frac * (double)n;  // rounded product (never fused with what follows)
-  const double tv = t;
-  const double r = std::floor(tv + 0.5);
-  const double k = (std::fabs(tv - r) <= 1e-9 * std::max(1.0, tv)) ? r : std::ceil(tv);
-  return std::min<int64_t>(std::max<int64_t>((int64_t)k, 1), n);
 }
 
 float key_to_float(uint32_t key) {
@@ -836,6 +852,7 @@ int fredopt_load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t 
     h->y64.release(); h->yall.release(); h->fout_a.release(); h->fout_b.release();
     h->vin_a.release(); h->vin_b.release();
   }
+  h->y64_zeroed = h->yall_zeroed = false;
   h->covf.release();
   h->ucoef.release();
   if (fmt == FREDOPT_FP32) {
@@ -1062,8 +1079,8 @@ int fredopt_load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t 
   h->off_g = h->off_bc + 2 * max_tiles;
   h->off_k2 = h->off_g + G.col_blocks;
   h->off_fin = h->off_k2 + 4 * G.row_blocks;
-  h->off_cnt = h->off_fin + 8 * G.row_blocks;
-  h->off_stage = h->off_cnt + 3 * G.row_blocks;
+  h->off_cnt = h->off_fin + 8 * h->geo_full.row_blocks;
+  h->off_stage = h->off_cnt + 3 * h->geo_full.row_blocks;
   h->off_btab = h->off_stage + 4 * kFinishBlocks;
   h->n_part = h->off_btab + kBetaTable;
   h->btab_alpha = -1.0;  // the table is refilled at the next fredopt_begin
@@ -1099,15 +1116,16 @@ int fredopt_set_constraints(fredopt_t h, int n, const fredopt_constraint* c) {
     h->tab.con[i].bound = c[i].bound;
     h->tab.con[i].prio = c[i].priority;
   }
+  const int fb = list_blocks(h);
   double* pc = h->part.p + h->off_cnt;
-  launch_count_rows(h->geo, h->tab, h->mask.p, h->mdd.p, h->mll.p, h->mdl.p, h->con_rows.p,
+  launch_count_rows(fb, h->tab, h->mask.p, h->mdd.p, h->mll.p, h->mdl.p, h->con_rows.p,
                     h->n_con_rows, pc, h->stream);
   CK(cudaGetLastError());
-  std::vector<double> hp(3 * h->geo.row_blocks);
+  std::vector<double> hp(3 * fb);
   CK(cudaMemcpyAsync(hp.data(), pc, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
   double nr = 0, nu = 0, W = 0;
-  for (int b = 0; b < h->geo.row_blocks; ++b) {
+  for (int b = 0; b < fb; ++b) {
     nr += hp[3 * b];
     nu += hp[3 * b + 1];
     W += hp[3 * b + 2];
@@ -1313,7 +1331,7 @@ int fredopt_end(fredopt_t h, float* w_out, float* dose_out, float* letd_out, fre
   if (!h->begun) return fail(h, FREDOPT_ERR_NOT_LOADED, "call fredopt_begin first");
   DeviceGuard dg(h->device);
   cudaStream_t s = h->stream;
-  const Geometry& G = h->geo;
+  const int fb = list_blocks(h);
   if (h->it_pending) {
     float ms = 0.f;
     CK(cudaEventSynchronize(h->ev_it1));
@@ -1321,7 +1339,8 @@ int fredopt_end(fredopt_t h, float* w_out, float* dose_out, float* letd_out, fre
     h->it_pending = false;
   }
   // final double-float-accumulated product over every row
-  CK(h->y64.ensure(std::max<int64_t>(1, h->V)));
+  rc = ready_y64(h);
+  if (rc) return rc;
   float* dptr = nullptr;
   float* lptr = nullptr;
   if (dose_out || letd_out) {
@@ -1335,7 +1354,6 @@ int fredopt_end(fredopt_t h, float* w_out, float* dose_out, float* letd_out, fre
       lptr = letd_out ? h->fout_b.p : nullptr;
     }
   }
-  CK(cudaMemsetAsync(h->y64.p, 0, std::max<int64_t>(1, h->V) * sizeof(double2), s));
   if (dptr) CK(cudaMemsetAsync(dptr, 0, h->V * sizeof(float), s));
   if (lptr) CK(cudaMemsetAsync(lptr, 0, h->V * sizeof(float), s));
   FwdArgs fa = fwd_args(h, false);
@@ -1343,11 +1361,11 @@ int fredopt_end(fredopt_t h, float* w_out, float* dose_out, float* letd_out, fre
   fa.y64 = h->y64.p;
   fa.dose_out = dptr;
   fa.letd_out = lptr;
-  run(h, 0, [&] { launch_forward(G, h->fmt, EPI_FINAL, false, fa, h->tab, s); });
+  run(h, 0, [&] { launch_forward(h->geo_full, h->fmt, EPI_FINAL, false, fa, h->tab, s); });
   double* pf = h->part.p + h->off_fin;
-  run(h, 5, [&] { launch_final_check(G, h->tab, h->y64.p, h->mask.p, h->mdd.p, h->mll.p, h->mdl.p, h->con_rows.p, h->n_con_rows, pf, s); });
+  run(h, 5, [&] { launch_final_check(fb, h->tab, h->y64.p, h->mask.p, h->mdd.p, h->mll.p, h->mdl.p, h->con_rows.p, h->n_con_rows, pf, s); });
   CK(cudaGetLastError());
-  std::vector<double> hp(8 * G.row_blocks);
+  std::vector<double> hp(8 * fb);
   CK(cudaMemcpyAsync(hp.data(), pf, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
   DevState d;
   CK(cudaMemcpyAsync(&d, h->st.p, sizeof(DevState), cudaMemcpyDeviceToHost, s));
@@ -1367,7 +1385,7 @@ int fredopt_end(fredopt_t h, float* w_out, float* dose_out, float* letd_out, fre
     rep->n_rows = h->n_rows_reach;
     rep->unreachable_rows = h->n_unreach;
     double nv = 0.0, f = 0.0;
-    for (int b = 0; b < G.row_blocks; ++b) {
+    for (int b = 0; b < fb; ++b) {
       for (int q = 0; q < 6; ++q) rep->max_violation[q] = std::max(rep->max_violation[q], hp[8 * b + q]);
       nv += hp[8 * b + 6];
       f += hp[8 * b + 7];
@@ -1465,12 +1483,14 @@ int fredopt_forward(fredopt_t h, const float* w, float* dose_out, float* lw_out,
   join_in(h);
   rc = load_spot_vec(h, h->xbuf, w, flags);
   if (rc) return rc;
+  if (!h->yall.p || h->yall.n < (size_t)std::max<int64_t>(1, h->V)) h->yall_zeroed = false;
   CK(h->yall.ensure(std::max<int64_t>(1, h->V)));
-  CK(cudaMemsetAsync(h->yall.p, 0, std::max<int64_t>(1, h->V) * sizeof(float2), s));
+  if (!h->yall_zeroed) CK(cudaMemsetAsync(h->yall.p, 0, std::max<int64_t>(1, h->V) * sizeof(float2), s));
+  h->yall_zeroed = true;
   FwdArgs fa = fwd_args(h, false);
   fa.x = h->xbuf.p;
   fa.y = h->yall.p;
-  run(h, 0, [&] { launch_forward(h->geo, h->fmt, EPI_STORE, h->hint_fwd, fa, h->tab, s); });
+  run(h, 0, [&] { launch_forward(h->geo_full, h->fmt, EPI_STORE, h->hint_fwd, fa, h->tab, s); });
   float *da = dose_out, *db = lw_out;
   if (!dev_ptr(flags)) {
     CK(h->fout_a.ensure(std::max<int64_t>(1, h->V)));
@@ -1675,67 +1695,63 @@ int fredopt_volume_stats(fredopt_t h, const float* w, uint32_t flags, int n_req,
   DeviceGuard dg(h->device);
   cudaStream_t s = h->stream;
   join_in(h);
-  rc = final_pass_y64(h, w, flags);
+  rc = final_pass_y64(h, w, flags, true);
   if (rc) return rc;
 
-  // scratch: edges | counts | n_vox | digit histograms | selection slots
+  // scratch: inputs (edges | fractions), then results (counts | n_vox |
+  // selection slots), then digit histograms; one copy each way
   const int n_sel = (int)fracs.size();
-  const size_t o_edges = 0;
-  const size_t o_counts = o_edges + align256(std::max<size_t>(1, edges.size()) * sizeof(float));
+  const size_t o_fracs = align256(std::max<size_t>(1, edges.size()) * sizeof(float));
+  const size_t o_counts = o_fracs + align256(std::max(1, n_sel) * sizeof(double));
   const size_t o_nvox = o_counts + align256(std::max(1, n_bins) * sizeof(unsigned long long));
-  const size_t o_hist = o_nvox + align256(n_req * sizeof(unsigned long long));
-  const size_t o_slot = o_hist + align256(std::max(1, n_sel) * 256 * sizeof(uint32_t));
-  const size_t total = o_slot + align256(std::max(1, n_sel) * sizeof(SelSlot));
+  const size_t o_slot = o_nvox + align256(n_req * sizeof(unsigned long long));
+  const size_t o_hist = o_slot + align256(std::max(1, n_sel) * sizeof(SelSlot));
+  const size_t total = o_hist + align256(std::max(1, n_sel) * 256 * sizeof(uint32_t));
   CK(h->vol_buf.ensure(total));
   uint8_t* base = h->vol_buf.p;
-  CK(cudaMemsetAsync(base + o_counts, 0, o_slot - o_counts, s));
-  if (!edges.empty())
-    CK(cudaMemcpyAsync(base + o_edges, edges.data(), edges.size() * sizeof(float), cudaMemcpyHostToDevice, s));
+  std::vector<uint8_t> io(std::max(o_counts, o_hist - o_counts));
+  if (!edges.empty()) std::memcpy(io.data(), edges.data(), edges.size() * sizeof(float));
+  if (n_sel) std::memcpy(io.data() + o_fracs, fracs.data(), n_sel * sizeof(double));
+  CK(cudaMemsetAsync(base + o_counts, 0, total - o_counts, s));
+  CK(cudaMemcpyAsync(base, io.data(), o_counts, cudaMemcpyHostToDevice, s));
 
   va.y64 = h->y64.p;
   va.mask = h->mask.p;
-  va.n_rows = h->n_hot;  // every structure voxel is a streamed row
+  va.rows = h->con_rows.p;  // every structure voxel is a streamed row
+  va.n_rows = h->n_con_rows;
   va.c = h->tab.c;
   va.n_req = n_req;
   va.n_edges = (int)edges.size();
   va.n_bins = n_bins;
-  va.edges = reinterpret_cast<const float*>(base + o_edges);
+  va.edges = reinterpret_cast<const float*>(base);
   va.counts = reinterpret_cast<unsigned long long*>(base + o_counts);
   va.n_vox = reinterpret_cast<unsigned long long*>(base + o_nvox);
   run(h, 5, [&] { launch_vol_hist(h->geo, va, s); });
   CK(cudaGetLastError());
-  std::vector<unsigned long long> nvox(n_req);
-  CK(cudaMemcpyAsync(nvox.data(), va.n_vox, n_req * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-
-  std::vector<SelSlot> slots(std::max(1, n_sel));
   if (n_sel > 0) {
-    for (int j = 0; j < n_sel; ++j) {
-      const int64_t n = (int64_t)nvox[sel_req[j]];
-      slots[j].prefix = 0u;
-      slots[j].pad = 0u;
-      slots[j].k = n > 0 ? (uint64_t)at_volume_rank(fracs[j], n) : 0u;
-    }
+    for (int j = 0; j < n_sel; ++j) sa.req[j] = sel_req[j];
     sa.y64 = h->y64.p;
     sa.mask = h->mask.p;
-    sa.n_rows = h->n_hot;
+    sa.rows = h->con_rows.p;
+    sa.n_rows = h->n_con_rows;
     sa.c = h->tab.c;
     sa.any_bits = va.any_bits;
     sa.n_sel = n_sel;
+    sa.fracs = reinterpret_cast<const double*>(base + o_fracs);
+    sa.n_vox = va.n_vox;
     sa.hist = reinterpret_cast<uint32_t*>(base + o_hist);
     sa.st = reinterpret_cast<SelSlot*>(base + o_slot);
-    CK(cudaMemcpyAsync(sa.st, slots.data(), n_sel * sizeof(SelSlot), cudaMemcpyHostToDevice, s));
     run(h, 5, [&] { launch_vol_select(h->geo, sa, s); });
-    h->launches += 7;  // launch_vol_select enqueues 8 kernels
+    h->launches += kVolSelectLaunches - 1;
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(slots.data(), sa.st, n_sel * sizeof(SelSlot), cudaMemcpyDeviceToHost, s));
   }
-  std::vector<unsigned long long> counts(std::max(1, n_bins));
-  if (n_bins > 0)
-    CK(cudaMemcpyAsync(counts.data(), va.counts, n_bins * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+  CK(cudaMemcpyAsync(io.data(), base + o_counts, o_hist - o_counts, cudaMemcpyDeviceToHost, s));
   rc = check_sticky(h);
   collect_timers(h);
   if (rc) return rc;
+  const unsigned long long* counts = reinterpret_cast<const unsigned long long*>(io.data());
+  const unsigned long long* nvox = reinterpret_cast<const unsigned long long*>(io.data() + (o_nvox - o_counts));
+  const SelSlot* slots = reinterpret_cast<const SelSlot*>(io.data() + (o_slot - o_counts));
   int j = 0;
   for (int i = 0; i < n_req; ++i) {
     fredopt_volume_request& r = req[i];
@@ -1756,7 +1772,7 @@ int fredopt_quantity_map(fredopt_t h, const float* w, int quantity, float* out, 
   DeviceGuard dg(h->device);
   cudaStream_t s = h->stream;
   join_in(h);
-  rc = final_pass_y64(h, w, flags);
+  rc = final_pass_y64(h, w, flags, false);
   if (rc) return rc;
   float* dst = out;
   if (!dev_ptr(flags)) {

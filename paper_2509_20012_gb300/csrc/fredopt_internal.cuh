@@ -90,6 +90,7 @@ struct FwdArgs {
   const float* sD;       // row scales (16-bit storage) or null
   const float* sL;
   const int64_t* warp_row;  // [2 * n_warps]: row range [r0, r1) of each tile (nonempty rows)
+  const int64_t* rows;      // when set, tile j is the single row rows[j] (warp_row unused)
   unsigned int* sched;      // null: warp w streams tile w; else [2] counters of claimed tiles
   const float* x;
   int32_t n_x;           // number of spots
@@ -212,7 +213,7 @@ void launch_beta_table(double* out, long long n, double beta0, double alpha, cud
 void launch_finish(int step, const double* part_f, int nf, const double* part_bc, int nbc,
                    const double* part_g, int ng, DevState* st, double* stage, const double* btab,
                    long long n_btab, cudaStream_t s);
-void launch_count_rows(const Geometry& g, const Tables& t, const uint32_t* mask, const double* dd,
+void launch_count_rows(int grid, const Tables& t, const uint32_t* mask, const double* dd,
                        const double* ll, const double* dl, const int64_t* rows, int64_t n_list, double* part,
                        cudaStream_t s);
 void launch_scatter_y(const float2* y, const int64_t* voxel, int64_t n, float* a, float* b,
@@ -222,7 +223,7 @@ void launch_apply_step(int64_t n_hot, int n, float* w, const float* g, float2* y
 void launch_row_objective(const Geometry& g, const Tables& t, const float2* yw, const uint32_t* mask,
                           const float* sD, const float* sL, int64_t n_hot, float2* r_out,
                           double* part, cudaStream_t s);
-void launch_final_check(const Geometry& g, const Tables& t, const double2* y64, const uint32_t* mask,
+void launch_final_check(int grid, const Tables& t, const double2* y64, const uint32_t* mask,
                         const double* dd, const double* ll, const double* dl, const int64_t* rows, int64_t n_list,
                         double* part, cudaStream_t s);
 void launch_begin_state(DevState* st, cudaStream_t s);
@@ -364,6 +365,7 @@ constexpr int kMaxSel = 64;     // (request, fraction) selections per call
 struct VolArgs {
   const double2* y64;       // FP64 (Dw, Lw) per device row
   const uint32_t* mask;     // per device row
+  const int64_t* rows;      // the rows with a structure bit
   int64_t n_rows;
   double c;                 // cDL constant
   uint32_t any_bits;        // union of the requested structure bits
@@ -383,18 +385,23 @@ struct SelSlot {
 struct SelArgs {
   const double2* y64;
   const uint32_t* mask;
+  const int64_t* rows;
   int64_t n_rows;
   double c;
   uint32_t any_bits;
   int n_sel;
   int32_t q[kMaxSel], bit[kMaxSel];
+  int32_t req[kMaxSel];    // request of the selection
+  const double* fracs;     // [n_sel] fractions of the structure's volume
+  const unsigned long long* n_vox;  // voxels per request
   uint32_t* hist;  // [n_sel][256], zeroed by the caller
   SelSlot* st;     // [n_sel]
 };
 
 size_t vol_hist_smem(const VolArgs& a);
 void launch_vol_hist(const Geometry& g, const VolArgs& a, cudaStream_t s);
-void launch_vol_select(const Geometry& g, const SelArgs& a, cudaStream_t s);  // 8 launches
+constexpr int kVolSelectLaunches = 9;
+void launch_vol_select(const Geometry& g, const SelArgs& a, cudaStream_t s);
 void launch_vol_map(const Geometry& g, const double2* y64, const int64_t* voxel, int64_t n_rows, int q, double c,
                     float* out, cudaStream_t s);
 

@@ -668,7 +668,9 @@ __global__ void __launch_bounds__(kFwdThreads, 1024 / kFwdThreads) k_forward(Fwd
     }
   };
   while (job < a.n_warps) {
-    const int64_t r0 = a.warp_row[2 * job], r1 = a.warp_row[2 * job + 1];
+    // EPI_FINAL over listed rows: a tile is one row
+    const bool one = EPI == EPI_FINAL && a.rows != nullptr;
+    const int64_t r0 = one ? a.rows[job] : a.warp_row[2 * job], r1 = one ? r0 + 1 : a.warp_row[2 * job + 1];
     acc0 = 0.0;
     acc1 = 0.0;
     stream_segments<VT, Acc, S, true, (sizeof(VT) == 4 ? kFwdUnroll : kFwdUnroll16)>(
@@ -1465,18 +1467,18 @@ void launch_row_objective(const Geometry& g, const Tables& t, const float2* yw, 
   k_row_objective<<<g.row_blocks, kRowThreads, 0, s>>>(t, yw, mask, sD, sL, n_hot, r_out, part);
 }
 
-void launch_final_check(const Geometry& g, const Tables& t, const double2* y64, const uint32_t* mask,
+void launch_final_check(int grid, const Tables& t, const double2* y64, const uint32_t* mask,
                         const double* dd, const double* ll, const double* dl, const int64_t* rows, int64_t n_list,
                         double* part, cudaStream_t s) {
-  k_final_check<<<g.row_blocks, kRowThreads, 0, s>>>(t, y64, mask, dd, ll, dl, rows, n_list, part);
+  k_final_check<<<grid, kRowThreads, 0, s>>>(t, y64, mask, dd, ll, dl, rows, n_list, part);
 }
 
 void launch_begin_state(DevState* st, cudaStream_t s) { k_begin_state<<<1, 1, 0, s>>>(st); }
 
-void launch_count_rows(const Geometry& g, const Tables& t, const uint32_t* mask, const double* dd,
+void launch_count_rows(int grid, const Tables& t, const uint32_t* mask, const double* dd,
                        const double* ll, const double* dl, const int64_t* rows, int64_t n_list, double* part,
                        cudaStream_t s) {
-  k_count_rows<<<g.row_blocks, kRowThreads, 0, s>>>(t, mask, dd, ll, dl, rows, n_list, part);
+  k_count_rows<<<grid, kRowThreads, 0, s>>>(t, mask, dd, ll, dl, rows, n_list, part);
 }
 
 void launch_scatter_y(const float2* y, const int64_t* voxel, int64_t n, float* a, float* b,
