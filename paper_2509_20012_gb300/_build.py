@@ -1,6 +1,6 @@
 """In-tree build of libfredopt.so for sm_103a (nvcc; no cmake).
 
-The translation units (kernels, C ABI, plan load, server, no-allocation
+The translation units (kernels, C ABI, plan load, sweep, server, no-allocation
 product, volume statistics) compile in parallel, then link into
 paper_2509_20012_gb300/libfredopt.so with the CUDA runtime linked statically.
 `defines` builds variants elsewhere, e.g. the bounds-checked FO_CHECKED=1
@@ -20,8 +20,8 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(PKG, "libfredopt.so")
-SOURCES = ["fredopt_kernels.cu", "fredopt_api.cu", "fredopt_load.cu", "fredopt_server.cu", "fredopt_noalloc.cu",
-           "fredopt_volume.cu"]
+SOURCES = ["fredopt_kernels.cu", "fredopt_api.cu", "fredopt_load.cu", "fredopt_sweep.cu", "fredopt_server.cu",
+           "fredopt_noalloc.cu", "fredopt_volume.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE]
 

@@ -110,6 +110,7 @@ struct fredopt_ctx {
   int64_t row_cost = 0, chunk_cost = 0;  // warp-partition weights in use
   DBuf<int64_t> con_rows;        // streamed rows with a structure bit, ascending
   int64_t n_con_rows = 0, n_con_ne = 0;  // all of them; those with nonzeros (first in the list)
+  int64_t con_nnz = 0;                   // nonzeros of the structure rows
   uint64_t empty_bits[32] = {0};  // streamed rows without nonzeros, per structure bit
   DBuf<float2> ucoef;            // coefficients of fredopt_backward (kept apart from gam)
 
@@ -133,12 +134,11 @@ struct fredopt_ctx {
   // block-iterative sweep (built for sweep_m requested blocks; 0 = not built)
   int sweep_m = 0;
   int sweep_nb = 0;                          // blocks actually formed
-  std::vector<int64_t> h_sweep_bounds;       // [sweep_nb + 1] device rows
-  std::vector<int64_t> sweep_wr_off;         // [sweep_nb] offset (in pairs) of each block's warp ranges
-  std::vector<int> sweep_warps;              // [sweep_nb] warps of each block's forward product
-  DBuf<int64_t> sweep_wr, sweep_pos, sweep_bounds_d;
+  int64_t sweep_size = 0;                    // structure rows with nonzeros per block
+  DBuf<int64_t> sweep_pos, sweep_bounds_d;
+  DBuf<double> sweep_w, sweep_part;          // [sweep_nb] 1 / priority sum; violated rows' partial sums
   DBuf<float> xs;                            // the point being swept [n_pad]
-  DBuf<float2> ys;                           // forward product of the block rows [n_hot]
+  DBuf<float2> ys;                           // forward product of a block's rows [n_con_ne]
   DBuf<double> part;
   // steps beta0 alpha^s of the trial loop for s < kBetaTable (in `part` at
   // off_btab), filled on the device for (btab_alpha, btab_beta0)
@@ -384,11 +384,18 @@ ConArgs con_args(fredopt_t h) {
 }
 
 
+// 1 / priority sum of the sweep blocks' reachable rows (they change with the
+// constraint table only).
+void sweep_weights(fredopt_t h) {
+  launch_sweep_weights(h->tab, h->con_rows.p, h->n_con_ne, h->sweep_size, h->sweep_nb, h->mask.p, h->mdd.p, h->mll.p,
+                    h->mdl.p, h->sweep_w.p, h->stream);
+}
+
 // Blocks of the block-iterative sweep: the streamed rows with nonzeros that
 // lie in some structure, in device (= ascending voxel) order, cut into groups
-// of S = ceil(count / m) rows; block t covers the device rows from its first
-// structure row to the next block's first.  Builds each block's forward
-// schedule and the CSC position table of the block boundaries.
+// of S = ceil(count / m) rows.  Builds the CSC position table of the blocks'
+// boundaries (the device rows from a block's first structure row to the next
+// block's first).
 int build_sweep(fredopt_t h, int m) {
   if (h->sweep_m == m) return FREDOPT_OK;
   cudaStream_t s = h->stream;
@@ -397,41 +404,26 @@ int build_sweep(fredopt_t h, int m) {
     CK(cudaMemcpyAsync(C.data(), h->con_rows.p, C.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
   }
-  h->h_sweep_bounds.clear();
-  h->sweep_wr_off.clear();
-  h->sweep_warps.clear();
+  std::vector<int64_t> bnd;
   h->sweep_nb = 0;
+  h->sweep_size = 0;
   if (!C.empty()) {
     const int64_t S = ((int64_t)C.size() + m - 1) / m;
     const int nb = (int)(((int64_t)C.size() + S - 1) / S);
-    for (int t = 0; t < nb; ++t) h->h_sweep_bounds.push_back(C[(size_t)t * S]);
-    h->h_sweep_bounds.push_back(C.back() + 1);
+    for (int t = 0; t < nb; ++t) bnd.push_back(C[(size_t)t * S]);
     h->sweep_nb = nb;
+    h->sweep_size = S;
   }
-  int64_t n_wr = 0;
-  for (int t = 0; t < h->sweep_nb; ++t) {
-    const int64_t r0 = h->h_sweep_bounds[t], r1 = h->h_sweep_bounds[t + 1];
-    const int warps = (int)std::max<int64_t>(1, std::min<int64_t>(h->geo.fwd_warps, r1 - r0));
-    h->sweep_wr_off.push_back(n_wr);
-    h->sweep_warps.push_back(warps);
-    n_wr += warps;
-  }
-  CK(h->sweep_wr.alloc((size_t)std::max<int64_t>(1, n_wr) * 2));
-  for (int t = 0; t < h->sweep_nb; ++t) {
-    TileArgs q{TileArgs::PAIRS, h->rp.p, h->h_sweep_bounds[t], h->h_sweep_bounds[t + 1], 0, 0, h->sweep_warps[t], 0,
-               h->row_cost, h->sweep_wr.p + 2 * h->sweep_wr_off[t], nullptr};
-    launch_tiles(q, s);
-  }
-  const int nbnd = h->sweep_nb + 1;
-  std::vector<int64_t> bnd = h->h_sweep_bounds;
-  if (bnd.empty()) bnd.assign(1, 0);
+  bnd.push_back(C.empty() ? 0 : C.back() + 1);
   CK(upload_vec(h, h->sweep_bounds_d, bnd));
-  CK(h->sweep_pos.alloc((size_t)std::max(1, nbnd) * h->n));
-  if (h->sweep_nb > 0) launch_sweep_pos(h->cp.p, h->crow.p, h->n, h->sweep_bounds_d.p, nbnd, h->sweep_pos.p, s);
+  CK(h->sweep_pos.alloc(bnd.size() * h->n));
+  if (h->sweep_nb > 0)
+    launch_sweep_pos(h->cp.p, h->crow.p, h->n, h->sweep_bounds_d.p, (int)bnd.size(), h->sweep_pos.p, s);
+  CK(h->sweep_w.alloc(h->sweep_nb));
+  CK(h->sweep_part.alloc((size_t)((h->sweep_size + kSweepConThreads - 1) / kSweepConThreads)));
   CK(h->xs.ensure(h->n_pad));
   CK(cudaMemsetAsync(h->xs.p, 0, h->n_pad * sizeof(float), s));
-  CK(h->ys.ensure(std::max<int64_t>(1, h->n_hot)));
-  CK(cudaMemsetAsync(h->ys.p, 0, std::max<int64_t>(1, h->n_hot) * sizeof(float2), s));
+  CK(h->ys.ensure(h->n_con_ne));
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   h->sweep_m = m;
@@ -441,47 +433,48 @@ int build_sweep(fredopt_t h, int m) {
 // One block-iterative sweep from x = w + coef * g (use_coef) or x = w, into out.
 void enqueue_sweep(fredopt_t h, const float* w, int use_coef, double lam, double prio_scale, int norm,
                    int in_solve, float* out) {
-  const Geometry& G = h->geo;
   cudaStream_t s = h->stream;
   run(h, 5, [&] { launch_sweep_start(h->n, w, h->g.p, use_coef, h->xs.p, h->st.p, s); });
+  SweepArgs a{};
+  a.list = h->con_rows.p;
+  a.rp = h->rp.p;
+  a.col = h->col.p;
+  a.col16 = h->col16.p;
+  a.rD = h->Dv.p;
+  a.rL = h->Lv.p;
+  a.sD = h->fmt ? h->sD.p : nullptr;
+  a.sL = h->fmt ? h->sL.p : nullptr;
+  a.mask = h->mask.p;
+  a.dd = h->mdd.p;
+  a.ll = h->mll.p;
+  a.dl = h->mdl.p;
+  a.y = h->ys.p;
+  a.gam = h->gam.p;
+  a.part = h->sweep_part.p;
+  a.row = h->crow.p;
+  a.Dv = h->DTv.p;
+  a.Lv = h->LTv.p;
+  a.x = h->xs.p;
+  a.n = h->n;
+  a.norm = norm;
+  a.lam = lam;
+  a.prio_scale = prio_scale;
+  a.in_solve = in_solve;
+  a.st = h->st.p;
+  const double row_nnz = h->n_con_ne > 0 ? (double)h->con_nnz / (double)h->n_con_ne : 0.0;
+  const double col_nnz = (double)h->nnz_hot / ((double)std::max(1, h->sweep_nb) * (double)h->n);
   for (int t = 0; t < h->sweep_nb; ++t) {
-    FwdArgs fa = fwd_args(h, true);
-    fa.warp_row = h->sweep_wr.p + 2 * h->sweep_wr_off[t];
-    fa.n_warps = h->sweep_warps[t];
-    fa.sched = nullptr;  // the block's own static tiles
-    fa.x = h->xs.p;
-    fa.y = h->ys.p;
-    run(h, 0, [&] { launch_forward(G, h->fmt, EPI_STORE, h->hint_fwd, fa, h->tab, s); });
-    ConArgs k2 = con_args(h);
-    k2.yw = h->ys.p;
-    k2.yg = nullptr;
-    k2.use_coef = 0;
-    k2.rows = nullptr;  // the block's row range
-    k2.r0 = h->h_sweep_bounds[t];
-    k2.n_hot = h->h_sweep_bounds[t + 1];
-    // one CTA per 256 rows of the block, at most the usual grid
-    const int k2_grid = (int)std::max<int64_t>(
-        1, std::min<int64_t>(G.row_blocks, (k2.n_hot - k2.r0 + 255) / 256));
-    run(h, 2, [&] { launch_constraints(G, h->tab, k2, s, k2_grid); });
-    SweepArgs sa{};
-    sa.pos0 = h->sweep_pos.p + (size_t)t * h->n;
-    sa.pos1 = h->sweep_pos.p + (size_t)(t + 1) * h->n;
-    sa.row = h->crow.p;
-    sa.Dv = h->DTv.p;
-    sa.Lv = h->LTv.p;
-    sa.gam = h->gam.p;
-    sa.x = h->xs.p;
-    sa.n = h->n;
-    sa.k2part = h->part.p + h->off_k2;
-    sa.k2_blocks = k2_grid;
-    sa.norm = norm;
-    sa.lam = lam;
-    sa.prio_scale = prio_scale;
-    sa.in_solve = in_solve;
-    sa.st = h->st.p;
-    run(h, 1, [&] { launch_sweep_update(G, h->fmt, sa, s); });
+    a.i0 = t * h->sweep_size;
+    a.i1 = std::min(h->n_con_ne, a.i0 + h->sweep_size);
+    a.con_blocks = (int)((a.i1 - a.i0 + kSweepConThreads - 1) / kSweepConThreads);
+    a.winv = h->sweep_w.p + t;
+    a.pos0 = h->sweep_pos.p + (size_t)t * h->n;
+    a.pos1 = h->sweep_pos.p + (size_t)(t + 1) * h->n;
+    run(h, 0, [&] { launch_sweep_rows(h->fmt, row_nnz, a, s); });
+    run(h, 2, [&] { launch_sweep_con(h->tab, a, s); });
+    run(h, 1, [&] { launch_sweep_cols(h->fmt, col_nnz, a, s); });
   }
-  run(h, 3, [&] { launch_sweep_finish(G, h->n, h->xs.p, out, in_solve, h->st.p, h->log.p, s); });
+  run(h, 3, [&] { launch_sweep_finish(h->geo, h->n, h->xs.p, out, in_solve, h->st.p, h->log.p, s); });
 }
 
 // One superiorized iteration (Fig. 3 around the simultaneous Fig. 2).
@@ -862,7 +855,7 @@ int fredopt_load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t 
   h->V = n_vox; h->nnz = nnz; h->n = n_spots; h->n_pad = (n_spots + 3) & ~3;
   h->fmt = fmt; h->roi = roi; h->perm = perm; h->n_hot = n_hot; h->nnz_hot = nnz_hot;
   h->n_hot_ne = n_hot_ne; h->n_cold_ne = n_cold_ne;
-  h->n_con_ne = tot.c[5]; h->n_con_rows = tot.c[5] + tot.c[6];
+  h->n_con_ne = tot.c[5]; h->n_con_rows = tot.c[5] + tot.c[6]; h->con_nnz = (int64_t)tot.con_nnz;
   for (int b = 0; b < 32; ++b) h->empty_bits[b] = tot.empty_bits[b];
 
   CK(h->rp.fit(n_vox + 1));
@@ -1133,6 +1126,7 @@ int fredopt_set_constraints(fredopt_t h, int n, const fredopt_constraint* c) {
   h->n_rows_reach = (int64_t)nr;
   h->n_unreach = (int64_t)nu;
   h->W_all = W;
+  if (h->sweep_m > 0) sweep_weights(h);
   h->have_con = true;
   return FREDOPT_OK;
 }
@@ -1205,6 +1199,7 @@ int fredopt_begin(fredopt_t h, const float* w0, double alpha, double relaxation,
   h->prm = p;
   h->alpha = alpha;
   h->lam = relaxation;
+  if (p.sweep_blocks > 0) sweep_weights(h);
   h->beta0 = p.beta0 < 0.0 ? 0.1 * std::sqrt(nrm) : p.beta0;
   h->tab.c = p.c_cdl;
   CK(cudaMemcpyAsync(h->w.p, hw.data(), h->n * sizeof(float), cudaMemcpyHostToDevice, s));
@@ -1596,6 +1591,7 @@ int fredopt_sweep_step(fredopt_t h, const float* x, double relaxation, double pr
   join_in(h);
   rc = build_sweep(h, n_blocks);
   if (rc) return rc;
+  sweep_weights(h);
   rc = load_spot_vec(h, h->xbuf, x, flags);
   if (rc) return rc;
   CK(h->gtmp.ensure(h->n_pad));

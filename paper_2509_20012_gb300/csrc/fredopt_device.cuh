@@ -4,6 +4,8 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include "fredopt_internal.cuh"
+
 namespace fo {
 
 constexpr unsigned kFull = 0xffffffffu;
@@ -110,6 +112,173 @@ __device__ __forceinline__ void warp_sum2(Acc& a, Acc& b, int lane) {
   const Acc other = shfl_xor(keep, 16);
   a = up ? other : keep;
   b = up ? keep : other;
+}
+
+// ------------------------------------------------------------------ block reductions
+
+// Block reductions of one double per thread (blockDim = 256), in a fixed
+// order: a warp butterfly, then thread 0 adds the 8 warp results in warp
+// order.  GB300 runs FP64 at a small fraction of its FP32 rate, and every
+// FP64 warp instruction costs the same however few of its lanes are active,
+// so: a warp whose lanes all hold zero skips its butterfly (its sum is that
+// zero), maxima are of non-negative doubles, whose bit patterns order as
+// signed 64-bit integers (integer compares), and counts held in doubles are
+// added as 64-bit integers (exact, so in any order).
+__device__ __forceinline__ double warp_sum_nz(double v) {
+  if (!__any_sync(kFull, v != 0.0)) return v;
+  return warp_sum(v);
+}
+__device__ __forceinline__ long long warp_max_bits(long long b) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long c = __shfl_xor_sync(kFull, b, o);
+    b = c > b ? c : b;
+  }
+  return b;
+}
+__device__ __forceinline__ double warp_max_nonneg(double v) {
+  return __longlong_as_double(warp_max_bits(__double_as_longlong(v)));
+}
+__device__ __forceinline__ long long warp_isum(long long v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+  return v;
+}
+// red: at least 9 doubles of shared memory; every thread returns the result
+__device__ __forceinline__ double block_sum256(double v, double* red) {
+  v = warp_sum_nz(v);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double r = red[0];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) r += red[w];
+    red[8] = r;
+  }
+  __syncthreads();
+  // red[8] is rewritten only after the next call's first barrier, which
+  // every thread reaches after this read
+  return red[8];
+}
+// v >= 0
+__device__ __forceinline__ double block_max256(double v, double* red) {
+  long long* rb = reinterpret_cast<long long*>(red);
+  const long long b = warp_max_bits(__double_as_longlong(v));
+  if ((threadIdx.x & 31) == 0) rb[threadIdx.x >> 5] = b;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    long long r = rb[0];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) r = rb[w] > r ? rb[w] : r;
+    rb[8] = r;
+  }
+  __syncthreads();
+  return __longlong_as_double(rb[8]);
+}
+// integers held in doubles (|v| < 2^53), added exactly
+__device__ __forceinline__ double block_count256(long long v, double* red) {
+  long long* rb = reinterpret_cast<long long*>(red);
+  v = warp_isum(v);
+  if ((threadIdx.x & 31) == 0) rb[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    long long r = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) r += rb[w];
+    rb[8] = r;
+  }
+  __syncthreads();
+  return (double)rb[8];
+}
+// Sum of n doubles in a fixed order (strided per thread, then block_sum256).
+__device__ __forceinline__ double block_sum_array(const double* p, int n, double* red) {
+  double v = 0.0;
+  for (int i = threadIdx.x; i < n; i += 256) v += p[i];
+  return block_sum256(v, red);
+}
+// p[i] >= 0
+__device__ __forceinline__ double block_max_array(const double* p, int n, double* red) {
+  long long v = 0;
+  for (int i = threadIdx.x; i < n; i += 256) {
+    const long long b = __double_as_longlong(p[i]);
+    v = b > v ? b : v;
+  }
+  return block_max256(__longlong_as_double(v), red);
+}
+__device__ __forceinline__ double block_count_array(const double* p, int n, double* red) {
+  long long v = 0;
+  for (int i = threadIdx.x; i < n; i += 256) v += (long long)p[i];
+  return block_count256(v, red);
+}
+
+// ---- half-space evaluation of a voxel row (Fig. 2)
+// |a_r|^2 of constraint c for a row with moments dd, ll, dl
+__device__ __forceinline__ double row_norm2(const ConEntry& c, double cdl, double dd, double ll, double dl) {
+  const int fam = c.kind >> 1;  // 0 dose, 1 cDL, 2 LETd
+  return fam == 0 ? dd : fam == 1 ? cdl * cdl * ll : ll - 2.0 * c.bound * dl + c.bound * c.bound * dd;
+}
+// the constraint table in shared memory (a barrier follows at the caller)
+__device__ __forceinline__ void stage_constraints(const Tables& t, ConEntry* con) {
+  for (int q = threadIdx.x; q < t.n_con; q += blockDim.x) con[q] = t.con[q];
+}
+// bit q: constraint q applies to a voxel with structure mask m
+__device__ __forceinline__ uint32_t row_constraints(const ConEntry* con, int n_con, uint32_t m) {
+  uint32_t todo = 0u;
+  for (int q = 0; q < n_con; ++q) todo |= ((m >> con[q].bit) & 1u) << q;
+  return todo;
+}
+// Each lane walks the constraints of its own row, so a warp makes as many
+// FP64 steps (a division or two each) as one of its rows has constraints, not
+// as many as the table.  xd = (D x)_i, xl = (L x)_i; the sums run in table order.
+__device__ __forceinline__ void eval_constraints(const ConEntry* con, uint32_t todo, double cdl, double xd, double xl,
+                                                 double dd, double ll, double dl, double& gD, double& gL,
+                                                 double& psum, double& preach, unsigned& nv, double& mx) {
+  while (todo) {
+    const ConEntry c = con[__ffs(todo) - 1];
+    todo &= todo - 1u;
+    const double n2 = row_norm2(c, cdl, dd, ll, dl);
+    if (!(n2 > 0.0)) continue;  // unreachable row
+    preach += c.prio;
+    const int fam = c.kind >> 1;
+    const double v = fam == 0 ? xd : fam == 1 ? cdl * xl : xl - c.bound * xd;
+    const double b = fam == 2 ? 0.0 : c.bound;
+    const double viol = (c.kind & 1) ? v - b : b - v;
+    if (viol > 0.0) {
+      const double tt = c.prio * (b - v) / n2;
+      if (fam == 0) gD += tt;
+      else if (fam == 1) gL += cdl * tt;
+      else { gD -= c.bound * tt; gL += tt; }
+      psum += c.prio;
+      nv += 1u;
+      const double vu = (fam == 2) ? (xd > 0.0 ? viol / xd : 0.0) : viol;  // LETd in keV/um
+      mx = vu > mx ? vu : mx;
+    }
+  }
+}
+
+// ---- programmatic dependent launch
+// A kernel launched with launch_pdl may start while its predecessor on the
+// stream still runs.  It may read what no kernel of the chain writes at once;
+// pdl_wait() returns when the predecessor has finished and its writes are
+// visible (every thread calls it before it exits, so a chain stays ordered).
+// Then pdl_release() lets the successor start.  What the chain writes is read
+// with plain loads after the wait, never with the read-only path.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+void launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
 }  // namespace fo

@@ -64,7 +64,8 @@ struct DevState {
   int err;            // bit 0: bulk-copy wait timed out; bit 1: index out of range (FO_CHECKED builds)
   unsigned int done;  // last-block counter of the column finish
   int pad;
-  double sweep_nv, sweep_mx;  // block-iterative sweep: violated rows and largest violation
+  unsigned long long sweep_nv;  // block-iterative sweep: violated rows
+  long long sweep_mx;           // and largest violation (bits of a double >= 0)
   unsigned int done_fin;      // last-block counter of the scalar finish
   int pad2;
 };
@@ -243,6 +244,7 @@ struct RowTotals {
   long long c[7];
   unsigned int flags;
   unsigned int pad;
+  unsigned long long con_nnz;         // nonzeros of the structure rows
   unsigned long long empty_bits[32];  // streamed rows without nonzeros, per structure bit
 };
 size_t row_order_scratch(int64_t n_rows);  // int64 values
@@ -322,28 +324,54 @@ void launch_scale_coef(int64_t n, const float* aD, const float* aL, const int64_
 
 // ---- block-iterative sweep (fredopt_sweep.cu)
 struct SweepArgs {
-  const int64_t* pos0;   // [n]: first CSC position of each column at or after the block's first row
-  const int64_t* pos1;   // [n]: same for the next block
-  const int32_t* row;    // CSC row indices (streamed rows)
-  const void* Dv;        // CSC values
+  // the block's rows: list[i0 .. i1) (structure rows with nonzeros)
+  const int64_t* list;
+  int64_t i0, i1;
+  const int64_t* rp;       // CSR
+  const int32_t* col;      // indices, or null when col16 is set
+  const uint16_t* col16;
+  const void* rD;
+  const void* rL;
+  const float* sD;         // row scales (16-bit storage) or null
+  const float* sL;
+  const uint32_t* mask;
+  const double* dd;
+  const double* ll;
+  const double* dl;
+  float2* y;               // (Dx, Lx) per list entry
+  float2* gam;             // per streamed row (scaled like the transposed product's coefficients)
+  double* part;            // [con_blocks] priority sums of the violated rows
+  int con_blocks;
+  const double* winv;      // 1 / priority sum of the block's reachable rows (0 for none)
+  // columns
+  const int64_t* pos0;     // [n]: first CSC position of each column at or after the block's first row
+  const int64_t* pos1;     // [n]: same for the next block
+  const int32_t* row;      // CSC row indices (streamed rows)
+  const void* Dv;          // CSC values
   const void* Lv;
-  const float2* gam;     // per streamed row (scaled like the transposed product's coefficients)
-  float* x;              // [n], updated in place
+  float* x;                // [n], updated in place
   int32_t n;
-  const double* k2part;  // constraint partials of the block (4 slices of k2_blocks)
-  int32_t k2_blocks;
   int32_t norm;
   double lam;
-  double prio_scale;     // outside a solve
-  int32_t in_solve;      // 1: scale eta^k from DevState and count the block's violations
+  double prio_scale;       // outside a solve
+  int32_t in_solve;        // 1: scale eta^k from DevState and count the block's violations
   DevState* st;
 };
 
+constexpr int kSweepConThreads = 32;  // rows per CTA of the block's constraint kernel
 void launch_sweep_start(int n, const float* w, const float* g, int use_coef, float* x, DevState* st,
                         cudaStream_t s);
 void launch_sweep_pos(const int64_t* cp, const int32_t* row, int32_t n, const int64_t* bounds, int n_bounds,
                       int64_t* pos, cudaStream_t s);
-void launch_sweep_update(const Geometry& g, int fmt, const SweepArgs& a, cudaStream_t s);
+// winv[t] = 1 / priority sum of the reachable constraint rows of list[t * size .. (t + 1) * size), t < n_blk
+void launch_sweep_weights(const Tables& t, const int64_t* list, int64_t n_list, int64_t size, int n_blk,
+                       const uint32_t* mask, const double* dd, const double* ll, const double* dl, double* winv,
+                       cudaStream_t s);
+// forward product of the block's rows; warps per row by the mean row length
+void launch_sweep_rows(int fmt, double mean_nnz, const SweepArgs& a, cudaStream_t s);
+void launch_sweep_con(const Tables& t, const SweepArgs& a, cudaStream_t s);
+// lanes per column by the mean entries of a column in the block
+void launch_sweep_cols(int fmt, double mean_entries, const SweepArgs& a, cudaStream_t s);
 void launch_sweep_finish(const Geometry& g, int n, const float* x, float* out, int in_solve, DevState* st,
                          LogEntry* log, cudaStream_t s);
 // Based 16-bit CSC row indices over n_blk blocks of 128 elements (pass 1:

@@ -756,103 +756,6 @@ __global__ void __launch_bounds__(kBwdThreads, FO_BWD_MIN_BLOCKS) k_backward(Bwd
   }
 }
 
-// ------------------------------------------------------------------ block reductions
-
-// Block reductions of one double per thread (blockDim = 256), in a fixed
-// order: a warp butterfly, then thread 0 adds the 8 warp results in warp
-// order.  GB300 runs FP64 at a small fraction of its FP32 rate, and every
-// FP64 warp instruction costs the same however few of its lanes are active,
-// so: a warp whose lanes all hold zero skips its butterfly (its sum is that
-// zero), maxima are of non-negative doubles, whose bit patterns order as
-// signed 64-bit integers (integer compares), and counts held in doubles are
-// added as 64-bit integers (exact, so in any order).
-__device__ __forceinline__ double warp_sum_nz(double v) {
-  if (!__any_sync(kFull, v != 0.0)) return v;
-  return warp_sum(v);
-}
-__device__ __forceinline__ long long warp_max_bits(long long b) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const long long c = __shfl_xor_sync(kFull, b, o);
-    b = c > b ? c : b;
-  }
-  return b;
-}
-__device__ __forceinline__ double warp_max_nonneg(double v) {
-  return __longlong_as_double(warp_max_bits(__double_as_longlong(v)));
-}
-__device__ __forceinline__ long long warp_isum(long long v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-  return v;
-}
-// red: at least 9 doubles of shared memory; every thread returns the result
-__device__ __forceinline__ double block_sum256(double v, double* red) {
-  v = warp_sum_nz(v);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double r = red[0];
-#pragma unroll
-    for (int w = 1; w < 8; ++w) r += red[w];
-    red[8] = r;
-  }
-  __syncthreads();
-  // red[8] is rewritten only after the next call's first barrier, which
-  // every thread reaches after this read
-  return red[8];
-}
-// v >= 0
-__device__ __forceinline__ double block_max256(double v, double* red) {
-  long long* rb = reinterpret_cast<long long*>(red);
-  const long long b = warp_max_bits(__double_as_longlong(v));
-  if ((threadIdx.x & 31) == 0) rb[threadIdx.x >> 5] = b;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    long long r = rb[0];
-#pragma unroll
-    for (int w = 1; w < 8; ++w) r = rb[w] > r ? rb[w] : r;
-    rb[8] = r;
-  }
-  __syncthreads();
-  return __longlong_as_double(rb[8]);
-}
-// integers held in doubles (|v| < 2^53), added exactly
-__device__ __forceinline__ double block_count256(long long v, double* red) {
-  long long* rb = reinterpret_cast<long long*>(red);
-  v = warp_isum(v);
-  if ((threadIdx.x & 31) == 0) rb[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    long long r = 0;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) r += rb[w];
-    rb[8] = r;
-  }
-  __syncthreads();
-  return (double)rb[8];
-}
-// Sum of n doubles in a fixed order (strided per thread, then block_sum256).
-__device__ __forceinline__ double block_sum_array(const double* p, int n, double* red) {
-  double v = 0.0;
-  for (int i = threadIdx.x; i < n; i += 256) v += p[i];
-  return block_sum256(v, red);
-}
-// p[i] >= 0
-__device__ __forceinline__ double block_max_array(const double* p, int n, double* red) {
-  long long v = 0;
-  for (int i = threadIdx.x; i < n; i += 256) {
-    const long long b = __double_as_longlong(p[i]);
-    v = b > v ? b : v;
-  }
-  return block_max256(__longlong_as_double(v), red);
-}
-__device__ __forceinline__ double block_count_array(const double* p, int n, double* red) {
-  long long v = 0;
-  for (int i = threadIdx.x; i < n; i += 256) v += (long long)p[i];
-  return block_count256(v, red);
-}
-
 // ------------------------------------------------------------------ K3b
 
 // The end of an iteration (block-wide): its log entry (violated rows and
@@ -953,6 +856,9 @@ __global__ void __launch_bounds__(kColThreads) k_colfinish(ColArgs a) {
 // ------------------------------------------------------------------ K2
 
 __global__ void __launch_bounds__(kRowThreads) k_constraints(ConArgs a, Tables t) {
+  __shared__ ConEntry con[kMaxCon];
+  stage_constraints(t, con);
+  __syncthreads();
   // block b evaluates a contiguous slice of the rows: of [r0, n_hot), or of
   // the listed rows
   const int64_t lo = a.rows ? 0 : a.r0, hi = a.rows ? a.n_list : a.n_hot;
@@ -961,12 +867,12 @@ __global__ void __launch_bounds__(kRowThreads) k_constraints(ConArgs a, Tables t
   const int64_t j1 = min(hi, j0 + per);
   const double coef = a.use_coef ? a.st->coef : 0.0;
   double psum = 0.0, mx = 0.0, preach = 0.0;
-  long long nv = 0;
+  unsigned viol = 0u;
   for (int64_t j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
     const int64_t i = a.rows ? a.rows[j] : j;
-    const uint32_t m = a.mask[i];
+    const uint32_t todo = row_constraints(con, t.n_con, a.mask[i]);
     float2 out = make_float2(0.f, 0.f);
-    if (m) {
+    if (todo) {
       const float2 w2 = a.yw[i];
       double xd = w2.x, xl = w2.y;
       if (a.use_coef) {
@@ -975,41 +881,14 @@ __global__ void __launch_bounds__(kRowThreads) k_constraints(ConArgs a, Tables t
         xl += coef * (double)g2.y;
       }
       double gD = 0.0, gL = 0.0;
-      for (int q = 0; q < t.n_con; ++q) {
-        const ConEntry& c = t.con[q];
-        if (!((m >> c.bit) & 1u)) continue;
-        double v, n2, b;
-        const int fam = c.kind >> 1;  // 0 dose, 1 cDL, 2 LETd
-        if (fam == 0) {
-          v = xd; n2 = a.dd[i]; b = c.bound;
-        } else if (fam == 1) {
-          v = t.c * xl; n2 = t.c * t.c * a.ll[i]; b = c.bound;
-        } else {
-          v = xl - c.bound * xd;
-          n2 = a.ll[i] - 2.0 * c.bound * a.dl[i] + c.bound * c.bound * a.dd[i];
-          b = 0.0;
-        }
-        if (!(n2 > 0.0)) continue;  // unreachable row
-        preach += c.prio;
-        const bool upper = (c.kind & 1) != 0;
-        const double viol = upper ? v - b : b - v;
-        if (viol > 0.0) {
-          const double tt = c.prio * (b - v) / n2;
-          if (fam == 0) gD += tt;
-          else if (fam == 1) gL += t.c * tt;
-          else { gD -= c.bound * tt; gL += tt; }
-          psum += c.prio;
-          nv += 1;
-          const double vu = (fam == 2) ? (xd > 0.0 ? viol / xd : 0.0) : viol;  // LETd in keV/um
-          mx = vu > mx ? vu : mx;
-        }
-      }
+      eval_constraints(con, todo, t.c, xd, xl, a.dd[i], a.ll[i], a.dl[i], gD, gL, psum, preach, viol, mx);
       const double sd = a.sD ? (double)a.sD[i] : 1.0;
       const double sl = a.sL ? (double)a.sL[i] : 1.0;
       out = make_float2((float)(gD * sd), (float)(gL * sl));
     }
     a.gam[i] = out;
   }
+  long long nv = viol;
   // the block's two sums, its violated-row count and its largest violation
   // (>= 0): warp reductions (the FP64 butterflies skipped by warps without
   // violated or reachable rows), then the warp results in warp order
@@ -1580,145 +1459,6 @@ int init_kernels(Geometry* g, int device) {
   if (set_smem_all<__nv_bfloat16>(bytes) != cudaSuccess) return -2;
   if (set_smem_all<__half>(bytes) != cudaSuccess) return -2;
   return 0;
-}
-
-// ------------------------------------------------------------------ block-iterative sweep
-
-// x = w + coef * g (the perturbed point; coef = 0 without perturbation), and
-// the sweep's violation counters cleared.
-__global__ void k_sweep_start(int n, const float* __restrict__ w, const float* __restrict__ g, int use_coef,
-                              float* __restrict__ x, DevState* st) {
-  const double coef = use_coef ? st->coef : 0.0;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x)
-    x[j] = use_coef ? (float)((double)w[j] + coef * (double)g[j]) : w[j];
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    st->sweep_nv = 0.0;
-    st->sweep_mx = 0.0;
-  }
-}
-
-// pos[t * n + j] = first CSC position of column j whose row is >= bounds[t].
-__global__ void k_sweep_pos(const int64_t* __restrict__ cp, const int32_t* __restrict__ row, int32_t n,
-                            const int64_t* __restrict__ bounds, int n_bounds, int64_t* __restrict__ pos) {
-  const int64_t total = (int64_t)n_bounds * n;
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int t = (int)(idx / n);
-    const int j = (int)(idx - (int64_t)t * n);
-    const int64_t target = bounds[t];
-    int64_t lo = cp[j], hi = cp[j + 1];
-    while (lo < hi) {
-      const int64_t mid = (lo + hi) >> 1;
-      if ((int64_t)row[mid] < target) lo = mid + 1;
-      else hi = mid;
-    }
-    pos[idx] = lo;
-  }
-}
-
-// One block of the sweep: u_j = sum over the block's CSC entries of column j
-// of D_ij gamma_D[i] + L_ij gamma_L[i] (one warp per column, fixed order), then
-// x_j += lam * scale / W_B * u_j.  W_B and the violation counts come from the
-// block's constraint partials.
-template <typename VT>
-__global__ void __launch_bounds__(256) k_sweep_update(SweepArgs a) {
-  __shared__ double red[256];
-  __shared__ double sh_scale;
-  const double W = block_sum_array(a.k2part + (a.norm == 1 ? 0 : 3 * a.k2_blocks), a.k2_blocks, red);
-  if (a.in_solve && blockIdx.x == 0) {
-    const double nv = block_count_array(a.k2part + a.k2_blocks, a.k2_blocks, red);
-    const double mx = block_max_array(a.k2part + 2 * a.k2_blocks, a.k2_blocks, red);
-    if (threadIdx.x == 0) {
-      a.st->sweep_nv += nv;
-      a.st->sweep_mx = fmax(a.st->sweep_mx, mx);
-    }
-  }
-  if (threadIdx.x == 0) {
-    const double ps = a.in_solve ? (a.st->eta == 1.0 ? 1.0 : pow(a.st->eta, (double)a.st->k)) : a.prio_scale;
-    sh_scale = W > 0.0 ? a.lam * ps / W : 0.0;
-  }
-  __syncthreads();
-  const double scale = sh_scale;
-  if (scale == 0.0) return;
-  const VT* __restrict__ Dv = reinterpret_cast<const VT*>(a.Dv);
-  const VT* __restrict__ Lv = reinterpret_cast<const VT*>(a.Lv);
-  const int lane = threadIdx.x & 31;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; j < a.n; j += nw) {
-    const int64_t p0 = a.pos0[j], p1 = a.pos1[j];
-    if (p1 <= p0) continue;
-    float acc = 0.0f;
-    for (int64_t p = p0 + lane; p < p1; p += 32) {
-      const float2 c = a.gam[a.row[p]];
-      acc = fmaf(to_f(Dv[p]), c.x, acc);
-      acc = fmaf(to_f(Lv[p]), c.y, acc);
-    }
-    acc = warp_sum(acc);
-    if (lane == 0) a.x[j] = (float)((double)a.x[j] + scale * (double)acc);
-  }
-}
-
-// out = max(0, x); in a solve the last block writes the log entry and advances k.
-__global__ void __launch_bounds__(256) k_sweep_finish(int n, const float* __restrict__ x, float* __restrict__ out,
-                                                      int in_solve, DevState* st, LogEntry* log) {
-  __shared__ bool sh_last;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x)
-    out[j] = x[j] > 0.0f ? x[j] : 0.0f;
-  if (!in_solve) return;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned prev = atomicAdd(&st->done, 1u);
-    sh_last = (prev == gridDim.x - 1);
-  }
-  __syncthreads();
-  if (sh_last && threadIdx.x == 0) {
-    __threadfence();
-    if (st->log_cap > 0) {
-      LogEntry e;
-      e.k = st->k;
-      e.s = st->s;
-      e.accepted = st->accepted;
-      e.n_violated = (int)st->sweep_nv;
-      e.beta = st->beta_acc;
-      e.f_start = st->f_start;
-      e.f_end = st->f_cur;
-      e.gnorm = st->gnorm;
-      e.max_violation = st->sweep_mx;
-      log[st->k % st->log_cap] = e;
-    }
-    st->k += 1;
-    st->done = 0u;
-  }
-}
-
-void launch_sweep_start(int n, const float* w, const float* g, int use_coef, float* x, DevState* st,
-                        cudaStream_t s) {
-  k_sweep_start<<<std::max(1, std::min(1024, (n + 255) / 256)), 256, 0, s>>>(n, w, g, use_coef, x, st);
-}
-
-void launch_sweep_pos(const int64_t* cp, const int32_t* row, int32_t n, const int64_t* bounds, int n_bounds,
-                      int64_t* pos, cudaStream_t s) {
-  const int64_t total = (int64_t)n_bounds * n;
-  if (total == 0) return;
-  const unsigned gb = (unsigned)std::min<int64_t>((total + 255) / 256, 65535);
-  k_sweep_pos<<<gb, 256, 0, s>>>(cp, row, n, bounds, n_bounds, pos);
-}
-
-void launch_sweep_update(const Geometry& g, int fmt, const SweepArgs& a, cudaStream_t s) {
-  const unsigned gb = (unsigned)std::max(1, std::min(g.n_sms * 8, (a.n + 7) / 8));
-  if (fmt == 1)
-    k_sweep_update<__nv_bfloat16><<<gb, 256, 0, s>>>(a);
-  else if (fmt == 2)
-    k_sweep_update<__half><<<gb, 256, 0, s>>>(a);
-  else
-    k_sweep_update<float><<<gb, 256, 0, s>>>(a);
-}
-
-void launch_sweep_finish(const Geometry& g, int n, const float* x, float* out, int in_solve, DevState* st,
-                         LogEntry* log, cudaStream_t s) {
-  const unsigned gb = (unsigned)std::max(1, std::min(g.n_sms, (n + 255) / 256));
-  k_sweep_finish<<<gb, 256, 0, s>>>(n, x, out, in_solve, st, log);
 }
 
 // Based 16-bit row indices of the CSC (see BlockBase): one warp per block of

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(256) k_rows_count(const int64_t* __restrict__ 
   unsigned flags = 0u;
   if (blockIdx.x == 0 && tid == 0 && (rp[0] != 0 || rp[n] != nnz)) flags |= kRowsBadEnds;
   unsigned c[kRowCounters] = {0u, 0u, 0u, 0u, 0u, 0u, 0u};
-  long long z0 = 0, z2 = 0;
+  long long z0 = 0, z2 = 0, zc = 0;
   for (int k = 0; k < kRowItems; ++k) {
     const int64_t i = (int64_t)blockIdx.x * kRowBlk + k * 256 + tid;
     if (i >= n) break;
@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(256) k_rows_count(const int64_t* __restrict__ 
     c[5] += g == 0 && m != 0u;
     c[6] += g == 1 && m != 0u;
     if (g == 0) z0 += len;
+    if (g == 0 && m != 0u) zc += len;
     if (g == 2) z2 += len;
     if (g == 1)
       for (uint32_t b = m; b; b &= b - 1u) atomicAdd(&bits[__ffs(b) - 1], 1u);
@@ -79,6 +80,8 @@ __global__ void __launch_bounds__(256) k_rows_count(const int64_t* __restrict__ 
       if ((tid & 31) == 0 && v) atomicAdd(&sum[j], (unsigned long long)v);
     }
   }
+  zc = warp_sum(zc);
+  if ((tid & 31) == 0 && zc) atomicAdd(&tot->con_nnz, (unsigned long long)zc);
   flags = __reduce_or_sync(kFull, flags);
   if ((tid & 31) == 0 && flags) atomicOr(&tot->flags, flags);
   __syncthreads();

@@ -1,0 +1,372 @@
+// The block-iterative sweep: the block form of Fig. 2's row-action sweep.
+// Per block of structure rows, three kernels chained by programmatic dependent
+// launch:
+//   k_sweep_rows  forward product of the block's rows, several warps per row
+//   k_sweep_con   half-space evaluation, one row per thread
+//   k_sweep_cols  x_j += scale * sum over the block's entries of column j
+// A block of the clinical plan holds a few hundred rows (9 MB of matrix), so a
+// block is a chain of latencies, not of bytes: every kernel loads what does not
+// depend on its predecessor (matrix entries, positions, moments) before it waits
+// for it, and a row or column is spread over as many lanes as its length fills.
+// Clinical plan (5.7e7 nonzeros in structure rows, FP32), one sweep: 64 blocks
+// 3.60 -> 1.21 ms against plain launches of the streaming forward kernel (one
+// warp per row), the constraint kernel over 608 CTAs and one warp per column.
+#include "fredopt.h"
+#include "fredopt_device.cuh"
+#include "fredopt_internal.cuh"
+
+#include <algorithm>
+
+namespace fo {
+
+namespace {
+
+// x = w + coef * g (the perturbed point; coef = 0 without perturbation), and
+// the sweep's violation counters cleared.
+__global__ void k_sweep_start(int n, const float* __restrict__ w, const float* __restrict__ g, int use_coef,
+                              float* __restrict__ x, DevState* st) {
+  const double coef = use_coef ? st->coef : 0.0;
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x)
+    x[j] = use_coef ? (float)((double)w[j] + coef * (double)g[j]) : w[j];
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    st->sweep_nv = 0ull;
+    st->sweep_mx = 0ll;
+  }
+}
+
+// pos[t * n + j] = first CSC position of column j whose row is >= bounds[t].
+__global__ void k_sweep_pos(const int64_t* __restrict__ cp, const int32_t* __restrict__ row, int32_t n,
+                            const int64_t* __restrict__ bounds, int n_bounds, int64_t* __restrict__ pos) {
+  const int64_t total = (int64_t)n_bounds * n;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int t = (int)(idx / n);
+    const int j = (int)(idx - (int64_t)t * n);
+    const int64_t target = bounds[t];
+    int64_t lo = cp[j], hi = cp[j + 1];
+    while (lo < hi) {
+      const int64_t mid = (lo + hi) >> 1;
+      if ((int64_t)row[mid] < target) lo = mid + 1;
+      else hi = mid;
+    }
+    pos[idx] = lo;
+  }
+}
+
+__global__ void __launch_bounds__(256) k_sweep_weights(Tables t, const int64_t* list, int64_t n_list, int64_t size,
+                                                    const uint32_t* mask, const double* dd, const double* ll,
+                                                    const double* dl, double* winv) {
+  __shared__ double red[9];
+  const int64_t i0 = (int64_t)blockIdx.x * size, i1 = min(n_list, i0 + size);
+  double p = 0.0;
+  for (int64_t i = i0 + threadIdx.x; i < i1; i += 256) {
+    const int64_t r = list[i];
+    const uint32_t m = mask[r];
+    for (int q = 0; q < t.n_con; ++q)
+      if (((m >> t.con[q].bit) & 1u) && row_norm2(t.con[q], t.c, dd[r], ll[r], dl[r]) > 0.0) p += t.con[q].prio;
+  }
+  p = block_sum256(p, red);
+  if (threadIdx.x == 0) winv[blockIdx.x] = p > 0.0 ? 1.0 / p : 0.0;
+}
+
+// (Dx, Lx) of the block's rows, WPR warps per row: a lane takes every
+// (32 WPR)-th entry, four of them in flight, the next four requested before
+// the current ones are used.
+template <typename VT, typename IT, int WPR>
+__global__ void __launch_bounds__(256) k_sweep_rows(SweepArgs a) {
+  constexpr int K = 4, GS = 32 * WPR;
+  __shared__ float2 part[8];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t i = a.i0 + (int64_t)blockIdx.x * (8 / WPR) + wid / WPR;
+  const bool have = i < a.i1;
+  const int64_t r = have ? a.list[i] : 0;
+  const int64_t s = have ? a.rp[r] : 0;
+  const int len = have ? (int)(a.rp[r + 1] - s) : 0;
+  const IT* __restrict__ ci = (sizeof(IT) == 2 ? reinterpret_cast<const IT*>(a.col16) : reinterpret_cast<const IT*>(a.col)) + s;
+  const VT* __restrict__ Di = reinterpret_cast<const VT*>(a.rD) + s;
+  const VT* __restrict__ Li = reinterpret_cast<const VT*>(a.rL) + s;
+  const int first = (wid % WPR) * 32 + lane;
+  int c[K];
+  VT d[K], l[K];
+  auto load = [&](int e0) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const int e = e0 + k * GS;
+      c[k] = -1;
+      if (e < len) {
+        c[k] = (int)ci[e];
+        d[k] = Di[e];
+        l[k] = Li[e];
+      }
+    }
+  };
+  load(first);
+  pdl_wait();  // x is the last block's
+  pdl_release();
+  float sA = 0.0f, sB = 0.0f;
+  for (int e0 = first; __any_sync(kFull, e0 < len); e0 += K * GS) {
+    float x[K], dv[K], lv[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      x[k] = c[k] >= 0 ? a.x[c[k]] : 0.0f;
+      dv[k] = c[k] >= 0 ? to_f(d[k]) : 0.0f;
+      lv[k] = c[k] >= 0 ? to_f(l[k]) : 0.0f;
+    }
+    load(e0 + K * GS);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      sA = fmaf(dv[k], x[k], sA);
+      sB = fmaf(lv[k], x[k], sB);
+    }
+  }
+  warp_sum2(sA, sB, lane);
+  if (WPR > 1) {
+    if (lane == 0) part[wid] = make_float2(sA, sB);
+    __syncthreads();
+  }
+  if (have && first == 0) {
+    if (WPR > 1) {
+#pragma unroll
+      for (int k = 1; k < WPR; ++k) {
+        sA += part[wid + k].x;
+        sB += part[wid + k].y;
+      }
+    }
+    // row scales are powers of two: the FP32 product is exact
+    a.y[i] = a.sD ? make_float2(sA * a.sD[r], sB * a.sL[r]) : make_float2(sA, sB);
+  }
+}
+
+// One row per thread, one warp per CTA: the FP64 divisions spread over the SMs.
+__global__ void __launch_bounds__(kSweepConThreads) k_sweep_con(SweepArgs a, Tables t) {
+  __shared__ ConEntry con[kMaxCon];
+  stage_constraints(t, con);
+  const int64_t i = a.i0 + (int64_t)blockIdx.x * kSweepConThreads + threadIdx.x;
+  const bool have = i < a.i1;
+  const int64_t r = have ? a.list[i] : 0;
+  const uint32_t m = have ? a.mask[r] : 0u;
+  const double dd = have ? a.dd[r] : 0.0, ll = have ? a.ll[r] : 0.0, dl = have ? a.dl[r] : 0.0;
+  const double sd = have && a.sD ? (double)a.sD[r] : 1.0, sl = have && a.sL ? (double)a.sL[r] : 1.0;
+  __syncthreads();
+  const uint32_t todo = row_constraints(con, t.n_con, m);
+  pdl_wait();  // y of this block
+  pdl_release();
+  const float2 y = have ? a.y[i] : make_float2(0.0f, 0.0f);
+  double gD = 0.0, gL = 0.0, psum = 0.0, preach = 0.0, mx = 0.0;
+  unsigned nv = 0u;
+  eval_constraints(con, todo, t.c, y.x, y.y, dd, ll, dl, gD, gL, psum, preach, nv, mx);
+  if (have) a.gam[r] = make_float2((float)(gD * sd), (float)(gL * sl));
+  if (a.norm == FREDOPT_NORM_VIOLATED) {
+    psum = warp_sum_nz(psum);
+    if (threadIdx.x == 0) a.part[blockIdx.x] = psum;
+  }
+  if (a.in_solve) {  // exact whatever the order: integers, and a maximum of doubles >= 0 by their bits
+    nv = __reduce_add_sync(kFull, nv);
+    const long long bits = warp_max_bits(__double_as_longlong(mx));
+    if (threadIdx.x == 0 && nv) {
+      atomicAdd(&a.st->sweep_nv, (unsigned long long)nv);
+      atomicMax(&a.st->sweep_mx, bits);
+    }
+  }
+}
+
+// x_j += lam * scale / W_B * sum over the block's entries of column j of
+// D_ij gamma_D[i] + L_ij gamma_L[i].  LPC lanes per column, U columns per lane
+// group, their entries in flight together.  The FP64 update is left to the
+// CTA's first warps, one column per lane: GB300 issues an FP64 warp instruction
+// at the same low rate however few of its lanes are active, and one update per
+// column in the column's own warp was most of this kernel's time (19 us per
+// block of the clinical plan at 64 blocks).  A block's share of the columns is
+// uneven (its rows lie at one place), which is what is left.
+constexpr int kColsU = 2;  // columns per lane group (with 8 CTAs per SM: 3% faster than 4 with 4)
+template <typename VT, int LPC>
+__global__ void __launch_bounds__(256, 8) k_sweep_cols(SweepArgs a) {
+  constexpr int U = kColsU, CPW = 32 / LPC, COLS = 8 * U * CPW;  // columns per CTA
+  __shared__ float sums[COLS];
+  __shared__ double red[9];
+  __shared__ double sh_scale;
+  const int lane = threadIdx.x & 31;
+  const int sl = lane % LPC;
+  const int jw = (threadIdx.x >> 5) * (U * CPW) + lane / LPC;  // first column of the lane group, in the CTA
+  const int64_t jc = (int64_t)blockIdx.x * COLS;  // (columns dealt out with the grid's stride: 12% slower)
+  const VT* __restrict__ Dv = reinterpret_cast<const VT*>(a.Dv);
+  const VT* __restrict__ Lv = reinterpret_cast<const VT*>(a.Lv);
+  int p[U], left[U];  // positions are below 2^31
+  int most = 0;
+#pragma unroll
+  for (int k = 0; k < U; ++k) {
+    const int64_t j = jc + jw + k * CPW;
+    const int64_t p0 = j < a.n ? a.pos0[j] : 0, p1 = j < a.n ? a.pos1[j] : 0;
+    p[k] = (int)p0 + sl;
+    left[k] = (int)(p1 - p0) - sl;
+    most = max(most, left[k]);
+  }
+  int row[U];
+  VT d[U], l[U];
+  auto load = [&](int o) {
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      row[k] = -1;
+      if (o < left[k]) {
+        row[k] = a.row[p[k] + o];
+        d[k] = Dv[p[k] + o];
+        l[k] = Lv[p[k] + o];
+      }
+    }
+  };
+  load(0);
+  // the step: with NORM_ALL 1 / W_B is known before the predecessor ends
+  auto step_of = [&](double winv) {
+    if (threadIdx.x == 0) {
+      const double ps = a.in_solve ? (a.st->eta == 1.0 ? 1.0 : pow(a.st->eta, (double)a.st->k)) : a.prio_scale;
+      sh_scale = a.lam * ps * winv;
+    }
+  };
+  if (a.norm != FREDOPT_NORM_VIOLATED) step_of(*a.winv);
+  pdl_wait();  // gam (and the partial sums) of this block
+  pdl_release();
+  const int64_t jt = jc + threadIdx.x;
+  const bool mine = threadIdx.x < COLS && jt < a.n;  // this thread updates x[jt]
+  const float xj = mine ? a.x[jt] : 0.0f;
+  if (a.norm == FREDOPT_NORM_VIOLATED) {
+    double v = 0.0;
+    for (int i = threadIdx.x; i < a.con_blocks; i += 256) v += a.part[i];
+    v = block_sum256(v, red);
+    step_of(v > 0.0 ? 1.0 / v : 0.0);
+  }
+  float acc[U];
+#pragma unroll
+  for (int k = 0; k < U; ++k) acc[k] = 0.0f;
+  for (int o = 0; __any_sync(kFull, o < most); o += LPC) {
+    float2 g[U];
+    float dv[U], lv[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      g[k] = row[k] >= 0 ? a.gam[row[k]] : make_float2(0.0f, 0.0f);
+      dv[k] = row[k] >= 0 ? to_f(d[k]) : 0.0f;
+      lv[k] = row[k] >= 0 ? to_f(l[k]) : 0.0f;
+    }
+    load(o + LPC);
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      acc[k] = fmaf(dv[k], g[k].x, acc[k]);
+      acc[k] = fmaf(lv[k], g[k].y, acc[k]);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < U; ++k) {
+#pragma unroll
+    for (int o = LPC / 2; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(kFull, acc[k], o);
+    if (sl == 0) sums[jw + k * CPW] = acc[k];
+  }
+  __syncthreads();
+  if (mine) {
+    const float s = sums[threadIdx.x];
+    if (s != 0.0f) a.x[jt] = (float)((double)xj + sh_scale * (double)s);
+  }
+}
+
+// out = max(0, x); in a solve the last block writes the log entry and advances k.
+__global__ void __launch_bounds__(256) k_sweep_finish(int n, const float* __restrict__ x, float* __restrict__ out,
+                                                      int in_solve, DevState* st, LogEntry* log) {
+  __shared__ bool sh_last;
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x)
+    out[j] = x[j] > 0.0f ? x[j] : 0.0f;
+  if (!in_solve) return;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned prev = atomicAdd(&st->done, 1u);
+    sh_last = (prev == gridDim.x - 1);
+  }
+  __syncthreads();
+  if (sh_last && threadIdx.x == 0) {
+    __threadfence();
+    if (st->log_cap > 0) {
+      LogEntry e;
+      e.k = st->k;
+      e.s = st->s;
+      e.accepted = st->accepted;
+      e.n_violated = (int)st->sweep_nv;
+      e.beta = st->beta_acc;
+      e.f_start = st->f_start;
+      e.f_end = st->f_cur;
+      e.gnorm = st->gnorm;
+      e.max_violation = __longlong_as_double(st->sweep_mx);
+      log[st->k % st->log_cap] = e;
+    }
+    st->k += 1;
+    st->done = 0u;
+  }
+}
+
+template <typename VT, typename IT>
+void rows_inst(double mean_nnz, const SweepArgs& a, cudaStream_t s) {
+  const int64_t rows = a.i1 - a.i0;
+  auto go = [&](auto kernel, int wpr) {
+    launch_pdl(kernel, (unsigned)((rows * wpr + 7) / 8), 256, 0, s, a);
+  };
+  if (mean_nnz >= 1024.0) go(k_sweep_rows<VT, IT, 8>, 8);
+  else if (mean_nnz >= 512.0) go(k_sweep_rows<VT, IT, 4>, 4);
+  else if (mean_nnz >= 192.0) go(k_sweep_rows<VT, IT, 2>, 2);
+  else go(k_sweep_rows<VT, IT, 1>, 1);
+}
+
+template <typename VT>
+void cols_inst(double mean_entries, const SweepArgs& a, cudaStream_t s) {
+  constexpr int big = 8 * kColsU, small = 8 * kColsU * 4;  // columns per CTA
+  if (mean_entries > 12.0)
+    launch_pdl(k_sweep_cols<VT, 32>, (unsigned)(((int64_t)a.n + big - 1) / big), 256, 0, s, a);
+  else
+    launch_pdl(k_sweep_cols<VT, 8>, (unsigned)(((int64_t)a.n + small - 1) / small), 256, 0, s, a);
+}
+
+}  // namespace
+
+void launch_sweep_start(int n, const float* w, const float* g, int use_coef, float* x, DevState* st,
+                        cudaStream_t s) {
+  k_sweep_start<<<std::max(1, std::min(1024, (n + 255) / 256)), 256, 0, s>>>(n, w, g, use_coef, x, st);
+}
+
+void launch_sweep_pos(const int64_t* cp, const int32_t* row, int32_t n, const int64_t* bounds, int n_bounds,
+                      int64_t* pos, cudaStream_t s) {
+  const int64_t total = (int64_t)n_bounds * n;
+  if (total == 0) return;
+  const unsigned gb = (unsigned)std::min<int64_t>((total + 255) / 256, 65535);
+  k_sweep_pos<<<gb, 256, 0, s>>>(cp, row, n, bounds, n_bounds, pos);
+}
+
+void launch_sweep_weights(const Tables& t, const int64_t* list, int64_t n_list, int64_t size, int n_blk,
+                       const uint32_t* mask, const double* dd, const double* ll, const double* dl, double* winv,
+                       cudaStream_t s) {
+  if (n_blk > 0) k_sweep_weights<<<n_blk, 256, 0, s>>>(t, list, n_list, size, mask, dd, ll, dl, winv);
+}
+
+void launch_sweep_rows(int fmt, double mean_nnz, const SweepArgs& a, cudaStream_t s) {
+  auto by_index = [&](auto v) {
+    using VT = decltype(v);
+    if (a.col16) rows_inst<VT, uint16_t>(mean_nnz, a, s);
+    else rows_inst<VT, int32_t>(mean_nnz, a, s);
+  };
+  if (fmt == 1) by_index(__nv_bfloat16());
+  else if (fmt == 2) by_index(__half());
+  else by_index(float());
+}
+
+void launch_sweep_con(const Tables& t, const SweepArgs& a, cudaStream_t s) {
+  launch_pdl(k_sweep_con, (unsigned)a.con_blocks, kSweepConThreads, 0, s, a, t);
+}
+
+void launch_sweep_cols(int fmt, double mean_entries, const SweepArgs& a, cudaStream_t s) {
+  if (fmt == 1) cols_inst<__nv_bfloat16>(mean_entries, a, s);
+  else if (fmt == 2) cols_inst<__half>(mean_entries, a, s);
+  else cols_inst<float>(mean_entries, a, s);
+}
+
+void launch_sweep_finish(const Geometry& g, int n, const float* x, float* out, int in_solve, DevState* st,
+                         LogEntry* log, cudaStream_t s) {
+  const unsigned gb = (unsigned)std::max(1, std::min(g.n_sms, (n + 255) / 256));
+  k_sweep_finish<<<gb, 256, 0, s>>>(n, x, out, in_solve, st, log);
+}
+
+}  // namespace fo
