@@ -1083,6 +1083,7 @@ int fredopt_load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t 
 
   h->tab.n_con = 0;
   h->tab.n_obj = 0;
+  h->tab.obj_bits = 0u;
   h->have_con = false;
   h->obj_dose = false;
   h->W_all = 0.0;
@@ -1141,9 +1142,11 @@ int fredopt_set_objective(fredopt_t h, int n, const fredopt_objective_term* t) {
       return fail(h, FREDOPT_ERR_INVALID_ARG, "objective term " + std::to_string(i) + " invalid");
   free_graph(h);
   h->tab.n_obj = n;
+  h->tab.obj_bits = 0u;
   h->obj_dose = false;
   for (int i = 0; i < n; ++i) {
     h->tab.obj[i].bit = t[i].struct_bit;
+    h->tab.obj_bits |= 1u << t[i].struct_bit;
     h->tab.obj[i].q = t[i].quantity;
     h->tab.obj[i].target = t[i].target;
     h->tab.obj[i].weight = t[i].weight;

@@ -47,6 +47,7 @@ struct ObjEntry {
 struct Tables {
   int32_t n_con;
   int32_t n_obj;
+  uint32_t obj_bits;  // union of the objective terms' structure bits
   double c;  // cDL constant
   ConEntry con[kMaxCon];
   ObjEntry obj[kMaxObj];

@@ -636,34 +636,43 @@ __global__ void __launch_bounds__(kFwdThreads, 1024 / kFwdThreads) k_forward(Fwd
   auto flush = [&](int64_t base, int cnt, Acc myD, Acc myL) {
     if (lane >= cnt) return;
     const int64_t r = base + lane;
-    const double sd = a.sD ? (double)a.sD[r] : 1.0;
-    const double sl = a.sL ? (double)a.sL[r] : 1.0;
-    if (EPI == EPI_FINAL) {
-      const double Dx = (double)myD * sd, Lx = (double)myL * sl;
+    const float sd = a.sD ? a.sD[r] : 1.0f, sl = a.sL ? a.sL[r] : 1.0f;  // powers of two
+    if constexpr (EPI == EPI_FINAL) {
+      const double Dx = (double)myD * (double)sd, Lx = (double)myL * (double)sl;
       a.y64[r] = make_double2(Dx, Lx);
       const int64_t v = a.voxel ? a.voxel[r] : r;
       if (a.dose_out) a.dose_out[v] = (float)Dx;
       if (a.letd_out) a.letd_out[v] = Dx > 0.0 ? (float)(Lx / Dx) : 0.0f;
     } else {
-      const float Dx = (float)((double)myD * sd), Lx = (float)((double)myL * sl);
+      const float Dx = myD * sd, Lx = myL * sl;
       a.y[r] = make_float2(Dx, Lx);
-      if (EPI == EPI_OBJ) {
-        double f, rD, rL;
-        row_objective(t, a.mask[r], Dx, Lx, f, rD, rL);
-        a.r_out[r] = make_float2((float)(rD * sd), (float)(rL * sl));
-        acc0 += f;
-      } else if (EPI == EPI_BC) {
-        // B' = sum w (q(x) - T) q(g) = 1/2 (rD Dg + rL Lg); C' = sum w q(g)^2
-        const float2 rin = a.r_in[r];  // already multiplied by the row scales
-        acc0 += 0.5 * ((double)rin.x * (double)myD + (double)rin.y * (double)myL);
+      // FP64 only for rows with an objective term: GB300 issues an FP64 warp
+      // instruction in about 15 cycles per SM, however few lanes are active,
+      // and most warps hold no such row
+      if constexpr (EPI == EPI_OBJ) {
         const uint32_t m = a.mask[r];
-        double PD = 0.0, PL = 0.0;
-        for (int i = 0; i < t.n_obj; ++i) {
-          if (!((m >> t.obj[i].bit) & 1u)) continue;
-          if (t.obj[i].q == 0) PD += t.obj[i].weight;
-          else PL += t.obj[i].weight;
+        float2 res = make_float2(0.0f, 0.0f);
+        if (m & t.obj_bits) {
+          double f, rD, rL;
+          row_objective(t, m, Dx, Lx, f, rD, rL);
+          res = make_float2((float)(rD * (double)sd), (float)(rL * (double)sl));
+          acc0 += f;
         }
-        acc1 += PD * (double)Dx * (double)Dx + PL * t.c * t.c * (double)Lx * (double)Lx;
+        a.r_out[r] = res;
+      } else if constexpr (EPI == EPI_BC) {
+        const uint32_t m = a.mask[r];
+        if (m & t.obj_bits) {
+          // B' = sum w (q(x) - T) q(g) = 1/2 (rD Dg + rL Lg); C' = sum w q(g)^2
+          const float2 rin = a.r_in[r];  // already multiplied by the row scales
+          acc0 += 0.5 * ((double)rin.x * (double)myD + (double)rin.y * (double)myL);
+          double PD = 0.0, PL = 0.0;
+          for (int i = 0; i < t.n_obj; ++i) {
+            if (!((m >> t.obj[i].bit) & 1u)) continue;
+            if (t.obj[i].q == 0) PD += t.obj[i].weight;
+            else PL += t.obj[i].weight;
+          }
+          acc1 += PD * (double)Dx * (double)Dx + PL * t.c * t.c * (double)Lx * (double)Lx;
+        }
       }
     }
   };
@@ -677,7 +686,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1024 / kFwdThreads) k_forward(Fwd
         fwd_col<IT>(a), Dv, Lv, a.rp, r0, r1, lane, gather, flush, BlockBase{nullptr, nullptr, 0},
         SegCheck{a.n_elems, FO_CHECKED ? &a.st->err : nullptr});
     if (EPI == EPI_OBJ || EPI == EPI_BC) {  // partials per tile, summed later in tile order
-      const double s0 = warp_sum(acc0), s1 = warp_sum(acc1);
+      const double s0 = warp_sum_nz(acc0), s1 = EPI == EPI_BC ? warp_sum_nz(acc1) : 0.0;
       if (lane == 0) {
         a.part[job] = s0;
         if (EPI == EPI_BC) a.part[a.n_warps + job] = s1;
