@@ -301,8 +301,26 @@ bool claim_tiles(fredopt_t h) {
   return h->prm.tile_balance == 1 && h->nnz_hot >= kClaimMinNnzPerWarp * (int64_t)h->geo.fwd_warps;
 }
 
+// The kernels of a captured iteration form a dependent chain, each starting
+// while its predecessor drains (tiny plan: 62.3 -> 59.9 us per iteration).  Not
+// in long passes: CTAs placed early on the SMs that drain first unbalance them
+// (1.2e4 nonzeros per warp: 1% slower).  Not for plans that share the GPU:
+// CTAs that wait hold the slots of the other plans (six small plans in a batch:
+// 8.8 against 9.4 ms).  Not for single calls: a dependent launch costs the host
+// more than the few kernels gain (feasibility step of the tiny plan: 89 against
+// 95 us).
+constexpr int64_t kChainMaxNnzPerWarp = 4096;
+bool chained(fredopt_t h) {
+  return h->capturing && h->nnz_hot < kChainMaxNnzPerWarp * (int64_t)h->geo.fwd_warps &&
+         h->geo.n_sms == h->geo_full.n_sms;
+}
+
+// number of forward partials
+int n_parts(const Geometry& g, const FwdArgs& a) { return a.sched ? a.n_warps : forward_grid(g, a.n_warps); }
+
 FwdArgs fwd_args(fredopt_t h, bool hot) {
   FwdArgs a{};
+  a.pdl = chained(h);
   a.rp = h->rp.p;
   a.col = h->col.p;
   a.col16 = h->col16.p;
@@ -321,6 +339,7 @@ FwdArgs fwd_args(fredopt_t h, bool hot) {
   a.mask = h->mask.p;
   a.n_hot = h->n_hot;
   a.n_warps = a.sched ? h->n_tiles_hot : hot ? h->geo.fwd_warps : h->geo_full.fwd_warps;
+  a.part_stride = n_parts(h->geo, a);
   a.st = h->st.p;
   a.voxel = h->perm ? h->voxel.p : nullptr;
   return a;
@@ -343,6 +362,7 @@ BwdArgs bwd_args(fredopt_t h, const float2* coef) {
   b.coef = coef;
   b.chunk_sum = h->chunk_sum.p;
   b.n_warps = h->geo.bwd_warps;
+  b.pdl = chained(h);
   if (claim_tiles(h) && h->n_tiles_bwd > 0) {
     b.warp_chunk = h->tile_chunk.p;
     b.n_warps = h->n_tiles_bwd;
@@ -357,7 +377,8 @@ ColArgs col_args(fredopt_t h) {
   c.chunk_sum = h->chunk_sum.p;
   c.n = h->n;
   c.k2part = h->part.p + h->off_k2;
-  c.k2_blocks = h->geo.row_blocks;
+  c.k2_blocks = con_grid(h->geo, h->n_con_rows);
+  c.pdl = chained(h);
   c.W_all = h->W_all;
   c.st = h->st.p;
   c.log = h->log.p;
@@ -374,7 +395,7 @@ ConArgs con_args(fredopt_t h) {
   c.dl = h->mdl.p;
   c.sD = h->fmt ? h->sD.p : nullptr;
   c.sL = h->fmt ? h->sL.p : nullptr;
-  c.n_hot = h->n_hot;
+  c.pdl = chained(h);
   c.rows = h->con_rows.p;
   c.n_list = h->n_con_rows;
   c.gam = h->gam.p;
@@ -495,7 +516,7 @@ void enqueue_iteration(fredopt_t h) {
     fa.part = part_f;
     run(h, 0, [&] { launch_forward(G, h->fmt, EPI_OBJ, h->hint_fwd, fa, t, s); });
     for (int step = 0; step < N; ++step) {
-      int nf = fa.n_warps;
+      int nf = n_parts(G, fa);
       if (step > 0) {
         run(h, 5, [&] { launch_apply_step(h->n_hot, h->n, h->w.p, h->g.p, h->yw.p, h->yg.p, h->st.p, s); });
         run(h, 5, [&] {
@@ -517,8 +538,8 @@ void enqueue_iteration(fredopt_t h) {
       fb.part = part_bc;
       run(h, 0, [&] { launch_forward(G, h->fmt, EPI_BC, h->hint_fwd, fb, t, s); });
       run(h, 4, [&] {
-        launch_finish(step, part_f, nf, part_bc, fa.n_warps, part_g, G.col_blocks, h->st.p,
-                      h->part.p + h->off_stage, h->part.p + h->off_btab, kBetaTable, s);
+        launch_finish(step, part_f, nf, part_bc, n_parts(G, fa), part_g, col_grid(G, h->n), h->st.p,
+                      h->part.p + h->off_stage, h->part.p + h->off_btab, kBetaTable, chained(h), s);
       });
     }
   } else {
@@ -1071,7 +1092,7 @@ int fredopt_load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t 
   h->off_bc = h->off_f + std::max(max_tiles, G.row_blocks);
   h->off_g = h->off_bc + 2 * max_tiles;
   h->off_k2 = h->off_g + G.col_blocks;
-  h->off_fin = h->off_k2 + 4 * G.row_blocks;
+  h->off_fin = h->off_k2 + 4 * con_grid(G, std::numeric_limits<int64_t>::max() / 2);
   h->off_cnt = h->off_fin + 8 * h->geo_full.row_blocks;
   h->off_stage = h->off_cnt + 3 * h->geo_full.row_blocks;
   h->off_btab = h->off_stage + 4 * kFinishBlocks;
@@ -1630,7 +1651,7 @@ int fredopt_objective(fredopt_t h, const float* x, double* f_out, float* grad_ou
   ca.part = h->part.p + h->off_g;
   run(h, 3, [&] { launch_colfinish(G, COL_GRAD, ca, s); });
   CK(cudaGetLastError());
-  std::vector<double> hp(fa.n_warps);
+  std::vector<double> hp(n_parts(G, fa));
   CK(cudaMemcpyAsync(hp.data(), part_f, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
   if (grad_out) CK(copy_out(h, grad_out, h->gtmp.p, (size_t)h->n * sizeof(float), flags));
   rc = check_sticky(h);

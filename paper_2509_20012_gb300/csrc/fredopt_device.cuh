@@ -257,7 +257,7 @@ __device__ __forceinline__ void eval_constraints(const ConEntry* con, uint32_t t
 }
 
 // ---- programmatic dependent launch
-// A kernel launched with launch_pdl may start while its predecessor on the
+// A kernel launched as a link of a chain may start while its predecessor on the
 // stream still runs.  It may read what no kernel of the chain writes at once;
 // pdl_wait() returns when the predecessor has finished and its writes are
 // visible (every thread calls it before it exits, so a chain stays ordered).
@@ -266,8 +266,10 @@ __device__ __forceinline__ void eval_constraints(const ConEntry* con, uint32_t t
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Launch as a link of such a chain (pdl), or ordered after the whole predecessor.
 template <typename... P, typename... A>
-void launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A&&... args) {
+void launch_chain(bool pdl, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                  A&&... args) {
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
@@ -277,7 +279,7 @@ void launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = pdl ? 1 : 0;
   cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 

@@ -102,8 +102,10 @@ struct FwdArgs {
   int64_t n_hot;
   float2* r_out;         // EPI_OBJ: objective residual, scaled for the CSC
   const float2* r_in;    // EPI_BC: residual of EPI_OBJ
-  double* part;          // per-tile partials, stride n_warps (the tile count): [f] or [B', C']
-  int32_t n_warps;        // number of tiles in warp_row (the partials' stride)
+  double* part;          // partials [f] or [B', C']: one per claimed tile, or per CTA (static tiles)
+  int32_t part_stride;
+  int32_t n_warps;        // number of tiles in warp_row
+  bool pdl;              // launched as a link of a dependent chain
   DevState* st;
   // EPI_FINAL
   double2* y64;
@@ -129,6 +131,7 @@ struct BwdArgs {
   const float2* coef;         // per streamed row
   float* chunk_sum;
   int32_t n_warps;            // number of tiles
+  bool pdl;
 };
 
 struct ColArgs {
@@ -152,6 +155,7 @@ struct ColArgs {
   int32_t log_block;         // COL_PROJ in a solve with has_scale: 1 = one extra block closes the
                              // iteration (no block reads k), instead of the last block to finish
   int32_t use_u;             // 0: no transposed product (no constraints): u = 0
+  bool pdl;
   DevState* st;
   LogEntry* log;
 };
@@ -165,15 +169,13 @@ struct ConArgs {
   const double* dl;
   const float* sD;
   const float* sL;
-  int64_t r0;           // rows [r0, n_hot) are evaluated (0 for the whole set)
-  int64_t n_hot;
-  // when set, the rows evaluated are rows[0 .. n_list) instead (the rows
-  // with a structure bit, ascending); every other row's gam stays 0
+  // the rows with a structure bit, ascending; every other row's gam stays 0
   const int64_t* rows;
   int64_t n_list;
   float2* gam;
   double* part;         // per-block: [sum p violated, n violated, max violation, sum p reachable]
   int32_t use_coef;
+  bool pdl;
   DevState* st;
 };
 
@@ -206,15 +208,19 @@ void launch_forward(const Geometry& g, int fmt, int epi, bool stream_hint, const
 void launch_backward(const Geometry& g, int fmt, bool stream_hint, bool use_D, const BwdArgs& a,
                      cudaStream_t s);
 void launch_colfinish(const Geometry& g, int mode, const ColArgs& a, cudaStream_t s);
-// grid 0: g.row_blocks CTAs (the partials' stride); otherwise that many
-void launch_constraints(const Geometry& g, const Tables& t, const ConArgs& a, cudaStream_t s, int grid = 0);
+void launch_constraints(const Geometry& g, const Tables& t, const ConArgs& a, cudaStream_t s);
+// CTAs (the numbers of partials) of the forward product with n_warps tiles, of
+// the column finish and of the constraint evaluation
+int forward_grid(const Geometry& g, int n_warps);
+int col_grid(const Geometry& g, int n);
+int con_grid(const Geometry& g, int64_t n_list);
 constexpr int kFinishBlocks = 64;  // CTAs of the scalar finish; stage holds 4 * kFinishBlocks doubles
 // btab[s] = beta0 alpha^s for s < n_btab (filled at fredopt_begin)
 constexpr long long kBetaTable = 1 << 16;
 void launch_beta_table(double* out, long long n, double beta0, double alpha, cudaStream_t s);
 void launch_finish(int step, const double* part_f, int nf, const double* part_bc, int nbc,
                    const double* part_g, int ng, DevState* st, double* stage, const double* btab,
-                   long long n_btab, cudaStream_t s);
+                   long long n_btab, bool pdl, cudaStream_t s);
 void launch_count_rows(int grid, const Tables& t, const uint32_t* mask, const double* dd,
                        const double* ll, const double* dl, const int64_t* rows, int64_t n_list, double* part,
                        cudaStream_t s);

@@ -91,6 +91,8 @@ constexpr bool kBwdPingPong = FO_BWD_PP != 0;
 constexpr int kPrefetchUnits = FO_PREFETCH_UNITS;
 constexpr int kBwdThreads = 256;
 constexpr int kRowThreads = 256;
+constexpr int kConThreads = 64;
+constexpr int kFinishOne = 1024;  // partials per array up to which one CTA forms the scalar finish
 constexpr int kColThreads = 256;
 constexpr int kMbarSpins = FREDOPT_WAIT_POLLS;
 // Lane mapping of a block's 128 elements (element of value q of lane l):
@@ -376,12 +378,17 @@ __device__ __forceinline__ void load_blk_pairs(Blk<VT>& k, const IT* idx, const 
 // The arrays must be readable (zero padded) up to
 // round_up(ptr[r1], 32*V) + U*32*V elements (a prefetch starts below ptr[r1]
 // and covers U*32*V elements, within the same bound).
+// ready() runs when the first unit's loads are on their way and before the
+// first gather: it waits for what the gathers read, and false ends the call.
+struct NoWait {
+  __device__ bool operator()() const { return true; }
+};
 template <typename VT, typename Acc, bool S, bool USE_A, int U, bool BASED = false, int LM = 0,
-          typename IT, class Gather, class Flush, int PF = kPrefetchUnits, bool PP = false>
+          typename IT, class Gather, class Flush, class Ready, int PF = kPrefetchUnits, bool PP = false>
 __device__ __forceinline__ void stream_segments(const IT* __restrict__ idx,
                                                 const VT* __restrict__ Av, const VT* __restrict__ Bv,
                                                 const int64_t* __restrict__ ptr, int64_t r0, int64_t r1,
-                                                int lane, Gather gather, Flush flush,
+                                                int lane, Gather gather, Flush flush, Ready ready,
                                                 BlockBase bbase = BlockBase{nullptr, nullptr, 0},
                                                 SegCheck chk = SegCheck{0, nullptr}) {
   constexpr int V = VecOf<VT>::V;
@@ -532,6 +539,7 @@ __device__ __forceinline__ void stream_segments(const IT* __restrict__ idx,
     // of the other are in flight (no register copies of pending loads)
     Blk<VT> ua[U], ub[U];
     load_unit(ua, b);
+    if (!ready()) return;
     while (true) {
       if (b + UB < pe) load_unit(ub, b + UB);
       consume(ua, b);
@@ -546,10 +554,21 @@ __device__ __forceinline__ void stream_segments(const IT* __restrict__ idx,
     // one register unit: its U blocks are loaded together, then consumed;
     // latency is hidden by the other warps of the SM
     Blk<VT> ua[U];
-    while (!done) {
+    if constexpr (std::is_same<Ready, NoWait>::value) {
+      while (!done) {
+        load_unit(ua, b);
+        consume(ua, b);
+        b += UB;
+      }
+    } else {
       load_unit(ua, b);
-      consume(ua, b);
-      b += UB;
+      if (!ready()) return;
+      while (true) {
+        consume(ua, b);
+        if (done) break;
+        b += UB;
+        load_unit(ua, b);
+      }
     }
   }
 }
@@ -586,27 +605,40 @@ template <typename VT, int EPI, bool XS, bool S, typename IT>
 __global__ void __launch_bounds__(kFwdThreads, 1024 / kFwdThreads) k_forward(FwdArgs a, Tables t) {
   extern __shared__ __align__(128) unsigned char smem[];
   using Acc = typename std::conditional<EPI == EPI_FINAL, DF, float>::type;
-  const float* __restrict__ x = a.x;
+  const float* x = XS ? reinterpret_cast<const float*>(smem) : a.x;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + (size_t)a.n_x_pad * sizeof(float));
   if (XS) {
-    float* xs = reinterpret_cast<float*>(smem);
-    uint64_t* bar = reinterpret_cast<uint64_t*>(smem + (size_t)a.n_x_pad * sizeof(float));
     if (threadIdx.x == 0) {
       mbar_init(bar, 1);
       fence_mbar_init();
     }
     __syncthreads();
-    const uint32_t bytes = (uint32_t)a.n_x_pad * (uint32_t)sizeof(float);
-    if (threadIdx.x == 0) {
-      mbar_expect_tx(bar, bytes);
-      bulk_g2s(xs, a.x, bytes, bar);
-    }
-    if (!mbar_wait(bar, 0, kMbarSpins)) {
-      if (threadIdx.x == 0) atomicOr(&a.st->err, 1);
-      mbar_wait(bar, 0, kMbarSpins);  // let the copy in flight land before leaving
-      return;
-    }
-    x = xs;
   }
+  // Every warp runs this once: the predecessor has finished, and x is staged in
+  // shared memory (by thread 0's bulk copy) unless the bounded wait gives up.
+  // In passes that stay in L2 (S = false) a warp has its first loads on their way
+  // by then (1.4% of the tiny plan's iteration; 0.2% slower in the long passes).
+  bool waited = false, staged = true;
+  auto ready = [&]() -> bool {
+    if (waited) return staged;
+    waited = true;
+    pdl_wait();
+    pdl_release();
+    if (XS) {
+      if (threadIdx.x == 0) {
+        const uint32_t bytes = (uint32_t)a.n_x_pad * (uint32_t)sizeof(float);
+        mbar_expect_tx(bar, bytes);
+        bulk_g2s(smem, a.x, bytes, bar);
+      }
+      __syncwarp();
+      staged = __all_sync(kFull, mbar_wait(bar, 0, kMbarSpins));
+      if (!staged) {
+        if ((threadIdx.x & 31) == 0) atomicOr(&a.st->err, 1);
+        mbar_wait(bar, 0, kMbarSpins);  // let the copy in flight land before leaving
+      }
+    }
+    return staged;
+  };
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   // Tiles: a warp streams tile `warp` (static schedule) or claims tiles in
@@ -676,24 +708,45 @@ __global__ void __launch_bounds__(kFwdThreads, 1024 / kFwdThreads) k_forward(Fwd
       }
     }
   };
-  while (job < a.n_warps) {
+  if (S) ready();
+  while (job < a.n_warps && staged) {
     // EPI_FINAL over listed rows: a tile is one row
     const bool one = EPI == EPI_FINAL && a.rows != nullptr;
     const int64_t r0 = one ? a.rows[job] : a.warp_row[2 * job], r1 = one ? r0 + 1 : a.warp_row[2 * job + 1];
     acc0 = 0.0;
     acc1 = 0.0;
-    stream_segments<VT, Acc, S, true, (sizeof(VT) == 4 ? kFwdUnroll : kFwdUnroll16)>(
-        fwd_col<IT>(a), Dv, Lv, a.rp, r0, r1, lane, gather, flush, BlockBase{nullptr, nullptr, 0},
-        SegCheck{a.n_elems, FO_CHECKED ? &a.st->err : nullptr});
-    if (EPI == EPI_OBJ || EPI == EPI_BC) {  // partials per tile, summed later in tile order
+    const auto stream = [&](auto before) {
+      stream_segments<VT, Acc, S, true, (sizeof(VT) == 4 ? kFwdUnroll : kFwdUnroll16)>(
+          fwd_col<IT>(a), Dv, Lv, a.rp, r0, r1, lane, gather, flush, before, BlockBase{nullptr, nullptr, 0},
+          SegCheck{a.n_elems, FO_CHECKED ? &a.st->err : nullptr});
+    };
+    if constexpr (S) stream(NoWait());
+    else stream(ready);
+    if ((EPI == EPI_OBJ || EPI == EPI_BC) && a.sched) {  // partials per tile, summed later in tile order
       const double s0 = warp_sum_nz(acc0), s1 = EPI == EPI_BC ? warp_sum_nz(acc1) : 0.0;
       if (lane == 0) {
         a.part[job] = s0;
-        if (EPI == EPI_BC) a.part[a.n_warps + job] = s1;
+        if (EPI == EPI_BC) a.part[a.part_stride + job] = s1;
       }
     }
     if (!a.sched) break;
     job = claim();
+  }
+  ready();  // a warp without rows waits too: no CTA leaves with the copy in flight
+  if ((EPI == EPI_OBJ || EPI == EPI_BC) && !a.sched) {  // one tile per warp: a partial per CTA, in warp order
+    const int wid = threadIdx.x >> 5;
+    const double s0 = warp_sum_nz(acc0), s1 = EPI == EPI_BC ? warp_sum_nz(acc1) : 0.0;
+    __syncthreads();  // x is not read any more
+    double* red = reinterpret_cast<double*>(smem);
+    if (lane == 0) {
+      red[wid] = s0;
+      red[32 + wid] = s1;
+    }
+    __syncthreads();
+    if (wid < 2) {
+      const double v = warp_sum_nz(lane < kFwdThreads / 32 ? red[32 * wid + lane] : 0.0);
+      if (lane == 0 && (wid == 0 || EPI == EPI_BC)) a.part[wid * a.part_stride + blockIdx.x] = v;
+    }
   }
   if (a.sched && lane == 0) {
     __threadfence();
@@ -718,7 +771,7 @@ __global__ void __launch_bounds__(kBwdThreads, FO_BWD_MIN_BLOCKS) k_backward(Bwd
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const VT* __restrict__ Dv = reinterpret_cast<const VT*>(a.Dv);
   const VT* __restrict__ Lv = reinterpret_cast<const VT*>(a.Lv);
-  const float2* __restrict__ cf = a.coef;
+  const float2* cf = a.coef;  // the predecessor's output
   auto gather = [&](int r) {
 #if FO_CHECKED
     if ((uint64_t)(int64_t)r >= (uint64_t)a.n_rows) {
@@ -726,8 +779,9 @@ __global__ void __launch_bounds__(kBwdThreads, FO_BWD_MIN_BLOCKS) k_backward(Bwd
       r = 0;
     }
 #endif
-    if (!UD && FO_BWD_GATHER_Y) return make_float2(0.0f, __ldg(&cf[r].y));
-    return __ldg(&cf[r]);
+    // plain loads: what a chained predecessor wrote is not read-only
+    if (!UD && FO_BWD_GATHER_Y) return make_float2(0.0f, cf[r].y);
+    return cf[r];
   };
   float* out = a.chunk_sum;
   auto flush = [&](int64_t base, int cnt, float mA, float mB) {
@@ -741,16 +795,20 @@ __global__ void __launch_bounds__(kBwdThreads, FO_BWD_MIN_BLOCKS) k_backward(Bwd
     return (int)__shfl_sync(kFull, j, 0);
   };
   int job = a.sched ? claim() : warp;
+  // (the first unit's loads ahead of the wait, as in the forward product, cost
+  // registers that this kernel does not have)
+  pdl_wait();
+  pdl_release();
   while (job < a.n_warps) {
     if (NB)
       stream_segments<VT, float, S, UD, bwd_units<VT, UD>(), true, kBwdLaneMap<VT>,
-                      uint16_t, decltype(gather), decltype(flush), kPrefetchUnits, kBwdPingPong>(
-          a.row16, Dv, Lv, a.chunk_ptr, a.warp_chunk[job], a.warp_chunk[job + 1], lane, gather, flush,
+                      uint16_t, decltype(gather), decltype(flush), NoWait, kPrefetchUnits, kBwdPingPong>(
+          a.row16, Dv, Lv, a.chunk_ptr, a.warp_chunk[job], a.warp_chunk[job + 1], lane, gather, flush, NoWait(),
           BlockBase{a.hdr, a.ovf, a.n_ovf}, SegCheck{a.n_elems, FO_CHECKED ? &a.st->err : nullptr});
     else
       stream_segments<VT, float, S, UD, bwd_units<VT, UD>(), false, kBwdLaneMap<VT>,
-                      int32_t, decltype(gather), decltype(flush), kPrefetchUnits, kBwdPingPong>(
-          a.row, Dv, Lv, a.chunk_ptr, a.warp_chunk[job], a.warp_chunk[job + 1], lane, gather, flush,
+                      int32_t, decltype(gather), decltype(flush), NoWait, kPrefetchUnits, kBwdPingPong>(
+          a.row, Dv, Lv, a.chunk_ptr, a.warp_chunk[job], a.warp_chunk[job + 1], lane, gather, flush, NoWait(),
           BlockBase{nullptr, nullptr, 0}, SegCheck{a.n_elems, FO_CHECKED ? &a.st->err : nullptr});
     if (!a.sched) break;
     job = claim();
@@ -801,6 +859,8 @@ __global__ void __launch_bounds__(kColThreads) k_colfinish(ColArgs a) {
   // concurrently with the others (nothing else in the launch reads k), and
   // the other blocks split the columns
   const int nb = (int)gridDim.x - (MODE == COL_PROJ ? a.log_block : 0);
+  pdl_wait();
+  pdl_release();
   if (MODE == COL_PROJ && a.log_block && (int)blockIdx.x == nb) {
     close_iteration(a, red);
     return;
@@ -864,22 +924,35 @@ __global__ void __launch_bounds__(kColThreads) k_colfinish(ColArgs a) {
 
 // ------------------------------------------------------------------ K2
 
-__global__ void __launch_bounds__(kRowThreads) k_constraints(ConArgs a, Tables t) {
+// One listed row per thread and step.  Bound by FP64 instruction issue (an
+// FP64 warp instruction holds an SM's pipe for about 15 cycles), so the rows are
+// spread over CTAs of two warps and as many SMs as there are.
+__global__ void __launch_bounds__(kConThreads) k_constraints(ConArgs a, Tables t) {
+  constexpr int kWarps = kConThreads / 32;
   __shared__ ConEntry con[kMaxCon];
+  __shared__ double wred[3][kWarps];
+  __shared__ long long wcnt[kWarps];
   stage_constraints(t, con);
   __syncthreads();
-  // block b evaluates a contiguous slice of the rows: of [r0, n_hot), or of
-  // the listed rows
-  const int64_t lo = a.rows ? 0 : a.r0, hi = a.rows ? a.n_list : a.n_hot;
-  const int64_t per = (hi - lo + gridDim.x - 1) / gridDim.x;
-  const int64_t j0 = lo + (int64_t)blockIdx.x * per;
-  const int64_t j1 = min(hi, j0 + per);
+  const int64_t step = (int64_t)gridDim.x * kConThreads;
+  int64_t j = (int64_t)blockIdx.x * kConThreads + threadIdx.x;
+  int64_t i = 0;
+  uint32_t todo = 0u;
+  double dd = 0.0, ll = 0.0, dl = 0.0;
+  auto row = [&]() {  // what does not depend on the predecessor
+    i = a.rows[j];
+    todo = row_constraints(con, t.n_con, a.mask[i]);
+    dd = a.dd[i];
+    ll = a.ll[i];
+    dl = a.dl[i];
+  };
+  if (j < a.n_list) row();
+  pdl_wait();
+  pdl_release();
   const double coef = a.use_coef ? a.st->coef : 0.0;
   double psum = 0.0, mx = 0.0, preach = 0.0;
   unsigned viol = 0u;
-  for (int64_t j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
-    const int64_t i = a.rows ? a.rows[j] : j;
-    const uint32_t todo = row_constraints(con, t.n_con, a.mask[i]);
+  while (j < a.n_list) {
     float2 out = make_float2(0.f, 0.f);
     if (todo) {
       const float2 w2 = a.yw[i];
@@ -890,22 +963,20 @@ __global__ void __launch_bounds__(kRowThreads) k_constraints(ConArgs a, Tables t
         xl += coef * (double)g2.y;
       }
       double gD = 0.0, gL = 0.0;
-      eval_constraints(con, todo, t.c, xd, xl, a.dd[i], a.ll[i], a.dl[i], gD, gL, psum, preach, viol, mx);
-      const double sd = a.sD ? (double)a.sD[i] : 1.0;
-      const double sl = a.sL ? (double)a.sL[i] : 1.0;
-      out = make_float2((float)(gD * sd), (float)(gL * sl));
+      eval_constraints(con, todo, t.c, xd, xl, dd, ll, dl, gD, gL, psum, preach, viol, mx);
+      // the row scales are powers of two: exact in FP32
+      out = a.sD ? make_float2((float)gD * a.sD[i], (float)gL * a.sL[i]) : make_float2((float)gD, (float)gL);
     }
     a.gam[i] = out;
+    j += step;
+    if (j < a.n_list) row();
   }
-  long long nv = viol;
   // the block's two sums, its violated-row count and its largest violation
   // (>= 0): warp reductions (the FP64 butterflies skipped by warps without
   // violated or reachable rows), then the warp results in warp order
-  __shared__ double wred[3][kRowThreads / 32];
-  __shared__ long long wcnt[kRowThreads / 32];
   psum = warp_sum_nz(psum);
   preach = warp_sum_nz(preach);
-  nv = warp_isum(nv);
+  const long long nv = (long long)__reduce_add_sync(kFull, viol);
   mx = warp_max_nonneg(mx);
   if ((threadIdx.x & 31) == 0) {
     const int wi = threadIdx.x >> 5;
@@ -917,29 +988,17 @@ __global__ void __launch_bounds__(kRowThreads) k_constraints(ConArgs a, Tables t
   __syncthreads();
   if (threadIdx.x < 4) {
     const int k = threadIdx.x;
-    double t;
-    if (k == 1) {
-      long long c = 0;
+    double r = wred[k == 0 ? 0 : k == 3 ? 1 : 2][0];
+    long long c = wcnt[0];
 #pragma unroll
-      for (int w = 0; w < kRowThreads / 32; ++w) c += wcnt[w];
-      t = (double)c;
-    } else if (k == 2) {
-      long long b = 0;
-#pragma unroll
-      for (int w = 0; w < kRowThreads / 32; ++w) {
-        const long long x = __double_as_longlong(wred[2][w]);
-        b = x > b ? x : b;
-      }
-      t = __longlong_as_double(b);
-    } else {
-      const int src = k == 0 ? 0 : 1;
-      t = wred[src][0];
-#pragma unroll
-      for (int w = 1; w < kRowThreads / 32; ++w) t += wred[src][w];
+    for (int w = 1; w < kWarps; ++w) {
+      c += wcnt[w];
+      if (k == 2) r = fmax(r, wred[2][w]);
+      else if (k != 1) r += wred[k == 0 ? 0 : 1][w];
     }
     // partial slices: sum of priorities of violated rows, violated rows,
     // largest violation, sum of priorities of reachable rows
-    a.part[k * gridDim.x + blockIdx.x] = t;
+    a.part[k * gridDim.x + blockIdx.x] = k == 1 ? (double)c : r;
   }
 }
 
@@ -955,7 +1014,8 @@ __global__ void __launch_bounds__(kRowThreads) k_constraints(ConArgs a, Tables t
 // the two warps' results in warp order; the last CTA adds the 64 slice sums
 // of array k in warp k.  The solve state and the first trial steps are
 // loaded at the start, so that the last CTA's chain of dependent loads is
-// short.
+// short.  With at most kFinishOne partials per array (one per forward CTA
+// instead of one per claimed tile) a single CTA does it all.
 __global__ void __launch_bounds__(256) k_finish(int step, const double* part_f, int nf,
                                                 const double* part_bc, int nbc, const double* part_g,
                                                 int ng, DevState* st, double* stage, const double* btab,
@@ -975,6 +1035,8 @@ __global__ void __launch_bounds__(256) k_finish(int step, const double* part_f, 
     const long long si = s0 + lane;
     if (si < n_btab) beta_pre = btab[si];
   }
+  pdl_wait();
+  pdl_release();
   {
     const int k = wid >> 1, h = wid & 1;
     const double* arr = k == 0 ? part_f : k == 1 ? part_bc : k == 2 ? part_bc + nbc : part_g;
@@ -987,20 +1049,24 @@ __global__ void __launch_bounds__(256) k_finish(int step, const double* part_f, 
     if (lane == 0) wred[k][h] = v;
   }
   __syncthreads();
-  if (threadIdx.x < 4) stage[threadIdx.x * G + b] = wred[threadIdx.x][0] + wred[threadIdx.x][1];
-  if (threadIdx.x == 0) {
+  if (G == 1) {
+    if (threadIdx.x < 4) tot_sh[threadIdx.x] = wred[threadIdx.x][0] + wred[threadIdx.x][1];
+  } else {
+    if (threadIdx.x < 4) stage[threadIdx.x * G + b] = wred[threadIdx.x][0] + wred[threadIdx.x][1];
+    if (threadIdx.x == 0) {
+      __threadfence();
+      sh_last = atomicAdd(&st->done_fin, 1u) == (unsigned)G - 1;
+    }
+    __syncthreads();
+    if (!sh_last) return;
     __threadfence();
-    sh_last = atomicAdd(&st->done_fin, 1u) == (unsigned)G - 1;
-  }
-  __syncthreads();
-  if (!sh_last) return;
-  __threadfence();
-  // the slice sums, written by other CTAs of this launch: read past L1
-  if (wid < 4) {
-    double v = 0.0;
-    for (int i = lane; i < G; i += 32) v += __ldcg(&stage[wid * G + i]);
-    v = warp_sum_nz(v);
-    if (lane == 0) tot_sh[wid] = v;
+    // the slice sums, written by other CTAs of this launch: read past L1
+    if (wid < 4) {
+      double v = 0.0;
+      for (int i = lane; i < G; i += 32) v += __ldcg(&stage[wid * G + i]);
+      v = warp_sum_nz(v);
+      if (lane == 0) tot_sh[wid] = v;
+    }
   }
   __syncthreads();
   if (wid != 0) return;
@@ -1240,13 +1306,17 @@ __global__ void k_scatter_y(const float2* y, const int64_t* voxel, int64_t n, fl
 
 // ------------------------------------------------------------------ launch wrappers
 
+// only the CTAs that hold scheduled warps (all of them for a full pass)
+int forward_grid(const Geometry& g, int n_warps) {
+  const int wpb = g.fwd_threads / 32;
+  return std::max(1, std::min(g.fwd_blocks, (n_warps + wpb - 1) / wpb));
+}
+
 template <typename VT, int EPI, bool XS, bool S, typename IT = int32_t>
 static void fwd_inst(const Geometry& g, const FwdArgs& a, const Tables& t, cudaStream_t s) {
-  const size_t smem = XS ? (size_t)a.n_x_pad * sizeof(float) + 16 : 0;
-  // only the CTAs that hold scheduled warps (all of them for a full pass)
-  const int wpb = g.fwd_threads / 32;
-  const int blocks = std::max(1, std::min(g.fwd_blocks, (a.n_warps + wpb - 1) / wpb));
-  k_forward<VT, EPI, XS, S, IT><<<blocks, g.fwd_threads, smem, s>>>(a, t);
+  // x and its barrier; the epilogue's reduction takes the same place (512 bytes)
+  const size_t smem = std::max<size_t>(XS ? (size_t)a.n_x_pad * sizeof(float) + 16 : 0, 512);
+  launch_chain(a.pdl, k_forward<VT, EPI, XS, S, IT>, forward_grid(g, a.n_warps), g.fwd_threads, smem, s, a, t);
 }
 
 template <typename VT, int EPI>
@@ -1297,11 +1367,11 @@ void launch_forward(const Geometry& g, int fmt, int epi, bool stream_hint, const
 template <typename VT, bool NB>
 static void bwd_dispatch_nb(const Geometry& g, bool st, bool ud, const BwdArgs& a, cudaStream_t s) {
   if (st) {
-    if (ud) k_backward<VT, true, true, NB><<<g.bwd_blocks, g.bwd_threads, 0, s>>>(a);
-    else k_backward<VT, true, false, NB><<<g.bwd_blocks, g.bwd_threads, 0, s>>>(a);
+    if (ud) launch_chain(a.pdl, k_backward<VT, true, true, NB>, g.bwd_blocks, g.bwd_threads, 0, s, a);
+    else launch_chain(a.pdl, k_backward<VT, true, false, NB>, g.bwd_blocks, g.bwd_threads, 0, s, a);
   } else {
-    if (ud) k_backward<VT, false, true, NB><<<g.bwd_blocks, g.bwd_threads, 0, s>>>(a);
-    else k_backward<VT, false, false, NB><<<g.bwd_blocks, g.bwd_threads, 0, s>>>(a);
+    if (ud) launch_chain(a.pdl, k_backward<VT, false, true, NB>, g.bwd_blocks, g.bwd_threads, 0, s, a);
+    else launch_chain(a.pdl, k_backward<VT, false, false, NB>, g.bwd_blocks, g.bwd_threads, 0, s, a);
   }
 }
 template <typename VT>
@@ -1317,14 +1387,23 @@ void launch_backward(const Geometry& g, int fmt, bool stream_hint, bool use_D, c
   else bwd_dispatch<float>(g, stream_hint, use_D, a, s);
 }
 
+int col_grid(const Geometry& g, int n) { return std::max(1, std::min(g.col_blocks, (n + 127) / 128)); }
+
 void launch_colfinish(const Geometry& g, int mode, const ColArgs& a, cudaStream_t s) {
-  if (mode == COL_OUT) k_colfinish<COL_OUT><<<g.col_blocks, kColThreads, 0, s>>>(a);
-  else if (mode == COL_GRAD) k_colfinish<COL_GRAD><<<g.col_blocks, kColThreads, 0, s>>>(a);
-  else k_colfinish<COL_PROJ><<<g.col_blocks + a.log_block, kColThreads, 0, s>>>(a);
+  const int grid = col_grid(g, a.n);
+  if (mode == COL_OUT) launch_chain(a.pdl, k_colfinish<COL_OUT>, grid, kColThreads, 0, s, a);
+  else if (mode == COL_GRAD) launch_chain(a.pdl, k_colfinish<COL_GRAD>, grid, kColThreads, 0, s, a);
+  else launch_chain(a.pdl, k_colfinish<COL_PROJ>, grid + a.log_block, kColThreads, 0, s, a);
 }
 
-void launch_constraints(const Geometry& g, const Tables& t, const ConArgs& a, cudaStream_t s, int grid) {
-  k_constraints<<<grid > 0 ? grid : g.row_blocks, kRowThreads, 0, s>>>(a, t);
+int con_grid(const Geometry& g, int64_t n_list) {
+  // as many threads at most as row_blocks CTAs of the other row kernels have
+  const int64_t cap = (int64_t)g.row_blocks * (kRowThreads / kConThreads);
+  return (int)std::max<int64_t>(1, std::min<int64_t>(cap, (n_list + kConThreads - 1) / kConThreads));
+}
+
+void launch_constraints(const Geometry& g, const Tables& t, const ConArgs& a, cudaStream_t s) {
+  launch_chain(a.pdl, k_constraints, con_grid(g, a.n_list), kConThreads, 0, s, a, t);
 }
 
 __global__ void k_beta_table(double* out, long long n, double beta0, double alpha) {
@@ -1338,8 +1417,9 @@ void launch_beta_table(double* out, long long n, double beta0, double alpha, cud
 
 void launch_finish(int step, const double* part_f, int nf, const double* part_bc, int nbc,
                    const double* part_g, int ng, DevState* st, double* stage, const double* btab,
-                   long long n_btab, cudaStream_t s) {
-  k_finish<<<kFinishBlocks, 256, 0, s>>>(step, part_f, nf, part_bc, nbc, part_g, ng, st, stage, btab, n_btab);
+                   long long n_btab, bool pdl, cudaStream_t s) {
+  const bool one = std::max(std::max(nf, nbc), ng) <= kFinishOne;
+  launch_chain(pdl, k_finish, one ? 1 : kFinishBlocks, 256, 0, s, step, part_f, nf, part_bc, nbc, part_g, ng, st, stage, btab, n_btab);
 }
 
 void launch_apply_step(int64_t n_hot, int n, float* w, const float* g, float2* yw, const float2* yg,

@@ -304,7 +304,7 @@ template <typename VT, typename IT>
 void rows_inst(double mean_nnz, const SweepArgs& a, cudaStream_t s) {
   const int64_t rows = a.i1 - a.i0;
   auto go = [&](auto kernel, int wpr) {
-    launch_pdl(kernel, (unsigned)((rows * wpr + 7) / 8), 256, 0, s, a);
+    launch_chain(true, kernel, (unsigned)((rows * wpr + 7) / 8), 256, 0, s, a);
   };
   if (mean_nnz >= 1024.0) go(k_sweep_rows<VT, IT, 8>, 8);
   else if (mean_nnz >= 512.0) go(k_sweep_rows<VT, IT, 4>, 4);
@@ -316,9 +316,9 @@ template <typename VT>
 void cols_inst(double mean_entries, const SweepArgs& a, cudaStream_t s) {
   constexpr int big = 8 * kColsU, small = 8 * kColsU * 4;  // columns per CTA
   if (mean_entries > 12.0)
-    launch_pdl(k_sweep_cols<VT, 32>, (unsigned)(((int64_t)a.n + big - 1) / big), 256, 0, s, a);
+    launch_chain(true, k_sweep_cols<VT, 32>, (unsigned)(((int64_t)a.n + big - 1) / big), 256, 0, s, a);
   else
-    launch_pdl(k_sweep_cols<VT, 8>, (unsigned)(((int64_t)a.n + small - 1) / small), 256, 0, s, a);
+    launch_chain(true, k_sweep_cols<VT, 8>, (unsigned)(((int64_t)a.n + small - 1) / small), 256, 0, s, a);
 }
 
 }  // namespace
@@ -354,7 +354,7 @@ void launch_sweep_rows(int fmt, double mean_nnz, const SweepArgs& a, cudaStream_
 }
 
 void launch_sweep_con(const Tables& t, const SweepArgs& a, cudaStream_t s) {
-  launch_pdl(k_sweep_con, (unsigned)a.con_blocks, kSweepConThreads, 0, s, a, t);
+  launch_chain(true, k_sweep_con, (unsigned)a.con_blocks, kSweepConThreads, 0, s, a, t);
 }
 
 void launch_sweep_cols(int fmt, double mean_entries, const SweepArgs& a, cudaStream_t s) {
