@@ -544,7 +544,7 @@ int fredopt_server_destroy(fredopt_server_t s);
  * memory where they need it (for example a host program whose own pool owns
  * the GPU's memory, or a latency-critical loop that avoids cudaMalloc and
  * cudaFree because they can synchronise the device).  It needs no handle
- * and allocates nothing: its scratch is one fixed device array of 4.25 MiB
+ * and allocates nothing: its scratch is one fixed device array of 4 MiB
  * inside the library, which every GPU that loads the library keeps until
  * the process exits.
  *
