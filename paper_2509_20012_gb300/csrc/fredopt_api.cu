@@ -146,6 +146,10 @@ struct fredopt_ctx {
   DBuf<DevState> st;
   DBuf<LogEntry> log;
   DBuf<int> errw;
+  // pinned host memory: the error word that kernels set (mapped), and a staging
+  // area for the small results a call returns with
+  uint8_t* pin = nullptr;
+  int* err_dev = nullptr;  // device address of the error word
   size_t off_f = 0, off_bc = 0, off_g = 0, off_k2 = 0, off_fin = 0, off_cnt = 0, off_stage = 0, off_btab = 0,
          n_part = 0;
 
@@ -229,6 +233,11 @@ cudaError_t copy_out(fredopt_t h, void* dst, const void* src, size_t bytes, uint
   return cudaMemcpyAsync(dst, src, bytes, dev_ptr(flags) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                          h->stream);
 }
+
+constexpr size_t kPinStage = 64, kPinBytes = 64 + 64 * 1024;  // error word | staging
+constexpr int kStageDoubles = (int)((kPinBytes - kPinStage) / sizeof(double));
+double* stage(fredopt_t h) { return reinterpret_cast<double*>(h->pin + kPinStage); }
+volatile int* err_word(fredopt_t h) { return reinterpret_cast<volatile int*>(h->pin); }
 
 template <typename T>
 cudaError_t upload_vec(fredopt_t h, DBuf<T>& d, const std::vector<T>& v) {
@@ -559,6 +568,7 @@ void enqueue_iteration(fredopt_t h) {
   }
   ColArgs cc = col_args(h);
   cc.w = h->w.p;
+  cc.w_out = h->w.p;
   cc.g = h->g.p;
   cc.use_coef = pert ? 1 : 0;
   cc.use_u = t.n_con > 0 ? 1 : 0;
@@ -633,20 +643,34 @@ int need_loaded(fredopt_t h) {
   return FREDOPT_OK;
 }
 
-// Upload a spot vector (n floats) into a padded device buffer.
-int load_spot_vec(fredopt_t h, DBuf<float>& dst, const float* src, uint32_t flags) {
-  CK(copy_in(h, dst.p, src, (size_t)h->n * sizeof(float), flags));
+// A spot vector as the forward product takes it: the caller's device array in
+// place when the bulk copy of x can read it (16-byte aligned, no padding), else
+// a copy in xbuf.
+int spot_in(fredopt_t h, const float* src, uint32_t flags, const float** x) {
+  *x = src;
+  if (dev_ptr(flags) && h->n == h->n_pad && (reinterpret_cast<uintptr_t>(src) & 15) == 0) return FREDOPT_OK;
+  CK(copy_in(h, h->xbuf.p, src, (size_t)h->n * sizeof(float), flags));
+  *x = h->xbuf.p;
   return FREDOPT_OK;
+}
+
+// Where a kernel writes a spot vector for the caller: the caller's device array
+// (unless it overlaps `src`, read by the same kernel, in another way than
+// exactly), else `buf`, to be copied out.
+float* spot_out(fredopt_t h, float* dst, uint32_t flags, DBuf<float>& buf, const float* src = nullptr) {
+  if (!dst || !dev_ptr(flags)) return buf.p;
+  const uintptr_t d = reinterpret_cast<uintptr_t>(dst), x = reinterpret_cast<uintptr_t>(src);
+  const uintptr_t bytes = (uintptr_t)h->n * sizeof(float);
+  if (src && d != x && d < x + bytes && x < d + bytes) return buf.p;
+  return dst;
 }
 
 int check_sticky(fredopt_t h) {
   cudaError_t e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "stream synchronize");
-  int err = 0;
-  CK(cudaMemcpy(&err, &h->st.p->err, sizeof(int), cudaMemcpyDeviceToHost));
+  const int err = *err_word(h);
   if (err) {
-    const int zero = 0;
-    cudaMemcpy(&h->st.p->err, &zero, sizeof(int), cudaMemcpyHostToDevice);
+    *err_word(h) = 0;
     // a pass that gave up may have left its tile counters set
     if (h->fsched.p) cudaMemset(h->fsched.p, 0, 2 * sizeof(unsigned int));
     if (h->bsched.p) cudaMemset(h->bsched.p, 0, 2 * sizeof(unsigned int));
@@ -658,7 +682,7 @@ int check_sticky(fredopt_t h) {
 
 // CTAs of the passes over the listed structure rows
 int list_blocks(fredopt_t h) {
-  return (int)std::max<int64_t>(1, std::min<int64_t>(h->geo_full.row_blocks, (h->n_con_rows + 255) / 256));
+  return (int)std::max<int64_t>(1, std::min<int64_t>(std::min(608, h->geo_full.row_blocks), (h->n_con_rows + 255) / 256));
 }
 
 int ready_y64(fredopt_t h) {
@@ -677,9 +701,8 @@ int final_pass_y64(fredopt_t h, const float* w, uint32_t flags, bool structures)
   cudaStream_t s = h->stream;
   const float* x = nullptr;
   if (w) {
-    int rc = load_spot_vec(h, h->xbuf, w, flags);
+    const int rc = spot_in(h, w, flags, &x);
     if (rc) return rc;
-    x = h->xbuf.p;
   } else {
     if (!h->begun) return fail(h, FREDOPT_ERR_NOT_LOADED, "w is null and no solve is begun");
     x = h->w.p;
@@ -771,11 +794,15 @@ int fredopt_create(fredopt_t* out, int device, void* cuda_stream) {
   }
   if (cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreate(&h->ev_it0) != cudaSuccess || cudaEventCreate(&h->ev_it1) != cudaSuccess ||
-      h->st.alloc(1) != cudaSuccess || h->errw.alloc(1) != cudaSuccess) {
+      h->st.alloc(1) != cudaSuccess || h->errw.alloc(1) != cudaSuccess ||
+      cudaHostAlloc(reinterpret_cast<void**>(&h->pin), kPinBytes, cudaHostAllocMapped) != cudaSuccess ||
+      cudaHostGetDevicePointer(reinterpret_cast<void**>(&h->err_dev), h->pin, 0) != cudaSuccess) {
     fredopt_destroy(h);
     return FREDOPT_ERR_CUDA;
   }
-  cudaMemsetAsync(h->st.p, 0, sizeof(DevState), h->stream);
+  *err_word(h) = 0;
+  h->st_host.err = h->err_dev;
+  cudaMemcpyAsync(h->st.p, &h->st_host, sizeof(DevState), cudaMemcpyHostToDevice, h->stream);
   fredopt_default_params(&h->prm);
   h->tab.c = 0.04;
   cudaStreamSynchronize(h->stream);
@@ -796,6 +823,7 @@ int fredopt_destroy(fredopt_t h) {
   if (h->ev_it0) cudaEventDestroy(h->ev_it0);
   if (h->ev_it1) cudaEventDestroy(h->ev_it1);
   cudaStream_t own = h->own_stream ? h->stream : nullptr;
+  if (h->pin) cudaFreeHost(h->pin);
   delete h;  // frees every device buffer
   if (own) cudaStreamDestroy(own);
   return FREDOPT_OK;
@@ -1136,8 +1164,8 @@ int fredopt_set_constraints(fredopt_t h, int n, const fredopt_constraint* c) {
   launch_count_rows(fb, h->tab, h->mask.p, h->mdd.p, h->mll.p, h->mdl.p, h->con_rows.p,
                     h->n_con_rows, pc, h->stream);
   CK(cudaGetLastError());
-  std::vector<double> hp(3 * fb);
-  CK(cudaMemcpyAsync(hp.data(), pc, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  const double* hp = stage(h);
+  CK(cudaMemcpyAsync(stage(h), pc, 3 * fb * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
   double nr = 0, nu = 0, W = 0;
   for (int b = 0; b < fb; ++b) {
@@ -1202,18 +1230,27 @@ int fredopt_begin(fredopt_t h, const float* w0, double alpha, double relaxation,
   DeviceGuard dg(h->device);
   cudaStream_t s = h->stream;
   join_in(h);
-  std::vector<float> hw(h->n);
-  if (dev_ptr(flags)) {
-    CK(cudaMemcpyAsync(hw.data(), w0, h->n * sizeof(float), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-  } else {
-    std::memcpy(hw.data(), w0, h->n * sizeof(float));
-  }
   double nrm = 0.0;
-  for (float v : hw) {
-    if (!std::isfinite(v)) return fail(h, FREDOPT_ERR_NONFINITE, "w0 not finite");
-    if (v < 0.0f) return fail(h, FREDOPT_ERR_INVALID_ARG, "w0 must be >= 0");
-    nrm += (double)v * (double)v;
+  if (dev_ptr(flags)) {  // checked and summed on the device, in a fixed order
+    double* pw = h->part.p + h->off_fin;
+    launch_check_spots(w0, h->n, pw, s);
+    CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(stage(h), pw, 2 * kSpotCheckBlocks * sizeof(double), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    int bad = 0;
+    for (int b = 0; b < kSpotCheckBlocks; ++b) {
+      nrm += stage(h)[2 * b];
+      bad |= (int)stage(h)[2 * b + 1];
+    }
+    if (bad & 1) return fail(h, FREDOPT_ERR_NONFINITE, "w0 not finite");
+    if (bad & 2) return fail(h, FREDOPT_ERR_INVALID_ARG, "w0 must be >= 0");
+  } else {
+    for (int32_t j = 0; j < h->n; ++j) {
+      const float v = w0[j];
+      if (!std::isfinite(v)) return fail(h, FREDOPT_ERR_NONFINITE, "w0 not finite");
+      if (v < 0.0f) return fail(h, FREDOPT_ERR_INVALID_ARG, "w0 must be >= 0");
+      nrm += (double)v * (double)v;
+    }
   }
   free_graph(h);
   if (p.sweep_blocks > 0) {
@@ -1226,7 +1263,7 @@ int fredopt_begin(fredopt_t h, const float* w0, double alpha, double relaxation,
   if (p.sweep_blocks > 0) sweep_weights(h);
   h->beta0 = p.beta0 < 0.0 ? 0.1 * std::sqrt(nrm) : p.beta0;
   h->tab.c = p.c_cdl;
-  CK(cudaMemcpyAsync(h->w.p, hw.data(), h->n * sizeof(float), cudaMemcpyHostToDevice, s));
+  CK(copy_in(h, h->w.p, w0, h->n * sizeof(float), flags));
   if (h->btab_alpha != alpha || h->btab_beta0 != h->beta0) {
     // asynchronous: no allocation or host synchronisation in a served begin
     launch_beta_table(h->part.p + h->off_btab, kBetaTable, h->beta0, alpha, s);
@@ -1234,9 +1271,10 @@ int fredopt_begin(fredopt_t h, const float* w0, double alpha, double relaxation,
     h->btab_alpha = alpha;
     h->btab_beta0 = h->beta0;
   }
-  CK(h->log.alloc(std::max(1, p.log_capacity)));
+  CK(h->log.fit(std::max(1, p.log_capacity)));
   DevState& d = h->st_host;
   std::memset(&d, 0, sizeof(d));
+  d.err = h->err_dev;
   d.beta0 = h->beta0;
   d.alpha = alpha;
   d.lam = relaxation;
@@ -1248,7 +1286,8 @@ int fredopt_begin(fredopt_t h, const float* w0, double alpha, double relaxation,
   d.grad_normalize = p.grad_normalize ? 1 : 0;
   d.log_cap = p.log_capacity;
   d.f_empty = f_empty(h);
-  CK(cudaMemcpyAsync(h->st.p, &d, sizeof(DevState), cudaMemcpyHostToDevice, s));
+  std::memcpy(stage(h), &d, sizeof(d));
+  CK(cudaMemcpyAsync(h->st.p, stage(h), sizeof(DevState), cudaMemcpyHostToDevice, s));
   h->iters_run = 0;
   h->device_ms = 0.0;
   h->it_pending = false;
@@ -1384,10 +1423,12 @@ int fredopt_end(fredopt_t h, float* w_out, float* dose_out, float* letd_out, fre
   double* pf = h->part.p + h->off_fin;
   run(h, 5, [&] { launch_final_check(fb, h->tab, h->y64.p, h->mask.p, h->mdd.p, h->mll.p, h->mdl.p, h->con_rows.p, h->n_con_rows, pf, s); });
   CK(cudaGetLastError());
-  std::vector<double> hp(8 * fb);
-  CK(cudaMemcpyAsync(hp.data(), pf, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
-  DevState d;
-  CK(cudaMemcpyAsync(&d, h->st.p, sizeof(DevState), cudaMemcpyDeviceToHost, s));
+  // staged: the solve state, then the check's partials
+  constexpr size_t d_doubles = (sizeof(DevState) + sizeof(double) - 1) / sizeof(double);
+  static_assert(d_doubles + 8 * 608 <= (size_t)kStageDoubles, "staging area");
+  const double* hp = stage(h) + d_doubles;
+  CK(cudaMemcpyAsync(stage(h), h->st.p, sizeof(DevState), cudaMemcpyDeviceToHost, s));
+  CK(cudaMemcpyAsync(stage(h) + d_doubles, pf, 8 * fb * sizeof(double), cudaMemcpyDeviceToHost, s));
   CK(copy_out(h, w_out, h->w.p, (size_t)h->n * sizeof(float), flags));
   if (!dev_ptr(flags)) {
     if (dose_out) CK(cudaMemcpyAsync(dose_out, h->fout_a.p, h->V * sizeof(float), cudaMemcpyDeviceToHost, s));
@@ -1396,6 +1437,8 @@ int fredopt_end(fredopt_t h, float* w_out, float* dose_out, float* letd_out, fre
   rc = check_sticky(h);
   collect_timers(h);
   if (rc) return rc;
+  DevState d;
+  std::memcpy(&d, stage(h), sizeof(d));
   if (rep) {
     std::memset(rep, 0, sizeof(*rep));
     rep->iters = h->iters_run;
@@ -1500,14 +1543,15 @@ int fredopt_forward(fredopt_t h, const float* w, float* dose_out, float* lw_out,
   DeviceGuard dg(h->device);
   cudaStream_t s = h->stream;
   join_in(h);
-  rc = load_spot_vec(h, h->xbuf, w, flags);
+  const float* xin = nullptr;
+  rc = spot_in(h, w, flags, &xin);
   if (rc) return rc;
   if (!h->yall.p || h->yall.n < (size_t)std::max<int64_t>(1, h->V)) h->yall_zeroed = false;
   CK(h->yall.ensure(std::max<int64_t>(1, h->V)));
   if (!h->yall_zeroed) CK(cudaMemsetAsync(h->yall.p, 0, std::max<int64_t>(1, h->V) * sizeof(float2), s));
   h->yall_zeroed = true;
   FwdArgs fa = fwd_args(h, false);
-  fa.x = h->xbuf.p;
+  fa.x = xin;
   fa.y = h->yall.p;
   run(h, 0, [&] { launch_forward(h->geo_full, h->fmt, EPI_STORE, h->hint_fwd, fa, h->tab, s); });
   float *da = dose_out, *db = lw_out;
@@ -1550,10 +1594,10 @@ int fredopt_backward(fredopt_t h, const float* a_D, const float* a_L, float* u_o
   BwdArgs ba = bwd_args(h, h->ucoef.p);
   run(h, 1, [&] { launch_backward(h->geo, h->fmt, h->hint_bwd, true, ba, s); });
   ColArgs ca = col_args(h);
-  ca.out = h->gtmp.p;
+  ca.out = spot_out(h, u_out, flags, h->gtmp);
   run(h, 3, [&] { launch_colfinish(h->geo, COL_OUT, ca, s); });
   CK(cudaGetLastError());
-  CK(copy_out(h, u_out, h->gtmp.p, (size_t)h->n * sizeof(float), flags));
+  if (ca.out != u_out) CK(copy_out(h, u_out, ca.out, (size_t)h->n * sizeof(float), flags));
   rc = check_sticky(h);
   collect_timers(h);
   return rc;
@@ -1571,10 +1615,11 @@ int fredopt_feasibility_step(fredopt_t h, const float* x, double relaxation, dou
   cudaStream_t s = h->stream;
   const Geometry& G = h->geo;
   join_in(h);
-  rc = load_spot_vec(h, h->xbuf, x, flags);
+  const float* xin = nullptr;
+  rc = spot_in(h, x, flags, &xin);
   if (rc) return rc;
   FwdArgs fa = fwd_args(h, true);
-  fa.x = h->xbuf.p;
+  fa.x = xin;
   fa.y = h->yw.p;
   run(h, 0, [&] { launch_forward(G, h->fmt, EPI_STORE, h->hint_fwd, fa, h->tab, s); });
   ConArgs k2 = con_args(h);
@@ -1584,7 +1629,8 @@ int fredopt_feasibility_step(fredopt_t h, const float* x, double relaxation, dou
     run(h, 1, [&] { launch_backward(G, h->fmt, h->hint_bwd, true, bb, s); });
   }
   ColArgs cc = col_args(h);
-  cc.w = h->xbuf.p;
+  cc.w = xin;
+  cc.w_out = spot_out(h, w_out, flags, h->xbuf, xin);
   cc.use_u = h->tab.n_con > 0 ? 1 : 0;
   cc.norm = norm;
   cc.lam = relaxation;
@@ -1594,7 +1640,7 @@ int fredopt_feasibility_step(fredopt_t h, const float* x, double relaxation, dou
   cc.scale = h->W_all > 0.0 ? relaxation * prio_scale / h->W_all : 0.0;
   run(h, 3, [&] { launch_colfinish(G, COL_PROJ, cc, s); });
   CK(cudaGetLastError());
-  CK(copy_out(h, w_out, h->xbuf.p, (size_t)h->n * sizeof(float), flags));
+  if (cc.w_out != w_out) CK(copy_out(h, w_out, cc.w_out, (size_t)h->n * sizeof(float), flags));
   rc = check_sticky(h);
   collect_timers(h);
   return rc;
@@ -1616,12 +1662,13 @@ int fredopt_sweep_step(fredopt_t h, const float* x, double relaxation, double pr
   rc = build_sweep(h, n_blocks);
   if (rc) return rc;
   sweep_weights(h);
-  rc = load_spot_vec(h, h->xbuf, x, flags);
+  const float* xin = nullptr;
+  rc = spot_in(h, x, flags, &xin);
   if (rc) return rc;
-  CK(h->gtmp.ensure(h->n_pad));
-  enqueue_sweep(h, h->xbuf.p, 0, relaxation, prio_scale, norm, 0, h->gtmp.p);
+  float* dst = spot_out(h, w_out, flags, h->gtmp);
+  enqueue_sweep(h, xin, 0, relaxation, prio_scale, norm, 0, dst);
   CK(cudaGetLastError());
-  CK(copy_out(h, w_out, h->gtmp.p, (size_t)h->n * sizeof(float), flags));
+  if (dst != w_out) CK(copy_out(h, w_out, dst, (size_t)h->n * sizeof(float), flags));
   rc = check_sticky(h);
   collect_timers(h);
   return rc;
@@ -1635,11 +1682,12 @@ int fredopt_objective(fredopt_t h, const float* x, double* f_out, float* grad_ou
   cudaStream_t s = h->stream;
   const Geometry& G = h->geo;
   join_in(h);
-  rc = load_spot_vec(h, h->xbuf, x, flags);
+  const float* xin = nullptr;
+  rc = spot_in(h, x, flags, &xin);
   if (rc) return rc;
   double* part_f = h->part.p + h->off_f;
   FwdArgs fa = fwd_args(h, true);
-  fa.x = h->xbuf.p;
+  fa.x = xin;
   fa.y = h->yw.p;
   fa.r_out = h->r.p;
   fa.part = part_f;
@@ -1647,19 +1695,26 @@ int fredopt_objective(fredopt_t h, const float* x, double* f_out, float* grad_ou
   BwdArgs ba = bwd_args(h, h->r.p);
   run(h, 1, [&] { launch_backward(G, h->fmt, h->hint_bwd, h->obj_dose, ba, s); });
   ColArgs ca = col_args(h);
-  ca.out = h->gtmp.p;
+  ca.out = spot_out(h, grad_out, flags, h->gtmp);
   ca.part = h->part.p + h->off_g;
   run(h, 3, [&] { launch_colfinish(G, COL_GRAD, ca, s); });
+  // claimed tiles leave tens of thousands of partials: summed to kFinishBlocks first
+  int np = n_parts(G, fa);
+  const double* pf = part_f;
+  if (np > 1024) {
+    pf = h->part.p + h->off_stage;
+    launch_sum_slices(part_f, np, h->part.p + h->off_stage, s);
+    np = kFinishBlocks;
+  }
   CK(cudaGetLastError());
-  std::vector<double> hp(n_parts(G, fa));
-  CK(cudaMemcpyAsync(hp.data(), part_f, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
-  if (grad_out) CK(copy_out(h, grad_out, h->gtmp.p, (size_t)h->n * sizeof(float), flags));
+  CK(cudaMemcpyAsync(stage(h), pf, np * sizeof(double), cudaMemcpyDeviceToHost, s));
+  if (grad_out && ca.out != grad_out) CK(copy_out(h, grad_out, ca.out, (size_t)h->n * sizeof(float), flags));
   rc = check_sticky(h);
   collect_timers(h);
   if (rc) return rc;
   if (f_out) {
     double f = f_empty(h);
-    for (double v : hp) f += v;
+    for (int i = 0; i < np; ++i) f += stage(h)[i];
     *f_out = f;
   }
   return FREDOPT_OK;
@@ -2166,9 +2221,7 @@ int fredopt_batch_sync(fredopt_batch_t b, double* device_ms) {
   }
   if (device_ms) *device_ms = b->ms;
   for (fredopt_t h : b->hs) {
-    int err = 0;
-    cudaMemcpy(&err, &h->st.p->err, sizeof(int), cudaMemcpyDeviceToHost);
-    if (err) return FREDOPT_ERR_TIMEOUT;
+    if (*err_word(h)) return FREDOPT_ERR_TIMEOUT;
   }
   return FREDOPT_OK;
 }

@@ -62,7 +62,7 @@ struct DevState {
   long long k, s, accepted_total;
   int accepted;       // accepted steps in the current iteration
   int reductions, max_trials, norm, grad_normalize, log_cap;
-  int err;            // bit 0: bulk-copy wait timed out; bit 1: index out of range (FO_CHECKED builds)
+  int* err;           // mapped host word; bit 0: bulk-copy wait timed out; bit 1: index out of range (FO_CHECKED builds)
   unsigned int done;  // last-block counter of the column finish
   int pad;
   unsigned long long sweep_nv;  // block-iterative sweep: violated rows
@@ -139,7 +139,8 @@ struct ColArgs {
   const float* chunk_sum;
   int32_t n;
   float* out;                // COL_OUT / COL_GRAD (g)
-  float* w;                  // COL_PROJ: updated in place
+  const float* w;            // COL_PROJ: the point, and
+  float* w_out;              // its update (the same array in a solve)
   const float* g;            // COL_PROJ: gradient for the perturbed point
   double* part;              // per-block partials (COL_GRAD: ||g||^2)
   const double* k2part;      // COL_PROJ: constraint-evaluation partials
@@ -234,7 +235,11 @@ void launch_row_objective(const Geometry& g, const Tables& t, const float2* yw, 
 void launch_final_check(int grid, const Tables& t, const double2* y64, const uint32_t* mask,
                         const double* dd, const double* ll, const double* dl, const int64_t* rows, int64_t n_list,
                         double* part, cudaStream_t s);
-void launch_begin_state(DevState* st, cudaStream_t s);
+constexpr int kSpotCheckBlocks = 32;
+// part[2 b], part[2 b + 1]: sum of squares and flags (1 not finite, 2 negative) of block b's slice of x
+void launch_check_spots(const float* x, int32_t n, double* part, cudaStream_t s);
+// out[b] = sum of slice b of part[0 .. n), kFinishBlocks slices
+void launch_sum_slices(const double* part, int n, double* out, cudaStream_t s);
 
 // setup (K5, fredopt_load.cu)
 // Tiles that warps claim in order have guided sizes, 7 per warp: W tiles of

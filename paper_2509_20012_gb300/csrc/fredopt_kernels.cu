@@ -633,7 +633,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1024 / kFwdThreads) k_forward(Fwd
       __syncwarp();
       staged = __all_sync(kFull, mbar_wait(bar, 0, kMbarSpins));
       if (!staged) {
-        if ((threadIdx.x & 31) == 0) atomicOr(&a.st->err, 1);
+        if ((threadIdx.x & 31) == 0) atomicOr(a.st->err, 1);
         mbar_wait(bar, 0, kMbarSpins);  // let the copy in flight land before leaving
       }
     }
@@ -658,7 +658,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1024 / kFwdThreads) k_forward(Fwd
   auto gather = [&](int c) {
 #if FO_CHECKED
     if ((unsigned)c >= (unsigned)a.n_x) {
-      atomicOr(&a.st->err, 2);
+      atomicOr(a.st->err, 2);
       c = 0;
     }
 #endif
@@ -718,7 +718,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1024 / kFwdThreads) k_forward(Fwd
     const auto stream = [&](auto before) {
       stream_segments<VT, Acc, S, true, (sizeof(VT) == 4 ? kFwdUnroll : kFwdUnroll16)>(
           fwd_col<IT>(a), Dv, Lv, a.rp, r0, r1, lane, gather, flush, before, BlockBase{nullptr, nullptr, 0},
-          SegCheck{a.n_elems, FO_CHECKED ? &a.st->err : nullptr});
+          SegCheck{a.n_elems, FO_CHECKED ? a.st->err : nullptr});
     };
     if constexpr (S) stream(NoWait());
     else stream(ready);
@@ -775,7 +775,7 @@ __global__ void __launch_bounds__(kBwdThreads, FO_BWD_MIN_BLOCKS) k_backward(Bwd
   auto gather = [&](int r) {
 #if FO_CHECKED
     if ((uint64_t)(int64_t)r >= (uint64_t)a.n_rows) {
-      atomicOr(&a.st->err, 2);
+      atomicOr(a.st->err, 2);
       r = 0;
     }
 #endif
@@ -804,12 +804,12 @@ __global__ void __launch_bounds__(kBwdThreads, FO_BWD_MIN_BLOCKS) k_backward(Bwd
       stream_segments<VT, float, S, UD, bwd_units<VT, UD>(), true, kBwdLaneMap<VT>,
                       uint16_t, decltype(gather), decltype(flush), NoWait, kPrefetchUnits, kBwdPingPong>(
           a.row16, Dv, Lv, a.chunk_ptr, a.warp_chunk[job], a.warp_chunk[job + 1], lane, gather, flush, NoWait(),
-          BlockBase{a.hdr, a.ovf, a.n_ovf}, SegCheck{a.n_elems, FO_CHECKED ? &a.st->err : nullptr});
+          BlockBase{a.hdr, a.ovf, a.n_ovf}, SegCheck{a.n_elems, FO_CHECKED ? a.st->err : nullptr});
     else
       stream_segments<VT, float, S, UD, bwd_units<VT, UD>(), false, kBwdLaneMap<VT>,
                       int32_t, decltype(gather), decltype(flush), NoWait, kPrefetchUnits, kBwdPingPong>(
           a.row, Dv, Lv, a.chunk_ptr, a.warp_chunk[job], a.warp_chunk[job + 1], lane, gather, flush, NoWait(),
-          BlockBase{nullptr, nullptr, 0}, SegCheck{a.n_elems, FO_CHECKED ? &a.st->err : nullptr});
+          BlockBase{nullptr, nullptr, 0}, SegCheck{a.n_elems, FO_CHECKED ? a.st->err : nullptr});
     if (!a.sched) break;
     job = claim();
   }
@@ -898,7 +898,7 @@ __global__ void __launch_bounds__(kColThreads) k_colfinish(ColArgs a) {
       double xj = (double)a.w[j];
       if (a.use_coef) xj += coef * (double)a.g[j];
       const double wn = xj + scale * (double)s;
-      a.w[j] = wn > 0.0 ? (float)wn : 0.0f;
+      a.w_out[j] = wn > 0.0 ? (float)wn : 0.0f;
     }
   }
   if (MODE == COL_GRAD) {
@@ -1225,15 +1225,32 @@ __global__ void __launch_bounds__(kRowThreads) k_final_check(Tables t, const dou
   }
 }
 
-__global__ void k_begin_state(DevState* st) {
-  st->k = 0;
-  st->s = 0;
-  st->accepted_total = 0;
-  st->accepted = 0;
-  st->coef = 0.0;
-  st->f_start = st->f_cur = st->gnorm = st->beta_acc = 0.0;
-  st->err = 0;
-  st->done = 0u;
+__global__ void __launch_bounds__(256) k_check_spots(const float* __restrict__ x, int32_t n, double* part) {
+  __shared__ double red[9];
+  const int per = (n + (int)gridDim.x - 1) / (int)gridDim.x;
+  const int j0 = min(n, (int)blockIdx.x * per), j1 = min(n, j0 + per);
+  double sum = 0.0;
+  int bad = 0;
+  for (int j = j0 + threadIdx.x; j < j1; j += 256) {
+    const float v = x[j];
+    if (!isfinite(v)) bad |= 1;
+    if (v < 0.0f) bad |= 2;
+    sum += (double)v * (double)v;
+  }
+  sum = block_sum256(sum, red);
+  const int nonfinite = __syncthreads_or(bad & 1), negative = __syncthreads_or(bad & 2);
+  if (threadIdx.x == 0) {
+    part[2 * blockIdx.x] = sum;
+    part[2 * blockIdx.x + 1] = (double)((nonfinite ? 1 : 0) | (negative ? 2 : 0));
+  }
+}
+
+__global__ void __launch_bounds__(256) k_sum_slices(const double* __restrict__ part, int n, double* out) {
+  __shared__ double red[9];
+  const int per = (n + (int)gridDim.x - 1) / (int)gridDim.x;
+  const int i0 = min(n, (int)blockIdx.x * per), i1 = min(n, i0 + per);
+  const double v = block_sum_array(part + i0, i1 - i0, red);
+  if (threadIdx.x == 0) out[blockIdx.x] = v;
 }
 
 // ------------------------------------------------------------------ K5 setup
@@ -1441,7 +1458,13 @@ void launch_final_check(int grid, const Tables& t, const double2* y64, const uin
   k_final_check<<<grid, kRowThreads, 0, s>>>(t, y64, mask, dd, ll, dl, rows, n_list, part);
 }
 
-void launch_begin_state(DevState* st, cudaStream_t s) { k_begin_state<<<1, 1, 0, s>>>(st); }
+void launch_check_spots(const float* x, int32_t n, double* part, cudaStream_t s) {
+  k_check_spots<<<kSpotCheckBlocks, 256, 0, s>>>(x, n, part);
+}
+
+void launch_sum_slices(const double* part, int n, double* out, cudaStream_t s) {
+  k_sum_slices<<<kFinishBlocks, 256, 0, s>>>(part, n, out);
+}
 
 void launch_count_rows(int grid, const Tables& t, const uint32_t* mask, const double* dd,
                        const double* ll, const double* dl, const int64_t* rows, int64_t n_list, double* part,
@@ -1626,7 +1649,7 @@ __global__ void k_wait_check(int arrive, int spins, DevState* st) {
   }
   __syncthreads();
   if (arrive && threadIdx.x == 0) mbar_expect_tx(&bar, 0u);
-  if (!mbar_wait(&bar, 0, spins) && threadIdx.x == 0) atomicOr(&st->err, 1);
+  if (!mbar_wait(&bar, 0, spins) && threadIdx.x == 0) atomicOr(st->err, 1);
 }
 
 void launch_wait_check(int arrive, int spins, DevState* st, cudaStream_t s) {
