@@ -100,6 +100,8 @@ struct fredopt_ctx {
   DBuf<int64_t> warp_row_hot, warp_row_all, chunk_ptr;
   DBuf<int64_t> tile_row_hot;  // claimed tiles of the streamed rows (guided sizes)
   int n_tiles_hot = 0;
+  DBuf<int64_t> tile_row_all;  // the same for every row with nonzeros, whole-GPU shapes
+  int n_tiles_all = 0;
   DBuf<unsigned int> fsched;   // counters of the claimed tiles
   DBuf<int32_t> tile_chunk;    // claimed tiles of the transposed product: chunk bounds [n_tiles_bwd + 1]
   int n_tiles_bwd = 0;
@@ -310,6 +312,18 @@ bool claim_tiles(fredopt_t h) {
   return h->prm.tile_balance == 1 && h->nnz_hot >= kClaimMinNnzPerWarp * (int64_t)h->geo.fwd_warps;
 }
 
+// Passes over every row (whole-GPU shapes).  The double-float final pass does
+// about twice the work per nonzero, so claims pay from shorter passes on:
+// 7.3e8 nonzeros FP32 1.79 -> 1.41 ms, BF16 1.66 -> 1.18; 7.7e7 (1.6e4 per warp)
+// 0.205 -> 0.175; 2.2e7 (4.5e3 per warp) 78.6 -> 77.7 us.  The FP32 product:
+// 7.3e8 1.11 -> 1.05 ms, BF16 0.79 -> 0.65; at 7.7e7 equal and BF16 88 -> 94 us.
+constexpr int64_t kClaimMinNnzPerWarpFinal = 4096;
+bool claim_all_tiles(fredopt_t h, bool final_pass) {
+  if (h->prm.tile_balance == 2) return true;
+  return h->prm.tile_balance == 1 &&
+         h->nnz >= (final_pass ? kClaimMinNnzPerWarpFinal : kClaimMinNnzPerWarp) * (int64_t)h->geo_full.fwd_warps;
+}
+
 // The kernels of a captured iteration form a dependent chain, each starting
 // while its predecessor drains (tiny plan: 62.3 -> 59.9 us per iteration).  Not
 // in long passes: CTAs placed early on the SMs that drain first unbalance them
@@ -327,7 +341,7 @@ bool chained(fredopt_t h) {
 // number of forward partials
 int n_parts(const Geometry& g, const FwdArgs& a) { return a.sched ? a.n_warps : forward_grid(g, a.n_warps); }
 
-FwdArgs fwd_args(fredopt_t h, bool hot) {
+FwdArgs fwd_args(fredopt_t h, bool hot, bool final_pass = false) {
   FwdArgs a{};
   a.pdl = chained(h);
   a.rp = h->rp.p;
@@ -342,12 +356,15 @@ FwdArgs fwd_args(fredopt_t h, bool hot) {
   if (hot && claim_tiles(h) && h->n_tiles_hot > 0) {
     a.warp_row = h->tile_row_hot.p;
     a.sched = h->fsched.p;
+  } else if (!hot && claim_all_tiles(h, final_pass)) {
+    a.warp_row = h->tile_row_all.p;
+    a.sched = h->fsched.p;
   }
   a.n_x = h->n;
   a.n_x_pad = h->n_pad;
   a.mask = h->mask.p;
   a.n_hot = h->n_hot;
-  a.n_warps = a.sched ? h->n_tiles_hot : hot ? h->geo.fwd_warps : h->geo_full.fwd_warps;
+  a.n_warps = a.sched ? (hot ? h->n_tiles_hot : h->n_tiles_all) : hot ? h->geo.fwd_warps : h->geo_full.fwd_warps;
   a.part_stride = n_parts(h->geo, a);
   a.st = h->st.p;
   a.voxel = h->perm ? h->voxel.p : nullptr;
@@ -605,6 +622,14 @@ int set_fwd_schedule(fredopt_t h, int64_t row_cost) {
                         h->warp_row_all.p, nullptr}, h->stream);
   launch_tiles(TileArgs{TileArgs::GUIDED_PAIRS, rp, 0, hot, 0, 0, W, 0, row_cost, h->tile_row_hot.p, nullptr},
                h->stream);
+  CK(h->tile_row_all.fit(2 * (size_t)kGuidedTilesPerWarp * A));
+  if (w0 > 0)
+    launch_tiles(TileArgs{TileArgs::GUIDED_PAIRS, rp, 0, hot, 0, 0, w0, 0, row_cost, h->tile_row_all.p, nullptr},
+                 h->stream);
+  if (w0 < A)
+    launch_tiles(TileArgs{TileArgs::GUIDED_PAIRS, rp, h->n_hot, h->n_hot + cold, 0, 0, A - w0, 0, row_cost,
+                          h->tile_row_all.p + 2 * (size_t)kGuidedTilesPerWarp * w0, nullptr}, h->stream);
+  h->n_tiles_all = kGuidedTilesPerWarp * A;
   CK(cudaGetLastError());
   h->n_tiles_hot = kGuidedTilesPerWarp * W;
   h->row_cost = row_cost;
@@ -709,7 +734,7 @@ int final_pass_y64(fredopt_t h, const float* w, uint32_t flags, bool structures)
   }
   const int rc = ready_y64(h);
   if (rc) return rc;
-  FwdArgs fa = fwd_args(h, false);
+  FwdArgs fa = fwd_args(h, false, true);
   fa.x = x;
   fa.y64 = h->y64.p;
   fa.dose_out = nullptr;
@@ -1414,7 +1439,7 @@ int fredopt_end(fredopt_t h, float* w_out, float* dose_out, float* letd_out, fre
   }
   if (dptr) CK(cudaMemsetAsync(dptr, 0, h->V * sizeof(float), s));
   if (lptr) CK(cudaMemsetAsync(lptr, 0, h->V * sizeof(float), s));
-  FwdArgs fa = fwd_args(h, false);
+  FwdArgs fa = fwd_args(h, false, true);
   fa.x = h->w.p;
   fa.y64 = h->y64.p;
   fa.dose_out = dptr;

@@ -295,7 +295,7 @@ void launch_load_rows(int fmt, bool narrow, bool copy_values, const LoadRowsArgs
 struct TileArgs {
   enum Kind { PAIRS, BOUNDS64, BOUNDS32, GUIDED_PAIRS, GUIDED32 } kind;
   const int64_t* ptr;
-  int64_t a0, z0, a1, z1;  // ranges (the second for PAIRS; the guided kinds start at 0)
+  int64_t a0, z0, a1, z1;  // ranges (the second for PAIRS)
   int parts0, parts1;      // pieces of each range; warps for the guided kinds
   int64_t cost;
   int64_t* out64;

@@ -761,12 +761,12 @@ __device__ __forceinline__ int64_t even_bound(const int64_t* ptr, int64_t a, int
   return find_cost(ptr, a, z, cost, total * k / parts);
 }
 
-// Bound k of the guided tiles of [0, n) for W warps: W tiles of 1/2 of a warp's
+// Bound k of the guided tiles of [a, z) for W warps: W tiles of 1/2 of a warp's
 // share, W of 1/4, 1/8, 1/16 and 1/32 each, 2 W of 1/64.
-__device__ __forceinline__ int64_t guided_bound(const int64_t* ptr, int64_t n, int W, int64_t cost, int k) {
-  if (k <= 0) return 0;
-  if (k >= kGuidedTilesPerWarp * W) return n;
-  const double share = ((double)(ptr[n] - ptr[0]) + (double)cost * (double)n) / W;
+__device__ __forceinline__ int64_t guided_bound(const int64_t* ptr, int64_t a, int64_t z, int W, int64_t cost, int k) {
+  if (k <= 0) return a;
+  if (k >= kGuidedTilesPerWarp * W) return z;
+  const double share = ((double)(ptr[z] - ptr[a]) + (double)cost * (double)(z - a)) / W;
   double done = 0.0, f = 0.5;
   int left = k;
   for (int round = 0; round < 5 && left > 0; ++round, f *= 0.5) {
@@ -775,7 +775,7 @@ __device__ __forceinline__ int64_t guided_bound(const int64_t* ptr, int64_t n, i
     left -= t;
   }
   done += 0.015625 * left;
-  return find_cost(ptr, 0, n, cost, done * share);
+  return find_cost(ptr, a, z, cost, done * share);
 }
 
 __global__ void k_tiles(TileArgs q) {
@@ -793,10 +793,10 @@ __global__ void k_tiles(TileArgs q) {
     if (t <= q.parts0) q.out32[t] = (int32_t)even_bound(q.ptr, q.a0, q.z0, q.cost, t, q.parts0);
   } else if (q.kind == TileArgs::GUIDED_PAIRS) {
     if (t >= kGuidedTilesPerWarp * q.parts0) return;
-    q.out64[2 * t] = guided_bound(q.ptr, q.z0, q.parts0, q.cost, t);
-    q.out64[2 * t + 1] = guided_bound(q.ptr, q.z0, q.parts0, q.cost, t + 1);
+    q.out64[2 * t] = guided_bound(q.ptr, q.a0, q.z0, q.parts0, q.cost, t);
+    q.out64[2 * t + 1] = guided_bound(q.ptr, q.a0, q.z0, q.parts0, q.cost, t + 1);
   } else {  // GUIDED32
-    if (t <= kGuidedTilesPerWarp * q.parts0) q.out32[t] = (int32_t)guided_bound(q.ptr, q.z0, q.parts0, q.cost, t);
+    if (t <= kGuidedTilesPerWarp * q.parts0) q.out32[t] = (int32_t)guided_bound(q.ptr, q.a0, q.z0, q.parts0, q.cost, t);
   }
 }
 
