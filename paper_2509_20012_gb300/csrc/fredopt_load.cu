@@ -325,6 +325,17 @@ __global__ void __launch_bounds__(256) k_load_rows(LoadRowsArgs a) {
 
 // ------------------------------------------------------------------ counts
 
+template <typename IT>
+__device__ __forceinline__ int lower_bound_col(const IT* __restrict__ col, int len, int key) {
+  int lo = 0, hi = len;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if ((int)col[mid] < key) lo = mid + 1;
+    else hi = mid;
+  }
+  return lo;
+}
+
 constexpr int kCountThreads = 1024;
 constexpr int kCountK = 8;
 
@@ -350,28 +361,19 @@ __global__ void __launch_bounds__(kCountThreads) k_csc_count(const int64_t* __re
   for (int64_t r = strip_row[blockIdx.x] + (threadIdx.x >> 5); r < r1; r += kCountThreads / 32) {
     const int64_t s = rp[r];
     const int len = (int)(rp[r + 1] - s);
-    int32_t* first = split ? split + r * (n_grp + 1) : nullptr;
-    int last = -1;  // group of the entry before this chunk of 32
-    for (int i0 = 0; i0 < len; i0 += 32 * kCountK) {
+    const IT* __restrict__ cc = col + s;
+    for (int i0 = lane; i0 < len; i0 += 32 * kCountK) {
       int c[kCountK];  // the loads of kCountK chunks in flight
 #pragma unroll
-      for (int k = 0; k < kCountK; ++k) c[k] = i0 + 32 * k + lane < len ? (int)col[s + i0 + 32 * k + lane] : -1;
+      for (int k = 0; k < kCountK; ++k) c[k] = i0 + 32 * k < len ? (int)cc[i0 + 32 * k] : -1;
 #pragma unroll
-      for (int k = 0; k < kCountK; ++k) {
-        const int i = i0 + 32 * k;
-        if (i >= len) break;
+      for (int k = 0; k < kCountK; ++k)
         if (c[k] >= 0) atomicAdd(&hist[c[k]], 1);
-        if (first) {
-          const int g = c[k] >= 0 ? c[k] >> gshift : last;
-          int before = __shfl_up_sync(kFull, g, 1);
-          if (lane == 0) before = last;
-          for (int q = before + 1; q <= g; ++q) first[q] = i + lane;  // none past the row's end
-          last = __shfl_sync(kFull, g, min(31, len - 1 - i));
-        }
-      }
     }
-    if (first)
-      for (int q = last + 1 + lane; q <= n_grp; q += 32) first[q] = len;
+    // one group boundary per lane, found in the row just read
+    if (split)
+      for (int q = lane; q <= n_grp; q += 32)
+        split[r * (n_grp + 1) + q] = q < n_grp ? lower_bound_col(cc, len, q << gshift) : len;
   }
   if (SMEM) {
     __syncthreads();
@@ -429,28 +431,41 @@ __global__ void k_csc_offsets(int32_t* __restrict__ cnt, int n_strip, int32_t n_
 // that stores entry by entry.  The CTAs that run at one time write a few
 // groups' column frontiers, which stay in L2 until their lines are full.  With
 // `split` a row's piece of the group is looked up, else found by bisection.
-// 7.3e8 FP32 nonzeros: 9.6 ms, where 16-row steps with one 16-byte record
-// store per entry and a pass to split the records took 17.7 ms.
-#ifndef FO_FILL_THREADS
-#define FO_FILL_THREADS 512
-#endif
-#ifndef FO_FILL_K
-#define FO_FILL_K 4
-#endif
-constexpr int kFillThreads = FO_FILL_THREADS;
+// 7.3e8 FP32 nonzeros: 8.3 ms, where 16-row steps with one 16-byte record
+// store per entry and a pass to split the records took 17.7 ms.  Bound by the
+// barriers and load latencies of its short tiles (a row has about 140 entries in
+// an occupied group) and by frontier lines that leave L2 half full.  Four CTAs of
+// 384 threads per SM: 8.3 ms; three of 512 8.5, four of 256 8.7, two of 768 14.8;
+// groups of 512 columns 11.4, of 2048 10.1.
+constexpr int kFillThreads = 384;
+constexpr int kFillCtas = 4;       // per SM
+constexpr int kFillGroupShift = 10;
 constexpr int kFillWarps = kFillThreads / 32;
-constexpr int kFillK = FO_FILL_K;  // chunks of 32 entries of a row in flight per warp
+constexpr int kFillK = 5;  // chunks of 32 entries of a row in flight per warp
+
+// the two values of an entry as one shared-memory word
+template <typename VT> struct ValPair;
+template <> struct ValPair<float> {
+  using T = float2;
+  static __device__ __forceinline__ T make(float d, float l) { return make_float2(d, l); }
+  static __device__ __forceinline__ float d(T p) { return p.x; }
+  static __device__ __forceinline__ float l(T p) { return p.y; }
+};
+template <> struct ValPair<uint16_t> {
+  using T = uint32_t;
+  static __device__ __forceinline__ T make(uint16_t d, uint16_t l) { return (uint32_t)d | ((uint32_t)l << 16); }
+  static __device__ __forceinline__ uint16_t d(T p) { return (uint16_t)(p & 0xffffu); }
+  static __device__ __forceinline__ uint16_t l(T p) { return (uint16_t)(p >> 16); }
+};
 
 template <typename VT>
 struct FillSmem {  // byte offsets for T slots and G columns
-  size_t dv, lv, row, colq, mask, first, delta, cur, off, src, scan, bytes;
+  size_t val, rc, mask, first, delta, cur, off, src, scan, bytes;
   __host__ __device__ FillSmem(int T, int G) {
     size_t o = 0;
     auto take = [&](size_t b) { const size_t at = o; o = (o + b + 15) & ~(size_t)15; return at; };
-    dv = take(sizeof(VT) * (size_t)T);
-    lv = take(sizeof(VT) * (size_t)T);
-    row = take((size_t)T);
-    colq = take(2 * (size_t)T);
+    val = take(2 * sizeof(VT) * (size_t)T);
+    rc = take(4 * (size_t)T);  // column << 5 | row of the tile
     mask = take(4 * (size_t)G);
     first = take(2 * (size_t)G);
     delta = take(4 * (size_t)G);
@@ -485,17 +500,6 @@ __device__ __forceinline__ int block_excl_scan(int v, int* wsum, int* total) {
   return before + x - v;
 }
 
-template <typename IT>
-__device__ __forceinline__ int lower_bound_col(const IT* __restrict__ col, int len, int key) {
-  int lo = 0, hi = len;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if ((int)col[mid] < key) lo = mid + 1;
-    else hi = mid;
-  }
-  return lo;
-}
-
 template <typename VT, typename IT>
 __global__ void __launch_bounds__(kFillThreads) k_csc_fill(
     const int64_t* __restrict__ rp, const IT* __restrict__ col, const VT* __restrict__ Dv,
@@ -505,10 +509,9 @@ __global__ void __launch_bounds__(kFillThreads) k_csc_fill(
   extern __shared__ __align__(16) unsigned char fill_sh[];
   const int G = 1 << gshift;
   const FillSmem<VT> m(T, G);
-  VT* sD = reinterpret_cast<VT*>(fill_sh + m.dv);
-  VT* sL = reinterpret_cast<VT*>(fill_sh + m.lv);
-  uint8_t* sRow = fill_sh + m.row;
-  uint16_t* sCol = reinterpret_cast<uint16_t*>(fill_sh + m.colq);
+  using VP = ValPair<VT>;
+  typename VP::T* sVal = reinterpret_cast<typename VP::T*>(fill_sh + m.val);
+  uint32_t* sRC = reinterpret_cast<uint32_t*>(fill_sh + m.rc);
   uint32_t* mask = reinterpret_cast<uint32_t*>(fill_sh + m.mask);
   uint16_t* first = reinterpret_cast<uint16_t*>(fill_sh + m.first);
   int32_t* delta = reinterpret_cast<int32_t*>(fill_sh + m.delta);
@@ -623,10 +626,8 @@ __global__ void __launch_bounds__(kFillThreads) k_csc_fill(
           for (int q = 0; q < kFillK; ++q)
             if (c[q] >= 0) {
               const int pos = first[c[q]] + __popc(mask[c[q]] & below);
-              sD[pos] = d[q];
-              sL[pos] = v[q];
-              sRow[pos] = (uint8_t)(j - j0);
-              sCol[pos] = (uint16_t)c[q];
+              sVal[pos] = VP::make(d[q], v[q]);
+              sRC[pos] = ((uint32_t)c[q] << 5) | (uint32_t)(j - j0);
             }
         }
       }
@@ -634,10 +635,12 @@ __global__ void __launch_bounds__(kFillThreads) k_csc_fill(
       // ---- 4: slots to the output; the masks cleared for the next tile
       const int rb = (int)(r + j0);
       for (int i = tid; i < total; i += kFillThreads) {
-        const int64_t dst = delta[sCol[i]] + i;
-        row_out[dst] = rb + sRow[i];
-        DT[dst] = sD[i];
-        LT[dst] = sL[i];
+        const uint32_t rc = sRC[i];
+        const typename VP::T v = sVal[i];
+        const int dst = delta[rc >> 5] + i;
+        row_out[dst] = rb + (int)(rc & 31u);
+        DT[dst] = VP::d(v);
+        LT[dst] = VP::l(v);
       }
       for (int k = tid; k < G / 4; k += kFillThreads) reinterpret_cast<uint4*>(mask)[k] = make_uint4(0u, 0u, 0u, 0u);
       __syncthreads();
@@ -802,14 +805,7 @@ __global__ void k_tiles(TileArgs q) {
 
 }  // namespace
 
-#ifndef FO_FILL_GSHIFT
-#define FO_FILL_GSHIFT 10
-#endif
-#ifndef FO_FILL_CTAS
-#define FO_FILL_CTAS 3
-#endif
-
-// Groups of 1024 columns and two CTAs per SM; more columns than 65536 take
+// Groups of 1024 columns and kFillCtas CTAs per SM; more columns than 65536 take
 // groups of 4096 (fewer pieces per row) and one CTA per SM.  Two strips of rows
 // per SM.  The tile takes the shared memory that is left; a slot's position fits
 // 16 bits.
@@ -818,13 +814,13 @@ CscShape csc_shape(const Geometry& g, int fmt, int64_t n_rows, int32_t n_cols, i
   q.n_rows = n_rows;
   q.n_cols = n_cols;
   const bool many = n_cols > 65536;
-  q.gshift = many ? 12 : FO_FILL_GSHIFT;
+  q.gshift = many ? 12 : kFillGroupShift;
   while (q.gshift > 6 && (1 << (q.gshift - 1)) >= n_cols) --q.gshift;
   const int G = 1 << q.gshift;
   q.n_grp = (int)(((int64_t)n_cols + G - 1) >> q.gshift);
   q.n_strip = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)g.n_sms * (many ? 1 : 2), n_rows));
-  const size_t budget = many ? g.smem_limit : std::min<size_t>(g.smem_limit, (g.smem_limit - 1024 * (FO_FILL_CTAS - 1)) / FO_FILL_CTAS);
-  const int per = fmt == 0 ? 11 : 7;
+  const size_t budget = many ? g.smem_limit : std::min<size_t>(g.smem_limit, (g.smem_limit - 1024 * (kFillCtas - 1)) / kFillCtas);
+  const int per = fmt == 0 ? 12 : 8;
   const size_t fixed = fmt == 0 ? FillSmem<float>(0, G).bytes : FillSmem<uint16_t>(0, G).bytes;
   q.tile = (int)std::min<size_t>(16384, (budget - fixed - 64) / per) & ~15;
   // the table of the groups' starts pays when it stays below the matrix itself
