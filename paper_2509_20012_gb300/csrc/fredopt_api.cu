@@ -600,6 +600,14 @@ void enqueue_iteration(fredopt_t h) {
   run(h, 3, [&] { launch_colfinish(G, COL_PROJ, cc, s); });
 }
 
+// Tile weights: a row end or a chunk end (warp reductions and bookkeeping) costs
+// about as much as streaming this many nonzeros; 16-bit values stream faster
+// (fredopt_autotune can pick other weights).  Measured over the clinical, tiny,
+// half-resolution and batched plans: 100 against 64 for 16-bit rows, six plans
+// 8.56 -> 8.37 ms; 48 against 16 per chunk, clinical plan in ROI rows
+// 20.78 -> 20.69 ms, tiny plan 5.95 -> 5.91.
+constexpr int64_t kRowCost = 64, kRowCost16 = 100, kChunkCost = 48;
+
 // Warp partitions.  A segment's sum does not depend on which warp streams it
 // (lanes take elements by their absolute block-aligned position and add them
 // in order), so these weights change the speed, never a result bit.
@@ -1098,23 +1106,18 @@ int fredopt_load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t 
     } else {
       h->crow16.release();
     }
-    const int rc = set_bwd_schedule(h, 16);
+    const int rc = set_bwd_schedule(h, kChunkCost);
     if (rc) return rc;
     CK(cudaStreamSynchronize(s));  // the scratch of this block is freed here
   }
 
-  // ---- row schedules of the forward product (rows with nonzeros only);
-  // a row end (two warp reductions and bookkeeping) costs about as much as
-  // streaming FO_ROW_COST nonzeros (fredopt_autotune can pick another weight)
-#ifndef FO_ROW_COST
-#define FO_ROW_COST 64
-#endif
+  // ---- row schedules of the forward product (rows with nonzeros only)
   CK(h->fsched.ensure(2));
   CK(cudaMemsetAsync(h->fsched.p, 0, 2 * sizeof(unsigned int), s));
   CK(h->bsched.ensure(2));
   CK(cudaMemsetAsync(h->bsched.p, 0, 2 * sizeof(unsigned int), s));
   {
-    const int rc = set_fwd_schedule(h, FO_ROW_COST);
+    const int rc = set_fwd_schedule(h, fmt == FREDOPT_FP32 ? kRowCost : kRowCost16);
     if (rc) return rc;
   }
   // streaming (evict-first) loads when the streamed matrices do not fit in L2
