@@ -862,10 +862,10 @@ int fredopt_destroy(fredopt_t h) {
   return FREDOPT_OK;
 }
 
-int fredopt_load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t nnz,
+static int load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t nnz,
                            const int64_t* row_ptr, const int32_t* col, const float* D_val,
                            const float* L_val, const uint32_t* voxel_mask, int format,
-                           uint32_t flags) {
+                           uint32_t flags, bool* keep) {
   if (!h) return FREDOPT_ERR_INVALID_ARG;
   const int fmt = format & 0xff;
   const bool roi = (format & FREDOPT_ROWS_ROI) != 0;
@@ -917,9 +917,10 @@ int fredopt_load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t 
 
   // ---- the previous plan's buffers: kept where the new plan needs at least
   // half of them (a plan re-planned on the same handle), else all freed first
-  const bool similar = h->Dv.p && h->Dv.n >= (size_t)nnz_alloc * vb && h->Dv.n / 2 <= (size_t)nnz_alloc * vb &&
+  const bool similar = *keep && h->Dv.p && h->Dv.n >= (size_t)nnz_alloc * vb && h->Dv.n / 2 <= (size_t)nnz_alloc * vb &&
                        h->DTv.n >= (size_t)nh_alloc * vb && h->DTv.n / 2 <= (size_t)nh_alloc * vb && h->V >= n_vox &&
                        h->V / 2 <= n_vox;
+  *keep = similar;
   if (!similar) {
     h->rp.release(); h->col.release(); h->col16.release(); h->Dv.release(); h->Lv.release();
     h->voxel.release(); h->mask.release(); h->con_rows.release(); h->cp.release();
@@ -1167,6 +1168,19 @@ int fredopt_load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t 
   h->n_rows_reach = h->n_unreach = 0;
   h->loaded = true;
   return FREDOPT_OK;
+}
+
+int fredopt_load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t nnz,
+                           const int64_t* row_ptr, const int32_t* col, const float* D_val,
+                           const float* L_val, const uint32_t* voxel_mask, int format,
+                           uint32_t flags) {
+  bool keep = true;
+  int rc = load_influence(h, n_vox, n_spots, nnz, row_ptr, col, D_val, L_val, voxel_mask, format, flags, &keep);
+  if (rc == FREDOPT_ERR_OOM && keep) {  // kept buffers are up to twice what the plan needs: without them
+    keep = false;
+    rc = load_influence(h, n_vox, n_spots, nnz, row_ptr, col, D_val, L_val, voxel_mask, format, flags, &keep);
+  }
+  return rc;
 }
 
 int fredopt_set_constraints(fredopt_t h, int n, const fredopt_constraint* c) {
