@@ -681,19 +681,19 @@ def volume_benchmark(plan, w, local, stream, hbm, reps=20):
         kt = h.get_timing()
         h.set_timing(False)
         other_ms = kt["other"][0] / reps
-        # each pass reads the mask of every streamed row and the FP64 pair of the structure rows
-        by = n_pass * (plan.n_vox * 4 + n_struct * 16)
+        # each pass reads row number, mask and FP64 pair of the listed structure rows
+        by = n_pass * n_struct * (8 + 4 + 16)
         out[name] = {"requests": len(reqs), "ms_per_call": wall * 1e3, "final_pass_ms": kt["forward"][0] / reps,
-                     "stats_kernels_ms": other_ms, "stats_launches": 1 if n_pass == 1 else 9,
+                     "stats_kernels_ms": other_ms, "stats_launches": 1 if n_pass == 1 else 10,
                      "stats_bytes": by, "stats_achieved_gbs": by / (other_ms * 1e-3) / 1e9 if other_ms else None,
                      "peak": hbm}
         if name == "values_at_volume":
             out[name]["results"] = {f"{r['quantity']}:{r['struct_bit']}": [float(x) for x in v["at_volume"]]
                                     for r, v in zip(reqs, res)}
     h.close()
-    out["note"] = ("%d structure voxels of %d rows; the statistics kernels read 4 B of mask per row and 16 B of "
-                   "FP64 (Dw, Lw) per structure voxel per pass, mostly from L2 right after the final pass: "
-                   "launch- and L2-bound, not an HBM roofline" % (n_struct, plan.n_vox))
+    out["note"] = ("%d structure voxels of %d rows; the final pass runs over the structure rows, the statistics "
+                   "kernels read 28 B per structure voxel per pass, mostly from L2: launch-bound, not an HBM "
+                   "roofline" % (n_struct, plan.n_vox))
     return out
 
 
