@@ -73,9 +73,10 @@ extern "C" {
  * other plans (a batch graph, a server with several plans in flight): about
  * one SM's worth of CTAs per 400000 nonzeros of the streamed rows (the whole
  * GPU from 6.08e7 nonzeros on GB300), so that small plans leave SMs to the
- * others.  Results depend only on the plan and its launch shapes: a plan
- * loaded with and without the flag agrees to rounding, and bit for bit with
- * itself alone and in a batch. */
+ * others (fredopt_forward and the final passes, whose sums do not depend on
+ * it, take the whole GPU).  Results depend only on the plan and its launch
+ * shapes: a plan loaded with and without the flag agrees to rounding, and bit
+ * for bit with itself alone and in a batch. */
 #define FREDOPT_SHARED 0x400
 
 /* ---- constraint kinds (Fig. 2 half-spaces; the LETd limit LETd <= Lambda as the half-space (L - Lambda D) w <= 0) ----
