@@ -129,8 +129,9 @@ typedef struct fredopt_params {
   int32_t sweep_blocks;   /* 0 (default): simultaneous feasibility step (Cimmino).  M in
                              1..FREDOPT_MAX_SWEEP_BLOCKS: block-iterative sweep of Fig. 2 over M
                              voxel blocks (see fredopt_sweep_step) */
-  int32_t tile_balance;   /* 1 (default): in passes of at least 16384 nonzeros per warp (final
-                             pass: 4096), the forward and transposed products' warps claim tiles of decreasing
+  int32_t tile_balance;   /* 1 (default): in long passes (from 20000 to 48000 nonzeros per warp
+                             on, by product and storage; final pass: 4096), the forward and
+                             transposed products' warps claim tiles of decreasing
                              size from a counter, so SMs that stream faster take more of them
                              (the SMs of a GB300 differ by up to ~13% in streaming rate);
                              2: claim tiles in every pass; 0: one static tile per warp.

@@ -304,12 +304,22 @@ void collect_timers(fredopt_t h) {
 }
 
 // Claimed tiles pay off when a pass is long enough for the SMs' different
-// streaming rates to matter; below kClaimMinNnzPerWarp nonzeros per warp the
-// claims cost more than they balance (tile_balance 2 claims always).
-constexpr int64_t kClaimMinNnzPerWarp = 16384;
-bool claim_tiles(fredopt_t h) {
+// streaming rates to matter; in shorter passes the claims cost more than they
+// balance (tile_balance 2 claims always).  The lines lie, in nonzeros per
+// forward warp, where static and claimed tiles took the same time; per launch,
+// static -> claimed, in us:
+//   per warp           1.6e4          2.5e4          3.8e4          6.7e4          1.5e5
+//   forward FP32       132 -> 133     196 -> 193     293 -> 284     499 -> 473     1071 -> 1026
+//   forward 16-bit      85 ->  93     123 -> 130     184 -> 184     306 -> 298      692 ->  640
+//   transposed FP32    112 -> 120     170 -> 174     251 -> 251     423 -> 412      890 ->  847
+//   transposed 16-bit   89 -> 100     139 -> 146     201 -> 204     339 -> 330      698 ->  662
+int64_t claim_min_nnz(fredopt_t h, bool transposed) {
+  if (h->fmt == FREDOPT_FP32) return transposed ? 38000 : 20000;
+  return transposed ? 48000 : 38000;
+}
+bool claim_tiles(fredopt_t h, bool transposed) {
   if (h->prm.tile_balance == 2) return true;
-  return h->prm.tile_balance == 1 && h->nnz_hot >= kClaimMinNnzPerWarp * (int64_t)h->geo.fwd_warps;
+  return h->prm.tile_balance == 1 && h->nnz_hot >= claim_min_nnz(h, transposed) * (int64_t)h->geo.fwd_warps;
 }
 
 // Passes over every row (whole-GPU shapes).  The double-float final pass does
@@ -321,7 +331,7 @@ constexpr int64_t kClaimMinNnzPerWarpFinal = 4096;
 bool claim_all_tiles(fredopt_t h, bool final_pass) {
   if (h->prm.tile_balance == 2) return true;
   return h->prm.tile_balance == 1 &&
-         h->nnz >= (final_pass ? kClaimMinNnzPerWarpFinal : kClaimMinNnzPerWarp) * (int64_t)h->geo_full.fwd_warps;
+         h->nnz >= (final_pass ? kClaimMinNnzPerWarpFinal : claim_min_nnz(h, false)) * (int64_t)h->geo_full.fwd_warps;
 }
 
 // The kernels of a captured iteration form a dependent chain, each starting
@@ -353,7 +363,7 @@ FwdArgs fwd_args(fredopt_t h, bool hot, bool final_pass = false) {
   a.sD = h->fmt ? h->sD.p : nullptr;
   a.sL = h->fmt ? h->sL.p : nullptr;
   a.warp_row = hot ? h->warp_row_hot.p : h->warp_row_all.p;
-  if (hot && claim_tiles(h) && h->n_tiles_hot > 0) {
+  if (hot && claim_tiles(h, false) && h->n_tiles_hot > 0) {
     a.warp_row = h->tile_row_hot.p;
     a.sched = h->fsched.p;
   } else if (!hot && claim_all_tiles(h, final_pass)) {
@@ -389,7 +399,7 @@ BwdArgs bwd_args(fredopt_t h, const float2* coef) {
   b.chunk_sum = h->chunk_sum.p;
   b.n_warps = h->geo.bwd_warps;
   b.pdl = chained(h);
-  if (claim_tiles(h) && h->n_tiles_bwd > 0) {
+  if (claim_tiles(h, true) && h->n_tiles_bwd > 0) {
     b.warp_chunk = h->tile_chunk.p;
     b.n_warps = h->n_tiles_bwd;
     b.sched = h->bsched.p;

@@ -17,7 +17,7 @@
 //   K3b k_colfinish  per spot: sum of its chunks in order, then the
 //                    gradient, or the clip w <- max(0, x + u) (Fig. 2, last
 //                    loop); closes the iteration (log entry, k).
-//   K4 k_finish      64 blocks, then the last one: deterministic two-level
+//   K4 k_finish      one block, or 64 and then the last one: deterministic
 //                    reduction of the partials and the closed-form
 //                    non-ascent trial loop (Fig. 3) in one warp.
 //   K5 setup         in fredopt_load.cu (row order, values, CSC copy, tiles);
