@@ -964,8 +964,13 @@ __global__ void __launch_bounds__(kConThreads) k_constraints(ConArgs a, Tables t
       }
       double gD = 0.0, gL = 0.0;
       eval_constraints(con, todo, t.c, xd, xl, dd, ll, dl, gD, gL, psum, preach, viol, mx);
-      // the row scales are powers of two: exact in FP32
-      out = a.sD ? make_float2((float)gD * a.sD[i], (float)gL * a.sL[i]) : make_float2((float)gD, (float)gL);
+      // scaled in FP64 and rounded once: g itself is about 1 / |a_r|, which leaves the
+      // FP32 range for rows of very small or large values, where g times the scale does not
+      if (a.sD) {
+        gD *= (double)a.sD[i];
+        gL *= (double)a.sL[i];
+      }
+      out = make_float2((float)gD, (float)gL);
     }
     a.gam[i] = out;
     j += step;
