@@ -697,6 +697,17 @@ int spot_in(fredopt_t h, const float* src, uint32_t flags, const float** x) {
   return FREDOPT_OK;
 }
 
+// Checks n spots of w0 and adds their squares to *nrm, in order.
+int check_spots(fredopt_t h, const float* w, int32_t n, double* nrm) {
+  for (int32_t j = 0; j < n; ++j) {
+    const float v = w[j];
+    if (!std::isfinite(v)) return fail(h, FREDOPT_ERR_NONFINITE, "w0 not finite");
+    if (v < 0.0f) return fail(h, FREDOPT_ERR_INVALID_ARG, "w0 must be >= 0");
+    *nrm += (double)v * (double)v;
+  }
+  return FREDOPT_OK;
+}
+
 // Where a kernel writes a spot vector for the caller: the caller's device array
 // (unless it overlaps `src`, read by the same kernel, in another way than
 // exactly), else `buf`, to be copied out.
@@ -1283,26 +1294,16 @@ int fredopt_begin(fredopt_t h, const float* w0, double alpha, double relaxation,
   cudaStream_t s = h->stream;
   join_in(h);
   double nrm = 0.0;
-  if (dev_ptr(flags)) {  // checked and summed on the device, in a fixed order
-    double* pw = h->part.p + h->off_fin;
-    launch_check_spots(w0, h->n, pw, s);
-    CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(stage(h), pw, 2 * kSpotCheckBlocks * sizeof(double), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    int bad = 0;
-    for (int b = 0; b < kSpotCheckBlocks; ++b) {
-      nrm += stage(h)[2 * b];
-      bad |= (int)stage(h)[2 * b + 1];
+  if (dev_ptr(flags)) {  // through the staging area, in order: the same sum as for a host array
+    const int32_t m = 2 * kStageDoubles;
+    for (int32_t j = 0; j < h->n; j += m) {
+      const int32_t k = std::min(m, h->n - j);
+      CK(cudaMemcpyAsync(stage(h), w0 + j, k * sizeof(float), cudaMemcpyDeviceToHost, s));
+      CK(cudaStreamSynchronize(s));
+      if ((rc = check_spots(h, reinterpret_cast<const float*>(stage(h)), k, &nrm))) return rc;
     }
-    if (bad & 1) return fail(h, FREDOPT_ERR_NONFINITE, "w0 not finite");
-    if (bad & 2) return fail(h, FREDOPT_ERR_INVALID_ARG, "w0 must be >= 0");
-  } else {
-    for (int32_t j = 0; j < h->n; ++j) {
-      const float v = w0[j];
-      if (!std::isfinite(v)) return fail(h, FREDOPT_ERR_NONFINITE, "w0 not finite");
-      if (v < 0.0f) return fail(h, FREDOPT_ERR_INVALID_ARG, "w0 must be >= 0");
-      nrm += (double)v * (double)v;
-    }
+  } else if ((rc = check_spots(h, w0, h->n, &nrm))) {
+    return rc;
   }
   free_graph(h);
   if (p.sweep_blocks > 0) {

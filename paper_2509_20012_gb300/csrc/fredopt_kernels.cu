@@ -1230,26 +1230,6 @@ __global__ void __launch_bounds__(kRowThreads) k_final_check(Tables t, const dou
   }
 }
 
-__global__ void __launch_bounds__(256) k_check_spots(const float* __restrict__ x, int32_t n, double* part) {
-  __shared__ double red[9];
-  const int per = (n + (int)gridDim.x - 1) / (int)gridDim.x;
-  const int j0 = min(n, (int)blockIdx.x * per), j1 = min(n, j0 + per);
-  double sum = 0.0;
-  int bad = 0;
-  for (int j = j0 + threadIdx.x; j < j1; j += 256) {
-    const float v = x[j];
-    if (!isfinite(v)) bad |= 1;
-    if (v < 0.0f) bad |= 2;
-    sum += (double)v * (double)v;
-  }
-  sum = block_sum256(sum, red);
-  const int nonfinite = __syncthreads_or(bad & 1), negative = __syncthreads_or(bad & 2);
-  if (threadIdx.x == 0) {
-    part[2 * blockIdx.x] = sum;
-    part[2 * blockIdx.x + 1] = (double)((nonfinite ? 1 : 0) | (negative ? 2 : 0));
-  }
-}
-
 __global__ void __launch_bounds__(256) k_sum_slices(const double* __restrict__ part, int n, double* out) {
   __shared__ double red[9];
   const int per = (n + (int)gridDim.x - 1) / (int)gridDim.x;
@@ -1461,10 +1441,6 @@ void launch_final_check(int grid, const Tables& t, const double2* y64, const uin
                         const double* dd, const double* ll, const double* dl, const int64_t* rows, int64_t n_list,
                         double* part, cudaStream_t s) {
   k_final_check<<<grid, kRowThreads, 0, s>>>(t, y64, mask, dd, ll, dl, rows, n_list, part);
-}
-
-void launch_check_spots(const float* x, int32_t n, double* part, cudaStream_t s) {
-  k_check_spots<<<kSpotCheckBlocks, 256, 0, s>>>(x, n, part);
 }
 
 void launch_sum_slices(const double* part, int n, double* out, cudaStream_t s) {
