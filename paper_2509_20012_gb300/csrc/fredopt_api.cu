@@ -719,15 +719,20 @@ float* spot_out(fredopt_t h, float* dst, uint32_t flags, DBuf<float>& buf, const
   return dst;
 }
 
+// The error word, and the tile counters, which a pass that gave up may have left
+// set.  Nothing of the handle is in flight.
+void clear_error(fredopt_t h) {
+  *err_word(h) = 0;
+  if (h->fsched.p) cudaMemsetAsync(h->fsched.p, 0, 2 * sizeof(unsigned int), h->stream);
+  if (h->bsched.p) cudaMemsetAsync(h->bsched.p, 0, 2 * sizeof(unsigned int), h->stream);
+}
+
 int check_sticky(fredopt_t h) {
   cudaError_t e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "stream synchronize");
   const int err = *err_word(h);
   if (err) {
-    *err_word(h) = 0;
-    // a pass that gave up may have left its tile counters set
-    if (h->fsched.p) cudaMemset(h->fsched.p, 0, 2 * sizeof(unsigned int));
-    if (h->bsched.p) cudaMemset(h->bsched.p, 0, 2 * sizeof(unsigned int));
+    clear_error(h);
     if (err & 2) return fail(h, FREDOPT_ERR_PATTERN, "checked build: an index or tile range out of bounds");
     return fail(h, FREDOPT_ERR_TIMEOUT, "a bounded device-side wait gave up (bulk copy)");
   }
@@ -1395,6 +1400,7 @@ int fredopt_begin(fredopt_t h, const float* w0, double alpha, double relaxation,
     CK(cudaGraphInstantiate(&h->gexec, h->graph, 0));
   }
   CK(cudaStreamSynchronize(s));
+  if (*err_word(h)) clear_error(h);  // of an earlier solve that no call reported
   h->begun = true;
   return FREDOPT_OK;
 }

@@ -1,0 +1,85 @@
+"""What the library's host code does when a runtime call or a device-side wait
+fails, on the CPU: fredopt_api.cu compiled over a stand-in CUDA runtime whose
+"kernels" compute nothing (fake_cuda.cpp).  No GPU is involved."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2509_20012_gb300 import fredopt
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    if not os.path.exists(os.path.join(CUDA, "include", "cuda_runtime.h")):
+        pytest.skip("no CUDA headers")
+    so = str(tmp_path_factory.mktemp("fake") / "libfake.so")
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-w", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I",
+                           os.path.join(ROOT, "include"), "-I", os.path.join(CUDA, "include"),
+                           os.path.join(ROOT, "tests", "fake_cuda.cpp"), "-o", so])
+    lib = ctypes.CDLL(so)
+    for name, (res, args) in fredopt._SIGS.items():
+        if hasattr(lib, name):
+            getattr(lib, name).restype, getattr(lib, name).argtypes = res, args
+    lib.fake_used.restype = lib.fake_peak.restype = ctypes.c_size_t
+    lib.fake_limit.argtypes = [ctypes.c_size_t]
+    yield lib
+    lib.fake_limit(2 ** 63)
+
+
+class Plan:
+    """A handle of the stand-in library with n_vox rows of `per` nonzeros."""
+
+    def __init__(self, lib, n_vox, per, n=64):
+        self.lib, self.n = lib, n
+        self.h = ctypes.c_void_p()
+        assert lib.fredopt_create(ctypes.byref(self.h), 0, None) == 0
+        assert self.load(n_vox, per) == 0
+
+    def load(self, n_vox, per, fmt=0):
+        rp = np.arange(n_vox + 1, dtype=np.int64) * per
+        col = np.zeros(n_vox * per, np.int32)
+        val = np.zeros(n_vox * per, np.float32)
+        mask = np.ones(n_vox, np.uint32)
+        return self.lib.fredopt_load_influence(self.h, n_vox, self.n, n_vox * per, rp.ctypes.data, col.ctypes.data,
+                                               val.ctypes.data, val.ctypes.data, mask.ctypes.data, fmt, 0)
+
+    def begin(self, **kw):
+        p = fredopt.Params(beta0=-1.0, eta=1.0, reductions=1, max_trials=50, c_cdl=0.04, use_graphs=0, tile_balance=1)
+        for k, v in kw.items():
+            setattr(p, k, v)
+        w0 = np.ones(self.n, np.float32)
+        return self.lib.fredopt_begin(self.h, w0.ctypes.data, 0.99, 1.0, ctypes.byref(p), 0)
+
+    def end(self):
+        return self.lib.fredopt_end(self.h, None, None, None, None, 0)
+
+    def close(self):
+        self.lib.fredopt_destroy(self.h)
+
+
+def test_begin_drops_the_error_of_an_abandoned_solve(fake):
+    """A wait that gave up in a solve that is never ended belongs to that solve:
+    the next one on the handle, alone or in a batch, does not report it."""
+    a = Plan(fake, 50, 3)
+    assert a.begin() == 0
+    fake.fake_fail_waits(1)
+    assert fake.fredopt_iterate(a.h, 2) == 0
+    assert a.begin() == 0
+    assert fake.fredopt_iterate(a.h, 2) == 0
+    assert a.end() == 0
+    # in a batch: reported by its synchronisation, and by that call alone
+    b = ctypes.c_void_p()
+    hs = (ctypes.c_void_p * 1)(a.h)
+    for give_up in (1, 0):
+        assert a.begin() == 0
+        fake.fake_fail_waits(give_up)
+        assert fake.fredopt_batch_create(ctypes.byref(b), hs, 1) == 0  # the stand-in runs what is captured
+        assert fake.fredopt_batch_sync(b, None) == (fredopt.ERR_TIMEOUT if give_up else 0)
+        assert fake.fredopt_batch_destroy(b) == 0
+    a.close()
