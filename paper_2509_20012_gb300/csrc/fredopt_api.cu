@@ -888,6 +888,17 @@ int fredopt_destroy(fredopt_t h) {
   return FREDOPT_OK;
 }
 
+// Frees what a plan's size determines.
+static void release_plan(fredopt_t h) {
+  h->rp.release(); h->col.release(); h->col16.release(); h->Dv.release(); h->Lv.release();
+  h->sD.release(); h->sL.release(); h->mdd.release(); h->mll.release(); h->mdl.release();
+  h->voxel.release(); h->mask.release(); h->con_rows.release(); h->cp.release(); h->covf.release();
+  h->crow.release(); h->crow16.release(); h->chdr.release(); h->DTv.release(); h->LTv.release();
+  h->yw.release(); h->yg.release(); h->r.release(); h->gam.release(); h->ucoef.release();
+  h->y64.release(); h->yall.release(); h->fout_a.release(); h->fout_b.release();
+  h->vin_a.release(); h->vin_b.release(); h->ys.release(); h->sweep_pos.release();
+}
+
 static int load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t nnz,
                            const int64_t* row_ptr, const int32_t* col, const float* D_val,
                            const float* L_val, const uint32_t* voxel_mask, int format,
@@ -907,6 +918,7 @@ static int load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t n
   h->begun = false;
   h->sweep_m = 0;
   cudaStream_t s = h->stream;
+  if (!*keep) release_plan(h);
   join_in(h);
   const bool host = !dev_ptr(flags);
   const int vb = value_bytes(fmt);
@@ -947,13 +959,7 @@ static int load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t n
                        h->DTv.n >= (size_t)nh_alloc * vb && h->DTv.n / 2 <= (size_t)nh_alloc * vb && h->V >= n_vox &&
                        h->V / 2 <= n_vox;
   *keep = similar;
-  if (!similar) {
-    h->rp.release(); h->col.release(); h->col16.release(); h->Dv.release(); h->Lv.release();
-    h->voxel.release(); h->mask.release(); h->con_rows.release(); h->cp.release();
-    h->crow.release(); h->crow16.release(); h->chdr.release(); h->DTv.release(); h->LTv.release();
-    h->y64.release(); h->yall.release(); h->fout_a.release(); h->fout_b.release();
-    h->vin_a.release(); h->vin_b.release();
-  }
+  if (!similar) release_plan(h);
   h->y64_zeroed = h->yall_zeroed = false;
   h->covf.release();
   h->ucoef.release();

@@ -83,3 +83,33 @@ def test_begin_drops_the_error_of_an_abandoned_solve(fake):
         assert fake.fredopt_batch_sync(b, None) == (fredopt.ERR_TIMEOUT if give_up else 0)
         assert fake.fredopt_batch_destroy(b) == 0
     a.close()
+
+
+@pytest.mark.parametrize("per", [1, 40])
+def test_reload_frees_the_old_plan_when_memory_runs_out(fake, per):
+    """A reload for which there is no room beside the old plan's buffers, from the
+    first allocation on, frees them and loads: whatever fits on its own fits."""
+    sizes = (4000, 3000)
+    alone = []  # peak of each plan in a fresh handle
+    for n_vox in sizes:
+        fake.fake_limit(2 ** 63)
+        before = fake.fake_used()
+        p = Plan(fake, n_vox, per)
+        alone.append(fake.fake_peak() - before)
+        p.close()
+        assert fake.fake_used() == before
+    p = Plan(fake, sizes[0], per)
+    assert p.begin() == 0 and p.end() == 0
+    held = fake.fake_used()
+    base = held  # every handle before is closed
+    for room in list(range(0, 4 * alone[1], alone[1] // 16)):
+        limit = max(held + room, 0)
+        fake.fake_limit(limit)
+        rc = p.load(sizes[1], per)
+        if limit >= alone[1]:
+            assert rc == 0, (room, rc)
+        fake.fake_limit(2 ** 63)
+        assert p.load(sizes[0], per) == 0
+        held = fake.fake_used()
+    p.close()
+    assert fake.fake_used() < base
