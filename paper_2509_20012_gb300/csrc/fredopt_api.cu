@@ -137,8 +137,11 @@ struct fredopt_ctx {
   int sweep_m = 0;
   int sweep_nb = 0;                          // blocks actually formed
   int64_t sweep_size = 0;                    // structure rows with nonzeros per block
+  int sweep_warps = 0;                       // > 0: the streaming forward product takes the blocks' rows,
+  DBuf<int64_t> sweep_tiles;                 // in this many tiles per block
   DBuf<int64_t> sweep_pos, sweep_bounds_d;
-  DBuf<double> sweep_w, sweep_part;          // [sweep_nb] 1 / priority sum; violated rows' partial sums
+  DBuf<double> sweep_w, sweep_wpart;         // [sweep_nb] 1 / priority sum; its slices' sums
+  DBuf<double> sweep_part;                   // violated rows' partial priority sums of a block
   DBuf<float> xs;                            // the point being swept [n_pad]
   DBuf<float2> ys;                           // forward product of a block's rows [n_con_ne]
   DBuf<double> part;
@@ -441,12 +444,20 @@ ConArgs con_args(fredopt_t h) {
 }
 
 
-// 1 / priority sum of the sweep blocks' reachable rows (they change with the
-// constraint table only).
+// 1 / priority sum of the sweep blocks' reachable rows.  Formed when the blocks
+// are built, and again when the constraint table or c_cdl changes.
 void sweep_weights(fredopt_t h) {
   launch_sweep_weights(h->tab, h->con_rows.p, h->n_con_ne, h->sweep_size, h->sweep_nb, h->mask.p, h->mdd.p, h->mll.p,
-                    h->mdl.p, h->sweep_w.p, h->stream);
+                       h->mdl.p, h->sweep_wpart.p, h->sweep_w.p, h->stream);
 }
+
+// Rows of a sweep's blocks by the streaming forward product, when the list of
+// structure rows is the device rows in order (FREDOPT_ROWS_ROI), from this many
+// nonzeros per block on: it keeps more entries in flight, but stages all of x
+// per block.  Rows of one sweep, in us, k_sweep_rows -> streaming:
+//   FP32    4.6e7 per block 116 -> 101   1.5e7 134 -> 130   1.0e7 230 -> 211   5.0e6 307 -> 312   2.9e6 255 -> 483
+//   16-bit  8.0e7 per block 155 ->  79   1.0e7 226 -> 161   5.0e6 287 -> 253   1.2e6 606 -> 929
+int64_t sweep_stream_nnz(fredopt_t h) { return h->fmt == FREDOPT_FP32 ? 10000000 : 4000000; }
 
 // Blocks of the block-iterative sweep: the streamed rows with nonzeros that
 // lie in some structure, in device (= ascending voxel) order, cut into groups
@@ -472,15 +483,27 @@ int build_sweep(fredopt_t h, int m) {
     h->sweep_size = S;
   }
   bnd.push_back(C.empty() ? 0 : C.back() + 1);
+  h->sweep_warps = 0;
+  if (!C.empty() && C.back() + 1 == (int64_t)C.size() &&
+      h->con_nnz >= sweep_stream_nnz(h) * h->sweep_nb) {
+    const int W = (int)std::min<int64_t>(h->geo.fwd_warps, h->sweep_size);
+    CK(h->sweep_tiles.alloc(2 * (size_t)W * h->sweep_nb));
+    for (int t = 0; t < h->sweep_nb; ++t)
+      launch_tiles(TileArgs{TileArgs::PAIRS, h->rp.p, bnd[t], bnd[t + 1], 0, 0, W, 0, h->row_cost,
+                            h->sweep_tiles.p + 2 * (size_t)W * t, nullptr}, s);
+    h->sweep_warps = W;
+  }
   CK(upload_vec(h, h->sweep_bounds_d, bnd));
   CK(h->sweep_pos.alloc(bnd.size() * h->n));
   if (h->sweep_nb > 0)
     launch_sweep_pos(h->cp.p, h->crow.p, h->n, h->sweep_bounds_d.p, (int)bnd.size(), h->sweep_pos.p, s);
   CK(h->sweep_w.alloc(h->sweep_nb));
+  CK(h->sweep_wpart.alloc((size_t)h->sweep_nb * sweep_weight_slices(h->sweep_size)));
   CK(h->sweep_part.alloc((size_t)((h->sweep_size + kSweepConThreads - 1) / kSweepConThreads)));
   CK(h->xs.ensure(h->n_pad));
   CK(cudaMemsetAsync(h->xs.p, 0, h->n_pad * sizeof(float), s));
   CK(h->ys.ensure(h->n_con_ne));
+  sweep_weights(h);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   h->sweep_m = m;
@@ -527,7 +550,18 @@ void enqueue_sweep(fredopt_t h, const float* w, int use_coef, double lam, double
     a.winv = h->sweep_w.p + t;
     a.pos0 = h->sweep_pos.p + (size_t)t * h->n;
     a.pos1 = h->sweep_pos.p + (size_t)(t + 1) * h->n;
-    run(h, 0, [&] { launch_sweep_rows(h->fmt, row_nnz, a, s); });
+    if (h->sweep_warps > 0) {
+      FwdArgs fa = fwd_args(h, true);
+      fa.pdl = true;
+      fa.warp_row = h->sweep_tiles.p + 2 * (size_t)h->sweep_warps * t;
+      fa.n_warps = h->sweep_warps;
+      fa.sched = nullptr;
+      fa.x = h->xs.p;
+      fa.y = h->ys.p;
+      run(h, 0, [&] { launch_forward(h->geo, h->fmt, EPI_STORE, h->hint_fwd, fa, h->tab, s); });
+    } else {
+      run(h, 0, [&] { launch_sweep_rows(h->fmt, row_nnz, a, s); });
+    }
     run(h, 2, [&] { launch_sweep_con(h->tab, a, s); });
     run(h, 1, [&] { launch_sweep_cols(h->fmt, col_nnz, a, s); });
   }
@@ -896,7 +930,7 @@ static void release_plan(fredopt_t h) {
   h->crow.release(); h->crow16.release(); h->chdr.release(); h->DTv.release(); h->LTv.release();
   h->yw.release(); h->yg.release(); h->r.release(); h->gam.release(); h->ucoef.release();
   h->y64.release(); h->yall.release(); h->fout_a.release(); h->fout_b.release();
-  h->vin_a.release(); h->vin_b.release(); h->ys.release(); h->sweep_pos.release();
+  h->vin_a.release(); h->vin_b.release(); h->ys.release(); h->sweep_pos.release(); h->sweep_tiles.release();
 }
 
 static int load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t nnz,
@@ -1324,9 +1358,11 @@ int fredopt_begin(fredopt_t h, const float* w0, double alpha, double relaxation,
   h->prm = p;
   h->alpha = alpha;
   h->lam = relaxation;
-  if (p.sweep_blocks > 0) sweep_weights(h);
   h->beta0 = p.beta0 < 0.0 ? 0.1 * std::sqrt(nrm) : p.beta0;
-  h->tab.c = p.c_cdl;
+  if (h->tab.c != p.c_cdl) {
+    h->tab.c = p.c_cdl;
+    if (h->sweep_m > 0) sweep_weights(h);
+  }
   CK(copy_in(h, h->w.p, w0, h->n * sizeof(float), flags));
   if (h->btab_alpha != alpha || h->btab_beta0 != h->beta0) {
     // asynchronous: no allocation or host synchronisation in a served begin
@@ -1726,7 +1762,6 @@ int fredopt_sweep_step(fredopt_t h, const float* x, double relaxation, double pr
   join_in(h);
   rc = build_sweep(h, n_blocks);
   if (rc) return rc;
-  sweep_weights(h);
   const float* xin = nullptr;
   rc = spot_in(h, x, flags, &xin);
   if (rc) return rc;

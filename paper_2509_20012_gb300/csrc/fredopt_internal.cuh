@@ -372,10 +372,12 @@ void launch_sweep_start(int n, const float* w, const float* g, int use_coef, flo
                         cudaStream_t s);
 void launch_sweep_pos(const int64_t* cp, const int32_t* row, int32_t n, const int64_t* bounds, int n_bounds,
                       int64_t* pos, cudaStream_t s);
-// winv[t] = 1 / priority sum of the reachable constraint rows of list[t * size .. (t + 1) * size), t < n_blk
+// winv[t] = 1 / priority sum of the reachable constraint rows of list[t * size .. (t + 1) * size), t < n_blk;
+// part: n_blk * sweep_weight_slices(size) values
+int sweep_weight_slices(int64_t size);
 void launch_sweep_weights(const Tables& t, const int64_t* list, int64_t n_list, int64_t size, int n_blk,
-                       const uint32_t* mask, const double* dd, const double* ll, const double* dl, double* winv,
-                       cudaStream_t s);
+                          const uint32_t* mask, const double* dd, const double* ll, const double* dl, double* part,
+                          double* winv, cudaStream_t s);
 // forward product of the block's rows; warps per row by the mean row length
 void launch_sweep_rows(int fmt, double mean_nnz, const SweepArgs& a, cudaStream_t s);
 void launch_sweep_con(const Tables& t, const SweepArgs& a, cudaStream_t s);

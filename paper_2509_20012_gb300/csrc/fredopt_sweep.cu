@@ -2,6 +2,7 @@
 // Per block of structure rows, three kernels chained by programmatic dependent
 // launch:
 //   k_sweep_rows  forward product of the block's rows, several warps per row
+//                 (long blocks of consecutive rows: k_forward)
 //   k_sweep_con   half-space evaluation, one row per thread
 //   k_sweep_cols  x_j += scale * sum over the block's entries of column j
 // A block of the clinical plan holds a few hundred rows (9 MB of matrix), so a
@@ -10,7 +11,9 @@
 // for it, and a row or column is spread over as many lanes as its length fills.
 // Clinical plan (5.7e7 nonzeros in structure rows, FP32), one sweep: 64 blocks
 // 3.60 -> 1.21 ms against plain launches of the streaming forward kernel (one
-// warp per row), the constraint kernel over 608 CTAs and one warp per column.
+// warp per row), the constraint kernel over 608 CTAs and one warp per column;
+// 1 block 0.44 -> 0.28 ms.  The chain is kept in batches too, where it was
+// measured: six plans of 64 blocks 1.77 -> 0.76 ms per iteration.
 #include "fredopt.h"
 #include "fredopt_device.cuh"
 #include "fredopt_internal.cuh"
@@ -53,11 +56,15 @@ __global__ void k_sweep_pos(const int64_t* __restrict__ cp, const int32_t* __res
   }
 }
 
+// Priority sum of the reachable constraint rows of slice blockIdx.y of block
+// blockIdx.x (`rows` rows).  One CTA over a whole block of 79 thousand rows took
+// 0.46 ms.
 __global__ void __launch_bounds__(256) k_sweep_weights(Tables t, const int64_t* list, int64_t n_list, int64_t size,
-                                                    const uint32_t* mask, const double* dd, const double* ll,
-                                                    const double* dl, double* winv) {
+                                                       int64_t rows, const uint32_t* mask, const double* dd,
+                                                       const double* ll, const double* dl, double* part) {
   __shared__ double red[9];
-  const int64_t i0 = (int64_t)blockIdx.x * size, i1 = min(n_list, i0 + size);
+  const int64_t b0 = (int64_t)blockIdx.x * size, b1 = min(n_list, b0 + size);
+  const int64_t i0 = b0 + (int64_t)blockIdx.y * rows, i1 = min(b1, i0 + rows);
   double p = 0.0;
   for (int64_t i = i0 + threadIdx.x; i < i1; i += 256) {
     const int64_t r = list[i];
@@ -66,6 +73,12 @@ __global__ void __launch_bounds__(256) k_sweep_weights(Tables t, const int64_t* 
       if (((m >> t.con[q].bit) & 1u) && row_norm2(t.con[q], t.c, dd[r], ll[r], dl[r]) > 0.0) p += t.con[q].prio;
   }
   p = block_sum256(p, red);
+  if (threadIdx.x == 0) part[(int64_t)blockIdx.x * gridDim.y + blockIdx.y] = p;
+}
+
+__global__ void __launch_bounds__(256) k_sweep_winv(const double* part, int slices, double* winv) {
+  __shared__ double red[9];
+  const double p = block_sum_array(part + (int64_t)blockIdx.x * slices, slices, red);
   if (threadIdx.x == 0) winv[blockIdx.x] = p > 0.0 ? 1.0 / p : 0.0;
 }
 
@@ -172,16 +185,17 @@ __global__ void __launch_bounds__(kSweepConThreads) k_sweep_con(SweepArgs a, Tab
 
 // x_j += lam * scale / W_B * sum over the block's entries of column j of
 // D_ij gamma_D[i] + L_ij gamma_L[i].  LPC lanes per column, U columns per lane
-// group, their entries in flight together.  The FP64 update is left to the
+// group, K entries of each in flight together: four of one long column, or one
+// each of two short ones.  The FP64 update is left to the
 // CTA's first warps, one column per lane: GB300 issues an FP64 warp instruction
 // at the same low rate however few of its lanes are active, and one update per
 // column in the column's own warp was most of this kernel's time (19 us per
 // block of the clinical plan at 64 blocks).  A block's share of the columns is
 // uneven (its rows lie at one place), which is what is left.
 constexpr int kColsU = 2;  // columns per lane group (with 8 CTAs per SM: 3% faster than 4 with 4)
-template <typename VT, int LPC>
-__global__ void __launch_bounds__(256, 8) k_sweep_cols(SweepArgs a) {
-  constexpr int U = kColsU, CPW = 32 / LPC, COLS = 8 * U * CPW;  // columns per CTA
+template <typename VT, int LPC, int U, int K, int CTAS>
+__global__ void __launch_bounds__(256, CTAS) k_sweep_cols(SweepArgs a) {
+  constexpr int CPW = 32 / LPC, COLS = 8 * U * CPW;  // columns per CTA
   __shared__ float sums[COLS];
   __shared__ double red[9];
   __shared__ double sh_scale;
@@ -201,16 +215,19 @@ __global__ void __launch_bounds__(256, 8) k_sweep_cols(SweepArgs a) {
     left[k] = (int)(p1 - p0) - sl;
     most = max(most, left[k]);
   }
-  int row[U];
-  VT d[U], l[U];
+  int row[U][K];
+  VT d[U][K], l[U][K];
   auto load = [&](int o) {
 #pragma unroll
     for (int k = 0; k < U; ++k) {
-      row[k] = -1;
-      if (o < left[k]) {
-        row[k] = a.row[p[k] + o];
-        d[k] = Dv[p[k] + o];
-        l[k] = Lv[p[k] + o];
+#pragma unroll
+      for (int e = 0; e < K; ++e) {
+        row[k][e] = -1;
+        if (o + e * LPC < left[k]) {
+          row[k][e] = a.row[p[k] + o + e * LPC];
+          d[k][e] = Dv[p[k] + o + e * LPC];
+          l[k][e] = Lv[p[k] + o + e * LPC];
+        }
       }
     }
   };
@@ -237,20 +254,26 @@ __global__ void __launch_bounds__(256, 8) k_sweep_cols(SweepArgs a) {
   float acc[U];
 #pragma unroll
   for (int k = 0; k < U; ++k) acc[k] = 0.0f;
-  for (int o = 0; __any_sync(kFull, o < most); o += LPC) {
-    float2 g[U];
-    float dv[U], lv[U];
+  for (int o = 0; __any_sync(kFull, o < most); o += LPC * K) {
+    float2 g[U][K];
+    float dv[U][K], lv[U][K];
 #pragma unroll
     for (int k = 0; k < U; ++k) {
-      g[k] = row[k] >= 0 ? a.gam[row[k]] : make_float2(0.0f, 0.0f);
-      dv[k] = row[k] >= 0 ? to_f(d[k]) : 0.0f;
-      lv[k] = row[k] >= 0 ? to_f(l[k]) : 0.0f;
+#pragma unroll
+      for (int e = 0; e < K; ++e) {
+        g[k][e] = row[k][e] >= 0 ? a.gam[row[k][e]] : make_float2(0.0f, 0.0f);
+        dv[k][e] = row[k][e] >= 0 ? to_f(d[k][e]) : 0.0f;
+        lv[k][e] = row[k][e] >= 0 ? to_f(l[k][e]) : 0.0f;
+      }
     }
-    load(o + LPC);
+    load(o + LPC * K);
 #pragma unroll
     for (int k = 0; k < U; ++k) {
-      acc[k] = fmaf(dv[k], g[k].x, acc[k]);
-      acc[k] = fmaf(lv[k], g[k].y, acc[k]);
+#pragma unroll
+      for (int e = 0; e < K; ++e) {
+        acc[k] = fmaf(dv[k][e], g[k][e].x, acc[k]);
+        acc[k] = fmaf(lv[k][e], g[k][e].y, acc[k]);
+      }
     }
   }
 #pragma unroll
@@ -314,11 +337,20 @@ void rows_inst(double mean_nnz, const SweepArgs& a, cudaStream_t s) {
 
 template <typename VT>
 void cols_inst(double mean_entries, const SweepArgs& a, cudaStream_t s) {
-  constexpr int big = 8 * kColsU, small = 8 * kColsU * 4;  // columns per CTA
-  if (mean_entries > 12.0)
-    launch_chain(true, k_sweep_cols<VT, 32>, (unsigned)(((int64_t)a.n + big - 1) / big), 256, 0, s, a);
-  else
-    launch_chain(true, k_sweep_cols<VT, 8>, (unsigned)(((int64_t)a.n + small - 1) / small), 256, 0, s, a);
+  auto go = [&](auto kernel, int cols) {
+    launch_chain(true, kernel, (unsigned)(((int64_t)a.n + cols - 1) / cols), 256, 0, s, a);
+  };
+  // The update of one sweep, in us, two columns and one entry each in flight per
+  // lane -> one column and four entries, by mean entries per column and block:
+  //   24 (64 blocks of the clinical plan)   994 -> 1144    42   1400 -> 1240
+  //   96                                    491 ->  394   380   3660 -> 2420
+  //   1500 (one block)                      236 ->  140
+  // Plans of few columns leave the second a last wave that is nearly empty (6480
+  // columns: an iteration of 64 blocks, 72 entries, 562 -> 621 us; of 16 blocks,
+  // 290 entries, 224 and 224; of 4 blocks, 1160 entries, 163 -> 132).
+  if (mean_entries > 512.0 || (mean_entries > 32.0 && a.n >= 16384)) go(k_sweep_cols<VT, 32, 1, 4, 4>, 8);
+  else if (mean_entries > 12.0) go(k_sweep_cols<VT, 32, kColsU, 1, 8>, 8 * kColsU);
+  else go(k_sweep_cols<VT, 8, kColsU, 1, 8>, 8 * kColsU * 4);
 }
 
 }  // namespace
@@ -336,10 +368,18 @@ void launch_sweep_pos(const int64_t* cp, const int32_t* row, int32_t n, const in
   k_sweep_pos<<<gb, 256, 0, s>>>(cp, row, n, bounds, n_bounds, pos);
 }
 
+int sweep_weight_slices(int64_t size) {
+  return (int)std::min<int64_t>(4096, std::max<int64_t>(1, (size + 1023) / 1024));
+}
+
 void launch_sweep_weights(const Tables& t, const int64_t* list, int64_t n_list, int64_t size, int n_blk,
-                       const uint32_t* mask, const double* dd, const double* ll, const double* dl, double* winv,
-                       cudaStream_t s) {
-  if (n_blk > 0) k_sweep_weights<<<n_blk, 256, 0, s>>>(t, list, n_list, size, mask, dd, ll, dl, winv);
+                          const uint32_t* mask, const double* dd, const double* ll, const double* dl, double* part,
+                          double* winv, cudaStream_t s) {
+  if (n_blk == 0) return;
+  const int slices = sweep_weight_slices(size);
+  k_sweep_weights<<<dim3(n_blk, slices), 256, 0, s>>>(t, list, n_list, size, (size + slices - 1) / slices, mask, dd, ll, dl,
+                                                      part);
+  k_sweep_winv<<<n_blk, 256, 0, s>>>(part, slices, winv);
 }
 
 void launch_sweep_rows(int fmt, double mean_nnz, const SweepArgs& a, cudaStream_t s) {

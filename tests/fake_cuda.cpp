@@ -176,8 +176,9 @@ void launch_wait_check(int arrive, int, DevState* st, cudaStream_t) {
 }
 void launch_sweep_start(int, const float*, const float*, int, float*, DevState*, cudaStream_t) {}
 void launch_sweep_pos(const int64_t*, const int32_t*, int32_t, const int64_t*, int, int64_t*, cudaStream_t) {}
+int sweep_weight_slices(int64_t) { return 1; }
 void launch_sweep_weights(const Tables&, const int64_t*, int64_t, int64_t, int, const uint32_t*, const double*,
-                          const double*, const double*, double*, cudaStream_t) {}
+                          const double*, const double*, double*, double*, cudaStream_t) {}
 void launch_sweep_rows(int, double, const SweepArgs&, cudaStream_t) {}
 void launch_sweep_con(const Tables&, const SweepArgs&, cudaStream_t) {}
 void launch_sweep_cols(int, double, const SweepArgs&, cudaStream_t) {}
