@@ -314,6 +314,7 @@ struct CscShape {
   int n_grp;
   int tile;        // entries a CTA sorts at a time
   bool use_split;  // keep (n_grp + 1) * n_rows group starts
+  bool short_pieces;  // few entries per row and group: scattered entry by entry
 };
 CscShape csc_shape(const Geometry& g, int fmt, int64_t n_rows, int32_t n_cols, int64_t nnz);
 // cnt: n_strip * n_cols, zeroed; split: n_rows * (n_grp + 1) or null
@@ -324,7 +325,7 @@ void launch_csc_colsum(const int32_t* cnt, int n_strip, int32_t n_cols, int64_t*
 void launch_csc_offsets(int32_t* cnt, int n_strip, int32_t n_cols, const int64_t* cp, cudaStream_t s);
 void launch_csc_fill(const CscShape& q, int fmt, const int64_t* rp, const int32_t* col, const uint16_t* col16,
                      const void* Dv, const void* Lv, const int64_t* strip_row, const int32_t* split,
-                     const int32_t* cursor, int32_t* row_out, void* DT, void* LT, cudaStream_t s);
+                     int32_t* cursor, int32_t* row_out, void* DT, void* LT, cudaStream_t s);
 void launch_dequant_csc(int fmt, const int64_t* cp, int32_t n_cols, const int32_t* row, const void* DT,
                         const void* LT, const float* sD, const float* sL, float* Dout, float* Lout,
                         cudaStream_t s);

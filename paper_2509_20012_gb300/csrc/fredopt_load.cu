@@ -12,6 +12,7 @@
 //   k_csc_offsets  (strip, column)
 //   k_csc_fill     one CTA per (strip, column group) sorts tiles of entries by
 //                  column in shared memory and writes them as runs
+//   k_csc_scatter  the same for rows with very few entries per group
 //   k_csc_columns, column pointers; the chunks of the transposed product
 //   k_chunk_fill
 //   k_tiles        bounds of the tiles that warps stream, by bisection of the
@@ -649,6 +650,130 @@ __global__ void __launch_bounds__(kFillThreads) k_csc_fill(
   }
 }
 
+// The same transpose for rows with few entries per column group: then a tile of
+// 32 rows holds too few entries for its passes over the group's columns, and the
+// CTAs' look-ups of every (row, group) piece outgrow the entries.  One CTA takes
+// the entries of strip b in CSR order, up to kScatEntries of up to 64 rows at a
+// time, whatever their columns:
+//   1  an entry finds its column's slot in a hash table (at most half full) and
+//      sets its row's bit in the slot's 64-bit mask;
+//   2  it goes to output cursor[c] + (its bits below its own): row order;
+//   3  the first entry of a column advances the cursor and clears the slot.
+// Entries of a tile rarely share a column, so every entry is a store of its own in
+// each of the three arrays, which binds it: 12 to 15 ms per 1e8 entries whatever
+// the shape.  Loads in ms, k_csc_fill (groups of 1024) -> k_csc_scatter, by mean
+// entries per row and group:
+//   9e-4 (9 per row, 3e6 columns, 1.8e7 entries)  184.8 -> 13.8   1.3   45.6 -> 27.7
+//   0.1 (98, 1e6, 3.9e7)                          103.8 -> 11.9   2.5   23.8 -> 23.7
+//   0.3 (19, 70000, 7.5e7)                         61.0 -> 15.0   3.3   27.0 -> 28.0
+//   0.6 (19, 30000, 7.5e7)                         37.7 -> 15.0   6.6    6.1 -> 11.3
+// Rows whose entries lie in a few of the groups favour k_csc_fill, so the line is 2.
+// More than 65536 columns take one strip per SM, not two (their counters are 4
+// bytes per strip and column): 17.8 -> 13.8 ms for 3e6 columns.
+constexpr int kScatThreads = 512, kScatPer = 8, kScatEntries = kScatThreads * kScatPer;
+constexpr int kScatSlotBits = 13, kScatSlots = 1 << kScatSlotBits;
+constexpr int kScatRows = 1024;  // row pointers staged at a time
+constexpr size_t kScatSmem = kScatSlots * (sizeof(unsigned long long) + sizeof(int32_t)) + (kScatRows + 1) * sizeof(int64_t);
+static_assert(2 * kScatEntries <= kScatSlots, "hash table at most half full: every probe ends");
+
+template <typename VT, typename IT>
+__global__ void __launch_bounds__(kScatThreads, 2) k_csc_scatter(
+    const int64_t* __restrict__ rp, const IT* __restrict__ col, const VT* __restrict__ Dv, const VT* __restrict__ Lv,
+    const int64_t* __restrict__ strip_row, int32_t n_cols, int32_t* cursor, int32_t* __restrict__ row_out,
+    VT* __restrict__ DT, VT* __restrict__ LT) {
+  extern __shared__ __align__(16) unsigned char fill_sh[];
+  unsigned long long* mask = reinterpret_cast<unsigned long long*>(fill_sh);
+  int64_t* srp = reinterpret_cast<int64_t*>(mask + kScatSlots);
+  int32_t* key = reinterpret_cast<int32_t*>(srp + kScatRows + 1);
+  const int tid = threadIdx.x;
+  for (int j = tid; j < kScatSlots; j += kScatThreads) {
+    mask[j] = 0ull;
+    key[j] = -1;
+  }
+  int32_t* cur = cursor + (int64_t)blockIdx.x * n_cols;
+  const int64_t r_end = strip_row[blockIdx.x + 1];
+  for (int64_t r0 = strip_row[blockIdx.x]; r0 < r_end; r0 += kScatRows) {
+    const int nr = (int)min((int64_t)kScatRows, r_end - r0);
+    for (int i = tid; i <= nr; i += kScatThreads) srp[i] = rp[r0 + i];
+    __syncthreads();
+    int64_t p0 = srp[0];
+    for (int a = 0; a < nr;) {  // the tile starts at entry p0, in row a of the staged ones
+      const int z = min(a + 64, nr);
+      const int64_t p1 = min(p0 + kScatEntries, srp[z]);
+      int c[kScatPer], hk[kScatPer];  // column or -1; slot | row of the tile << kScatSlotBits
+#pragma unroll
+      for (int q = 0; q < kScatPer; ++q) {
+        const int64_t p = p0 + tid + q * kScatThreads;
+        c[q] = p < p1 ? (int)col[p] : -1;
+      }
+#pragma unroll
+      for (int q = 0; q < kScatPer; ++q) {
+        if (c[q] < 0) continue;
+        const int64_t p = p0 + tid + q * kScatThreads;
+        int lo = a, hi = z;  // the last row that starts at or before p
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if (srp[mid] <= p) lo = mid;
+          else hi = mid;
+        }
+        unsigned h = ((unsigned)c[q] * 2654435761u) >> (32 - kScatSlotBits);
+        while (true) {
+          const int32_t k = atomicCAS(&key[h], -1, c[q]);
+          if (k == -1 || k == c[q]) break;
+          h = (h + 1) & (kScatSlots - 1);
+        }
+        atomicOr(&mask[h], 1ull << (lo - a));
+        hk[q] = (int)h | ((lo - a) << kScatSlotBits);
+      }
+      __syncthreads();
+      int next[kScatPer];  // the column's new cursor, where this entry is its first
+#pragma unroll
+      for (int q = 0; q < kScatPer; ++q) {
+        next[q] = -1;
+        if (c[q] < 0) continue;
+        const int64_t p = p0 + tid + q * kScatThreads;
+        const unsigned long long m = mask[hk[q] & (kScatSlots - 1)];
+        const int row = hk[q] >> kScatSlotBits;
+        const int rank = __popcll(m & ((1ull << row) - 1ull));
+        const int base = cur[c[q]], pos = base + rank;
+        row_out[pos] = (int)(r0 + a + row);
+        DT[pos] = Dv[p];
+        LT[pos] = Lv[p];
+        if (rank == 0) next[q] = base + __popcll(m);
+      }
+      __syncthreads();
+#pragma unroll
+      for (int q = 0; q < kScatPer; ++q) {
+        if (next[q] < 0) continue;
+        const int h = hk[q] & (kScatSlots - 1);
+        cur[c[q]] = next[q];
+        key[h] = -1;
+        mask[h] = 0ull;
+      }
+      if (p1 == srp[z]) {
+        a = z;
+      } else {  // the tile ended inside a row, or where one starts
+        int hi = z;
+        while (hi - a > 1) {
+          const int mid = (a + hi) >> 1;
+          if (srp[mid] <= p1) a = mid;
+          else hi = mid;
+        }
+      }
+      p0 = p1;
+      __syncthreads();
+    }
+  }
+}
+
+template <typename VT, typename IT>
+void scatter_inst(const CscShape& q, const int64_t* rp, const IT* col, const void* Dv, const void* Lv,
+                  const int64_t* strip_row, int32_t* cursor, int32_t* row_out, void* DT, void* LT, cudaStream_t s) {
+  cudaFuncSetAttribute(k_csc_scatter<VT, IT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScatSmem);
+  k_csc_scatter<VT, IT><<<(unsigned)q.n_strip, kScatThreads, kScatSmem, s>>>(
+      rp, col, (const VT*)Dv, (const VT*)Lv, strip_row, q.n_cols, cursor, row_out, (VT*)DT, (VT*)LT);
+}
+
 template <typename VT, typename IT>
 void fill_inst(const CscShape& q, const int64_t* rp, const IT* col, const void* Dv, const void* Lv,
                const int64_t* strip_row, const int32_t* split, const int32_t* cursor, int32_t* row_out, void* DT,
@@ -805,26 +930,25 @@ __global__ void k_tiles(TileArgs q) {
 
 }  // namespace
 
-// Groups of 1024 columns and kFillCtas CTAs per SM; more columns than 65536 take
-// groups of 4096 (fewer pieces per row) and one CTA per SM.  Two strips of rows
-// per SM.  The tile takes the shared memory that is left; a slot's position fits
-// 16 bits.
+// Groups of 1024 columns and kFillCtas CTAs per SM.  The tile takes the shared
+// memory that is left; a slot's position fits 16 bits.
+constexpr double kShortPiece = 2.0;  // mean entries per row and group below which k_csc_scatter takes over
 CscShape csc_shape(const Geometry& g, int fmt, int64_t n_rows, int32_t n_cols, int64_t nnz) {
   CscShape q{};
   q.n_rows = n_rows;
   q.n_cols = n_cols;
-  const bool many = n_cols > 65536;
-  q.gshift = many ? 12 : kFillGroupShift;
+  q.gshift = kFillGroupShift;
   while (q.gshift > 6 && (1 << (q.gshift - 1)) >= n_cols) --q.gshift;
   const int G = 1 << q.gshift;
   q.n_grp = (int)(((int64_t)n_cols + G - 1) >> q.gshift);
-  q.n_strip = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)g.n_sms * (many ? 1 : 2), n_rows));
-  const size_t budget = many ? g.smem_limit : std::min<size_t>(g.smem_limit, (g.smem_limit - 1024 * (kFillCtas - 1)) / kFillCtas);
+  q.short_pieces = (double)nnz < kShortPiece * (double)n_rows * (double)q.n_grp;
+  q.n_strip = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)g.n_sms * (q.short_pieces && n_cols > 65536 ? 1 : 2), n_rows));
+  const size_t budget = (g.smem_limit - 1024 * (kFillCtas - 1)) / kFillCtas;
   const int per = fmt == 0 ? 12 : 8;
   const size_t fixed = fmt == 0 ? FillSmem<float>(0, G).bytes : FillSmem<uint16_t>(0, G).bytes;
   q.tile = (int)std::min<size_t>(16384, (budget - fixed - 64) / per) & ~15;
   // the table of the groups' starts pays when it stays below the matrix itself
-  q.use_split = (double)(q.n_grp + 1) * 4.0 * (double)n_rows <= 8.0 * (double)nnz;
+  q.use_split = !q.short_pieces && (double)(q.n_grp + 1) * 4.0 * (double)n_rows <= 8.0 * (double)nnz;
   return q;
 }
 
@@ -844,14 +968,16 @@ void launch_csc_offsets(int32_t* cnt, int n_strip, int32_t n_cols, const int64_t
 
 void launch_csc_fill(const CscShape& q, int fmt, const int64_t* rp, const int32_t* col, const uint16_t* col16,
                      const void* Dv, const void* Lv, const int64_t* strip_row, const int32_t* split,
-                     const int32_t* cursor, int32_t* row_out, void* DT, void* LT, cudaStream_t s) {
-  if (fmt == 0) {
-    if (col16) fill_inst<float>(q, rp, col16, Dv, Lv, strip_row, split, cursor, row_out, DT, LT, s);
-    else fill_inst<float>(q, rp, col, Dv, Lv, strip_row, split, cursor, row_out, DT, LT, s);
-  } else {
-    if (col16) fill_inst<uint16_t>(q, rp, col16, Dv, Lv, strip_row, split, cursor, row_out, DT, LT, s);
-    else fill_inst<uint16_t>(q, rp, col, Dv, Lv, strip_row, split, cursor, row_out, DT, LT, s);
-  }
+                     int32_t* cursor, int32_t* row_out, void* DT, void* LT, cudaStream_t s) {
+  auto go = [&](auto v, auto cols) {
+    using VT = decltype(v);
+    if (q.short_pieces) scatter_inst<VT>(q, rp, cols, Dv, Lv, strip_row, cursor, row_out, DT, LT, s);
+    else fill_inst<VT>(q, rp, cols, Dv, Lv, strip_row, split, cursor, row_out, DT, LT, s);
+  };
+  if (fmt == 0 && col16) go(float(), col16);
+  else if (fmt == 0) go(float(), col);
+  else if (col16) go(uint16_t(), col16);
+  else go(uint16_t(), col);
 }
 
 void launch_csc_columns(const int64_t* tot, int32_t n, int64_t C, int64_t* cp, int32_t* col_chunk, cudaStream_t s) {

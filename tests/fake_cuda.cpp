@@ -164,7 +164,7 @@ void launch_csc_count(const CscShape&, size_t, const int64_t*, const int32_t*, c
 void launch_csc_colsum(const int32_t*, int, int32_t, int64_t*, cudaStream_t) {}
 void launch_csc_offsets(int32_t*, int, int32_t, const int64_t*, cudaStream_t) {}
 void launch_csc_fill(const CscShape&, int, const int64_t*, const int32_t*, const uint16_t*, const void*, const void*,
-                     const int64_t*, const int32_t*, const int32_t*, int32_t*, void*, void*, cudaStream_t) {}
+                     const int64_t*, const int32_t*, int32_t*, int32_t*, void*, void*, cudaStream_t) {}
 void launch_dequant_csc(int, const int64_t*, int32_t, const int32_t*, const void*, const void*, const float*,
                         const float*, float*, float*, cudaStream_t) {}
 void launch_scale_coef(int64_t, const float*, const float*, const int64_t*, const float*, const float*, float2*,
