@@ -198,7 +198,11 @@ struct Geometry {
   size_t smem_limit;    // bytes of opt-in shared memory per block
 };
 
-int init_kernels(Geometry* g, int device);  // sets function attributes once per device
+// Sets the kernels' shared-memory limits on the current device, always to the same
+// value: a limit is one per device and process, so a launch must not set its own.
+int init_kernels(Geometry* g, int device);
+cudaError_t init_load_kernels(int smem_bytes);    // (parts of init_kernels)
+cudaError_t init_volume_kernels(int smem_bytes);
 // binary and PTX architecture versions (major * 10 + minor) of the loaded
 // forward and transposed-product kernels on the current device
 cudaError_t kernel_arch(int* fwd_binary, int* bwd_binary, int* ptx_version);

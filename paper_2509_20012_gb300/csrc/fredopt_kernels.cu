@@ -1551,6 +1551,7 @@ int init_kernels(Geometry* g, int device) {
   if (set_smem_all<float>(bytes) != cudaSuccess) return -2;
   if (set_smem_all<__nv_bfloat16>(bytes) != cudaSuccess) return -2;
   if (set_smem_all<__half>(bytes) != cudaSuccess) return -2;
+  if (init_load_kernels(bytes) != cudaSuccess || init_volume_kernels(bytes) != cudaSuccess) return -2;
   return 0;
 }
 

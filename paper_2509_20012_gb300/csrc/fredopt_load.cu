@@ -769,7 +769,6 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_csc_scatter(
 template <typename VT, typename IT>
 void scatter_inst(const CscShape& q, const int64_t* rp, const IT* col, const void* Dv, const void* Lv,
                   const int64_t* strip_row, int32_t* cursor, int32_t* row_out, void* DT, void* LT, cudaStream_t s) {
-  cudaFuncSetAttribute(k_csc_scatter<VT, IT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScatSmem);
   k_csc_scatter<VT, IT><<<(unsigned)q.n_strip, kScatThreads, kScatSmem, s>>>(
       rp, col, (const VT*)Dv, (const VT*)Lv, strip_row, q.n_cols, cursor, row_out, (VT*)DT, (VT*)LT);
 }
@@ -779,7 +778,6 @@ void fill_inst(const CscShape& q, const int64_t* rp, const IT* col, const void* 
                const int64_t* strip_row, const int32_t* split, const int32_t* cursor, int32_t* row_out, void* DT,
                void* LT, cudaStream_t s) {
   const FillSmem<VT> m(q.tile, 1 << q.gshift);
-  cudaFuncSetAttribute(k_csc_fill<VT, IT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m.bytes);
   k_csc_fill<VT, IT><<<(unsigned)(q.n_strip * q.n_grp), kFillThreads, m.bytes, s>>>(
       rp, col, (const VT*)Dv, (const VT*)Lv, strip_row, q.n_strip, q.n_cols, q.gshift, q.n_grp, q.tile, split, cursor,
       row_out, (VT*)DT, (VT*)LT);
@@ -790,7 +788,6 @@ void count_inst(const CscShape& q, size_t smem_limit, const int64_t* rp, const I
                 int32_t* cnt, int32_t* split, cudaStream_t s) {
   const size_t smem = (size_t)q.n_cols * sizeof(int32_t);
   if (smem <= smem_limit) {
-    cudaFuncSetAttribute(k_csc_count<true, IT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     k_csc_count<true, IT><<<q.n_strip, kCountThreads, smem, s>>>(rp, col, strip_row, q.n_cols, q.gshift, q.n_grp, cnt,
                                                                  split);
   } else {
@@ -1012,6 +1009,23 @@ void launch_rows_place(const int64_t* rp, const uint32_t* mask, int64_t n, bool 
                        float* sD, float* sL, cudaStream_t s) {
   k_rows_place<<<(unsigned)row_order_blocks(n), 256, 0, s>>>(rp, mask, n, roi ? 1 : 0, blk, tot, rp_out, voxel,
                                                              mask_out, con_rows, sD, sL);
+}
+
+template <typename IT>
+static cudaError_t init_load_it(int bytes) {
+  const void* k[] = {(const void*)k_csc_count<true, IT>,       (const void*)k_csc_fill<float, IT>,
+                     (const void*)k_csc_fill<uint16_t, IT>,    (const void*)k_csc_scatter<float, IT>,
+                     (const void*)k_csc_scatter<uint16_t, IT>};
+  for (const void* f : k) {
+    const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t init_load_kernels(int smem_bytes) {
+  const cudaError_t e = init_load_it<int32_t>(smem_bytes);
+  return e != cudaSuccess ? e : init_load_it<uint16_t>(smem_bytes);
 }
 
 template <typename VT, bool COPY>

@@ -160,19 +160,23 @@ unsigned vol_grid(const Geometry& g, int64_t n_rows) {
 
 }  // namespace
 
+cudaError_t init_volume_kernels(int smem_bytes) {
+  const cudaError_t e = cudaFuncSetAttribute(k_vol_hist, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_vol_digits, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+}
+
 size_t vol_hist_smem(const VolArgs& a) {
   return (size_t)(a.n_edges + a.n_bins + a.n_req) * sizeof(uint32_t);
 }
 
 void launch_vol_hist(const Geometry& g, const VolArgs& a, cudaStream_t s) {
   const size_t smem = vol_hist_smem(a);
-  cudaFuncSetAttribute(k_vol_hist, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   k_vol_hist<<<vol_grid(g, a.n_rows), 256, smem, s>>>(a);
 }
 
 void launch_vol_select(const Geometry& g, const SelArgs& a, cudaStream_t s) {
   const size_t smem = (size_t)a.n_sel * 256 * sizeof(uint32_t);
-  cudaFuncSetAttribute(k_vol_digits, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   k_vol_rank<<<1, kMaxSel, 0, s>>>(a);
   for (int shift = 24; shift >= 0; shift -= 8) {
     k_vol_digits<<<vol_grid(g, a.n_rows), 256, smem, s>>>(a, shift);
