@@ -354,13 +354,24 @@ bool chained(fredopt_t h) {
 // number of forward partials
 int n_parts(const Geometry& g, const FwdArgs& a) { return a.sched ? a.n_warps : forward_grid(g, a.n_warps); }
 
+// Elements that every array of the CSR, or of the CSC with 16- or 32-bit rows,
+// holds (kept buffers differ in length).
+int64_t csr_elems(fredopt_t h) {
+  const size_t vb = (size_t)value_bytes(h->fmt);
+  return (int64_t)std::min({h->col16.p ? h->col16.n : h->col.n, h->Dv.n / vb, h->Lv.n / vb});
+}
+int64_t csc_elems(fredopt_t h, bool row16) {
+  const size_t vb = (size_t)value_bytes(h->fmt);
+  return (int64_t)std::min({row16 ? h->crow16.n : h->crow.n, h->DTv.n / vb, h->LTv.n / vb});
+}
+
 FwdArgs fwd_args(fredopt_t h, bool hot, bool final_pass = false) {
   FwdArgs a{};
   a.pdl = chained(h);
   a.rp = h->rp.p;
   a.col = h->col.p;
   a.col16 = h->col16.p;
-  a.n_elems = (int64_t)(h->col16.p ? h->col16.n : h->col.n);
+  a.n_elems = csr_elems(h);
   a.Dv = h->Dv.p;
   a.Lv = h->Lv.p;
   a.sD = h->fmt ? h->sD.p : nullptr;
@@ -388,7 +399,7 @@ BwdArgs bwd_args(fredopt_t h, const float2* coef) {
   BwdArgs b{};
   b.st = h->st.p;
   b.n_rows = h->n_hot;
-  b.n_elems = (int64_t)h->crow.n;
+  b.n_elems = csc_elems(h, h->crow16.p != nullptr);
   b.n_ovf = (int32_t)h->n_wide_blocks;
   b.row = h->crow.p;
   b.row16 = h->crow16.p;
@@ -517,6 +528,9 @@ void enqueue_sweep(fredopt_t h, const float* w, int use_coef, double lam, double
   run(h, 5, [&] { launch_sweep_start(h->n, w, h->g.p, use_coef, h->xs.p, h->st.p, s); });
   SweepArgs a{};
   a.list = h->con_rows.p;
+  a.n_rows = h->n_hot;
+  a.n_elems = csr_elems(h);
+  a.n_csc = csc_elems(h, false);
   a.rp = h->rp.p;
   a.col = h->col.p;
   a.col16 = h->col16.p;

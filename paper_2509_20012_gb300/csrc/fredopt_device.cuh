@@ -114,6 +114,39 @@ __device__ __forceinline__ void warp_sum2(Acc& a, Acc& b, int lane) {
   b = up ? keep : other;
 }
 
+// ------------------------------------------------------------------ checked builds
+
+// Checked builds (FO_CHECKED=1, a debug aid in place of a memory checker): the
+// kernels that stream the matrices check every tile's, row's and column's element
+// range against the allocated length, every gathered index against its table and
+// every overflow slot, record a failure in bit 1 of the error word (reported as
+// FREDOPT_ERR_PATTERN) and skip the access.  Results are otherwise
+// bit-identical to the default build.
+#ifndef FO_CHECKED
+#define FO_CHECKED 0
+#endif
+// i, or 0 with the failure recorded when i lies outside [0, n)
+template <typename I>
+__device__ __forceinline__ I checked_index(I i, int64_t n, const DevState* st) {
+#if FO_CHECKED
+  if ((int64_t)i < 0 || (int64_t)i >= n) {
+    atomicOr(st->err, 2);
+    return 0;
+  }
+#endif
+  return i;
+}
+// e, or s with the failure recorded unless 0 <= s <= e <= n
+__device__ __forceinline__ int64_t checked_end(int64_t s, int64_t e, int64_t n, const DevState* st) {
+#if FO_CHECKED
+  if (s < 0 || e < s || e > n) {
+    atomicOr(st->err, 2);
+    return s;
+  }
+#endif
+  return e;
+}
+
 // ------------------------------------------------------------------ block reductions
 
 // Block reductions of one double per thread (blockDim = 256), in a fixed

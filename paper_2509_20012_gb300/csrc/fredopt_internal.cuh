@@ -341,6 +341,8 @@ struct SweepArgs {
   // the block's rows: list[i0 .. i1) (structure rows with nonzeros)
   const int64_t* list;
   int64_t i0, i1;
+  int64_t n_rows;          // streamed rows
+  int64_t n_elems, n_csc;  // allocated elements of the CSR and CSC arrays
   const int64_t* rp;       // CSR
   const int32_t* col;      // indices, or null when col16 is set
   const uint16_t* col16;

@@ -262,15 +262,6 @@ struct BlockBase {
   int32_t n_ovf;
 };
 
-// Checked builds (FO_CHECKED=1, a debug aid in place of a memory checker):
-// the streaming kernels check every tile's element range against the
-// allocated length, every gathered index against its table and every
-// overflow slot, record a failure in bit 1 of the error word (reported as
-// FREDOPT_ERR_PATTERN) and skip the access.  Results are otherwise
-// bit-identical to the default build.
-#ifndef FO_CHECKED
-#define FO_CHECKED 0
-#endif
 struct SegCheck {
   int64_t n_elems;
   int* err;
@@ -656,12 +647,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1024 / kFwdThreads) k_forward(Fwd
   const VT* __restrict__ Lv = reinterpret_cast<const VT*>(a.Lv);
   double acc0 = 0.0, acc1 = 0.0;  // per-lane partials of the epilogue reductions
   auto gather = [&](int c) {
-#if FO_CHECKED
-    if ((unsigned)c >= (unsigned)a.n_x) {
-      atomicOr(a.st->err, 2);
-      c = 0;
-    }
-#endif
+    c = checked_index(c, a.n_x, a.st);
     const float v = x[c];
     return make_float2(v, v);
   };
@@ -773,12 +759,7 @@ __global__ void __launch_bounds__(kBwdThreads, FO_BWD_MIN_BLOCKS) k_backward(Bwd
   const VT* __restrict__ Lv = reinterpret_cast<const VT*>(a.Lv);
   const float2* cf = a.coef;  // the predecessor's output
   auto gather = [&](int r) {
-#if FO_CHECKED
-    if ((uint64_t)(int64_t)r >= (uint64_t)a.n_rows) {
-      atomicOr(a.st->err, 2);
-      r = 0;
-    }
-#endif
+    r = checked_index(r, a.n_rows, a.st);
     // plain loads: what a chained predecessor wrote is not read-only
     if (!UD && FO_BWD_GATHER_Y) return make_float2(0.0f, cf[r].y);
     return cf[r];

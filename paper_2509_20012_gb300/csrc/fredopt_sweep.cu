@@ -92,9 +92,9 @@ __global__ void __launch_bounds__(256) k_sweep_rows(SweepArgs a) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t i = a.i0 + (int64_t)blockIdx.x * (8 / WPR) + wid / WPR;
   const bool have = i < a.i1;
-  const int64_t r = have ? a.list[i] : 0;
+  const int64_t r = have ? checked_index(a.list[i], a.n_rows, a.st) : 0;
   const int64_t s = have ? a.rp[r] : 0;
-  const int len = have ? (int)(a.rp[r + 1] - s) : 0;
+  const int len = have ? (int)(checked_end(s, a.rp[r + 1], a.n_elems, a.st) - s) : 0;
   const IT* __restrict__ ci = (sizeof(IT) == 2 ? reinterpret_cast<const IT*>(a.col16) : reinterpret_cast<const IT*>(a.col)) + s;
   const VT* __restrict__ Di = reinterpret_cast<const VT*>(a.rD) + s;
   const VT* __restrict__ Li = reinterpret_cast<const VT*>(a.rL) + s;
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(256) k_sweep_rows(SweepArgs a) {
     float x[K], dv[K], lv[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-      x[k] = c[k] >= 0 ? a.x[c[k]] : 0.0f;
+      x[k] = c[k] >= 0 ? a.x[checked_index(c[k], a.n, a.st)] : 0.0f;
       dv[k] = c[k] >= 0 ? to_f(d[k]) : 0.0f;
       lv[k] = c[k] >= 0 ? to_f(l[k]) : 0.0f;
     }
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kSweepConThreads) k_sweep_con(SweepArgs a, Tab
   stage_constraints(t, con);
   const int64_t i = a.i0 + (int64_t)blockIdx.x * kSweepConThreads + threadIdx.x;
   const bool have = i < a.i1;
-  const int64_t r = have ? a.list[i] : 0;
+  const int64_t r = have ? checked_index(a.list[i], a.n_rows, a.st) : 0;
   const uint32_t m = have ? a.mask[r] : 0u;
   const double dd = have ? a.dd[r] : 0.0, ll = have ? a.ll[r] : 0.0, dl = have ? a.dl[r] : 0.0;
   const double sd = have && a.sD ? (double)a.sD[r] : 1.0, sl = have && a.sL ? (double)a.sL[r] : 1.0;
@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(256, CTAS) k_sweep_cols(SweepArgs a) {
 #pragma unroll
   for (int k = 0; k < U; ++k) {
     const int64_t j = jc + jw + k * CPW;
-    const int64_t p0 = j < a.n ? a.pos0[j] : 0, p1 = j < a.n ? a.pos1[j] : 0;
+    const int64_t p0 = j < a.n ? a.pos0[j] : 0, p1 = j < a.n ? checked_end(p0, a.pos1[j], a.n_csc, a.st) : 0;
     p[k] = (int)p0 + sl;
     left[k] = (int)(p1 - p0) - sl;
     most = max(most, left[k]);
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(256, CTAS) k_sweep_cols(SweepArgs a) {
     for (int k = 0; k < U; ++k) {
 #pragma unroll
       for (int e = 0; e < K; ++e) {
-        g[k][e] = row[k][e] >= 0 ? a.gam[row[k][e]] : make_float2(0.0f, 0.0f);
+        g[k][e] = row[k][e] >= 0 ? a.gam[checked_index(row[k][e], a.n_rows, a.st)] : make_float2(0.0f, 0.0f);
         dv[k][e] = row[k][e] >= 0 ? to_f(d[k][e]) : 0.0f;
         lv[k][e] = row[k][e] >= 0 ? to_f(l[k][e]) : 0.0f;
       }

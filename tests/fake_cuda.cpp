@@ -13,6 +13,12 @@ size_t g_used = 0, g_peak = 0, g_limit = ~(size_t)0;
 int g_fail_waits = 0;      // forward products whose bounded wait gives up
 int g_fail_captures = 0;   // cudaStreamBeginCapture calls that fail
 int g_capturing = 0, g_stray_external = 0;
+int g_long_checks = 0;     // products whose stated array length is not that of every array
+void check_length(int64_t n, const void* idx, size_t ib, const void* d, const void* l, int fmt) {
+  const size_t vb = fmt == 0 ? 4 : 2;
+  for (auto [p, b] : {std::pair{idx, ib}, std::pair{d, vb}, std::pair{l, vb}})
+    if ((size_t)n * b > g_blocks[const_cast<void*>(p)]) ++g_long_checks;
+}
 long long g_nnz_hot = 0;
 }  // namespace
 
@@ -23,6 +29,7 @@ void fake_limit(size_t bytes) { g_limit = bytes; g_peak = g_used; }
 void fake_fail_waits(int n) { g_fail_waits = n; }
 void fake_fail_captures(int n) { g_fail_captures = n; }
 int fake_stray_external() { return g_stray_external; }
+int fake_long_checks() { return g_long_checks; }
 
 // ---- CUDA runtime
 cudaError_t cudaMalloc(void** p, size_t n) {
@@ -111,13 +118,16 @@ bool forward_uses_smem(const Geometry&, int) { return true; }
 int forward_grid(const Geometry& g, int) { return g.fwd_blocks; }
 int col_grid(const Geometry& g, int) { return g.col_blocks; }
 int con_grid(const Geometry& g, int64_t) { return g.row_blocks; }
-void launch_forward(const Geometry&, int, int, bool, const FwdArgs& a, const Tables&, cudaStream_t) {
+void launch_forward(const Geometry&, int fmt, int, bool, const FwdArgs& a, const Tables&, cudaStream_t) {
+  check_length(a.n_elems, a.col16 ? (const void*)a.col16 : a.col, a.col16 ? 2 : 4, a.Dv, a.Lv, fmt);
   if (g_fail_waits > 0) {
     --g_fail_waits;
     *a.st->err |= 1;
   }
 }
-void launch_backward(const Geometry&, int, bool, bool, const BwdArgs&, cudaStream_t) {}
+void launch_backward(const Geometry&, int fmt, bool, bool, const BwdArgs& a, cudaStream_t) {
+  check_length(a.n_elems, a.row16 ? (const void*)a.row16 : a.row, a.row16 ? 2 : 4, a.Dv, a.Lv, fmt);
+}
 void launch_colfinish(const Geometry&, int, const ColArgs&, cudaStream_t) {}
 void launch_constraints(const Geometry&, const Tables&, const ConArgs&, cudaStream_t) {}
 void launch_beta_table(double*, long long, double, double, cudaStream_t) {}
@@ -179,7 +189,10 @@ void launch_sweep_pos(const int64_t*, const int32_t*, int32_t, const int64_t*, i
 int sweep_weight_slices(int64_t) { return 1; }
 void launch_sweep_weights(const Tables&, const int64_t*, int64_t, int64_t, int, const uint32_t*, const double*,
                           const double*, const double*, double*, double*, cudaStream_t) {}
-void launch_sweep_rows(int, double, const SweepArgs&, cudaStream_t) {}
+void launch_sweep_rows(int fmt, double, const SweepArgs& a, cudaStream_t) {
+  check_length(a.n_elems, a.col16 ? (const void*)a.col16 : a.col, a.col16 ? 2 : 4, a.rD, a.rL, fmt);
+  check_length(a.n_csc, a.row, 4, a.Dv, a.Lv, fmt);
+}
 void launch_sweep_con(const Tables&, const SweepArgs&, cudaStream_t) {}
 void launch_sweep_cols(int, double, const SweepArgs&, cudaStream_t) {}
 void launch_sweep_finish(const Geometry&, int, const float*, float*, int, DevState*, LogEntry*, cudaStream_t) {}

@@ -113,3 +113,21 @@ def test_reload_frees_the_old_plan_when_memory_runs_out(fake, per):
         held = fake.fake_used()
     p.close()
     assert fake.fake_used() < base
+
+
+def test_checked_lengths_hold_for_every_array(fake):
+    """The element count that checked builds test ranges against is one that each of
+    the arrays has, also where a reload kept longer buffers for some of them."""
+    INDEX32, ROI = 0x200, 0x100
+    p = Plan(fake, 300, 20)
+    x, a, u = np.ones(p.n, np.float32), np.ones(2000, np.float32), np.zeros(2000, np.float32)
+    con = (fredopt.Constraint * 1)(fredopt.Constraint(0, 0, 1.0, 1.0))
+    for n_vox, per, fmt in ((300, 20, INDEX32), (200, 20, 0), (300, 20, 1), (250, 21, INDEX32 | 2), (300, 20, 0),
+                            (160, 20, INDEX32 | ROI), (160, 39, 1), (1200, 20, 0), (700, 20, 2)):
+        assert p.load(n_vox, per, fmt) == 0
+        assert p.lib.fredopt_set_constraints(p.h, 1, con) == 0
+        assert p.lib.fredopt_forward(p.h, x.ctypes.data, u.ctypes.data, None, 0) == 0
+        assert p.lib.fredopt_backward(p.h, a.ctypes.data, a.ctypes.data, u.ctypes.data, 0) == 0
+        assert p.lib.fredopt_sweep_step(p.h, x.ctypes.data, 1.0, 1.0, 0, 3, u.ctypes.data, 0) == 0
+        assert fake.fake_long_checks() == 0, (n_vox, per, fmt)
+    p.close()

@@ -28,3 +28,16 @@ def test_function_attributes_are_set_at_initialisation_only():
     calls = functions_calling("cudaFuncSetAttribute")
     assert len(calls) >= 3
     assert [c for c in calls if not c[1].startswith(("init_", "set_smem"))] == []
+
+
+def test_checked_build_covers_the_streaming_kernels():
+    """Every kernel that gathers by an index, or streams a range, that it reads from
+    memory checks both in FO_CHECKED builds."""
+    text = "".join(open(os.path.join(CSRC, f)).read() for f in ("fredopt_kernels.cu", "fredopt_sweep.cu"))
+    body = {}
+    for m in re.finditer(r"__global__ [^{;]*?(k_\w+)\([^{;]*\{", text):
+        body[m.group(1)] = text[m.end():text.index("\n}\n", m.end())]
+    for kernel in ("k_forward", "k_backward", "k_sweep_rows", "k_sweep_cols", "k_sweep_con"):
+        assert "checked_index(" in body[kernel], kernel
+    for kernel in ("k_sweep_rows", "k_sweep_cols"):
+        assert "checked_end(" in body[kernel], kernel
