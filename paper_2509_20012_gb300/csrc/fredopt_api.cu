@@ -659,12 +659,21 @@ void enqueue_iteration(fredopt_t h) {
 }
 
 // Tile weights: a row end or a chunk end (warp reductions and bookkeeping) costs
-// about as much as streaming this many nonzeros; 16-bit values stream faster
-// (fredopt_autotune can pick other weights).  Measured over the clinical, tiny,
-// half-resolution and batched plans: 100 against 64 for 16-bit rows, six plans
-// 8.56 -> 8.37 ms; 48 against 16 per chunk, clinical plan in ROI rows
-// 20.78 -> 20.69 ms, tiny plan 5.95 -> 5.91.
-constexpr int64_t kRowCost = 64, kRowCost16 = 100, kChunkCost = 48;
+// about as much as streaming this many nonzeros; 16-bit values stream faster.
+// fredopt_autotune picks among the candidates, which hold the weights of a load.
+// Measured over the clinical, tiny, half-resolution and batched plans: 128 against
+// 64 for 16-bit rows, six plans 8.57 -> 8.38 ms; 64 against 16 per chunk, clinical
+// plan in ROI rows 20.75 -> 20.69 ms, an ROI plan of 1e7 nonzeros 2.46 -> 2.40.
+constexpr int64_t kRowCosts[] = {16, 32, 64, 128, 256, 512}, kChunkCosts[] = {4, 16, 64, 256, 1024};
+constexpr int64_t kRowCost = 64, kRowCost16 = 128, kChunkCost = 64;
+template <size_t N>
+constexpr bool among(const int64_t (&list)[N], int64_t v) {
+  for (int64_t x : list)
+    if (x == v) return true;
+  return false;
+}
+static_assert(among(kRowCosts, kRowCost) && among(kRowCosts, kRowCost16) && among(kChunkCosts, kChunkCost),
+              "fredopt_autotune can keep the weights of a load");
 
 // Warp partitions.  A segment's sum does not depend on which warp streams it
 // (lanes take elements by their absolute block-aligned position and add them
@@ -2157,7 +2166,7 @@ int fredopt_autotune(fredopt_t h, int reps, int64_t* row_cost, int64_t* chunk_co
   fa.y = h->yw.p;
   int64_t best_row = h->row_cost;
   float best_f = 1e30f;
-  for (int64_t c : {16, 32, 64, 128, 256, 512}) {
+  for (int64_t c : kRowCosts) {
     if ((rc = set_fwd_schedule(h, c))) break;
     const float t = time_ms([&] { launch_forward(G, h->fmt, EPI_STORE, h->hint_fwd, fa, h->tab, s); });
     if (t < best_f) { best_f = t; best_row = c; }
@@ -2165,7 +2174,7 @@ int fredopt_autotune(fredopt_t h, int reps, int64_t* row_cost, int64_t* chunk_co
   BwdArgs ba = bwd_args(h, h->gam.p);
   int64_t best_chunk = h->chunk_cost;
   float best_b = 1e30f;
-  for (int64_t c : {4, 16, 64, 256, 1024}) {
+  for (int64_t c : kChunkCosts) {
     if (rc || (rc = set_bwd_schedule(h, c))) break;
     const float t = time_ms([&] { launch_backward(G, h->fmt, h->hint_bwd, true, ba, s); });
     if (t < best_b) { best_b = t; best_chunk = c; }

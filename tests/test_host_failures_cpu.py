@@ -131,3 +131,15 @@ def test_checked_lengths_hold_for_every_array(fake):
         assert p.lib.fredopt_sweep_step(p.h, x.ctypes.data, 1.0, 1.0, 0, 3, u.ctypes.data, 0) == 0
         assert fake.fake_long_checks() == 0, (n_vox, per, fmt)
     p.close()
+
+
+@pytest.mark.parametrize("fmt", [0, 1, 2])
+def test_autotune_can_keep_the_weights_of_a_load(fake, fmt):
+    """The tile weights that a load sets are among those that fredopt_autotune times
+    and returns (rows 16..512 and chunks 4..1024, as test_gpu_batch has them)."""
+    p = Plan(fake, 100, 20)
+    assert p.load(100, 20, fmt) == 0
+    r, c = ctypes.c_int64(), ctypes.c_int64()
+    assert fake.fredopt_get_tuning(p.h, ctypes.byref(r), ctypes.byref(c)) == 0
+    assert r.value in (16, 32, 64, 128, 256, 512) and c.value in (4, 16, 64, 256, 1024)
+    p.close()
