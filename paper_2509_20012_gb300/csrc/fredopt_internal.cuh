@@ -208,6 +208,14 @@ cudaError_t init_volume_kernels(int smem_bytes);
 cudaError_t kernel_arch(int* fwd_binary, int* bwd_binary, int* ptx_version);
 
 bool forward_uses_smem(const Geometry& g, int n_x_pad);
+// Shared memory of the forward product: x (n_x_pad floats) from the start, over
+// which the epilogue's reduction (kFwdRedBytes) is written when x is not read any
+// more, and behind both the barrier of x's bulk copy, whose place nothing else takes.
+constexpr size_t kFwdRedBytes = 512, kFwdBarBytes = 16;
+__host__ __device__ inline size_t fwd_bar_offset(int n_x_pad) {
+  const size_t x = (size_t)n_x_pad * sizeof(float);
+  return x > kFwdRedBytes ? x : kFwdRedBytes;
+}
 void launch_forward(const Geometry& g, int fmt, int epi, bool stream_hint, const FwdArgs& a,
                     const Tables& t, cudaStream_t s);
 void launch_backward(const Geometry& g, int fmt, bool stream_hint, bool use_D, const BwdArgs& a,

@@ -597,7 +597,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1024 / kFwdThreads) k_forward(Fwd
   extern __shared__ __align__(128) unsigned char smem[];
   using Acc = typename std::conditional<EPI == EPI_FINAL, DF, float>::type;
   const float* x = XS ? reinterpret_cast<const float*>(smem) : a.x;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + (size_t)a.n_x_pad * sizeof(float));
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + fwd_bar_offset(a.n_x_pad));
   if (XS) {
     if (threadIdx.x == 0) {
       mbar_init(bar, 1);
@@ -724,6 +724,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1024 / kFwdThreads) k_forward(Fwd
     const double s0 = warp_sum_nz(acc0), s1 = EPI == EPI_BC ? warp_sum_nz(acc1) : 0.0;
     __syncthreads();  // x is not read any more
     double* red = reinterpret_cast<double*>(smem);
+    static_assert(2 * 32 * sizeof(double) <= kFwdRedBytes && kFwdThreads <= 1024, "two sums per warp");
     if (lane == 0) {
       red[wid] = s0;
       red[32 + wid] = s1;
@@ -1297,8 +1298,7 @@ int forward_grid(const Geometry& g, int n_warps) {
 
 template <typename VT, int EPI, bool XS, bool S, typename IT = int32_t>
 static void fwd_inst(const Geometry& g, const FwdArgs& a, const Tables& t, cudaStream_t s) {
-  // x and its barrier; the epilogue's reduction takes the same place (512 bytes)
-  const size_t smem = std::max<size_t>(XS ? (size_t)a.n_x_pad * sizeof(float) + 16 : 0, 512);
+  const size_t smem = XS ? fwd_bar_offset(a.n_x_pad) + kFwdBarBytes : kFwdRedBytes;
   launch_chain(a.pdl, k_forward<VT, EPI, XS, S, IT>, forward_grid(g, a.n_warps), g.fwd_threads, smem, s, a, t);
 }
 
@@ -1336,7 +1336,7 @@ static void fwd_dispatch_epi(const Geometry& g, int epi, bool xs, bool st, const
 }
 
 bool forward_uses_smem(const Geometry& g, int n_x_pad) {
-  return FO_FWD_XS && (size_t)n_x_pad * sizeof(float) + 16 <= g.smem_limit;
+  return FO_FWD_XS && fwd_bar_offset(n_x_pad) + kFwdBarBytes <= g.smem_limit;
 }
 
 void launch_forward(const Geometry& g, int fmt, int epi, bool stream_hint, const FwdArgs& a,

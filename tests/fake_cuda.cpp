@@ -30,6 +30,7 @@ void fake_fail_waits(int n) { g_fail_waits = n; }
 void fake_fail_captures(int n) { g_fail_captures = n; }
 int fake_stray_external() { return g_stray_external; }
 int fake_long_checks() { return g_long_checks; }
+size_t fake_bar_offset(int n_x_pad) { return fo::fwd_bar_offset(n_x_pad); }
 
 // ---- CUDA runtime
 cudaError_t cudaMalloc(void** p, size_t n) {

@@ -143,3 +143,12 @@ def test_autotune_can_keep_the_weights_of_a_load(fake, fmt):
     assert fake.fredopt_get_tuning(p.h, ctypes.byref(r), ctypes.byref(c)) == 0
     assert r.value in (16, 32, 64, 128, 256, 512) and c.value in (4, 16, 64, 256, 1024)
     p.close()
+
+
+def test_the_barrier_of_the_forward_product_has_its_own_place(fake):
+    """Behind x (4 bytes per spot) and behind the 512 bytes of the reduction that is
+    written over x, on an 8-byte boundary, for every padded number of spots."""
+    fake.fake_bar_offset.restype = ctypes.c_size_t
+    for n_pad in (4, 8, 60, 124, 128, 132, 30000, 58100):
+        at = fake.fake_bar_offset(n_pad)
+        assert at == max(4 * n_pad, 512) and at % 8 == 0
