@@ -1417,8 +1417,8 @@ int fredopt_begin(fredopt_t h, const float* w0, double alpha, double relaxation,
   if (p.use_graphs) {
     const int64_t before = h->launches;
     const size_t t0 = h->timers_used;
-    h->capturing = true;
     CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+    h->capturing = true;
     enqueue_iteration(h);
     cudaError_t e = cudaStreamEndCapture(s, &h->graph);
     h->capturing = false;

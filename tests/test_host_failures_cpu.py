@@ -152,3 +152,17 @@ def test_the_barrier_of_the_forward_product_has_its_own_place(fake):
     for n_pad in (4, 8, 60, 124, 128, 132, 30000, 58100):
         at = fake.fake_bar_offset(n_pad)
         assert at == max(4 * n_pad, 512) and at % 8 == 0
+
+
+def test_a_capture_that_cannot_start_leaves_plain_launches(fake):
+    """After a begin whose stream capture is refused, a begin without graphs runs and
+    times its iterations as plain launches: no event is recorded as a graph node."""
+    p = Plan(fake, 50, 3)
+    assert fake.fredopt_set_timing(p.h, 1) == 0
+    fake.fake_fail_captures(1)
+    assert p.begin(use_graphs=1) == -7
+    assert p.begin(use_graphs=0) == 0
+    assert fake.fredopt_iterate(p.h, 2) == 0
+    assert p.end() == 0
+    assert fake.fake_stray_external() == 0
+    p.close()
