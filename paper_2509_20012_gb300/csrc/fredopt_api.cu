@@ -16,6 +16,7 @@
 #include <cstdio>
 #include <cstring>
 #include <limits>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -58,6 +59,18 @@ struct Timer {
 struct GraphTimer {
   cudaGraphNode_t a = nullptr, b = nullptr;
   int cls = 0;
+};
+
+// Blocks of the block-iterative sweep (built for m requested blocks; 0 = not built)
+struct Sweep {
+  int m = 0;
+  int nb = 0;                      // blocks actually formed
+  int64_t size = 0;                // structure rows with nonzeros per block
+  int warps = 0;                   // > 0: the streaming forward product takes the blocks' rows,
+  DBuf<int64_t> tiles;             // in this many tiles per block
+  DBuf<int64_t> pos, bounds;
+  DBuf<double> w, wpart;           // [nb] 1 / priority sum; its slices' sums
+  DBuf<double> part;               // violated rows' partial priority sums of a block
 };
 
 }  // namespace
@@ -133,15 +146,7 @@ struct fredopt_ctx {
   DBuf<float> chunk_sum, fout_a, fout_b, vin_a, vin_b;
   DBuf<uint8_t> vol_buf;  // volume statistics scratch
 
-  // block-iterative sweep (built for sweep_m requested blocks; 0 = not built)
-  int sweep_m = 0;
-  int sweep_nb = 0;                          // blocks actually formed
-  int64_t sweep_size = 0;                    // structure rows with nonzeros per block
-  int sweep_warps = 0;                       // > 0: the streaming forward product takes the blocks' rows,
-  DBuf<int64_t> sweep_tiles;                 // in this many tiles per block
-  DBuf<int64_t> sweep_pos, sweep_bounds_d;
-  DBuf<double> sweep_w, sweep_wpart;         // [sweep_nb] 1 / priority sum; its slices' sums
-  DBuf<double> sweep_part;                   // violated rows' partial priority sums of a block
+  std::unique_ptr<Sweep> sw{new Sweep()};    // blocks of the begun solve's sweeps, or of the last single sweep
   DBuf<float> xs;                            // the point being swept [n_pad]
   DBuf<float2> ys;                           // forward product of a block's rows [n_con_ne]
   DBuf<double> part;
@@ -458,8 +463,8 @@ ConArgs con_args(fredopt_t h) {
 // 1 / priority sum of the sweep blocks' reachable rows.  Formed when the blocks
 // are built, and again when the constraint table or c_cdl changes.
 void sweep_weights(fredopt_t h) {
-  launch_sweep_weights(h->tab, h->con_rows.p, h->n_con_ne, h->sweep_size, h->sweep_nb, h->mask.p, h->mdd.p, h->mll.p,
-                       h->mdl.p, h->sweep_wpart.p, h->sweep_w.p, h->stream);
+  launch_sweep_weights(h->tab, h->con_rows.p, h->n_con_ne, h->sw->size, h->sw->nb, h->mask.p, h->mdd.p, h->mll.p,
+                       h->mdl.p, h->sw->wpart.p, h->sw->w.p, h->stream);
 }
 
 // Rows of a sweep's blocks by the streaming forward product, when the list of
@@ -476,7 +481,7 @@ int64_t sweep_stream_nnz(fredopt_t h) { return h->fmt == FREDOPT_FP32 ? 10000000
 // boundaries (the device rows from a block's first structure row to the next
 // block's first).
 int build_sweep(fredopt_t h, int m) {
-  if (h->sweep_m == m) return FREDOPT_OK;
+  if (h->sw->m == m) return FREDOPT_OK;
   cudaStream_t s = h->stream;
   std::vector<int64_t> C(h->n_con_ne);  // structure rows with nonzeros, ascending
   if (!C.empty()) {
@@ -484,40 +489,41 @@ int build_sweep(fredopt_t h, int m) {
     CK(cudaStreamSynchronize(s));
   }
   std::vector<int64_t> bnd;
-  h->sweep_nb = 0;
-  h->sweep_size = 0;
+  h->sw->m = 0;
+  h->sw->nb = 0;
+  h->sw->size = 0;
   if (!C.empty()) {
     const int64_t S = ((int64_t)C.size() + m - 1) / m;
     const int nb = (int)(((int64_t)C.size() + S - 1) / S);
     for (int t = 0; t < nb; ++t) bnd.push_back(C[(size_t)t * S]);
-    h->sweep_nb = nb;
-    h->sweep_size = S;
+    h->sw->nb = nb;
+    h->sw->size = S;
   }
   bnd.push_back(C.empty() ? 0 : C.back() + 1);
-  h->sweep_warps = 0;
+  h->sw->warps = 0;
   if (!C.empty() && C.back() + 1 == (int64_t)C.size() &&
-      h->con_nnz >= sweep_stream_nnz(h) * h->sweep_nb) {
-    const int W = (int)std::min<int64_t>(h->geo.fwd_warps, h->sweep_size);
-    CK(h->sweep_tiles.alloc(2 * (size_t)W * h->sweep_nb));
-    for (int t = 0; t < h->sweep_nb; ++t)
+      h->con_nnz >= sweep_stream_nnz(h) * h->sw->nb) {
+    const int W = (int)std::min<int64_t>(h->geo.fwd_warps, h->sw->size);
+    CK(h->sw->tiles.alloc(2 * (size_t)W * h->sw->nb));
+    for (int t = 0; t < h->sw->nb; ++t)
       launch_tiles(TileArgs{TileArgs::PAIRS, h->rp.p, bnd[t], bnd[t + 1], 0, 0, W, 0, h->row_cost,
-                            h->sweep_tiles.p + 2 * (size_t)W * t, nullptr}, s);
-    h->sweep_warps = W;
+                            h->sw->tiles.p + 2 * (size_t)W * t, nullptr}, s);
+    h->sw->warps = W;
   }
-  CK(upload_vec(h, h->sweep_bounds_d, bnd));
-  CK(h->sweep_pos.alloc(bnd.size() * h->n));
-  if (h->sweep_nb > 0)
-    launch_sweep_pos(h->cp.p, h->crow.p, h->n, h->sweep_bounds_d.p, (int)bnd.size(), h->sweep_pos.p, s);
-  CK(h->sweep_w.alloc(h->sweep_nb));
-  CK(h->sweep_wpart.alloc((size_t)h->sweep_nb * sweep_weight_slices(h->sweep_size)));
-  CK(h->sweep_part.alloc((size_t)((h->sweep_size + kSweepConThreads - 1) / kSweepConThreads)));
+  CK(upload_vec(h, h->sw->bounds, bnd));
+  CK(h->sw->pos.alloc(bnd.size() * h->n));
+  if (h->sw->nb > 0)
+    launch_sweep_pos(h->cp.p, h->crow.p, h->n, h->sw->bounds.p, (int)bnd.size(), h->sw->pos.p, s);
+  CK(h->sw->w.alloc(h->sw->nb));
+  CK(h->sw->wpart.alloc((size_t)h->sw->nb * sweep_weight_slices(h->sw->size)));
+  CK(h->sw->part.alloc((size_t)((h->sw->size + kSweepConThreads - 1) / kSweepConThreads)));
   CK(h->xs.ensure(h->n_pad));
   CK(cudaMemsetAsync(h->xs.p, 0, h->n_pad * sizeof(float), s));
   CK(h->ys.ensure(h->n_con_ne));
   sweep_weights(h);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
-  h->sweep_m = m;
+  h->sw->m = m;
   return FREDOPT_OK;
 }
 
@@ -544,7 +550,7 @@ void enqueue_sweep(fredopt_t h, const float* w, int use_coef, double lam, double
   a.dl = h->mdl.p;
   a.y = h->ys.p;
   a.gam = h->gam.p;
-  a.part = h->sweep_part.p;
+  a.part = h->sw->part.p;
   a.row = h->crow.p;
   a.Dv = h->DTv.p;
   a.Lv = h->LTv.p;
@@ -556,19 +562,19 @@ void enqueue_sweep(fredopt_t h, const float* w, int use_coef, double lam, double
   a.in_solve = in_solve;
   a.st = h->st.p;
   const double row_nnz = h->n_con_ne > 0 ? (double)h->con_nnz / (double)h->n_con_ne : 0.0;
-  const double col_nnz = (double)h->nnz_hot / ((double)std::max(1, h->sweep_nb) * (double)h->n);
-  for (int t = 0; t < h->sweep_nb; ++t) {
-    a.i0 = t * h->sweep_size;
-    a.i1 = std::min(h->n_con_ne, a.i0 + h->sweep_size);
+  const double col_nnz = (double)h->nnz_hot / ((double)std::max(1, h->sw->nb) * (double)h->n);
+  for (int t = 0; t < h->sw->nb; ++t) {
+    a.i0 = t * h->sw->size;
+    a.i1 = std::min(h->n_con_ne, a.i0 + h->sw->size);
     a.con_blocks = (int)((a.i1 - a.i0 + kSweepConThreads - 1) / kSweepConThreads);
-    a.winv = h->sweep_w.p + t;
-    a.pos0 = h->sweep_pos.p + (size_t)t * h->n;
-    a.pos1 = h->sweep_pos.p + (size_t)(t + 1) * h->n;
-    if (h->sweep_warps > 0) {
+    a.winv = h->sw->w.p + t;
+    a.pos0 = h->sw->pos.p + (size_t)t * h->n;
+    a.pos1 = h->sw->pos.p + (size_t)(t + 1) * h->n;
+    if (h->sw->warps > 0) {
       FwdArgs fa = fwd_args(h, true);
       fa.pdl = true;
-      fa.warp_row = h->sweep_tiles.p + 2 * (size_t)h->sweep_warps * t;
-      fa.n_warps = h->sweep_warps;
+      fa.warp_row = h->sw->tiles.p + 2 * (size_t)h->sw->warps * t;
+      fa.n_warps = h->sw->warps;
       fa.sched = nullptr;
       fa.x = h->xs.p;
       fa.y = h->ys.p;
@@ -953,7 +959,7 @@ static void release_plan(fredopt_t h) {
   h->crow.release(); h->crow16.release(); h->chdr.release(); h->DTv.release(); h->LTv.release();
   h->yw.release(); h->yg.release(); h->r.release(); h->gam.release(); h->ucoef.release();
   h->y64.release(); h->yall.release(); h->fout_a.release(); h->fout_b.release();
-  h->vin_a.release(); h->vin_b.release(); h->ys.release(); h->sweep_pos.release(); h->sweep_tiles.release();
+  h->vin_a.release(); h->vin_b.release(); h->ys.release(); h->sw.reset(new Sweep());
 }
 
 static int load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t nnz,
@@ -973,7 +979,7 @@ static int load_influence(fredopt_t h, int64_t n_vox, int32_t n_spots, int64_t n
   free_graph(h);
   h->loaded = false;
   h->begun = false;
-  h->sweep_m = 0;
+  h->sw->m = 0;
   cudaStream_t s = h->stream;
   if (!*keep) release_plan(h);
   join_in(h);
@@ -1307,7 +1313,7 @@ int fredopt_set_constraints(fredopt_t h, int n, const fredopt_constraint* c) {
   h->n_rows_reach = (int64_t)nr;
   h->n_unreach = (int64_t)nu;
   h->W_all = W;
-  if (h->sweep_m > 0) sweep_weights(h);
+  if (h->sw->m > 0) sweep_weights(h);
   h->have_con = true;
   return FREDOPT_OK;
 }
@@ -1384,7 +1390,7 @@ int fredopt_begin(fredopt_t h, const float* w0, double alpha, double relaxation,
   h->beta0 = p.beta0 < 0.0 ? 0.1 * std::sqrt(nrm) : p.beta0;
   if (h->tab.c != p.c_cdl) {
     h->tab.c = p.c_cdl;
-    if (h->sweep_m > 0) sweep_weights(h);
+    if (h->sw->m > 0) sweep_weights(h);
   }
   CK(copy_in(h, h->w.p, w0, h->n * sizeof(float), flags));
   if (h->btab_alpha != alpha || h->btab_beta0 != h->beta0) {
@@ -1779,10 +1785,25 @@ int fredopt_sweep_step(fredopt_t h, const float* x, double relaxation, double pr
   if (norm != FREDOPT_NORM_ALL && norm != FREDOPT_NORM_VIOLATED) return fail(h, FREDOPT_ERR_INVALID_ARG, "bad norm");
   if (n_blocks < 1 || n_blocks > FREDOPT_MAX_SWEEP_BLOCKS)
     return fail(h, FREDOPT_ERR_INVALID_ARG, "need 1 <= n_blocks <= FREDOPT_MAX_SWEEP_BLOCKS");
-  if (h->begun && h->gexec && h->prm.sweep_blocks > 0 && h->sweep_m != n_blocks)
+  if (h->begun && h->gexec && h->prm.sweep_blocks > 0 && h->sw->m != n_blocks)
     return fail(h, FREDOPT_ERR_INVALID_ARG, "the begun solve sweeps another number of blocks");
   DeviceGuard dg(h->device);
   join_in(h);
+  // a begun solve that sweeps other blocks (in plain launches or a batch graph)
+  // keeps its own: this call's are built aside and freed at its end
+  struct Aside {
+    fredopt_t h;
+    std::unique_ptr<Sweep> own;
+    ~Aside() {
+      if (!own) return;
+      cudaStreamSynchronize(h->stream);
+      h->sw = std::move(own);
+    }
+  } aside{h, nullptr};
+  if (h->begun && h->prm.sweep_blocks > 0 && h->sw->m != n_blocks) {
+    aside.own = std::move(h->sw);
+    h->sw.reset(new Sweep());
+  }
   rc = build_sweep(h, n_blocks);
   if (rc) return rc;
   const float* xin = nullptr;

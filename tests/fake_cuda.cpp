@@ -13,6 +13,8 @@ size_t g_used = 0, g_peak = 0, g_limit = ~(size_t)0;
 int g_fail_waits = 0;      // forward products whose bounded wait gives up
 int g_fail_captures = 0;   // cudaStreamBeginCapture calls that fail
 int g_capturing = 0, g_stray_external = 0;
+int g_sweep_blocks = 0;
+const void *g_sweep_pos = nullptr, *g_captured_pos = nullptr;
 int g_long_checks = 0;     // products whose stated array length is not that of every array
 void check_length(int64_t n, const void* idx, size_t ib, const void* d, const void* l, int fmt) {
   const size_t vb = fmt == 0 ? 4 : 2;
@@ -29,6 +31,13 @@ void fake_limit(size_t bytes) { g_limit = bytes; g_peak = g_used; }
 void fake_fail_waits(int n) { g_fail_waits = n; }
 void fake_fail_captures(int n) { g_fail_captures = n; }
 int fake_stray_external() { return g_stray_external; }
+int fake_sweep_blocks() {  // blocks swept since the last call
+  const int n = g_sweep_blocks;
+  g_sweep_blocks = 0;
+  return n;
+}
+void fake_capture_pos() { g_captured_pos = g_sweep_pos; }  // the tables of the last sweep
+int fake_captured_alive() { return g_blocks.count(const_cast<void*>(g_captured_pos)); }
 int fake_long_checks() { return g_long_checks; }
 size_t fake_bar_offset(int n_x_pad) { return fo::fwd_bar_offset(n_x_pad); }
 
@@ -45,8 +54,7 @@ cudaError_t cudaMalloc(void** p, size_t n) {
 cudaError_t cudaFree(void* p) {
   g_used -= g_blocks[p];
   g_blocks.erase(p);
-  std::free(p);
-  return cudaSuccess;
+  return cudaSuccess;  // not handed out again: a stale pointer shows
 }
 cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { *p = std::calloc(1, n); return cudaSuccess; }
 cudaError_t cudaHostGetDevicePointer(void** d, void* h, unsigned) { *d = h; return cudaSuccess; }
@@ -193,6 +201,8 @@ void launch_sweep_weights(const Tables&, const int64_t*, int64_t, int64_t, int, 
 void launch_sweep_rows(int fmt, double, const SweepArgs& a, cudaStream_t) {
   check_length(a.n_elems, a.col16 ? (const void*)a.col16 : a.col, a.col16 ? 2 : 4, a.rD, a.rL, fmt);
   check_length(a.n_csc, a.row, 4, a.Dv, a.Lv, fmt);
+  if (a.i0 == 0) g_sweep_pos = a.pos0;
+  ++g_sweep_blocks;
 }
 void launch_sweep_con(const Tables&, const SweepArgs&, cudaStream_t) {}
 void launch_sweep_cols(int, double, const SweepArgs&, cudaStream_t) {}

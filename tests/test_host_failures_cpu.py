@@ -166,3 +166,29 @@ def test_a_capture_that_cannot_start_leaves_plain_launches(fake):
     assert p.end() == 0
     assert fake.fake_stray_external() == 0
     p.close()
+
+
+def test_a_single_sweep_leaves_the_solve_its_blocks(fake):
+    """A begun solve that sweeps 4 blocks, in plain launches or captured in a batch,
+    goes on with its own 4 after a single sweep of 7, whose tables are not built in
+    the place of the solve's."""
+    p = Plan(fake, 100, 3)
+    con = (fredopt.Constraint * 1)(fredopt.Constraint(0, 0, 1.0, 1.0))
+    assert fake.fredopt_set_constraints(p.h, 1, con) == 0
+    x, w = np.ones(p.n, np.float32), np.zeros(p.n, np.float32)
+    sweep = lambda n: fake.fredopt_sweep_step(p.h, x.ctypes.data, 1.0, 1.0, 0, n, w.ctypes.data, 0)
+    assert p.begin(sweep_blocks=4) == 0
+    b = ctypes.c_void_p()
+    fake.fake_sweep_blocks()
+    assert fake.fredopt_batch_create(ctypes.byref(b), (ctypes.c_void_p * 1)(p.h), 1) == 0
+    assert fake.fake_sweep_blocks() == 4
+    fake.fake_capture_pos()
+    assert sweep(7) == 0 and fake.fake_sweep_blocks() == 7
+    assert fake.fake_captured_alive() == 1
+    assert fake.fredopt_iterate(p.h, 2) == 0 and fake.fake_sweep_blocks() == 8
+    assert sweep(4) == 0 and fake.fake_sweep_blocks() == 4
+    assert fake.fredopt_batch_destroy(b) == 0
+    # a captured solve refuses another number, as it did
+    assert p.begin(sweep_blocks=4, use_graphs=1) == 0
+    assert sweep(7) == -1
+    p.close()
