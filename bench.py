@@ -7,7 +7,9 @@ and LETd limits; w0 = 1, alpha 0.99, relaxation 1.  One step = one
 superiorized iteration (Fig. 3 around the simultaneous Fig. 2): two fused
 forward products and two transposed products over every voxel row.
 
-Output: one JSON line (rank 0).  `value` is device throughput with the plan
+Output: one JSON line of at most 4000 characters (rank 0), and the full record
+as a JSON file (--detail, default _build/bench_detail.json), of whose further
+entries the line keeps the leading numbers.  `value` is device throughput with the plan
 resident in HBM, timed over K graph replays of the iteration (the library's
 path); `e2e` is one full plan re-optimisation (500 iterations) through the
 public C ABI from pinned host buffers; `roofline` is the dominant kernel's
@@ -81,6 +83,52 @@ def peaks():
         return float(d["hbm_gbs"]), "measured"
     except Exception:
         return 6800.0, "fallback"
+
+
+# what the printed line always holds, as it is; the record's other entries follow as
+# far as LINE_CHARS allows
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks")
+LINE_CHARS = 4000
+
+
+def _short(v, depth=2):
+    """The numbers, truth values and short texts of a record, floats to 5 digits,
+    nested dicts to `depth` levels; None when nothing of that is in it."""
+    if isinstance(v, bool) or v is None or isinstance(v, int):
+        return v
+    if isinstance(v, float):
+        return float(f"{v:.5g}")
+    if isinstance(v, str):
+        return v if len(v) <= 32 else None
+    if isinstance(v, dict) and depth:
+        out = {k: _short(x, depth - 1) for k, x in v.items()}
+        return {k: x for k, x in out.items() if x is not None} or None
+    return None
+
+
+def headline(record: dict, limit: int = LINE_CHARS) -> str:
+    """The printed line: LINE_KEYS unchanged, then the other entries shortened, in
+    order, each as long as the line stays within `limit` characters."""
+    line = {k: record[k] for k in LINE_KEYS if k in record}
+    for k, v in record.items():
+        if k in line:
+            continue
+        for depth in (2, 1):
+            s = _short(v, depth)
+            if s is not None and len(json.dumps({**line, k: s})) <= limit:
+                line[k] = s
+                break
+    return json.dumps(line)
+
+
+def write_record(record: dict, path: str):
+    try:
+        os.makedirs(os.path.dirname(os.path.abspath(path)), exist_ok=True)
+        with open(path, "w") as f:
+            json.dump(record, f, indent=1)
+    except OSError as e:
+        print(f"bench: record not written to {path}: {e}", file=sys.stderr)
 
 
 class ClockSampler:
@@ -419,7 +467,8 @@ def run_gpu_arm(args):
                                 "n_rows": roi["sizes"]["n_rows"], "nnz_rows": roi["sizes"]["nnz_rows"],
                                 "forward": roi["fwd"], "backward": roi["bwd"], "clocks": roi["clocks"],
                                 "max_abs_w_diff_vs_all_rows": float(np.max(np.abs(roi["w"] - main["w"])))}
-        print(json.dumps(line))
+        write_record(line, args.detail)
+        print(headline(line))
     if ws > 1:
         import torch.distributed as dist
         dist.barrier()
@@ -988,6 +1037,8 @@ def main():
     ap.add_argument("--warmup", type=int, default=5)
     ap.add_argument("--impl", default="gb300", choices=["gb300", "reference"])
     ap.add_argument("--seed", type=int, default=0)
+    ap.add_argument("--detail", default=os.path.join(ROOT, "_build", "bench_detail.json"),
+                    help="file for the full record, of which the printed line is the head")
     ap.add_argument("--no-roi", dest="roi", action="store_false")
     ap.add_argument("--e2e-iters", type=int, default=500)
     ap.add_argument("--cpu-iters", type=int, default=2,
