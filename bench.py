@@ -89,6 +89,7 @@ def peaks():
 # far as LINE_CHARS allows
 LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
              "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks")
+LINE_NEXT = {"roofline": 1, "cpu_baseline": 1, "serving": 2, "batching": 2, "roi_rows": 1, "precision": 2}  # entry: levels
 LINE_CHARS = 4000
 
 
@@ -108,14 +109,14 @@ def _short(v, depth=2):
 
 
 def headline(record: dict, limit: int = LINE_CHARS) -> str:
-    """The printed line: LINE_KEYS unchanged, then the other entries shortened, in
-    order, each as long as the line stays within `limit` characters."""
+    """The printed line: LINE_KEYS unchanged, then the other entries shortened,
+    LINE_NEXT first, each if the line stays within `limit` characters."""
     line = {k: record[k] for k in LINE_KEYS if k in record}
-    for k, v in record.items():
-        if k in line:
+    for k in (*LINE_NEXT, *record):
+        if k in line or k not in record:
             continue
-        for depth in (2, 1):
-            s = _short(v, depth)
+        for depth in range(LINE_NEXT.get(k, 2), 0, -1):
+            s = _short(record[k], depth)
             if s is not None and len(json.dumps({**line, k: s})) <= limit:
                 line[k] = s
                 break
