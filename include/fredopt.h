@@ -73,8 +73,8 @@ extern "C" {
  * other plans (a batch graph, a server with several plans in flight): about
  * one SM's worth of CTAs per 400000 nonzeros of the streamed rows (the whole
  * GPU from 6.08e7 nonzeros on GB300), so that small plans leave SMs to the
- * others (fredopt_forward and the final passes, whose sums do not depend on
- * it, take the whole GPU).  Results depend only on the plan and its launch
+ * others (fredopt_forward, the final passes and the sweep's blocks, whose sums
+ * do not depend on it, take the whole GPU).  Results depend only on the plan and its launch
  * shapes: a plan loaded with and without the flag agrees to rounding, and bit
  * for bit with itself alone and in a batch. */
 #define FREDOPT_SHARED 0x400
@@ -282,9 +282,9 @@ int fredopt_objective(fredopt_t h, const float* x, double* f_out, float* grad_ou
  * PTV rule "98% of the volume receives at least 95% of the prescription") ----
  *
  * The voxel values are those of fredopt_end's final pass: (D w)_i and
- * (L w)_i accumulated in double-float (about 48 bits; exact products, relative
- * error per addition <= 3 * 2^-48) over the stored values, then rounded once to
- * FP32 as dose = (D w)_i, LETd = (L w)_i / (D w)_i (0 where (D w)_i <= 0),
+ * (L w)_i accumulated in double-float over the stored values (exact products;
+ * for a row of n nonzeros the error is at most (3 n / 128 + 40) 2^-48 of the sum
+ * of the products' magnitudes), then rounded once to FP32 as dose = (D w)_i, LETd = (L w)_i / (D w)_i (0 where (D w)_i <= 0),
  * cDL = c_cdl (L w)_i, with c_cdl of the last begin (default 0.04 um/keV).
  * A structure is the set of voxels whose mask has bit struct_bit set.
  *

@@ -345,11 +345,10 @@ bool claim_all_tiles(fredopt_t h, bool final_pass) {
 // The kernels of a captured iteration form a dependent chain, each starting
 // while its predecessor drains (tiny plan: 62.3 -> 59.9 us per iteration).  Not
 // in long passes: CTAs placed early on the SMs that drain first unbalance them
-// (1.2e4 nonzeros per warp: 1% slower).  Not for plans that share the GPU:
-// CTAs that wait hold the slots of the other plans (six small plans in a batch:
-// 8.8 against 9.4 ms).  Not for single calls: a dependent launch costs the host
-// more than the few kernels gain (feasibility step of the tiny plan: 89 against
-// 95 us).
+// (1.2e4 nonzeros per warp: 1% slower).  Not for plans that share the GPU, which
+// it does not help (six small plans in a batch: 8.42 and 8.40 ms).  Not for single
+// calls: a dependent launch costs the host 1 us more (feasibility step of the tiny
+// plan: 62.9 against 65.1 us; a gradient of 1.1e7 nonzeros would gain, 83 -> 74 us).
 constexpr int64_t kChainMaxNnzPerWarp = 4096;
 bool chained(fredopt_t h) {
   return h->capturing && h->nnz_hot < kChainMaxNnzPerWarp * (int64_t)h->geo.fwd_warps &&

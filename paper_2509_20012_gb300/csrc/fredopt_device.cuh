@@ -25,7 +25,7 @@ __device__ __forceinline__ T warp_sum(T v) {
 // A value hi + lo held in two FP32 numbers (|lo| <= ulp(hi) / 2): about 48
 // significant bits at FP32 speed.  GB300's FP64 rate is a small fraction of
 // its FP32 rate, so the final FP64-class pass accumulates in this form.
-// Products are exact (TwoProd with an FMA); additions use the accurate
+// Sums of two such values use the accurate
 // double-word sum of Joldes, Muller and Popescu (ACM TOMS 44(2), 2017,
 // relative error <= 3 * 2^-48), built from Knuth's TwoSum and Dekker's
 // FastTwoSum.  Every operation is an explicitly rounded intrinsic, so the
@@ -53,11 +53,6 @@ __device__ __forceinline__ DF df_add(DF x, DF y) {
   const DF v = fast_two_sum(s.hi, __fadd_rn(s.lo, t.hi));
   return fast_two_sum(v.hi, __fadd_rn(t.lo, v.lo));
 }
-// c + a * b
-__device__ __forceinline__ DF acc_fma(float a, float b, DF c) {
-  const float p = __fmul_rn(a, b);
-  return df_add(c, DF(p, __fmaf_rn(a, b, -p)));  // a * b = p + (a * b - p) exactly
-}
 template <>
 __device__ __forceinline__ DF warp_sum(DF v) {
 #pragma unroll
@@ -67,14 +62,25 @@ __device__ __forceinline__ DF warp_sum(DF v) {
   }
   return v;
 }
-// c + sum of four products in double-float: the products exact (TwoProd), the
-// three sums of their high parts exact (TwoSum), the seven error terms added
-// in FP32, and one renormalised addition to c.  Against four acc_fma steps
-// this is 43 FP32 operations instead of 88, and one rounding of the pair
-// instead of four: over rows of 128 to 3072 nonzeros (positive, mixed-sign
-// and wide-ranged values) its largest error against 64-bit-exact sums is the
-// same or smaller (5e-15 against 6e-15 of the sum of magnitudes).  The final
-// pass is bound by these operations: 7.3e8 nonzeros, FP32 2.70 -> 1.46 ms,
+// c + sum of four products in double-float: the products exact (TwoProd with an
+// FMA: a x = p + fma(a, x, -p)), the three sums of their high parts exact (TwoSum),
+// the seven error terms added in FP32, and joined to c by a TwoSum of the high parts
+// and two FP32 additions.  With u = 2^-24 and M the four products' magnitudes, the
+// error terms are at most 3 u M in all and pass three additions each, 8 u^2 M; the
+// two that join them err by u^2 (|c| + 3 M) and u^2 (2 |c| + 4 M); when c and the sum
+// nearly cancel, the last FastTwoSum's operands may lie the other way round, for no
+// more than u^2 (|c| + 3 M) where the addition before it saves u^2 (|c| + M).  A
+// step's error is at most 2^-48 (17 M + 3 |c|).  A row of n nonzeros takes n / 128
+// steps per lane (two more where it starts and ends inside a block), and the lanes'
+// sums are joined by five accurate additions, so
+// its sum is within (3 n / 128 + 40) 2^-48 of its sum of magnitudes (absolutely: terms
+// that cancel leave a larger relative error).  Four accurate double-word
+// additions instead (88 FP32 operations, not 43; 3 u^2 of the partial sum each) bound
+// it no better and measure the same or worse: largest errors in units of 2^-48 of the
+// sum of magnitudes, four additions / this, over rows of
+//   384 to 3072 nonzeros    positive 1.4 / 1.5   mixed signs 0.2 / 0.2   2^-30..2^30 1.0 / 0.9
+//   58112 nonzeros          positive 2.2 / 2.1   mixed signs 0.1 / 0.1   2^-30..2^30 0.5 / 0.3
+// The final pass is bound by these operations: 7.3e8 nonzeros, FP32 2.70 -> 1.46 ms,
 // FP16 2.59 -> 1.63 ms (its streaming floor is 1.07 and 0.65 ms).
 __device__ __forceinline__ DF df_dot4(const float* a, const float* x, DF c) {
   float p[4], e[4];

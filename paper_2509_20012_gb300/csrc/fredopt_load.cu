@@ -211,9 +211,8 @@ __device__ __forceinline__ void store_as(float v, __half* q) { *q = __float2half
 //   - values to Dv, Lv in their storage type, 16-bit ones after a power-of-two
 //     row scale (COPY = false: the input arrays are the storage already);
 //   - for streamed rows the moments |D_i|^2, |L_i|^2, <D_i, L_i> of the stored
-//     values in double-float (exact products, df_dot4; relative error of these
-//     nonnegative terms <= 3 * 2^-48 per addition), scales applied at the end,
-//     exactly.
+//     values in double-float (exact products; error bound at df_dot4), scales
+//     applied at the end, exactly.
 // Bound by its bytes: 12 read and 10 written per FP32 nonzero, 2.50 ms for
 // 7.3e8 (6.4 TB/s).  Separate passes (validation 1.49 ms, row gather 5.87,
 // moments 2.06, index narrowing 0.66) took 10.1 ms.
