@@ -759,15 +759,56 @@ int spot_in(fredopt_t h, const float* src, uint32_t flags, const float** x) {
   return FREDOPT_OK;
 }
 
-// Checks n spots of w0 and adds their squares to *nrm, in order.
-int check_spots(fredopt_t h, const float* w, int32_t n, double* nrm) {
-  for (int32_t j = 0; j < n; ++j) {
-    const float v = w[j];
-    if (!std::isfinite(v)) return fail(h, FREDOPT_ERR_NONFINITE, "w0 not finite");
-    if (v < 0.0f) return fail(h, FREDOPT_ERR_INVALID_ARG, "w0 must be >= 0");
-    *nrm += (double)v * (double)v;
+// Sum of squares of n values in the order of k_check_spots: 256 interleaved sums
+// (exact products), each 32 joined by halves, then the eight in order.
+double slice_squares(const float* x, int32_t n) {
+  double v[256] = {0.0};
+  for (int32_t j = 0; j < n; ++j) v[j & 255] += (double)x[j] * (double)x[j];
+  double sum = 0.0;
+  for (int w = 0; w < 8; ++w) {
+    double* t = v + 32 * w;
+    for (int o = 16; o > 0; o >>= 1)
+      for (int l = 0; l < o; ++l) t[l] += t[l + o];
+    sum = w ? sum + t[0] : t[0];
   }
-  return FREDOPT_OK;
+  return sum;
+}
+
+// Checks w0 (host or device) and sums its squares into *nrm; a host and a device
+// array give the same bits and the same error, that of the first bad element.
+int check_spots(fredopt_t h, const float* w0, uint32_t flags, double* nrm) {
+  double part[2 * kSpotSlices];
+  if (dev_ptr(flags)) {
+    double* pw = h->part.p + h->off_fin;
+    launch_check_spots(w0, h->n, pw, h->stream);
+    CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(stage(h), pw, sizeof(part), cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaStreamSynchronize(h->stream));
+    std::memcpy(part, stage(h), sizeof(part));
+  } else {
+    const int32_t per = (h->n + kSpotSlices - 1) / kSpotSlices;
+    for (int b = 0; b < kSpotSlices; ++b) {
+      const int64_t j0 = std::min<int64_t>(h->n, (int64_t)b * per), j1 = std::min<int64_t>(h->n, j0 + per);
+      part[2 * b] = slice_squares(w0 + j0, (int32_t)(j1 - j0));
+      part[2 * b + 1] = (double)kNoSpot;
+      bool bad = false;
+      for (int64_t j = j0; j < j1; ++j) bad |= !(w0[j] >= 0.0f && w0[j] <= std::numeric_limits<float>::max());
+      for (int64_t j = j0; bad && j < j1; ++j) {
+        const bool neg = w0[j] < 0.0f && std::isfinite(w0[j]);
+        if (!neg && std::isfinite(w0[j])) continue;
+        part[2 * b + 1] = (double)(2 * j + neg);
+        break;
+      }
+    }
+  }
+  double first = (double)kNoSpot;
+  for (int b = 0; b < kSpotSlices; ++b) {
+    *nrm += part[2 * b];
+    first = std::min(first, part[2 * b + 1]);
+  }
+  if (first == (double)kNoSpot) return FREDOPT_OK;
+  if ((unsigned long long)first & 1) return fail(h, FREDOPT_ERR_INVALID_ARG, "w0 must be >= 0");
+  return fail(h, FREDOPT_ERR_NONFINITE, "w0 not finite");
 }
 
 // Where a kernel writes a spot vector for the caller: the caller's device array
@@ -1367,17 +1408,7 @@ int fredopt_begin(fredopt_t h, const float* w0, double alpha, double relaxation,
   cudaStream_t s = h->stream;
   join_in(h);
   double nrm = 0.0;
-  if (dev_ptr(flags)) {  // through the staging area, in order: the same sum as for a host array
-    const int32_t m = 2 * kStageDoubles;
-    for (int32_t j = 0; j < h->n; j += m) {
-      const int32_t k = std::min(m, h->n - j);
-      CK(cudaMemcpyAsync(stage(h), w0 + j, k * sizeof(float), cudaMemcpyDeviceToHost, s));
-      CK(cudaStreamSynchronize(s));
-      if ((rc = check_spots(h, reinterpret_cast<const float*>(stage(h)), k, &nrm))) return rc;
-    }
-  } else if ((rc = check_spots(h, w0, h->n, &nrm))) {
-    return rc;
-  }
+  if ((rc = check_spots(h, w0, flags, &nrm))) return rc;
   free_graph(h);
   if (p.sweep_blocks > 0) {
     rc = build_sweep(h, p.sweep_blocks);

@@ -247,6 +247,9 @@ void launch_row_objective(const Geometry& g, const Tables& t, const float2* yw, 
 void launch_final_check(int grid, const Tables& t, const double2* y64, const uint32_t* mask,
                         const double* dd, const double* ll, const double* dl, const int64_t* rows, int64_t n_list,
                         double* part, cudaStream_t s);
+constexpr int kSpotSlices = 32;
+constexpr unsigned long long kNoSpot = 1ull << 40;
+void launch_check_spots(const float* x, int32_t n, double* part, cudaStream_t s);  // part: 2 kSpotSlices values
 // out[b] = sum of slice b of part[0 .. n), kFinishBlocks slices
 void launch_sum_slices(const double* part, int n, double* out, cudaStream_t s);
 

@@ -1212,6 +1212,31 @@ __global__ void __launch_bounds__(kRowThreads) k_final_check(Tables t, const dou
   }
 }
 
+// Slice b of x (kSpotSlices slices): part[2 b] the sum of its squares, in the order
+// that the host takes too (fredopt_api.cu, slice_squares); part[2 b + 1] twice the
+// index of its first element that is not finite, or one more than that of its first
+// negative one, whichever comes first; kNoSpot without either.
+__global__ void __launch_bounds__(256) k_check_spots(const float* __restrict__ x, int32_t n, double* part) {
+  __shared__ double red[9];
+  __shared__ unsigned long long first;
+  if (threadIdx.x == 0) first = kNoSpot;
+  __syncthreads();
+  const int per = (n + kSpotSlices - 1) / kSpotSlices;
+  const int j0 = min((int64_t)n, (int64_t)blockIdx.x * per), j1 = min((int64_t)n, (int64_t)j0 + per);
+  double sum = 0.0;
+  for (int j = j0 + threadIdx.x; j < j1; j += 256) {
+    const float v = x[j];
+    if (!isfinite(v)) atomicMin(&first, 2ull * j);
+    else if (v < 0.0f) atomicMin(&first, 2ull * j + 1ull);
+    sum += (double)v * (double)v;
+  }
+  sum = block_sum256(sum, red);  // (its barriers order `first` too)
+  if (threadIdx.x == 0) {
+    part[2 * blockIdx.x] = sum;
+    part[2 * blockIdx.x + 1] = (double)first;
+  }
+}
+
 __global__ void __launch_bounds__(256) k_sum_slices(const double* __restrict__ part, int n, double* out) {
   __shared__ double red[9];
   const int per = (n + (int)gridDim.x - 1) / (int)gridDim.x;
@@ -1422,6 +1447,10 @@ void launch_final_check(int grid, const Tables& t, const double2* y64, const uin
                         const double* dd, const double* ll, const double* dl, const int64_t* rows, int64_t n_list,
                         double* part, cudaStream_t s) {
   k_final_check<<<grid, kRowThreads, 0, s>>>(t, y64, mask, dd, ll, dl, rows, n_list, part);
+}
+
+void launch_check_spots(const float* x, int32_t n, double* part, cudaStream_t s) {
+  k_check_spots<<<kSpotSlices, 256, 0, s>>>(x, n, part);
 }
 
 void launch_sum_slices(const double* part, int n, double* out, cudaStream_t s) {

@@ -152,6 +152,9 @@ void launch_row_objective(const Geometry&, const Tables&, const float2*, const u
                           int64_t, float2*, double*, cudaStream_t) {}
 void launch_final_check(int, const Tables&, const double2*, const uint32_t*, const double*, const double*,
                         const double*, const int64_t*, int64_t, double*, cudaStream_t) {}
+void launch_check_spots(const float*, int32_t, double* part, cudaStream_t) {
+  for (int b = 0; b < kSpotSlices; ++b) part[2 * b + 1] = (double)kNoSpot;
+}
 void launch_sum_slices(const double*, int, double*, cudaStream_t) {}
 size_t row_order_scratch(int64_t n) { return (size_t)n / 256 + 8; }
 void launch_rows_count(const int64_t* rp, const uint32_t* mask, int64_t n, int64_t nnz, bool, int64_t*, RowTotals* t,
