@@ -659,8 +659,9 @@ __global__ void __launch_bounds__(kFillThreads) k_csc_fill(
 //   2  it goes to output cursor[c] + (its bits below its own): row order;
 //   3  the first entry of a column advances the cursor and clears the slot.
 // Entries of a tile rarely share a column, so every entry is a store of its own in
-// each of the three arrays, which binds it: 12 to 15 ms per 1e8 entries whatever
-// the shape.  Loads in ms, k_csc_fill (groups of 1024) -> k_csc_scatter, by mean
+// each of the three arrays (4 sectors written per entry, most of them leaving L2 half
+// empty; half of the stall cycles wait for the cursors): 12 to 15 ms per 1e8 entries
+// whatever the shape.  Loads in ms, k_csc_fill (groups of 1024) -> k_csc_scatter, by mean
 // entries per row and group:
 //   9e-4 (9 per row, 3e6 columns, 1.8e7 entries)  184.8 -> 13.8   1.3   45.6 -> 27.7
 //   0.1 (98, 1e6, 3.9e7)                          103.8 -> 11.9   2.5   23.8 -> 23.7
