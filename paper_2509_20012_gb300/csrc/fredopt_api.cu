@@ -69,6 +69,8 @@ struct Sweep {
   int warps = 0;                   // > 0: the streaming forward product takes the blocks' rows,
   DBuf<int64_t> tiles;             // in this many tiles per block
   DBuf<int64_t> pos, bounds;
+  DBuf<double> lens;               // scratch of the build
+  double own_entries = 0.0;        // entries of a block in the column that an entry lies in, on average
   DBuf<double> w, wpart;           // [nb] 1 / priority sum; its slices' sums
   DBuf<double> part;               // violated rows' partial priority sums of a block
 };
@@ -466,13 +468,24 @@ void sweep_weights(fredopt_t h) {
                        h->mdl.p, h->sw->wpart.p, h->sw->w.p, h->stream);
 }
 
-// Rows of a sweep's blocks by the streaming forward product, when the list of
-// structure rows is the device rows in order (FREDOPT_ROWS_ROI), from this many
-// nonzeros per block on: it keeps more entries in flight, but stages all of x
-// per block.  Rows of one sweep, in us, k_sweep_rows -> streaming:
-//   FP32    4.6e7 per block 116 -> 101   1.5e7 134 -> 130   1.0e7 230 -> 211   5.0e6 307 -> 312   2.9e6 255 -> 483
-//   16-bit  8.0e7 per block 155 ->  79   1.0e7 226 -> 161   5.0e6 287 -> 253   1.2e6 606 -> 929
-int64_t sweep_stream_nnz(fredopt_t h) { return h->fmt == FREDOPT_FP32 ? 10000000 : 4000000; }
+// Whether the streaming forward product takes the rows of a sweep's nb blocks, with
+// the rows between them.  k_sweep_rows takes the structure rows alone, a few entries
+// per lane in flight, and a warp at least per row; the other keeps more in flight,
+// but stages all of x per block, leaves its successor no room to start early, and
+// streams a row with one warp.  Estimates in us per block, fitted to the times of
+// whole sweeps, k_sweep_rows / streaming:
+//   5.7e7 nonzeros, 23 thousand rows, FP32    1 block 285 / 277    2 318 / 330    3 338 / 356
+//   8.0e7, 79 thousand rows                   FP32: 1 374 / 347, 4 493 / 487, 8 570 / 607;  BF16: 350 / 284, 474 / 423, 547 / 544
+//   2.6e7, 2.8e6 rows, FP32                   1 1894 / 1298    16 2022 / 1448    32 2116 / 1988    100 2789 / 5314
+//   7.5e7, 3765 rows, FP32                    1 373 / 358    2 457 / 465    4 607 / 725
+//   4.2e7 of 7.7e7 in structure rows, FP32    1 283 / 320
+bool sweep_streams(fredopt_t h, int nb) {
+  const bool fp32 = h->fmt == FREDOPT_FP32;
+  const double rows = ((double)h->con_nnz / 5.4e5 + (double)h->n_con_ne * 0.28e-3) / nb;
+  const double all = ((double)h->nnz_hot + 64.0 * (double)h->n_hot_ne) / (fp32 ? 7.0e5 : 1.2e6) / nb;
+  const double row = (double)h->con_nnz / (double)h->n_con_ne / (fp32 ? 250.0 : 400.0);
+  return 15.0 + std::max(all, row) < rows;
+}
 
 // Blocks of the block-iterative sweep: the streamed rows with nonzeros that
 // lie in some structure, in device (= ascending voxel) order, cut into groups
@@ -500,9 +513,8 @@ int build_sweep(fredopt_t h, int m) {
   }
   bnd.push_back(C.empty() ? 0 : C.back() + 1);
   h->sw->warps = 0;
-  if (!C.empty() && C.back() + 1 == (int64_t)C.size() &&
-      h->con_nnz >= sweep_stream_nnz(h) * h->sw->nb) {
-    const int W = (int)std::min<int64_t>(h->geo.fwd_warps, h->sw->size);
+  if (!C.empty() && sweep_streams(h, h->sw->nb)) {
+    const int W = h->geo_full.fwd_warps;
     CK(h->sw->tiles.alloc(2 * (size_t)W * h->sw->nb));
     for (int t = 0; t < h->sw->nb; ++t)
       launch_tiles(TileArgs{TileArgs::PAIRS, h->rp.p, bnd[t], bnd[t + 1], 0, 0, W, 0, h->row_cost,
@@ -518,8 +530,22 @@ int build_sweep(fredopt_t h, int m) {
   CK(h->sw->part.alloc((size_t)((h->sw->size + kSweepConThreads - 1) / kSweepConThreads)));
   CK(h->xs.ensure(h->n_pad));
   CK(cudaMemsetAsync(h->xs.p, 0, h->n_pad * sizeof(float), s));
-  CK(h->ys.ensure(h->n_con_ne));
+  CK(h->ys.ensure(h->n_hot));
   sweep_weights(h);
+  h->sw->own_entries = 0.0;
+  if (h->sw->nb > 0) {
+    CK(h->sw->lens.alloc(2 * (size_t)h->sw->nb));
+    launch_sweep_lengths(h->sw->pos.p, h->n, h->sw->nb, h->sw->lens.p, s);
+    std::vector<double> len(2 * (size_t)h->sw->nb);
+    CK(cudaMemcpyAsync(len.data(), h->sw->lens.p, len.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    double s1 = 0.0, s2 = 0.0;
+    for (int t = 0; t < h->sw->nb; ++t) {
+      s1 += len[2 * t];
+      s2 += len[2 * t + 1];
+    }
+    h->sw->own_entries = s1 > 0.0 ? s2 / s1 : 0.0;
+  }
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   h->sw->m = m;
@@ -577,12 +603,12 @@ void enqueue_sweep(fredopt_t h, const float* w, int use_coef, double lam, double
       fa.sched = nullptr;
       fa.x = h->xs.p;
       fa.y = h->ys.p;
-      run(h, 0, [&] { launch_forward(h->geo, h->fmt, EPI_STORE, h->hint_fwd, fa, h->tab, s); });
+      run(h, 0, [&] { launch_forward(h->geo_full, h->fmt, EPI_STORE, h->hint_fwd, fa, h->tab, s); });
     } else {
       run(h, 0, [&] { launch_sweep_rows(h->fmt, row_nnz, a, s); });
     }
     run(h, 2, [&] { launch_sweep_con(h->tab, a, s); });
-    run(h, 1, [&] { launch_sweep_cols(h->fmt, col_nnz, a, s); });
+    run(h, 1, [&] { launch_sweep_cols(h->fmt, col_nnz, h->sw->own_entries, a, s); });
   }
   run(h, 3, [&] { launch_sweep_finish(h->geo, h->n, h->xs.p, out, in_solve, h->st.p, h->log.p, s); });
 }

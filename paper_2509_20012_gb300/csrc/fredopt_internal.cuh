@@ -365,7 +365,7 @@ struct SweepArgs {
   const double* dd;
   const double* ll;
   const double* dl;
-  float2* y;               // (Dx, Lx) per list entry
+  float2* y;               // (Dx, Lx) per streamed row
   float2* gam;             // per streamed row (scaled like the transposed product's coefficients)
   double* part;            // [con_blocks] priority sums of the violated rows
   int con_blocks;
@@ -399,8 +399,11 @@ void launch_sweep_weights(const Tables& t, const int64_t* list, int64_t n_list, 
 // forward product of the block's rows; warps per row by the mean row length
 void launch_sweep_rows(int fmt, double mean_nnz, const SweepArgs& a, cudaStream_t s);
 void launch_sweep_con(const Tables& t, const SweepArgs& a, cudaStream_t s);
-// lanes per column by the mean entries of a column in the block
-void launch_sweep_cols(int fmt, double mean_entries, const SweepArgs& a, cudaStream_t s);
+// out: 2 values per block
+void launch_sweep_lengths(const int64_t* pos, int32_t n, int n_blk, double* out, cudaStream_t s);
+// lanes per column by the mean entries of a column in the block, entries in flight
+// by those of the column that an entry lies in, on average
+void launch_sweep_cols(int fmt, double mean_entries, double own_entries, const SweepArgs& a, cudaStream_t s);
 void launch_sweep_finish(const Geometry& g, int n, const float* x, float* out, int in_solve, DevState* st,
                          LogEntry* log, cudaStream_t s);
 // Based 16-bit CSC row indices over n_blk blocks of 128 elements (pass 1:

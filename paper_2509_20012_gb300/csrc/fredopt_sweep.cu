@@ -2,7 +2,7 @@
 // Per block of structure rows, three kernels chained by programmatic dependent
 // launch:
 //   k_sweep_rows  forward product of the block's rows, several warps per row
-//                 (long blocks of consecutive rows: k_forward)
+//                 (blocks of many nonzeros or many short rows: k_forward)
 //   k_sweep_con   half-space evaluation, one row per thread
 //   k_sweep_cols  x_j += scale * sum over the block's entries of column j
 // A block of the clinical plan holds a few hundred rows (9 MB of matrix), so a
@@ -53,6 +53,25 @@ __global__ void k_sweep_pos(const int64_t* __restrict__ cp, const int32_t* __res
       else hi = mid;
     }
     pos[idx] = lo;
+  }
+}
+
+// Per block, over its columns: out[2 t] = entries, out[2 t + 1] = sum of their squares
+// (their ratio is the length of the column that an entry lies in, on average).
+__global__ void __launch_bounds__(256) k_sweep_lengths(const int64_t* __restrict__ pos, int32_t n, double* out) {
+  __shared__ double red[9];
+  const int64_t* p = pos + (int64_t)blockIdx.x * n;
+  double s1 = 0.0, s2 = 0.0;
+  for (int j = threadIdx.x; j < n; j += 256) {
+    const double l = (double)(p[n + j] - p[j]);
+    s1 += l;
+    s2 += l * l;
+  }
+  s1 = block_sum256(s1, red);
+  s2 = block_sum256(s2, red);
+  if (threadIdx.x == 0) {
+    out[2 * blockIdx.x] = s1;
+    out[2 * blockIdx.x + 1] = s2;
   }
 }
 
@@ -146,7 +165,7 @@ __global__ void __launch_bounds__(256) k_sweep_rows(SweepArgs a) {
       }
     }
     // row scales are powers of two: the FP32 product is exact
-    a.y[i] = a.sD ? make_float2(sA * a.sD[r], sB * a.sL[r]) : make_float2(sA, sB);
+    a.y[r] = a.sD ? make_float2(sA * a.sD[r], sB * a.sL[r]) : make_float2(sA, sB);
   }
 }
 
@@ -164,7 +183,7 @@ __global__ void __launch_bounds__(kSweepConThreads) k_sweep_con(SweepArgs a, Tab
   const uint32_t todo = row_constraints(con, t.n_con, m);
   pdl_wait();  // y of this block
   pdl_release();
-  const float2 y = have ? a.y[i] : make_float2(0.0f, 0.0f);
+  const float2 y = have ? a.y[r] : make_float2(0.0f, 0.0f);
   double gD = 0.0, gL = 0.0, psum = 0.0, preach = 0.0, mx = 0.0;
   unsigned nv = 0u;
   eval_constraints(con, todo, t.c, y.x, y.y, dd, ll, dl, gD, gL, psum, preach, nv, mx);
@@ -336,19 +355,20 @@ void rows_inst(double mean_nnz, const SweepArgs& a, cudaStream_t s) {
 }
 
 template <typename VT>
-void cols_inst(double mean_entries, const SweepArgs& a, cudaStream_t s) {
+void cols_inst(double mean_entries, double own_entries, const SweepArgs& a, cudaStream_t s) {
   auto go = [&](auto kernel, int cols) {
     launch_chain(true, kernel, (unsigned)(((int64_t)a.n + cols - 1) / cols), 256, 0, s, a);
   };
   // The update of one sweep, in us, two columns and one entry each in flight per
-  // lane -> one column and four entries, by mean entries per column and block:
-  //   24 (64 blocks of the clinical plan)   994 -> 1144    42   1400 -> 1240
-  //   96                                    491 ->  394   380   3660 -> 2420
-  //   1500 (one block)                      236 ->  140
-  // Plans of few columns leave the second a last wave that is nearly empty (6480
-  // columns: an iteration of 64 blocks, 72 entries, 562 -> 621 us; of 16 blocks,
-  // 290 entries, 224 and 224; of 4 blocks, 1160 entries, 163 -> 132).
-  if (mean_entries > 512.0 || (mean_entries > 32.0 && a.n >= 16384)) go(k_sweep_cols<VT, 32, 1, 4, 4>, 8);
+  // lane -> one column and four entries, by the entries of the column that an entry
+  // lies in (a block's columns are uneven):
+  //   30000 columns   161  993 -> 1136   318  602 -> 635   478  498 ->  399   865  803 -> 494   2028 3674 -> 2422
+  //   70000           107  290 ->  351   425  228 -> 223        50000   333  269 ->  316   666  228 -> 229
+  //   2000            142 1153 ->  854   440  662 -> 373   879  533 ->  260
+  // Few columns are few warps either way; short ones share the GPU worse then (six
+  // plans of 640 to 6480 columns in a batch: 77 to 185 entries 375 -> 400 us per
+  // iteration, 224 to 575 290 -> 274).
+  if (own_entries > (a.n < 8192 ? 200.0 : 400.0)) go(k_sweep_cols<VT, 32, 1, 4, 4>, 8);
   else if (mean_entries > 12.0) go(k_sweep_cols<VT, 32, kColsU, 1, 8>, 8 * kColsU);
   else go(k_sweep_cols<VT, 8, kColsU, 1, 8>, 8 * kColsU * 4);
 }
@@ -397,10 +417,14 @@ void launch_sweep_con(const Tables& t, const SweepArgs& a, cudaStream_t s) {
   launch_chain(true, k_sweep_con, (unsigned)a.con_blocks, kSweepConThreads, 0, s, a, t);
 }
 
-void launch_sweep_cols(int fmt, double mean_entries, const SweepArgs& a, cudaStream_t s) {
-  if (fmt == 1) cols_inst<__nv_bfloat16>(mean_entries, a, s);
-  else if (fmt == 2) cols_inst<__half>(mean_entries, a, s);
-  else cols_inst<float>(mean_entries, a, s);
+void launch_sweep_lengths(const int64_t* pos, int32_t n, int n_blk, double* out, cudaStream_t s) {
+  if (n_blk > 0) k_sweep_lengths<<<n_blk, 256, 0, s>>>(pos, n, out);
+}
+
+void launch_sweep_cols(int fmt, double mean_entries, double own_entries, const SweepArgs& a, cudaStream_t s) {
+  if (fmt == 1) cols_inst<__nv_bfloat16>(mean_entries, own_entries, a, s);
+  else if (fmt == 2) cols_inst<__half>(mean_entries, own_entries, a, s);
+  else cols_inst<float>(mean_entries, own_entries, a, s);
 }
 
 void launch_sweep_finish(const Geometry& g, int n, const float* x, float* out, int in_solve, DevState* st,

@@ -208,7 +208,10 @@ void launch_sweep_rows(int fmt, double, const SweepArgs& a, cudaStream_t) {
   ++g_sweep_blocks;
 }
 void launch_sweep_con(const Tables&, const SweepArgs&, cudaStream_t) {}
-void launch_sweep_cols(int, double, const SweepArgs&, cudaStream_t) {}
+void launch_sweep_lengths(const int64_t*, int32_t, int n, double* out, cudaStream_t) {
+  std::memset(out, 0, 2 * n * sizeof(double));
+}
+void launch_sweep_cols(int, double, double, const SweepArgs&, cudaStream_t) {}
 void launch_sweep_finish(const Geometry&, int, const float*, float*, int, DevState*, LogEntry*, cudaStream_t) {}
 size_t vol_hist_smem(const VolArgs&) { return 0; }
 void launch_vol_hist(const Geometry&, const VolArgs&, cudaStream_t) {}
