@@ -883,8 +883,9 @@ int ready_y64(fredopt_t h) {
 }
 
 // Double-float pass for w (host or device per flags; null = the current
-// iterate of a begun solve) into y64, as in fredopt_end: over every row, or
-// over the structure rows alone (one row per tile, claimed in order).
+// iterate of a begun solve) into y64, as in fredopt_end: over every row, or for the
+// structure rows over those alone (one row per tile, claimed in order) where that
+// takes less time.
 int final_pass_y64(fredopt_t h, const float* w, uint32_t flags, bool structures) {
   cudaStream_t s = h->stream;
   const float* x = nullptr;
@@ -902,8 +903,12 @@ int final_pass_y64(fredopt_t h, const float* w, uint32_t flags, bool structures)
   fa.y64 = h->y64.p;
   fa.dose_out = nullptr;
   fa.letd_out = nullptr;
-  if (structures) {
-    if (h->n_con_ne == 0) return FREDOPT_OK;  // every structure value is 0
+  if (structures && h->n_con_ne == 0) return FREDOPT_OK;  // every structure value is 0
+  // (a listed row restarts a warp's load chain: about 2.7 us of its time, in which it
+  // streams 300 nonzeros; a row end in a run of rows costs 64.  3e6 rows of 9, all in
+  // structures: 1.71 -> 0.43 ms; the clinical plan's 23 thousand rows of 6e6 98 us)
+  if (structures && (double)h->con_nnz + 300.0 * (double)h->n_con_ne <
+                        (double)h->nnz + 64.0 * (double)(h->n_hot_ne + h->n_cold_ne)) {
     fa.rows = h->con_rows.p;
     fa.sched = h->fsched.p;
     fa.n_warps = (int32_t)h->n_con_ne;
