@@ -24,8 +24,8 @@ def make(name):
     if name == "long":  # 24 million nonzeros in 17 thousand rows
         n_vox, n = 17003, 2001
         rp, col, D, L = phantom.random_csr(n_vox, n, 0.7, seed=8, empty_rows=21)
-    else:  # 400 thousand rows of at most 6
-        n_vox, n = 400007, 61
+    else:  # 400 thousand rows of at most 6; "wide": the fluence does not fit shared memory
+        n_vox, n = 400007, 61 if name == "short" else 60001
         c = np.sort(rng.integers(0, n, (n_vox, 6)), axis=1)
         keep = np.ones(c.shape, bool)
         keep[:, 1:] = c[:, 1:] != c[:, :-1]
@@ -46,12 +46,12 @@ def make(name):
 
 @pytest.fixture(scope="module")
 def plans():
-    return {name: make(name) for name in ("long", "short")}
+    return {name: make(name) for name in ("long", "short", "wide")}
 
 
 @pytest.mark.parametrize("name,fmt,n_blocks", [("long", "fp32", 1), ("long", "fp32", 2), ("long", "bf16", 1),
                                                ("long", "fp16", 5), ("short", "fp32", 1), ("short", "fp32", 3),
-                                               ("short", "bf16", 2), ("short", "fp32", 40)])
+                                               ("short", "bf16", 2), ("short", "fp32", 40), ("wide", "fp32", 2)])
 @pytest.mark.parametrize("norm", ["all", "violated"])
 def test_streamed_blocks(lib, plans, name, fmt, n_blocks, norm):
     rp, col, D, L, mask, n, x, cons = plans[name]
